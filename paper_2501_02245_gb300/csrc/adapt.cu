@@ -253,9 +253,9 @@ static bool ensure_dvm_capacity(gsis_ctx* c, long long Nd) {
     dev_free(c, c->recNew.scal); dev_free(c, c->recNew.tab); dev_free(c, c->enter_of);
     dev_free(c, c->SoVf); dev_free(c, c->itauf); dev_free(c, c->rho_wf);
     dev_free(c, c->sd_int); dev_free(c, c->sd_val);
-    dev_free(c, c->gx4); dev_free(c, c->gx1); dev_free(c, c->gy4); dev_free(c, c->gy1);
+    dev_free(c, c->gx4); dev_free(c, c->gy4);
     c->sd_int = nullptr; c->sd_val = nullptr;
-    c->gx4 = c->gx1 = c->gy4 = c->gy1 = nullptr;
+    c->gx4 = c->gy4 = nullptr;
     dev_free(c, c->recG.tabf); dev_free(c, c->recG.scalf); dev_free(c, c->recHalf.tabf);
     dev_free(c, c->recHalf.scalf); dev_free(c, c->recNew.tabf); dev_free(c, c->recNew.scalf);
     c->SoVf = nullptr; c->itauf = nullptr; c->rho_wf = nullptr;
@@ -283,10 +283,8 @@ static bool ensure_dvm_capacity(gsis_ctx* c, long long Nd) {
         c->sd_int = (int*)dev_alloc(c, cap * SD_INTS * sizeof(int));
         c->sd_val = dev_alloc(c, cap * SD_VALS * tb);
         c->gx4 = dev_alloc(c, cap * c->vg.nx * 4 * tb);
-        c->gx1 = dev_alloc(c, cap * c->vg.nx * tb);
         c->gy4 = dev_alloc(c, cap * nyz * 4 * tb);
-        c->gy1 = dev_alloc(c, cap * nyz * tb);
-        if (!c->sd_int || !c->sd_val || !c->gx4 || !c->gx1 || !c->gy4 || !c->gy1) return false;
+        if (!c->sd_int || !c->sd_val || !c->gx4 || !c->gy4) return false;
     }
     if (c->p.vdf_dtype != GSIS_F64) {
         c->SoVf = (float*)dev_alloc(c, cap * 18 * sizeof(float));

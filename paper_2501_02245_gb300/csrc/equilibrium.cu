@@ -310,13 +310,13 @@ __global__ void k_cell_eq(int Nd, const int* __restrict__ dvm_cell, const double
 // block per DVM cell, from the cell's record (Eq. updatef's corrected
 // Maxwellian tables) and 1/tau; formed in FP64 and stored in the sweep's
 // arithmetic type T:
-//   x(ix) = (E, E (B + R C2), E R, E C2 ; E C)             [gx4 ; gx1]
-//   y(q)  = E_yz/tau (D + R_yz C2_yz, 1, C2_yz, R_yz ; A)   [gy4 ; gy1]
-// so that g~/tau = sum of the five products x_i y_i.
+//   x(ix) = (E, E (B + R C2), E R, E C2)             [gx4]
+//   y(q)  = E_yz/tau (D + R_yz C2_yz, 1, C2_yz, R_yz)   [gy4]
+// so that g~/tau = sum of the four products x_i y_i (the Shakhov record has no
+// stress terms, see eval_g).
 template <typename T>
 __global__ void k_build_gtab(int Nd, Records rec, VGridDev vg, const double* __restrict__ itau,
-                             const float* __restrict__ itauf, T* __restrict__ gx4, T* __restrict__ gx1,
-                             T* __restrict__ gy4, T* __restrict__ gy1) {
+                             const float* __restrict__ itauf, T* __restrict__ gx4, T* __restrict__ gy4) {
     const int k = blockIdx.x;
     if (k >= Nd) return;
     const int NT = vg.NT, nx = vg.nx, ny = vg.ny, nyz = vg.ny * vg.nz;
@@ -328,55 +328,47 @@ __global__ void k_build_gtab(int Nd, Records rec, VGridDev vg, const double* __r
         // pipe (the bound of the FP64 form) is left alone.
         const float* tf = rec.tabf + (long long)k * NTAB * NT;
         const float* sf = rec.scalf + (long long)k * RS;
-        const float p0 = sf[RS_P0], pxy = sf[RS_P2XY], pxz = sf[RS_P2XZ], pyz = sf[RS_P2YZ];
+        const float p0 = sf[RS_P0];
         const float it = itauf[k];
         for (int ix = threadIdx.x; ix < nx; ix += blockDim.x) {
-            const float E = tf[ix], B = tf[NT + ix], C = tf[2 * NT + ix], C2 = tf[3 * NT + ix], R = tf[4 * NT + ix];
+            const float E = tf[ix], B = tf[NT + ix], C2 = tf[3 * NT + ix], R = tf[4 * NT + ix];
             *reinterpret_cast<float4*>(gx4 + ((long long)k * nx + ix) * 4) =
                 make_float4(E, E * (B + R * C2), E * R, E * C2);
-            gx1[(long long)k * nx + ix] = E * C;
         }
         for (int q = threadIdx.x; q < nyz; q += blockDim.x) {
             const int iz = q / ny, jy = nx + q - iz * ny, jz = nx + ny + iz;
-            const float Cy = tf[2 * NT + jy], Cz = tf[2 * NT + jz];
             const float Eyz = tf[jy] * tf[jz] * it;
-            const float D = p0 + (tf[NT + jy] + tf[NT + jz]) + 2.0f * pyz * Cy * Cz;
+            const float D = p0 + (tf[NT + jy] + tf[NT + jz]);
             const float Ryz = tf[4 * NT + jy] + tf[4 * NT + jz];
             const float C2yz = tf[3 * NT + jy] + tf[3 * NT + jz];
-            const float A = 2.0f * (pxy * Cy + pxz * Cz);
             *reinterpret_cast<float4*>(gy4 + ((long long)k * nyz + q) * 4) =
                 make_float4(Eyz * (D + Ryz * C2yz), Eyz, Eyz * C2yz, Eyz * Ryz);
-            gy1[(long long)k * nyz + q] = Eyz * A;
         }
         return;
     }
     const double* tab = rec.tab + (long long)k * NTAB * NT;
     const double* sc = rec.scal + (long long)k * RS;
-    const double p0 = sc[RS_P0], pxy = sc[RS_P2XY], pxz = sc[RS_P2XZ], pyz = sc[RS_P2YZ];
+    const double p0 = sc[RS_P0];
     const double it = itau[k];
     for (int ix = threadIdx.x; ix < nx; ix += blockDim.x) {
-        const double E = tab[ix], B = tab[NT + ix], C = tab[2 * NT + ix], C2 = tab[3 * NT + ix], R = tab[4 * NT + ix];
+        const double E = tab[ix], B = tab[NT + ix], C2 = tab[3 * NT + ix], R = tab[4 * NT + ix];
         T* o = gx4 + ((long long)k * nx + ix) * 4;
         o[0] = (T)E;
         o[1] = (T)(E * (B + R * C2));
         o[2] = (T)(E * R);
         o[3] = (T)(E * C2);
-        gx1[(long long)k * nx + ix] = (T)(E * C);
     }
     for (int q = threadIdx.x; q < nyz; q += blockDim.x) {
         const int jy = nx + q % ny, jz = nx + ny + q / ny;
-        const double Cy = tab[2 * NT + jy], Cz = tab[2 * NT + jz];
         const double Eyz = tab[jy] * tab[jz] * it * vg.vscale;   // g~/tau in stored units
-        const double D = p0 + (tab[NT + jy] + tab[NT + jz]) + 2.0 * pyz * Cy * Cz;
+        const double D = p0 + (tab[NT + jy] + tab[NT + jz]);
         const double Ryz = tab[4 * NT + jy] + tab[4 * NT + jz];
         const double C2yz = tab[3 * NT + jy] + tab[3 * NT + jz];
-        const double A = 2.0 * (pxy * Cy + pxz * Cz);
         T* o = gy4 + ((long long)k * nyz + q) * 4;
         o[0] = (T)(Eyz * (D + Ryz * C2yz));
         o[1] = (T)Eyz;
         o[2] = (T)(Eyz * C2yz);
         o[3] = (T)(Eyz * Ryz);
-        gy1[(long long)k * nyz + q] = (T)(Eyz * A);
     }
 }
 
@@ -390,10 +382,10 @@ void launch_cell_eq(gsis_ctx* c) {
     launch_build_records(c, c->recG, Nd, c->specs);
     if (c->p.vdf_dtype == GSIS_F64)
         k_build_gtab<double><<<Nd, 128, 0, c->stream>>>(Nd, c->recG, c->vg, c->itau, c->itauf, (double*)c->gx4,
-                                                        (double*)c->gx1, (double*)c->gy4, (double*)c->gy1);
+                                                        (double*)c->gy4);
     else
         k_build_gtab<float><<<Nd, 128, 0, c->stream>>>(Nd, c->recG, c->vg, c->itau, c->itauf, (float*)c->gx4,
-                                                       (float*)c->gx1, (float*)c->gy4, (float*)c->gy1);
+                                                       (float*)c->gy4);
     c->launches++;
 }
 

@@ -85,27 +85,48 @@ template <> __device__ __forceinline__ void ld16<float, __half>(const __half* p,
 }
 
 // ---------------------------------------------------------------- small math
-// minmod(a, b): 0 unless a and b share a sign, else the one nearer zero.
-template <typename T>
-__device__ __forceinline__ T minmod_t(T a, T b) {
-    const T m = fabs(a) < fabs(b) ? a : b;
-    return a * b > T(0) ? m : T(0);
-}
-
 // Half the minmod, 0.5 minmod(a, b).  FP64: decisions on the bit patterns and the halving as a decrement of the exponent field, all on the
 // integer pipe (GB300 issues FP64 at 1/64 of the FP32 rate).  Magnitudes of
 // IEEE doubles order like their bit patterns with the sign bit cleared, and
-// +-0 never shares a sign, so the result equals 0.5 minmod_t(a, b) for every
+// +-0 never shares a sign, so the result equals 0.5 minmod(a, b) for every
 // result of magnitude >= 2^-1021; a smaller one (300 orders of magnitude
 // below any value of the scheme) gives 0.
 template <typename T> __device__ __forceinline__ T hmm_t(T a, T b);
-template <> __device__ __forceinline__ float hmm_t<float>(float a, float b) { return 0.5f * minmod_t<float>(a, b); }
+
+// minmod for the sweeps.  FP32: min.xorsign.abs gives the smaller magnitude
+// with the product's sign, so a positive result means equal signs; max with 0
+// and a's sign finish it: three instructions for the compare-and-select
+// form's five, and no product that could underflow in the Maxwellian tails.  (A
+// NaN on either side gives a zero slope, as the comparisons did.)
+template <typename T> __device__ __forceinline__ T mm_t(T a, T b);
+template <> __device__ __forceinline__ float mm_t<float>(float a, float b) {
+    float x;
+    asm("min.NaN.xorsign.abs.f32 %0, %1, %2;" : "=f"(x) : "f"(a), "f"(b));
+    return __uint_as_float(__float_as_uint(fmaxf(x, 0.0f)) | (__float_as_uint(a) & 0x80000000u));
+}
+// FP64: on the bit patterns (see hmm_t below).  The sign bit is cleared by an
+// explicit 32-bit AND: written as a 64-bit mask, the compiler makes it an
+// absolute value, which is an FP64-pipe operation (two per limiter, a quarter
+// of the FP64 sweep's whole count).
+__device__ __forceinline__ unsigned long long mag_bits(double a) {
+    unsigned long long r;
+    asm("{\n\t.reg .b32 lo, hi;\n\tmov.b64 {lo, hi}, %1;\n\tand.b32 hi, hi, 0x7fffffff;\n\tmov.b64 %0, {lo, hi};\n\t}"
+        : "=l"(r) : "d"(a));
+    return r;
+}
+template <> __device__ __forceinline__ double mm_t<double>(double a, double b) {
+    const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
+    const bool a_smaller = mag_bits(a) < mag_bits(b);
+    return (ia ^ ib) >= 0 ? __longlong_as_double(a_smaller ? ia : ib) : 0.0;
+}
+template <> __device__ __forceinline__ float hmm_t<float>(float a, float b) { return 0.5f * mm_t<float>(a, b); }
 template <> __device__ __forceinline__ double hmm_t<double>(double a, double b) {
     const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
-    const long long ma = ia & 0x7fffffffffffffffLL, mb = ib & 0x7fffffffffffffffLL;
+    const unsigned long long ma = mag_bits(a), mb = mag_bits(b);
     const bool a_smaller = ma < mb;
-    const long long m = a_smaller ? ia : ib, mm = a_smaller ? ma : mb;
-    const bool ok = (ia ^ ib) >= 0 && mm >= (2LL << 52);   // same sign, |result| >= 2^-1021 (so nonzero)
+    const long long m = a_smaller ? ia : ib;
+    const unsigned long long mm = a_smaller ? ma : mb;
+    const bool ok = (ia ^ ib) >= 0 && mm >= (2ULL << 52);   // same sign, |result| >= 2^-1021 (so nonzero)
     return ok ? __longlong_as_double(m - (1LL << 52)) : 0.0;
 }
 

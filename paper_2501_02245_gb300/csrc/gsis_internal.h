@@ -205,8 +205,8 @@ struct gsis_ctx {
     float *SoVf = nullptr, *itauf = nullptr, *rho_wf = nullptr;   // FP32 mirrors for the FP32 sweep
     int* sd_int = nullptr;         // [Nd][SD_INTS] packed sweep data per DVM cell (k_sweep_desc)
     void* sd_val = nullptr;        // [Nd][SD_VALS] S/V of the sides, in the sweep's arithmetic type
-    void *gx4 = nullptr, *gx1 = nullptr;   // [Nd][nx] x factor vectors of g~/tau (k_build_gtab)
-    void *gy4 = nullptr, *gy1 = nullptr;   // [Nd][ny*nz] y-z factor vectors
+    void* gx4 = nullptr;           // [Nd][nx] x factor vectors of g~/tau (k_build_gtab)
+    void* gy4 = nullptr;           // [Nd][ny*nz] y-z factor vectors
     void* f = nullptr;
     double *itau = nullptr, *mom = nullptr, *rho_w = nullptr, *wall_den = nullptr;
     double *wall_in = nullptr;     // [N][6][5] incoming half-range moments of the wall Maxwellian
@@ -266,6 +266,8 @@ gsis_status force_sweep_shape(gsis_ctx* c, const char* name);
 struct SweepArgs;
 size_t ring_bytes(gsis_ctx* c, int vt);
 bool launch_sweep_ring(gsis_ctx* c, const SweepArgs& a, int pass, int which);
+// sweep_col.cu (velocity columns, 2D meshes, FP64 storage)
+void launch_sweep_col(gsis_ctx* c, const SweepArgs& a, int pass, int shape);
 // batch.cu (persistent batched sweep; BatchSolve is declared in sweep_device.cuh)
 struct BatchSolve;
 int batch_num_shapes();

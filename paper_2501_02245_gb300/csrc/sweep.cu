@@ -156,13 +156,24 @@ static bool pair_ok(gsis_ctx* c) { return c->vg.nx % 2 == 0 && c->normal_compone
 static const char* kRingNames[] = {"ring_w8_v32", "ring_w4_v32", "ring_w8_v64"};
 constexpr int kRingShapes = 3;
 
+// After those, for FP64 storage: the velocity columns (sweep_col.cu; 2D meshes),
+// planes per column and warps per block.
+static const char* const kColNames[] = {"col_z4_g4", "col_z4_g8", "col_z3_g4", "col_z2_g8"};
+static int col_shapes(int dtype) { return dtype == GSIS_F64 ? (int)(sizeof(kColNames) / sizeof(kColNames[0])) : 0; }
+// FP64 on 2D meshes (the kernels keep a row's bytes in 32 bits)
+static bool col_ok(gsis_ctx* c) {
+    return c->p.vdf_dtype == GSIS_F64 && c->normal_components == 2 && (double)c->vg.Nv * sizeof(double) < 2147483648.0;
+}
+
 static int base_shapes(int dtype) {
     return dtype == GSIS_F64 ? (int)(sizeof(kShapesF64) / sizeof(kShapesF64[0]))
                              : (int)(sizeof(kShapesF32) / sizeof(kShapesF32[0]));
 }
-int sweep_num_shapes(int dtype) { return base_shapes(dtype) + kRingShapes; }
+int sweep_num_shapes(int dtype) { return base_shapes(dtype) + kRingShapes + col_shapes(dtype); }
+static int col_index(int dtype, int shape) { return shape - base_shapes(dtype) - kRingShapes; }
 const char* sweep_shape_name(int dtype, int shape) {
     if (shape < 0 || shape >= sweep_num_shapes(dtype)) return "?";
+    if (shape >= base_shapes(dtype) + kRingShapes) return kColNames[col_index(dtype, shape)];
     if (shape >= base_shapes(dtype)) return kRingNames[shape - base_shapes(dtype)];
     return dtype == GSIS_F64 ? kShapesF64[shape].name : kShapesF32[shape].name;
 }
@@ -199,6 +210,13 @@ static void sweep_f64_shape(gsis_ctx* c, const SweepArgs& a, int pass, int shape
 
 static void launch_sweep_shape(gsis_ctx* c, const SweepArgs& a, int pass, int shape) {
     const int nb = base_shapes(c->p.vdf_dtype);
+    if (shape >= nb + kRingShapes) {
+        if (col_ok(c)) {
+            launch_sweep_col(c, a, pass, col_index(c->p.vdf_dtype, shape));
+            return;
+        }
+        shape = 0;
+    }
     if (shape >= nb) {
         if (launch_sweep_ring(c, a, pass, shape - nb)) return;
         shape = 0;   // does not fit: register-stencil sweep
@@ -226,9 +244,7 @@ SweepArgs sweep_args(gsis_ctx* c) {
     a.recGhost = c->recGhost;
     a.recBC = c->recBC;
     a.gx4 = c->gx4;
-    a.gx1 = c->gx1;
     a.gy4 = c->gy4;
-    a.gy1 = c->gy1;
     a.vg = c->vg;
     return a;
 }
@@ -251,6 +267,21 @@ static std::map<std::string, int>& sweep_cache() {
     return m;
 }
 
+// Shapes the autotuner times: those that win somewhere.  FP64 on 2D meshes:
+// the columns, and the wide single-velocity blocks for small velocity grids
+// (the reduced distributions' 144 tiles: g16_v1_c1 7.5 ms, best column 11.6);
+// FP32 arithmetic: the velocity pairs and the widest single-velocity tile, the
+// single-velocity tiles where pairs cannot run.  The shared-memory windows and
+// the remaining tiles measured slower everywhere (cylinder FP64 120 ms against
+// 51.6, FP32 37 against 6.9) and run only when forced.
+static bool tune_candidate(gsis_ctx* c, int shape) {
+    const int nb = base_shapes(c->p.vdf_dtype);
+    if (shape >= nb + kRingShapes) return col_ok(c);
+    if (shape >= nb) return false;
+    if (c->p.vdf_dtype == GSIS_F64) return col_ok(c) ? shape >= 4 : true;
+    return pair_ok(c) ? (shape == 3 || pair_shape(c->p.vdf_dtype, shape)) : shape < 4;
+}
+
 // Fix the sweep tile shape by name (a test hook: every shape must give the
 // same result); GSIS_ERR_ARG if the name is unknown or the shape cannot run
 // this problem.
@@ -258,7 +289,10 @@ gsis_status force_sweep_shape(gsis_ctx* c, const char* name) {
     const int ns = sweep_num_shapes(c->p.vdf_dtype), nb = base_shapes(c->p.vdf_dtype);
     for (int sh = 0; sh < ns; ++sh) {
         if (std::string(sweep_shape_name(c->p.vdf_dtype, sh)) != name) continue;
-        if (sh >= nb) {
+        if (sh >= nb + kRingShapes) {
+            if (!col_ok(c))
+                return set_err(c, GSIS_ERR_ARG, std::string("sweep tile ") + name + " needs FP64 storage and a 2D mesh");
+        } else if (sh >= nb) {
             const int which = sh - nb;
             if (ring_bytes(c, which == 2 ? 64 : 32) == 0 || (c->p.vdf_dtype == GSIS_F64 && which == 2))
                 return set_err(c, GSIS_ERR_ARG, std::string("sweep tile ") + name + " does not fit this problem");
@@ -302,14 +336,11 @@ gsis_status tune_sweep(gsis_ctx* c) {
     cudaEventCreate(&e1);
     const SweepArgs a = sweep_args(c);
     const int ns = sweep_num_shapes(c->p.vdf_dtype);
-    int best = 0;
+    int best = 0;   // (always timed or overridden: every problem has candidates)
     float best_ms = 1e30f;
     std::string info = "tile timings (ms per pass pair):";
     for (int sh = 0; sh < ns; ++sh) {
-        const int nb = base_shapes(c->p.vdf_dtype);
-        if (sh >= nb && ring_bytes(c, sh - nb == 2 ? 64 : 32) == 0) continue;   // window does not fit
-        if (pair_shape(c->p.vdf_dtype, sh) && !pair_ok(c)) continue;
-        if (sh >= nb && c->p.vdf_dtype == GSIS_F64 && sh - nb == 2) continue;
+        if (!tune_candidate(c, sh)) continue;
         launch_sweep_shape(c, a, 1, sh);
         launch_sweep_shape(c, a, 0, sh);
         cudaEventRecord(e0, c->stream);

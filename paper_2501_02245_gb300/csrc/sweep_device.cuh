@@ -31,8 +31,8 @@ struct SweepArgs {
     const float* rho_wf;
     Records recGhost, recBC;
     // factor vectors of the reference distribution (k_build_gtab), in the
-    // arithmetic type: gx4/gx1 [Nd][nx] (4-vector, scalar), gy4/gy1 [Nd][ny*nz]
-    const void *gx4, *gx1, *gy4, *gy1;
+    // arithmetic type: gx4 [Nd][nx], gy4 [Nd][ny*nz] (4-vectors)
+    const void *gx4, *gy4;
     VGridDev vg;
 };
 
@@ -42,12 +42,30 @@ template <> __device__ __forceinline__ float neg_if<float>(float x, bool s) {
     return __uint_as_float(__float_as_uint(x) ^ ((unsigned)s << 31));
 }
 template <> __device__ __forceinline__ double neg_if<double>(double x, bool s) {
-    return __longlong_as_double(__double_as_longlong(x) ^ ((long long)s << 63));
+    double r;   // (an explicit 32-bit XOR: the compiler makes a 64-bit one an FP64-pipe negation)
+    asm("{\n\t.reg .b32 lo, hi;\n\tmov.b64 {lo, hi}, %1;\n\txor.b32 hi, hi, %2;\n\tmov.b64 %0, {lo, hi};\n\t}"
+        : "=d"(r) : "d"(x), "r"((unsigned)s << 31));
+    return r;
 }
 // x > 0 (FP64: on the bit pattern, integer pipe).
 template <typename T> __device__ __forceinline__ bool pos_t(T x);
 template <> __device__ __forceinline__ bool pos_t<float>(float x) { return x > 0.0f; }
 template <> __device__ __forceinline__ bool pos_t<double>(double x) { return __double_as_longlong(x) > 0; }
+
+// 1 / d for d in the range of div_t below: its reciprocal (FP64), the hardware
+// reciprocal (FP32, within 1 ulp).
+template <typename T> __device__ __forceinline__ T recip_t(T d);
+template <> __device__ __forceinline__ float recip_t<float>(float d) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return r;
+}
+template <> __device__ __forceinline__ double recip_t<double>(double d) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+    const float rf = recip_t<float>(__uint_as_float((unsigned)(b >> 29) - 0xC0000000u));
+    const double r = __longlong_as_double((long long)(((unsigned long long)__float_as_uint(rf) << 29) + (896ULL << 52)));
+    return r * fma(-d, r, 2.0);
+}
 
 // n / d for d > 0 with d and 1/d within the normal single-precision range
 // (the denominators of the sweep, 1/tau plus outflow terms, are).
@@ -65,14 +83,7 @@ template <> __device__ __forceinline__ bool pos_t<double>(double x) { return __d
 template <typename T> __device__ __forceinline__ T div_t(T n, T d);
 template <> __device__ __forceinline__ float div_t<float>(float n, float d) { return __fdividef(n, d); }
 template <> __device__ __forceinline__ double div_t<double>(double n, double d) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(d);
-    const unsigned fb = (unsigned)(b >> 29) - 0xC0000000u;   // (exponent - 896) << 23 | top 23 fraction bits
-    float rf;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(__uint_as_float(fb)));
-    const unsigned long long rb = ((unsigned long long)__float_as_uint(rf) << 29) + (896ULL << 52);
-    double r = __longlong_as_double((long long)rb);
-    r = r * fma(-d, r, 2.0);
-    return n * r;
+    return n * recip_t<double>(d);
 }
 
 template <typename T>
@@ -91,20 +102,18 @@ __device__ __forceinline__ V4<double> ld4(const double* p) {
 }
 
 // Reference distribution of cell k at velocity (ix, q = iy + ny iz), divided
-// by tau.  The record's E_x E_y E_z (p0 + sum B + sum R sum C2
-// + 2 sum_{i<j} P2_ij C_i C_j), split into its x and y-z parts, is the sum of
-// five products x_i y_i (k_build_gtab):
-//   x = (E_x, E_x (B_x + R_x C2_x), E_x R_x, E_x C2_x, E_x C_x)
-//   y = E_yz/tau (D + R_yz C2_yz, 1, C2_yz, R_yz, A)
-// with E_yz = E_y E_z, D = p0 + B_y + B_z + 2 P2_yz C_y C_z, R_yz = R_y + R_z,
-// C2_yz = C2_y + C2_z and A = 2 (P2_xy C_y + P2_xz C_z).
+// by tau.  The Shakhov record's E_x E_y E_z (p0 + sum B + sum R sum C2) (it
+// has no stress terms, P2 = 0), split into its x and y-z parts, is the sum of
+// four products x_i y_i (k_build_gtab):
+//   x = (E_x, E_x (B_x + R_x C2_x), E_x R_x, E_x C2_x)
+//   y = E_yz/tau (D + R_yz C2_yz, 1, C2_yz, R_yz)
+// with E_yz = E_y E_z, D = p0 + B_y + B_z, R_yz = R_y + R_z and C2_yz = C2_y + C2_z.
 template <typename T>
 __device__ __forceinline__ T eval_g(const SweepArgs& a, int k, int ix, int q) {
     const int kx = k * a.vg.nx + ix, ky = k * (a.vg.ny * a.vg.nz) + q;
     const V4<T> x = ld4(static_cast<const T*>(a.gx4) + 4 * (long long)kx);
     const V4<T> y = ld4(static_cast<const T*>(a.gy4) + 4 * (long long)ky);
-    T g = __ldg(static_cast<const T*>(a.gx1) + kx) * __ldg(static_cast<const T*>(a.gy1) + ky);
-    g = fma(x.x, y.x, g);
+    T g = x.x * y.x;
     g = fma(x.y, y.y, g);
     g = fma(x.z, y.z, g);
     return fma(x.w, y.w, g);

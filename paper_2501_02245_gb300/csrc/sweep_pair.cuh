@@ -99,17 +99,14 @@ __device__ __forceinline__ void make_vel2(const VGridDev& vg, long long vbase, i
     }
 }
 
-// g~ / tau at (ix, q) and (ix + 1, q): the five products of the x and y-z
+// g~ / tau at (ix, q) and (ix + 1, q): the four products of the x and y-z
 // factor vectors (eval_g), the y-z factors shared by the pair.
 __device__ __forceinline__ float2 eval_g2(const SweepArgs& a, int k, int ix, int q) {
     const int kx = k * a.vg.nx + ix, ky = k * (a.vg.ny * a.vg.nz) + q;
     const float* gx4 = static_cast<const float*>(a.gx4) + 4 * (long long)kx;
     const V4<float> xa = ld4(gx4), xb = ld4(gx4 + 4);
     const V4<float> y = ld4(static_cast<const float*>(a.gy4) + 4 * (long long)ky);
-    const float2 x1 = __ldg(reinterpret_cast<const float2*>(static_cast<const float*>(a.gx1) + kx));
-    const float y1 = __ldg(static_cast<const float*>(a.gy1) + ky);
-    float2 g = f2mul(x1, bc2(y1));
-    g = f2fma(make_float2(xa.x, xb.x), bc2(y.x), g);
+    float2 g = f2mul(make_float2(xa.x, xb.x), bc2(y.x));
     g = f2fma(make_float2(xa.y, xb.y), bc2(y.y), g);
     g = f2fma(make_float2(xa.z, xb.z), bc2(y.z), g);
     return f2fma(make_float2(xa.w, xb.w), bc2(y.w), g);
