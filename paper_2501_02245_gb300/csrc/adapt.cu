@@ -26,7 +26,7 @@ __global__ void k_kn_gll(int N, int ni, int nj, int nk, const int* __restrict__ 
     const double a = sqrt(GAMMA * T);
     const double lam = viscosity(T, mu0, omega) / (rho * T) * sqrt(PI * T / 2.0);
     auto nrm = [](const double* g) { return sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]); };
-    const double r = fmax(fmax(nrm(grho + c * 3) / rho, nrm(gU + c * 3) / fmax(U, a)), nrm(gT + c * 3) / T);
+    const double r = fmax(fmax(nrm(grho + c * 3) / rho, nrm(gU + c * 3) / fmax(U, a)), sqrt(gT[c] * gT[c] + gT[N + c] * gT[N + c] + gT[2 * N + c] * gT[2 * N + c]) / T);   // (gT is component-major)
     const double k = lam * r;
     kn[c] = k;
     bool f = k >= Kn_ref;

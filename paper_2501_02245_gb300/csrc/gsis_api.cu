@@ -338,7 +338,9 @@ struct BatchPlan {
     int n_jobs = 0;
     std::vector<int> big;                       // solves too large for the fused synthetic-solve kernel
     int nc = 1, shape = 1, grid = 0;
-    int macro_cluster = 1;                      // CTAs per solve of the fused synthetic-solve launch
+    // fused synthetic-solve launches: jobs [first, first + count) with `cluster` CTAs each
+    struct MacroClass { int first, count, cluster; };
+    std::vector<MacroClass> macro_classes;
     bool tuned = false;
     std::vector<double> tune_ms;
     cudaGraph_t graph = nullptr;
@@ -509,6 +511,7 @@ gsis_status build_plan(BatchPlan* P) {
         if (!cuda_ok(c, cudaStreamSynchronize(c->stream), "batch set-up")) return GSIS_ERR_CUDA;
     std::vector<BatchSolve> hs(n);
     std::vector<MacroJob> jobs;
+    std::vector<int> fused;   // solves of the fused synthetic-solve launches
     P->nc = 1;
     for (int i = 0; i < n; ++i) {
         gsis_ctx* c = P->ctxs[i];
@@ -517,19 +520,46 @@ gsis_status build_plan(BatchPlan* P) {
         hs[i].dtype = c->p.vdf_dtype;
         if (c->normal_components > 1) P->nc = 3;
         if (c->m.N <= MACRO_FUSED_MAX_CELLS)
-            jobs.push_back(macro_job(c, c->p.macro_steps, c->p.dt > 0.0));
+            fused.push_back(i);
         else
             P->big.push_back(i);
         P->W_at_capture.push_back(c->W);
     }
-    P->n_jobs = (int)jobs.size();
-    {   // spread the fused synthetic solves over the SMs: clusters of up to 8 CTAs, at most one
-        // resident CTA per SM (its 512 threads use the register file)
+    P->n_jobs = (int)fused.size();
+    {   // Spread the fused synthetic solves over the SMs (one resident CTA per SM: its 512 threads use
+        // the register file).  A phase lasts as long as the chunks of 32 faces on the busiest SM
+        // sub-partition, so each solve gets the fewest CTAs (a power of two, at most 8) that keep it at
+        // `most` chunks per sub-partition, for the smallest `most` whose clusters fit the SMs together;
+        // one launch per cluster size, the longest solves (largest clusters) first.
         int dev = 0, sms = 1;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int want = P->n_jobs > 0 ? std::max(1, sms / P->n_jobs) : 1;
-        P->macro_cluster = fused_cluster_size(want);
+        std::vector<int> chunks, cluster(P->n_jobs, 1);
+        int widest = 1;
+        for (int i : fused) {
+            gsis_ctx* c = P->ctxs[i];
+            chunks.push_back((c->m.N * c->normal_components + 31) / 32 + (c->m.nbside + 31) / 32);
+            widest = std::max(widest, chunks.back());
+        }
+        const int max_cs = fused_cluster_size(8);
+        for (int most = 1;; ++most) {
+            int total = 0;
+            for (int q = 0; q < P->n_jobs; ++q) {
+                int cs = 1;
+                while (cs < max_cs && chunks[q] > 4 * cs * most) cs *= 2;
+                cluster[q] = cs;
+                total += cs;
+            }
+            if (total <= sms || 4 * most >= widest) break;
+        }
+        for (int cs = 8; cs >= 1; cs /= 2) {
+            const int first = (int)jobs.size();
+            for (int q = 0; q < P->n_jobs; ++q) {
+                gsis_ctx* c = P->ctxs[fused[q]];
+                if (cluster[q] == cs) jobs.push_back(macro_job(c, c->p.macro_steps, c->p.dt > 0.0));
+            }
+            if ((int)jobs.size() > first) P->macro_classes.push_back({first, (int)jobs.size() - first, cs});
+        }
     }
     P->d_solves = (BatchSolve*)dev_alloc(o, n * sizeof(BatchSolve));
     P->d_ticket = (int*)dev_alloc(o, sizeof(int));
@@ -611,10 +641,14 @@ gsis_status build_plan(BatchPlan* P) {
         }
         cudaEventRecordWithFlags(P->ev[1], P->stream, cudaEventRecordExternal);
         branched(all, [](gsis_ctx* c) { stage_moments(c); }, none);
-        // the fused launch of the small solves, the large solves' synthetic solves beside it
+        // the fused launches of the small solves, the large solves' synthetic solves beside them
         branched(P->big, [](gsis_ctx* c) { macro_block(c, c->p.macro_steps, true, c->p.dt > 0.0, true); },
                  [&]() {
-                     if (P->n_jobs) launch_macro_fused(P->d_jobs, P->n_jobs, P->stream, P->macro_cluster);
+                     for (size_t q = 0; q < P->macro_classes.size(); ++q) {   // beside one another: one per stream
+                         const BatchPlan::MacroClass& m = P->macro_classes[q];
+                         launch_macro_fused(P->d_jobs + m.first, m.count, q == 0 ? P->stream : P->branch[(q - 1) % nbr],
+                                            m.cluster);
+                     }
                  });
         branched(all, [](gsis_ctx* c) {
             stage_residual(c, true);
@@ -632,13 +666,15 @@ gsis_status build_plan(BatchPlan* P) {
     ce = cudaGraphInstantiate(&P->exec, P->graph, 0);
     if (ce != cudaSuccess)
         return set_err(o, GSIS_ERR_CUDA, std::string("batch graph instantiation: ") + cudaGetErrorString(ce));
-    P->launches_per_iter = (l1 - l0) + 1 + (P->n_jobs ? 1 : 0);
+    P->launches_per_iter = (l1 - l0) + 1 + (long long)P->macro_classes.size();
+    std::string macro_info;
+    for (const BatchPlan::MacroClass& m : P->macro_classes)
+        macro_info += (macro_info.empty() ? "" : "+") + std::to_string(m.count) + "x" + std::to_string(m.cluster);
     size_t nodes = 0;
     cudaGraphGetNodes(P->graph, nullptr, &nodes);
     P->info = std::string("solves=") + std::to_string(n) + " items=" + std::to_string(P->n_items) +
               " tile=" + batch_shape_name(P->shape) + (P->tuned ? " (autotuned" : " (default") +
-              ") grid=" + std::to_string(P->grid) + " fused_macro=" + std::to_string(P->n_jobs) + "x" +
-              std::to_string(P->macro_cluster) +
+              ") grid=" + std::to_string(P->grid) + " fused_macro=" + macro_info +
               " graph_nodes=" + std::to_string(nodes) + " kernels_per_iteration=" + std::to_string(P->launches_per_iter);
     if (!P->tune_ms.empty()) {
         P->info += " tune_ms=";
@@ -925,7 +961,8 @@ gsis_status gsis_set_mesh(gsis_ctx* c, const gsis_mesh_desc* md) {
     c->F0 = (double*)dev_alloc(c, (size_t)N * 15 * sizeof(double));
     c->dFa = (double*)dev_alloc(c, (size_t)N * 15 * sizeof(double));
     c->dFb = (double*)dev_alloc(c, (size_t)N * 15 * sizeof(double));
-    c->fgeo = (double*)dev_alloc(c, (size_t)N * 3 * 8 * sizeof(double));
+    c->fgeo = (double*)dev_alloc(c, (size_t)N * 3 * FGEO_N * sizeof(double));
+    c->fst = (int4*)dev_alloc(c, (size_t)N * 3 * sizeof(int4));
     c->bgeo = (double*)dev_alloc(c, (size_t)N * 6 * 8 * sizeof(double));
     c->acell = (double*)dev_alloc(c, (size_t)N * sizeof(double));
     c->fields = (double*)dev_alloc(c, (size_t)N * FIELDS_N * sizeof(double));
@@ -959,7 +996,7 @@ gsis_status gsis_set_mesh(gsis_ctx* c, const gsis_mesh_desc* md) {
     c->recGhost.scal = (double*)dev_alloc(c, (size_t)N * RS * sizeof(double));
     c->recBC.scal = (double*)dev_alloc(c, 6 * RS * sizeof(double));
     if (!c->d_job || !c->d_bar || !m.cen || !m.vol || !m.Sout || !m.xf || !m.lsq_w || !m.nbr || !m.side_bc || !m.hyper || !m.bside || !c->Fbnd || !c->W || !c->Wmom ||
-        !c->Wh || !c->fgeo || !c->bgeo || !c->acell || !c->fields ||
+        !c->Wh || !c->fgeo || !c->fst || !c->bgeo || !c->acell || !c->fields ||
         !c->Wp || !c->Wm || !c->U || !c->Un || !c->dU || !c->dU2 || !c->R || !c->D || !c->lamS || !c->Ff ||
         !c->lamf || !c->F0 || !c->dFa || !c->dFb || !c->gu || !c->gT ||
         !c->grho || !c->gU || !c->hot || !c->kin || !c->nsf || !c->kn_gll || !c->wall_den || !c->wall_in ||

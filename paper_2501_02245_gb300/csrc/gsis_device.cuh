@@ -138,6 +138,16 @@ __device__ __forceinline__ double viscosity(double T, double mu0, double omega) 
     return mu0 * exp(omega * log(T));
 }
 
+// 1 / x to within two units in the last place (x a normal number, not 0): the
+// hardware's double-precision seed (20 bits) and two Newton-Raphson steps, four
+// FP64 operations where the division takes about ten.
+__device__ __forceinline__ double recip64(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+
 // ---------------------------------------------------------------- velocity index
 __device__ __forceinline__ void vsplit(long long v, int nx, int ny, int& ix, int& iy, int& iz) {
     ix = (int)(v % nx);

@@ -106,7 +106,8 @@ struct MacroArgs {
     const double* vol;
     const double* lsq_w;
     const double* bc_state;   // [6][5]
-    const double* fgeo;       // [N][3][8] high face of each direction: |S|, n (3), e (3), distance of centres
+    const double* fgeo;       // [N][3][FGEO_N] high face of each direction: |S|, n (3), e (3), distance of centres, 1/distance, S (3)
+    const int4* fst;          // [N][3] cells of that face's stencil: below L, R, beyond R (-1: none)
     const double* bgeo;       // [N][6][8] each side: |S|, n (3), unit cell-to-face vector (3), its length
     const int* bside;         // [nbside] far-field and wall sides, c * 6 + s
     int nbside;
@@ -123,10 +124,11 @@ struct MacroJob {
     double *Wm, *U;
     const double *Un, *hot, *wall_corr;
     double *gu, *gT, *Ff, *lamf, *R, *D, *lamS, *dU, *dU2, *acell;
-    double *F0, *dFa, *dFb;   // Euler flux tensor of U and its changes for the relaxation increments [N][15]
+    double *F0, *dFa, *dFb;   // Euler flux tensor of U and its changes for the relaxation increments [15][N]
     double* Fbnd;             // [N][6][6] boundary-side flux F.S_out (5) and lambda |S|
 };
 
+constexpr int FGEO_N = 12;      // face geometry values (MacroArgs::fgeo)
 constexpr int MACRO_FUSED_THREADS = 512;
 constexpr int MACRO_FUSED_MAX_CELLS = 4096;
 constexpr int MACRO_PERSISTENT_THREADS = 256;
@@ -186,6 +188,7 @@ struct gsis_ctx {
     double *Ff = nullptr, *lamf = nullptr;   // interior face fluxes [N][3][5] and lambda|S| [N][3] (high faces)
     double *F0 = nullptr, *dFa = nullptr, *dFb = nullptr;   // [N][15] Euler flux tensor and its changes (relaxation)
     double *fgeo = nullptr, *bgeo = nullptr; // face geometry (see MacroArgs)
+    int4* fst = nullptr;                     // cells of each face's stencil (see MacroArgs)
     double* acell = nullptr;                 // [N] sound speed of the current pseudo-time state
     double* fields = nullptr;                // [N][FIELDS_N] derived fields of gsis_moments
     double *gu = nullptr, *gT = nullptr, *grho = nullptr, *gU = nullptr;
@@ -302,7 +305,7 @@ void macro_block(gsis_ctx* c, int steps, bool with_hot, bool time_term, bool cap
 MacroJob macro_job(gsis_ctx* c, int steps, bool time_term);
 void launch_macro_fused(const MacroJob* d_jobs, int njobs, cudaStream_t stream, int cs);
 int fused_cluster_size(int want);
-int fused_cluster_for(int N);
+int fused_cluster_for(int N, int ndir, int nbside);
 void launch_eps(gsis_ctx* c, const double* Wn, const double* Wp);
 // adapt.cu
 void launch_kn_gll(gsis_ctx* c, const double* Wprim);

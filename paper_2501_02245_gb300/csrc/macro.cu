@@ -44,6 +44,7 @@ static MacroArgs margs(gsis_ctx* c) {
     a.bc_state = c->d_bc_state;
     a.fgeo = c->fgeo;
     a.bgeo = c->bgeo;
+    a.fst = c->fst;
     a.bside = c->m.bside;
     a.nbside = c->m.nbside;
     a.nd = c->normal_components;
@@ -56,47 +57,70 @@ static MacroArgs margs(gsis_ctx* c) {
 // ---------------------------------------------------------------------------- gradients
 // Least-squares gradient (face neighbours plus boundary face centres with the
 // boundary value: far field -> boundary state; wall -> u = 0, |u| = 0, T = T_w,
-// rho = cell value).  gu[c][j][i] = d u_j / d x_i.  ND: the LSQ weights have
-// components 0..ND-1 only (MacroArgs::fnd); the others are written as zero.
-template <int ND>
-__device__ __forceinline__ void gradients_nd(const MacroArgs& a, const double* Wp, int with_rho_U, double* gu,
-                                             double* gT, double* grho, double* gU, double* acell, int c) {
-    const double* wc = Wp + c * 5;
-    if (acell) acell[c] = sqrt(GAMMA * wc[4]);
-    const double Uc = with_rho_U ? sqrt(wc[1] * wc[1] + wc[2] * wc[2] + wc[3] * wc[3]) : 0.0;
-    double g[6][3];
-    for (int q = 0; q < 6; ++q) g[q][0] = g[q][1] = g[q][2] = 0.0;
-    for (int s = 0; s < 6; ++s) {
-        const int n = a.nbr[c * 6 + s];
-        const int bc = a.side_bc[c * 6 + s];
-        double val[6];   // ux, uy, uz, T, rho, U
-        if (n >= 0) {
-            const double* wn = Wp + n * 5;
-            val[0] = wn[1]; val[1] = wn[2]; val[2] = wn[3]; val[3] = wn[4]; val[4] = wn[0];
-            val[5] = with_rho_U ? sqrt(wn[1] * wn[1] + wn[2] * wn[2] + wn[3] * wn[3]) : 0.0;
-        } else if (bc == GSIS_BC_FARFIELD) {
-            const double* st = a.bc_state + s * 5;
-            val[0] = st[1]; val[1] = st[2]; val[2] = st[3]; val[3] = st[4]; val[4] = st[0];
-            val[5] = with_rho_U ? sqrt(st[1] * st[1] + st[2] * st[2] + st[3] * st[3]) : 0.0;
-        } else if (bc == GSIS_BC_WALL) {
-            const double* st = a.bc_state + s * 5;
-            val[0] = 0.0; val[1] = 0.0; val[2] = 0.0; val[3] = st[4]; val[4] = wc[0]; val[5] = 0.0;
-        } else {
-            continue;
-        }
-        const double phic[6] = {wc[1], wc[2], wc[3], wc[4], wc[0], Uc};
-        const double* w = a.lsq_w + ((long long)c * 6 + s) * 3;
-        const int nq = with_rho_U ? 6 : 4;
-        for (int q = 0; q < nq; ++q) {
-            const double dphi = val[q] - phic[q];
+// rho = cell value).  gu[(3 j + i) N + c] = d u_j / d x_i, gT[i N + c].  ND:
+// the LSQ weights have components 0..ND-1 only (MacroArgs::fnd) and the sides
+// of the other directions carry nothing; their entries are written as zero.
+// The neighbours' values are all loaded before any of them is used (a missing
+// neighbour repeats the cell: its difference is zero), so that a thread waits
+// for memory twice (indices, values) instead of twice per side.
+template <int ND, bool RHO_U>
+__device__ __forceinline__ void gradients_nd(const MacroArgs& a, const double* Wp, double* gu, double* gT,
+                                             double* grho, double* gU, double* acell, int c) {
+    constexpr int NS = 2 * ND, NQ = RHO_U ? 6 : 4;
+    const int N = a.N;
+    int n[NS];
 #pragma unroll
-            for (int i = 0; i < ND; ++i) g[q][i] += w[i] * dphi;
+    for (int d = 0; d < ND; ++d) {
+        const int2 v = *reinterpret_cast<const int2*>(a.nbr + c * 6 + 2 * d);
+        n[2 * d] = v.x;
+        n[2 * d + 1] = v.y;
+    }
+    double val[NS][6], w[NS][ND], phic[6];   // ux, uy, uz, T, rho, U
+    auto state = [](const double* p, double* o) {
+        o[0] = p[1]; o[1] = p[2]; o[2] = p[3]; o[3] = p[4];
+        if (RHO_U) {
+            o[4] = p[0];
+            o[5] = sqrt(p[1] * p[1] + p[2] * p[2] + p[3] * p[3]);
+        }
+    };
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        state(Wp + (n[s] >= 0 ? n[s] : c) * 5, val[s]);
+#pragma unroll
+        for (int i = 0; i < ND; ++i) w[s][i] = a.lsq_w[((long long)c * 6 + s) * 3 + i];
+    }
+    state(Wp + c * 5, phic);
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        if (n[s] >= 0) continue;
+        const int bc = a.side_bc[c * 6 + s];
+        const double* st = a.bc_state + s * 5;
+        if (bc == GSIS_BC_FARFIELD) {
+            state(st, val[s]);
+        } else if (bc == GSIS_BC_WALL) {
+            val[s][0] = 0.0; val[s][1] = 0.0; val[s][2] = 0.0; val[s][3] = st[4];
+            if (RHO_U) val[s][5] = 0.0;   // (rho keeps the cell's value)
         }
     }
+    if (acell) acell[c] = sqrt(GAMMA * phic[3]);
+    double g[6][3];
+    for (int q = 0; q < 6; ++q) g[q][0] = g[q][1] = g[q][2] = 0.0;
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const double dphi = val[s][q] - phic[q];
+#pragma unroll
+            for (int i = 0; i < ND; ++i) g[q][i] += w[s][i] * dphi;
+        }
+    }
+#pragma unroll
     for (int j = 0; j < 3; ++j)
-        for (int i = 0; i < 3; ++i) gu[(long long)c * 9 + j * 3 + i] = g[j][i];
-    for (int i = 0; i < 3; ++i) gT[(long long)c * 3 + i] = g[3][i];
-    if (with_rho_U) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) gu[(long long)(j * 3 + i) * N + c] = g[j][i];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) gT[(long long)i * N + c] = g[3][i];
+    if (RHO_U) {
         for (int i = 0; i < 3; ++i) {
             grho[(long long)c * 3 + i] = g[4][i];
             gU[(long long)c * 3 + i] = g[5][i];
@@ -104,20 +128,31 @@ __device__ __forceinline__ void gradients_nd(const MacroArgs& a, const double* W
     }
 }
 
-__device__ __forceinline__ void gradients_cell(const MacroArgs& a, const double* Wp, int with_rho_U, double* gu,
-                                               double* gT, double* grho, double* gU, double* acell, int c) {
+template <bool RHO_U>
+__device__ __forceinline__ void gradients_cell(const MacroArgs& a, const double* Wp, double* gu, double* gT,
+                                               double* grho, double* gU, double* acell, int c) {
     switch (a.fnd) {
-        case 1: gradients_nd<1>(a, Wp, with_rho_U, gu, gT, grho, gU, acell, c); break;
-        case 2: gradients_nd<2>(a, Wp, with_rho_U, gu, gT, grho, gU, acell, c); break;
-        default: gradients_nd<3>(a, Wp, with_rho_U, gu, gT, grho, gU, acell, c); break;
+        case 1: gradients_nd<1, RHO_U>(a, Wp, gu, gT, grho, gU, acell, c); break;
+        case 2: gradients_nd<2, RHO_U>(a, Wp, gu, gT, grho, gU, acell, c); break;
+        default: gradients_nd<3, RHO_U>(a, Wp, gu, gT, grho, gU, acell, c); break;
     }
+}
+
+// The gradients of cell c as the 3 x 3 and 3 arrays of nsf_of.
+__device__ __forceinline__ void cell_grad(const double* gu, const double* gT, int N, int c, double* u, double* T) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) u[i] = gu[(long long)i * N + c];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) T[i] = gT[(long long)i * N + c];
 }
 
 __global__ void k_gradients(MacroArgs a, const double* __restrict__ Wp, int with_rho_U, double* __restrict__ gu,
                             double* __restrict__ gT, double* __restrict__ grho, double* __restrict__ gU,
                             double* __restrict__ acell) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < a.N) gradients_cell(a, Wp, with_rho_U, gu, gT, grho, gU, acell, c);
+    if (c >= a.N) return;
+    if (with_rho_U) gradients_cell<true>(a, Wp, gu, gT, grho, gU, acell, c);
+    else gradients_cell<false>(a, Wp, gu, gT, nullptr, nullptr, acell, c);
 }
 
 void launch_gradients(gsis_ctx* c, const double* Wprim, bool with_rho_U) {
@@ -150,7 +185,9 @@ __global__ void k_nsf(int N, const double* __restrict__ Wp, const double* __rest
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
     const double mu = viscosity(Wp[c * 5 + 4], mu0, omega);
-    nsf_of(mu, gu + (long long)c * 9, gT + (long long)c * 3, out + (long long)c * HOTN, out + (long long)c * HOTN + 6);
+    double u[9], t[3];
+    cell_grad(gu, gT, N, c, u, t);
+    nsf_of(mu, u, t, out + (long long)c * HOTN, out + (long long)c * HOTN + 6);
 }
 
 void launch_nsf(gsis_ctx* c, const double* Wprim, double* out) {
@@ -172,10 +209,10 @@ __global__ void k_prim_to_cons(int N, const double* __restrict__ Wp, double* __r
     U[c * 5 + 4] = r * (1.5 * T + 0.5 * (ux * ux + uy * uy + uz * uz));
 }
 
-// (One FP64 division per state, its reciprocal reused: on GB300 a division
-// costs about ten FP64-pipe operations.)
+// (One reciprocal per state, reused: on GB300 an FP64 division costs about ten
+// FP64-pipe operations.)
 __device__ __forceinline__ void cons_to_prim(const double* U, double* Wp) {
-    const double r = U[0], ir = 1.0 / r;
+    const double r = U[0], ir = recip64(r);
     const double ux = U[1] * ir, uy = U[2] * ir, uz = U[3] * ir;
     Wp[0] = r;
     Wp[1] = ux;
@@ -192,9 +229,11 @@ __global__ void k_cons_to_prim(int N, const double* __restrict__ U, double* __re
 
 // Face geometry of the synthetic solve, computed once per mesh: for the high
 // face of each direction |S|, n = S/|S|, the unit vector e between the cell
-// centres and their distance; for every side |S|, n and the unit vector from
+// centres, their distance and its reciprocal, S, and the cells of the face's
+// stencil (MacroArgs::fst); for every side |S|, n and the unit vector from
 // the cell centre to the face centre and its length.
-__global__ void k_face_geometry(MacroArgs a, double* __restrict__ fgeo, double* __restrict__ bgeo) {
+__global__ void k_face_geometry(MacroArgs a, double* __restrict__ fgeo, double* __restrict__ bgeo,
+                                int4* __restrict__ fst) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= a.N) return;
     for (int s = 0; s < 6; ++s) {
@@ -211,8 +250,10 @@ __global__ void k_face_geometry(MacroArgs a, double* __restrict__ fgeo, double* 
         if (s & 1) {
             const int d = s >> 1;
             const int R = a.nbr[c * 6 + s];
-            double* G = fgeo + ((long long)c * 3 + d) * 8;
-            for (int q = 0; q < 8; ++q) G[q] = 0.0;
+            double* G = fgeo + ((long long)c * 3 + d) * FGEO_N;
+            for (int q = 0; q < FGEO_N; ++q) G[q] = 0.0;
+            // cells of the face's stencil: below L, L's neighbour R, beyond R
+            fst[(long long)c * 3 + d] = make_int4(a.nbr[c * 6 + s - 1], R, R >= 0 ? a.nbr[R * 6 + s] : -1, 0);
             if (R >= 0) {
                 double e[3];
                 for (int i = 0; i < 3; ++i) e[i] = a.cen[R * 3 + i] - a.cen[c * 3 + i];
@@ -221,6 +262,8 @@ __global__ void k_face_geometry(MacroArgs a, double* __restrict__ fgeo, double* 
                 for (int i = 0; i < 3; ++i) G[1 + i] = So[i] / Sabs;
                 for (int i = 0; i < 3; ++i) G[4 + i] = e[i] / dist;
                 G[7] = dist;
+                G[8] = 1.0 / dist;
+                for (int i = 0; i < 3; ++i) G[9 + i] = So[i];
             }
         }
     }
@@ -228,7 +271,7 @@ __global__ void k_face_geometry(MacroArgs a, double* __restrict__ fgeo, double* 
 
 void launch_face_geometry(gsis_ctx* c) {
     const int N = c->m.N;
-    k_face_geometry<<<(N + 127) / 128, 128, 0, c->stream>>>(margs(c), c->fgeo, c->bgeo);
+    k_face_geometry<<<(N + 127) / 128, 128, 0, c->stream>>>(margs(c), c->fgeo, c->bgeo, c->fst);
     c->launches++;
 }
 
@@ -296,8 +339,8 @@ template <int ND = 3>
 __device__ void kfvs(double rL, const double* uL, double pL, double rR, const double* uR, double pR,
                      const double* n, double* F) {
     for (int q = 0; q < 5; ++q) F[q] = 0.0;
-    half_range_add<ND>(rL, uL, pL / rL, n, 1.0, F);
-    half_range_add<ND>(rR, uR, pR / rR, n, -1.0, F);
+    half_range_add<ND>(rL, uL, pL * recip64(rL), n, 1.0, F);
+    half_range_add<ND>(rR, uR, pR * recip64(rR), n, -1.0, F);
 }
 
 // Euler flux tensor of conserved state U: F[q * 3 + i] = flux of component q
@@ -306,7 +349,7 @@ __device__ void kfvs(double rL, const double* uL, double pL, double rR, const do
 // along the others (ND = normal_components), F.S never reads them.
 template <int ND>
 __device__ __forceinline__ void euler_tensor(const double* U, double* F) {
-    const double r = U[0], ir = 1.0 / r;
+    const double r = U[0], ir = recip64(r);
     const double u[3] = {U[1] * ir, U[2] * ir, U[3] * ir};
     const double p = (GAMMA - 1.0) * (U[4] - 0.5 * r * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
 #pragma unroll
@@ -318,20 +361,23 @@ __device__ __forceinline__ void euler_tensor(const double* U, double* F) {
     }
 }
 
-// Change of the Euler flux tensor of cell c for the relaxation increment
-// dU_c, F(U_c + dU_c) - F(U_c), with F(U_c) kept in F0 for the pseudo-step:
-// each neighbour then reads the values instead of evaluating both fluxes
-// (and their divisions) itself.
+// Change of the Euler flux tensor of a cell for the relaxation increment
+// dU, F(U + dU) - F(U), with F(U) kept in F0 for the pseudo-step: each
+// neighbour then reads the values instead of evaluating both fluxes (and their
+// divisions) itself.  Arrays of the synthetic solve that neighbours or later
+// phases read are component-major ([component][N]): a warp's load of one
+// component touches two or three lines instead of one per lane.
 template <int ND>
-__device__ __forceinline__ void flux_change(const double* U, const double* dU, const double* F0, double* dF, int c) {
+__device__ __forceinline__ void flux_change(const double* U, const double* dU, const double* F0, double* dF, int N,
+                                            int c) {
     double Up[5], F1[15];
 #pragma unroll
-    for (int q = 0; q < 5; ++q) Up[q] = U[c * 5 + q] + dU[c * 5 + q];
+    for (int q = 0; q < 5; ++q) Up[q] = U[q] + dU[q];
     euler_tensor<ND>(Up, F1);
 #pragma unroll
     for (int q = 0; q < 5; ++q)
 #pragma unroll
-        for (int i = 0; i < ND; ++i) dF[(long long)c * 15 + q * 3 + i] = F1[q * 3 + i] - F0[(long long)c * 15 + q * 3 + i];
+        for (int i = 0; i < ND; ++i) dF[(long long)(q * 3 + i) * N + c] = F1[q * 3 + i] - F0[q * 3 + i];
 }
 
 __device__ __forceinline__ void prim5(const double* w, double* q) {   // (rho, u, p)
@@ -340,8 +386,8 @@ __device__ __forceinline__ void prim5(const double* w, double* q) {   // (rho, u
 
 // Interior face between L = cell c and R = its neighbour across side 2d+1
 // (area vector S pointing L -> R).  Writes the total face flux (inviscid +
-// viscous + HoT) F.S to Ff[c][d][5] and lambda |S| to lamf[c][d]; faces that
-// do not exist (boundary) get lamf = -1.
+// viscous + HoT) F.S to Ff[(5 d + q) N + c] and lambda |S| to lamf[d N + c];
+// faces that do not exist (boundary) get lamf = -1.
 // ND: on a mesh whose face normals, cell-to-cell vectors and LSQ weights have
 // components 0..ND-1 only (MacroArgs::fnd), the gradient entries along the
 // other directions are exact zeros and are not formed or multiplied: the same
@@ -349,42 +395,43 @@ __device__ __forceinline__ void prim5(const double* w, double* q) {   // (rho, u
 // the out-of-plane velocity of a 2D flow is zero only up to rounding -- and up
 // to the storage noise of BF16/FP16 VDFs -- and its viscous stress is what
 // damps it.)
+// What bounds it: FP64 instructions (a warp's holds the pipe of its SM
+// sub-partition for 64 cycles), so reciprocals that depend on the mesh are
+// stored, the others come from recip64, and the limiter runs on the integer pipe.
 template <int ND>
 __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* Wm, const double* gu,
-                                             const double* gT, const double* hot, const double* acell, int ndir,
+                                             const double* gT, const double* hot, const double* acell,
                                              double* Ff, double* lamf, int t) {
-    const int L = t / ndir, d = t % ndir;
-    const int Rr = a.nbr[L * 6 + 2 * d + 1];
-    double* F = Ff + ((long long)L * 3 + d) * 5;
+    const int N = a.N, d = t / N, L = t - d * N;
+    const int4 st = a.fst[(long long)L * 3 + d];
+    const int Rr = st.y;
     if (Rr < 0) {
-        lamf[(long long)L * 3 + d] = -1.0;
+        lamf[(long long)d * N + L] = -1.0;
         return;
     }
-    const double* S = a.Sout + ((long long)L * 6 + 2 * d + 1) * 3;
-    const double* G = a.fgeo + ((long long)L * 3 + d) * 8;
+    const double* G = a.fgeo + ((long long)L * 3 + d) * FGEO_N;
     const double Sabs = G[0];
-    const double nn[3] = {G[1], G[2], G[3]};
+    const double nn[3] = {G[1], G[2], G[3]}, S[3] = {G[9], G[10], G[11]};
     // MUSCL face states: q -/+ 0.5 minmod of the one-sided differences (the
     // halved limiter on the integer pipe), first order where the second
-    // neighbour is missing
-    double qL[5], qR[5], mL[5] = {0, 0, 0, 0, 0}, mR[5] = {0, 0, 0, 0, 0};
-    prim5(Wm + L * 5, qL);
-    prim5(Wm + Rr * 5, qR);
+    // neighbour is missing (the cell itself in its place: a zero difference)
+    double wL[5], wR[5], ql[5], qh[5];
     {
-        const int lo = a.nbr[L * 6 + 2 * d];
-        if (lo >= 0) {
-            double ql[5];
-            prim5(Wm + lo * 5, ql);
-            for (int q = 0; q < 5; ++q) mL[q] = hmm_t<double>(qL[q] - ql[q], qR[q] - qL[q]);
-        }
+        const double *pL = Wm + L * 5, *pR = Wm + Rr * 5, *pl = Wm + (st.x >= 0 ? st.x : L) * 5,
+                     *ph = Wm + (st.z >= 0 ? st.z : Rr) * 5;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) { wL[q] = pL[q]; wR[q] = pR[q]; }
+        prim5(pl, ql);
+        prim5(ph, qh);
     }
-    {
-        const int hi = a.nbr[Rr * 6 + 2 * d + 1];
-        if (hi >= 0) {
-            double qh[5];
-            prim5(Wm + hi * 5, qh);
-            for (int q = 0; q < 5; ++q) mR[q] = hmm_t<double>(qR[q] - qL[q], qh[q] - qR[q]);
-        }
+    double qL[5], qR[5], mL[5], mR[5];
+    prim5(wL, qL);
+    prim5(wR, qR);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        const double df = qR[q] - qL[q];
+        mL[q] = hmm_t<double>(qL[q] - ql[q], df);
+        mR[q] = hmm_t<double>(df, qh[q] - qR[q]);
     }
     double fl[5], fr[5];
     for (int q = 0; q < 5; ++q) { fl[q] = qL[q] + mL[q]; fr[q] = qR[q] - mR[q]; }
@@ -392,13 +439,11 @@ __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* W
     kfvs<ND>(fl[0], fl + 1, fl[4], fr[0], fr + 1, fr[4], nn, Fv);
     for (int q = 0; q < 5; ++q) Fv[q] *= Sabs;
     // viscous + HoT
-    const double* wL = Wm + L * 5;
-    const double* wR = Wm + Rr * 5;
     const double uf[3] = {0.5 * (wL[1] + wR[1]), 0.5 * (wL[2] + wR[2]), 0.5 * (wL[3] + wR[3])};
     const double Tf = 0.5 * (wL[4] + wR[4]);
     const double muf = viscosity(Tf, a.mu0, a.omega);
     const double e[3] = {G[4], G[5], G[6]};
-    const double dist = G[7], idist = 1.0 / dist;
+    const double dist = G[7], idist = G[8];
     // face gradients: cell average corrected along the line of centres, for every
     // velocity component j and the directions i below ND (the others are zero:
     // the LSQ weights and the line of centres have no such component)
@@ -408,7 +453,7 @@ __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* W
         double gav[3], ge = 0.0;
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
-            gav[i] = 0.5 * (gu[(long long)L * 9 + j * 3 + i] + gu[(long long)Rr * 9 + j * 3 + i]);
+            gav[i] = 0.5 * (gu[(long long)(j * 3 + i) * N + L] + gu[(long long)(j * 3 + i) * N + Rr]);
             ge = i == 0 ? gav[0] * e[0] : ge + gav[i] * e[i];
         }
         const double corr = (wR[1 + j] - wL[1 + j]) * idist - ge;
@@ -419,7 +464,7 @@ __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* W
         double gav[3], ge = 0.0;
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
-            gav[i] = 0.5 * (gT[(long long)L * 3 + i] + gT[(long long)Rr * 3 + i]);
+            gav[i] = 0.5 * (gT[(long long)i * N + L] + gT[(long long)i * N + Rr]);
             ge = i == 0 ? gav[0] * e[0] : ge + gav[i] * e[i];
         }
         const double corr = (wR[4] - wL[4]) * idist - ge;
@@ -461,34 +506,37 @@ __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* W
     }
 #pragma unroll
     for (int k = 1; k < ND; ++k) QS += Q[k] * S[k];
+    double* F = Ff + (long long)(5 * d) * N + L;
     F[0] = Fv[0];
-    F[1] = Fv[1] + SigS[0];
-    F[2] = Fv[2] + SigS[1];
-    F[3] = Fv[3] + SigS[2];
-    F[4] = Fv[4] + ((SigS[0] * uf[0] + SigS[1] * uf[1] + SigS[2] * uf[2]) + QS);
+    F[(long long)N] = Fv[1] + SigS[0];
+    F[(long long)2 * N] = Fv[2] + SigS[1];
+    F[(long long)3 * N] = Fv[3] + SigS[2];
+    F[(long long)4 * N] = Fv[4] + ((SigS[0] * uf[0] + SigS[1] * uf[1] + SigS[2] * uf[2]) + QS);
     const double aL = acell[L], aR = acell[Rr];
     double un = uf[0] * nn[0];
 #pragma unroll
     for (int k = 1; k < ND; ++k) un += uf[k] * nn[k];
-    const double lam = fabs(un) + 0.5 * (aL + aR) + 5.0 * muf / (0.5 * (wL[0] + wR[0]) * dist);
-    lamf[(long long)L * 3 + d] = lam * Sabs;
+    const double lam = fabs(un) + 0.5 * (aL + aR) + 5.0 * muf * recip64(0.5 * (wL[0] + wR[0]) * dist);
+    lamf[(long long)d * N + L] = lam * Sabs;
 }
 
 __device__ __forceinline__ void face_flux_one(const MacroArgs& a, const double* Wm, const double* gu,
-                                              const double* gT, const double* hot, const double* acell, int ndir,
+                                              const double* gT, const double* hot, const double* acell,
                                               double* Ff, double* lamf, int t) {
     switch (a.fnd) {
-        case 1: face_flux_nd<1>(a, Wm, gu, gT, hot, acell, ndir, Ff, lamf, t); break;
-        case 2: face_flux_nd<2>(a, Wm, gu, gT, hot, acell, ndir, Ff, lamf, t); break;
-        default: face_flux_nd<3>(a, Wm, gu, gT, hot, acell, ndir, Ff, lamf, t); break;
+        case 1: face_flux_nd<1>(a, Wm, gu, gT, hot, acell, Ff, lamf, t); break;
+        case 2: face_flux_nd<2>(a, Wm, gu, gT, hot, acell, Ff, lamf, t); break;
+        default: face_flux_nd<3>(a, Wm, gu, gT, hot, acell, Ff, lamf, t); break;
     }
 }
 
-// NSF flux through wall side s of cell c at state w (prim) with cell gradients
-// gu, gT: no mass flux, cell pressure, NSF stress and heat flux at u = 0,
+// NSF flux through wall side s of cell c at state w (prim) with the cells' gradients
+// guN, gTN (component-major): no mass flux, cell pressure, NSF stress and heat flux at u = 0,
 // T = T_w from the cell gradient corrected along the cell-to-face line.
-__device__ void wall_nsf_flux(const MacroArgs& a, const double* w, const double* gu, const double* gT, int c, int s,
+__device__ void wall_nsf_flux(const MacroArgs& a, const double* w, const double* guN, const double* gTN, int c, int s,
                               double* Fb) {
+    double gu[9], gT[3];
+    cell_grad(guN, gTN, a.N, c, gu, gT);
     const double* So = a.Sout + ((long long)c * 6 + s) * 3;
     const double Tw = a.bc_state[s * 5 + 4];
     const double* G = a.bgeo + ((long long)c * 6 + s) * 8;
@@ -529,7 +577,7 @@ __global__ void k_wall_corr(MacroArgs a, const int* __restrict__ cell2dvm, const
         double* o = wall_corr + ((long long)c * 6 + s) * 5;
         if (a.nbr[c * 6 + s] < 0 && a.side_bc[c * 6 + s] == GSIS_BC_WALL && cell2dvm[c] >= 0) {
             double F[5];
-            wall_nsf_flux(a, Wh + c * 5, gu + (long long)c * 9, gT + (long long)c * 3, c, s, F);
+            wall_nsf_flux(a, Wh + c * 5, gu, gT, c, s, F);
             const double* kin = wall_kin + ((long long)c * 6 + s) * 5;
             for (int q = 0; q < 5; ++q) o[q] = kin[q] - F[q];
         } else {
@@ -563,7 +611,7 @@ __global__ void k_wall_loads(MacroArgs a, const int* __restrict__ cell2dvm, cons
         if (cell2dvm[c] >= 0) {
             for (int q = 0; q < 5; ++q) F[q] = wall_kin[((long long)c * 6 + s) * 5 + q];
         } else {
-            wall_nsf_flux(a, W + c * 5, gu + (long long)c * 9, gT + (long long)c * 3, c, s, F);
+            wall_nsf_flux(a, W + c * 5, gu, gT, c, s, F);
         }
         const double* G = a.bgeo + ((long long)c * 6 + s) * 8;   // |S|, unit normal
         const double Fn = F[1] * G[1] + F[2] * G[2] + F[3] * G[3];
@@ -586,7 +634,9 @@ __global__ void k_constitutive(int N, const double* __restrict__ W, const double
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
     double sig[6], q[3];
-    nsf_of(viscosity(W[c * 5 + 4], mu0, omega), gu + (long long)c * 9, gT + (long long)c * 3, sig, q);
+    double u[9], t[3];
+    cell_grad(gu, gT, N, c, u, t);
+    nsf_of(viscosity(W[c * 5 + 4], mu0, omega), u, t, sig, q);
     double* o = out + (long long)c * FIELDS_N;
     const double* h = hot + (long long)c * HOTN;
     for (int k = 0; k < 6; ++k) o[k] = sig[k] + h[k];
@@ -644,7 +694,7 @@ __device__ __forceinline__ void boundary_flux_one(const MacroArgs& a, const doub
         Fb[4] += (SigS[0] * ufb[0] + SigS[1] * ufb[1] + SigS[2] * ufb[2]) +
                  (h[6] * So[0] + h[7] * So[1] + h[8] * So[2]);
     } else {
-        wall_nsf_flux(a, wc, gu + (long long)c * 9, gT + (long long)c * 3, c, s, Fb);
+        wall_nsf_flux(a, wc, gu, gT, c, s, Fb);
         const double* wcr = wall_corr + (long long)cs * 5;
         for (int q = 0; q < 5; ++q) Fb[q] += wcr[q];
     }
@@ -657,6 +707,10 @@ __device__ __forceinline__ void boundary_flux_one(const MacroArgs& a, const doub
     o[5] = lam * Sabs;
 }
 
+// Faces, rounded up to whole warps so that no warp mixes interior faces and
+// boundary sides (it would run both).
+__host__ __device__ __forceinline__ int face_items(int N, int ndir) { return (N * ndir + 31) / 32 * 32; }
+
 // Face phase of the per-phase kernels: interior faces (N * ndir threads), then
 // the far-field and wall sides.
 __global__ void k_face_flux(MacroArgs a, const double* __restrict__ Wm, const double* __restrict__ gu,
@@ -664,73 +718,103 @@ __global__ void k_face_flux(MacroArgs a, const double* __restrict__ Wm, const do
                             const double* __restrict__ acell, int ndir, double* __restrict__ Ff,
                             double* __restrict__ lamf, const double* __restrict__ wall_corr,
                             double* __restrict__ Fbnd) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x, nf = a.N * ndir;
-    if (t < nf) face_flux_one(a, Wm, gu, gT, hot, acell, ndir, Ff, lamf, t);
-    else if (t < nf + a.nbside) boundary_flux_one(a, Wm, gu, gT, hot, wall_corr, Fbnd, t - nf);
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, nf = a.N * ndir, nfp = face_items(a.N, ndir);
+    if (t < nf) face_flux_one(a, Wm, gu, gT, hot, acell, Ff, lamf, t);
+    else if (t >= nfp && t < nfp + a.nbside) boundary_flux_one(a, Wm, gu, gT, hot, wall_corr, Fbnd, t - nfp);
 }
 
 // Cell residual R_c = -sum_F F.S_out (gathering the face fluxes in side
 // order: interior faces from Ff, far-field and wall sides from Fbnd), lambda|S|
 // per side, the reciprocal 1/D of the diagonal (in D) and dU0 = R/D.
-__device__ __forceinline__ void cell_residual_one(const MacroArgs& a, const double* Wm, const double* U,
-                                                  const double* Un, const double* gu, const double* gT,
-                                                  const double* hot, const double* Ff, const double* lamf,
-                                                  const double* Fbnd, double cfl, double dt, double* R, double* D,
-                                                  double* lamS, double* dU, double* F0, double* dF, int c) {
+// (ND index directions carry flux; every load is issued before the sums.)
+template <int ND>
+__device__ __forceinline__ void cell_residual_nd(const MacroArgs& a, const double* U, const double* Un,
+                                                 const double* Ff, const double* lamf, const double* Fbnd, double cfl,
+                                                 double dt, double* R, double* D, double* lamS, double* dU, double* F0,
+                                                 double* dF, int c) {
+    constexpr int NS = 2 * ND;
+    const int N = a.N;
+    int n[NS];
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        const int2 v = *reinterpret_cast<const int2*>(a.nbr + c * 6 + 2 * d);
+        n[2 * d] = v.x;
+        n[2 * d + 1] = v.y;
+    }
+    double F[NS][5], ls[NS], Uc[5];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {   // the face's low cell: this one for high sides, the neighbour for low sides
+        const int d = s >> 1, L = (s & 1) || n[s] < 0 ? c : n[s];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) F[s][q] = Ff[(long long)(5 * d + q) * N + L];
+        ls[s] = lamf[(long long)d * N + L];
+    }
+#pragma unroll
+    for (int q = 0; q < 5; ++q) Uc[q] = U[c * 5 + q];
     double Rc[5] = {0, 0, 0, 0, 0};
     double lam_sum = 0.0;
-    for (int s = 0; s < 6; ++s) {
-        const int n = a.nbr[c * 6 + s];
-        const int bc = a.side_bc[c * 6 + s];
-        const int d = s >> 1;
-        if (n >= 0) {
-            const bool isL = (s & 1) != 0;
-            const int L = isL ? c : n;
-            const double* F = Ff + ((long long)L * 3 + d) * 5;
-            const double sgn = isL ? -1.0 : 1.0;
-            for (int q = 0; q < 5; ++q) Rc[q] += sgn * F[q];
-            const double ls = lamf[(long long)L * 3 + d];
-            lamS[(long long)c * 6 + s] = ls;
-            lam_sum += ls;
-        } else if (bc == GSIS_BC_FARFIELD || bc == GSIS_BC_WALL) {   // formed in the face phase
-            const double* Fb = Fbnd + ((long long)c * 6 + s) * 6;
-            for (int q = 0; q < 5; ++q) Rc[q] -= Fb[q];
-            lamS[(long long)c * 6 + s] = Fb[5];
-            lam_sum += Fb[5];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        if (n[s] >= 0) {
+#pragma unroll
+            for (int q = 0; q < 5; ++q) Rc[q] = (s & 1) ? Rc[q] - F[s][q] : Rc[q] + F[s][q];
         } else {
-            lamS[(long long)c * 6 + s] = 0.0;
+            const int bc = a.side_bc[c * 6 + s];
+            ls[s] = 0.0;
+            if (bc == GSIS_BC_FARFIELD || bc == GSIS_BC_WALL) {   // formed in the face phase
+                const double* Fb = Fbnd + ((long long)c * 6 + s) * 6;
+                for (int q = 0; q < 5; ++q) Rc[q] -= Fb[q];
+                ls[s] = Fb[5];
+            }
         }
+        lamS[(long long)s * N + c] = ls[s];
+        lam_sum += ls[s];
     }
     double Dc = (1.0 / cfl + 0.5) * lam_sum;
     if (dt > 0.0) {
         const double Vdt = a.vol[c] / dt;
-        for (int q = 0; q < 5; ++q) Rc[q] -= Vdt * (U[c * 5 + q] - Un[c * 5 + q]);
+#pragma unroll
+        for (int q = 0; q < 5; ++q) Rc[q] -= Vdt * (Uc[q] - Un[c * 5 + q]);
         Dc += Vdt;
     }
     const double iD = 1.0 / Dc;
     D[c] = iD;   // the relaxation sweeps multiply by the reciprocal
+    double dUc[5];
+#pragma unroll
     for (int q = 0; q < 5; ++q) {
-        R[c * 5 + q] = Rc[q];
-        dU[c * 5 + q] = Rc[q] * iD;
+        dUc[q] = Rc[q] * iD;
+        R[(long long)q * N + c] = Rc[q];
+        dU[(long long)q * N + c] = dUc[q];
     }
     if (dF) {   // relaxation sweeps follow: the flux tensor of U_c and its change for dU_c
-        switch (a.nd) {
-            case 1: euler_tensor<1>(U + c * 5, F0 + (long long)c * 15); flux_change<1>(U, dU, F0, dF, c); break;
-            case 2: euler_tensor<2>(U + c * 5, F0 + (long long)c * 15); flux_change<2>(U, dU, F0, dF, c); break;
-            default: euler_tensor<3>(U + c * 5, F0 + (long long)c * 15); flux_change<3>(U, dU, F0, dF, c); break;
-        }
+        double T[15];
+        euler_tensor<ND>(Uc, T);
+#pragma unroll
+        for (int q = 0; q < 5; ++q)
+#pragma unroll
+            for (int i = 0; i < ND; ++i) F0[(long long)(q * 3 + i) * N + c] = T[q * 3 + i];
+        flux_change<ND>(Uc, dUc, T, dF, N, c);
     }
 }
 
-__global__ void k_cell_residual(MacroArgs a, const double* __restrict__ Wm, const double* __restrict__ U,
-                                const double* __restrict__ Un, const double* __restrict__ gu,
-                                const double* __restrict__ gT, const double* __restrict__ hot,
+__device__ __forceinline__ void cell_residual_one(const MacroArgs& a, const double* U, const double* Un,
+                                                  const double* Ff, const double* lamf, const double* Fbnd, double cfl,
+                                                  double dt, double* R, double* D, double* lamS, double* dU, double* F0,
+                                                  double* dF, int c) {
+    switch (a.nd) {
+        case 1: cell_residual_nd<1>(a, U, Un, Ff, lamf, Fbnd, cfl, dt, R, D, lamS, dU, F0, dF, c); break;
+        case 2: cell_residual_nd<2>(a, U, Un, Ff, lamf, Fbnd, cfl, dt, R, D, lamS, dU, F0, dF, c); break;
+        default: cell_residual_nd<3>(a, U, Un, Ff, lamf, Fbnd, cfl, dt, R, D, lamS, dU, F0, dF, c); break;
+    }
+}
+
+__global__ void k_cell_residual(MacroArgs a, const double* __restrict__ U, const double* __restrict__ Un,
                                 const double* __restrict__ Ff, const double* __restrict__ lamf,
                                 const double* __restrict__ Fbnd, double cfl, double dt,
                                 double* __restrict__ R, double* __restrict__ D, double* __restrict__ lamS,
                                 double* __restrict__ dU, double* __restrict__ F0, double* __restrict__ dF) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < a.N) cell_residual_one(a, Wm, U, Un, gu, gT, hot, Ff, lamf, Fbnd, cfl, dt, R, D, lamS, dU, F0, dF, c);
+    if (c < a.N) cell_residual_one(a, U, Un, Ff, lamf, Fbnd, cfl, dt, R, D, lamS, dU, F0, dF, c);
 }
 
 // One Jacobi sweep: dU_new = (R - 1/2 sum_j [dF_j . S_out - lambda|S| dU_j]) / D,
@@ -738,39 +822,73 @@ __global__ void k_cell_residual(MacroArgs a, const double* __restrict__ Wm, cons
 // (dFin); with dFout the cell's own tensor for dU_new follows for the next sweep.
 // The two sums are accumulated apart (FMA chains over the normal components
 // that can be nonzero) and combined once.
+// The loads of all sides are issued before the sums.  The new increment is
+// left in dUc (registers) and, with dUout, stored.
 template <int ND>
 __device__ __forceinline__ void relax_nd(const MacroArgs& a, const double* U, const double* R, const double* D,
                                          const double* lamS, const double* dUin, double* dUout, const double* dFin,
-                                         double* dFout, const double* F0, int c) {
-    double fs[5] = {0, 0, 0, 0, 0}, ld[5] = {0, 0, 0, 0, 0};
-    for (int s = 0; s < 6; ++s) {
-        const int n = a.nbr[c * 6 + s];
-        if (n < 0) continue;
-        const double* So = a.Sout + ((long long)c * 6 + s) * 3;
-        const double* dF = dFin + (long long)n * 15;
-        const double ls = lamS[(long long)c * 6 + s];
+                                         double* dFout, const double* F0, int c, double* dUc) {
+    constexpr int NS = 2 * ND;
+    const int N = a.N;
+    int n[NS];
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        const int2 v = *reinterpret_cast<const int2*>(a.nbr + c * 6 + 2 * d);
+        n[2 * d] = v.x;
+        n[2 * d + 1] = v.y;
+    }
+    double dF[NS][5][ND], dn[NS][5], So[NS][ND], ls[NS], Rc[5];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        const int m = n[s] >= 0 ? n[s] : c;
 #pragma unroll
         for (int q = 0; q < 5; ++q) {
-            double t = fs[q];
 #pragma unroll
-            for (int i = 0; i < ND; ++i) t = fma(dF[q * 3 + i], So[i], t);
-            fs[q] = t;
-            ld[q] = fma(ls, dUin[n * 5 + q], ld[q]);
+            for (int i = 0; i < ND; ++i) dF[s][q][i] = dFin[(long long)(q * 3 + i) * N + m];
+            dn[s][q] = dUin[(long long)q * N + m];
+        }
+#pragma unroll
+        for (int i = 0; i < ND; ++i) So[s][i] = a.Sout[((long long)c * 6 + s) * 3 + i];
+        ls[s] = lamS[(long long)s * N + c];
+    }
+#pragma unroll
+    for (int q = 0; q < 5; ++q) Rc[q] = R[(long long)q * N + c];
+    const double iD = D[c];   // 1 / D
+    double fs[5] = {0, 0, 0, 0, 0}, ld[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        if (n[s] < 0) continue;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+#pragma unroll
+            for (int i = 0; i < ND; ++i) fs[q] = fma(dF[s][q][i], So[s][i], fs[q]);
+            ld[q] = fma(ls[s], dn[s][q], ld[q]);
         }
     }
-    const double iD = D[c];   // 1 / D
 #pragma unroll
-    for (int q = 0; q < 5; ++q) dUout[c * 5 + q] = (R[c * 5 + q] - 0.5 * (fs[q] - ld[q])) * iD;
-    if (dFout) flux_change<ND>(U, dUout, F0, dFout, c);
+    for (int q = 0; q < 5; ++q) {
+        dUc[q] = (Rc[q] - 0.5 * (fs[q] - ld[q])) * iD;
+        if (dUout) dUout[(long long)q * N + c] = dUc[q];
+    }
+    if (dFout) {
+        double Uc[5], T[15];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+            Uc[q] = U[c * 5 + q];
+#pragma unroll
+            for (int i = 0; i < ND; ++i) T[q * 3 + i] = F0[(long long)(q * 3 + i) * N + c];
+        }
+        flux_change<ND>(Uc, dUc, T, dFout, N, c);
+    }
 }
 
 __device__ __forceinline__ void relax_one(const MacroArgs& a, const double* U, const double* R, const double* D,
                                           const double* lamS, const double* dUin, double* dUout, const double* dFin,
-                                          double* dFout, const double* F0, int c) {
+                                          double* dFout, const double* F0, int c, double* dUc) {
     switch (a.nd) {
-        case 1: relax_nd<1>(a, U, R, D, lamS, dUin, dUout, dFin, dFout, F0, c); break;
-        case 2: relax_nd<2>(a, U, R, D, lamS, dUin, dUout, dFin, dFout, F0, c); break;
-        default: relax_nd<3>(a, U, R, D, lamS, dUin, dUout, dFin, dFout, F0, c); break;
+        case 1: relax_nd<1>(a, U, R, D, lamS, dUin, dUout, dFin, dFout, F0, c, dUc); break;
+        case 2: relax_nd<2>(a, U, R, D, lamS, dUin, dUout, dFin, dFout, F0, c, dUc); break;
+        default: relax_nd<3>(a, U, R, D, lamS, dUin, dUout, dFin, dFout, F0, c, dUc); break;
     }
 }
 
@@ -779,32 +897,48 @@ __global__ void k_relax(MacroArgs a, const double* __restrict__ U, const double*
                         double* __restrict__ dUout, const double* __restrict__ dFin, double* __restrict__ dFout,
                         const double* __restrict__ F0) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < a.N) relax_one(a, U, R, D, lamS, dUin, dUout, dFin, dFout, F0, c);
+    double dUc[5];
+    if (c < a.N) relax_one(a, U, R, D, lamS, dUin, dUout, dFin, dFout, F0, c, dUc);
 }
 
-
-__device__ __forceinline__ void update_one(double* U, const double* dU, double* Wm, int c) {
-    for (int q = 0; q < 5; ++q) U[c * 5 + q] += dU[c * 5 + q];
-    cons_to_prim(U + c * 5, Wm + c * 5);
+// U += dU (dU of this cell), primitive state Wm.
+__device__ __forceinline__ void update_one(double* U, const double* dUc, double* Wm, int c) {
+    double Uc[5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        Uc[q] = U[c * 5 + q] + dUc[q];
+        U[c * 5 + q] = Uc[q];
+    }
+    cons_to_prim(Uc, Wm + c * 5);
 }
 
 __global__ void k_update(int N, double* __restrict__ U, const double* __restrict__ dU, double* __restrict__ Wm) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < N) update_one(U, dU, Wm, c);
+    if (c >= N) return;
+    double dUc[5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) dUc[q] = dU[(long long)q * N + c];
+    update_one(U, dUc, Wm, c);
 }
 
 // The last Jacobi sweep of a pseudo-step followed by the update of the
 // cell's own state (U += dU, primitive Wm): the sweep reads U only through the
 // flux change, which the last sweep does not form, so each cell may update
-// its state in place (one launch instead of two, the same values).
+// its state in place (one phase instead of two, the same values).
+__device__ __forceinline__ void relax_update_one(const MacroArgs& a, double* U, const double* R, const double* D,
+                                                 const double* lamS, const double* dUin, const double* dFin, double* Wm,
+                                                 int c) {
+    double dUc[5];
+    relax_one(a, U, R, D, lamS, dUin, nullptr, dFin, nullptr, nullptr, c, dUc);
+    update_one(U, dUc, Wm, c);
+}
+
 __global__ void k_relax_update(MacroArgs a, double* __restrict__ U, const double* __restrict__ R,
                                const double* __restrict__ D, const double* __restrict__ lamS,
-                               const double* __restrict__ dUin, double* __restrict__ dUout,
-                               const double* __restrict__ dFin, double* __restrict__ Wm) {
+                               const double* __restrict__ dUin, const double* __restrict__ dFin,
+                               double* __restrict__ Wm) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= a.N) return;
-    relax_one(a, U, R, D, lamS, dUin, dUout, dFin, nullptr, nullptr, c);
-    update_one(U, dUout, Wm, c);
+    if (c < a.N) relax_update_one(a, U, R, D, lamS, dUin, dFin, Wm, c);
 }
 
 // The whole pseudo-time block of one solve in one thread-block cluster of
@@ -812,9 +946,14 @@ __global__ void k_relax_update(MacroArgs a, double* __restrict__ U, const double
 // batches).  The same per-cell and per-face functions as the multi-block
 // kernels, separated by cluster barriers (release/acquire at cluster scope,
 // so every CTA of the cluster sees the others' global-memory writes of the
-// previous phase), so the result is identical.  A batch of solves uses
-// clusters to occupy the SMs its solves alone would leave idle (64 solves:
-// clusters of two, 5 % faster).  Jobs are clusters 0, 1, ... of the grid.
+// previous phase), so the result is identical.  Jobs are clusters 0, 1, ...
+// of the grid.
+// What bounds it: a warp's FP64 instruction holds the FP64 pipe of its SM
+// sub-partition for 64 cycles, so a phase lasts (FP64 instructions per item) x
+// 64 cycles x the chunks of 32 items on the busiest sub-partition.  Chunk g goes
+// to warp g / cs of CTA g mod cs: the chunks spread over all 4 cs
+// sub-partitions of the cluster (a CTA-major order put every cell of a solve
+// of up to 512 cells on one SM).
 __device__ __forceinline__ void fused_sync(int cs) {
     if (cs > 1)
         cg::this_cluster().sync();
@@ -824,32 +963,43 @@ __device__ __forceinline__ void fused_sync(int cs) {
 
 __global__ void __launch_bounds__(MACRO_FUSED_THREADS, 1) k_macro_fused(const MacroJob* __restrict__ jobs, int cs) {
     const MacroJob& J = jobs[blockIdx.x / cs];
-    const int first = (blockIdx.x % cs) * blockDim.x + threadIdx.x, stride = cs * blockDim.x;
+    const int first = (((threadIdx.x >> 5) * cs + blockIdx.x % cs) << 5) + (threadIdx.x & 31), stride = cs * blockDim.x;
     const MacroArgs a = J.a;
-    const int N = a.N;
+    const int N = a.N, nf = N * J.ndir, nfp = face_items(N, J.ndir);
     for (int it = 0; it < J.steps; ++it) {
         for (int c = first; c < N; c += stride)
-            gradients_cell(a, J.Wm, 0, J.gu, J.gT, nullptr, nullptr, J.acell, c);
+            gradients_cell<false>(a, J.Wm, J.gu, J.gT, nullptr, nullptr, J.acell, c);
         fused_sync(cs);
-        for (int t = first; t < N * J.ndir + a.nbside; t += stride) {
-            if (t < N * J.ndir) face_flux_one(a, J.Wm, J.gu, J.gT, J.hot, J.acell, J.ndir, J.Ff, J.lamf, t);
-            else boundary_flux_one(a, J.Wm, J.gu, J.gT, J.hot, J.wall_corr, J.Fbnd, t - N * J.ndir);
+        for (int t = first; t < nfp + a.nbside; t += stride) {
+            if (t < nf) face_flux_one(a, J.Wm, J.gu, J.gT, J.hot, J.acell, J.Ff, J.lamf, t);
+            else if (t >= nfp) boundary_flux_one(a, J.Wm, J.gu, J.gT, J.hot, J.wall_corr, J.Fbnd, t - nfp);
         }
         fused_sync(cs);
         for (int c = first; c < N; c += stride)
-            cell_residual_one(a, J.Wm, J.U, J.Un, J.gu, J.gT, J.hot, J.Ff, J.lamf, J.Fbnd, J.cfl, J.dt, J.R,
-                              J.D, J.lamS, J.dU, J.F0, J.k_sub > 0 ? J.dFa : nullptr, c);
+            cell_residual_one(a, J.U, J.Un, J.Ff, J.lamf, J.Fbnd, J.cfl, J.dt, J.R, J.D, J.lamS, J.dU, J.F0,
+                              J.k_sub > 0 ? J.dFa : nullptr, c);
         fused_sync(cs);
         double* din = J.dU;
         double* dout = J.dU2;
-        for (int s = 0; s < J.k_sub; ++s) {
+        for (int s = 0; s + 1 < J.k_sub; ++s) {
             double* fin = (s & 1) ? J.dFb : J.dFa;
-            double* fout = s + 1 < J.k_sub ? ((s & 1) ? J.dFa : J.dFb) : nullptr;
-            for (int c = first; c < N; c += stride) relax_one(a, J.U, J.R, J.D, J.lamS, din, dout, fin, fout, J.F0, c);
+            double* fout = (s & 1) ? J.dFa : J.dFb;
+            double dUc[5];
+            for (int c = first; c < N; c += stride)
+                relax_one(a, J.U, J.R, J.D, J.lamS, din, dout, fin, fout, J.F0, c, dUc);
             fused_sync(cs);
             double* t = din; din = dout; dout = t;
         }
-        for (int c = first; c < N; c += stride) update_one(J.U, din, J.Wm, c);
+        if (J.k_sub > 0) {
+            for (int c = first; c < N; c += stride)
+                relax_update_one(a, J.U, J.R, J.D, J.lamS, din, (J.k_sub - 1) & 1 ? J.dFb : J.dFa, J.Wm, c);
+        } else {
+            for (int c = first; c < N; c += stride) {
+                double dUc[5];
+                for (int q = 0; q < 5; ++q) dUc[q] = din[(long long)q * N + c];
+                update_one(J.U, dUc, J.Wm, c);
+            }
+        }
         fused_sync(cs);
     }
 }
@@ -923,12 +1073,13 @@ void launch_macro_fused(const MacroJob* d_jobs, int njobs, cudaStream_t stream, 
     k_macro_fused<<<njobs, MACRO_FUSED_THREADS, 0, stream>>>(d_jobs, 1);
 }
 
-// Cluster size for one fused solve alone: one CTA (measured on the 200-cell
-// shock: a cluster of two CTAs was 8 % slower -- the phases are bound by
-// their dependent loads and the barriers, not by one SM's FP64 rate).
-int fused_cluster_for(int N) {
-    (void)N;
-    return 1;
+// Cluster size of one fused solve alone: the fewest CTAs (a power of two, at
+// most 8) that give every chunk of 32 faces a sub-partition of its own.
+int fused_cluster_for(int N, int ndir, int nbside) {
+    const int chunks = (face_items(N, ndir) + nbside + 31) / 32;
+    int want = 1;
+    while (want < 8 && 4 * want < chunks) want *= 2;
+    return fused_cluster_size(want);
 }
 
 // ---------------------------------------------------------------------------- persistent kernel
@@ -986,34 +1137,44 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier* bar, unsigned expected
 __global__ void __launch_bounds__(MACRO_PERSISTENT_THREADS, 2)
     k_macro_persistent(MacroJob J, GridBarrier* bar, unsigned long long spin_limit, int stall) {
     const MacroArgs a = J.a;
-    const int N = a.N;
+    const int N = a.N, nf = N * J.ndir, nfp = face_items(N, J.ndir);
     const int first = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
     // stall (test hook): the barrier waits for one block more than the grid
     // holds, so its wait can only end by running out of spin_limit polls
     const unsigned expected = gridDim.x + (stall ? 1u : 0u);
     for (int it = 0; it < J.steps; ++it) {
         for (int c = first; c < N; c += stride)
-            gradients_cell(a, J.Wm, 0, J.gu, J.gT, nullptr, nullptr, J.acell, c);
+            gradients_cell<false>(a, J.Wm, J.gu, J.gT, nullptr, nullptr, J.acell, c);
         if (!grid_barrier(bar, expected, spin_limit)) return;
-        for (int t = first; t < N * J.ndir + a.nbside; t += stride) {
-            if (t < N * J.ndir) face_flux_one(a, J.Wm, J.gu, J.gT, J.hot, J.acell, J.ndir, J.Ff, J.lamf, t);
-            else boundary_flux_one(a, J.Wm, J.gu, J.gT, J.hot, J.wall_corr, J.Fbnd, t - N * J.ndir);
+        for (int t = first; t < nfp + a.nbside; t += stride) {
+            if (t < nf) face_flux_one(a, J.Wm, J.gu, J.gT, J.hot, J.acell, J.Ff, J.lamf, t);
+            else if (t >= nfp) boundary_flux_one(a, J.Wm, J.gu, J.gT, J.hot, J.wall_corr, J.Fbnd, t - nfp);
         }
         if (!grid_barrier(bar, expected, spin_limit)) return;
         for (int c = first; c < N; c += stride)
-            cell_residual_one(a, J.Wm, J.U, J.Un, J.gu, J.gT, J.hot, J.Ff, J.lamf, J.Fbnd, J.cfl, J.dt, J.R,
-                              J.D, J.lamS, J.dU, J.F0, J.k_sub > 0 ? J.dFa : nullptr, c);
+            cell_residual_one(a, J.U, J.Un, J.Ff, J.lamf, J.Fbnd, J.cfl, J.dt, J.R, J.D, J.lamS, J.dU, J.F0, J.k_sub > 0 ? J.dFa : nullptr, c);
         if (!grid_barrier(bar, expected, spin_limit)) return;
         double* din = J.dU;
         double* dout = J.dU2;
-        for (int s = 0; s < J.k_sub; ++s) {
+        for (int s = 0; s + 1 < J.k_sub; ++s) {
             double* fin = (s & 1) ? J.dFb : J.dFa;
-            double* fout = s + 1 < J.k_sub ? ((s & 1) ? J.dFa : J.dFb) : nullptr;
-            for (int c = first; c < N; c += stride) relax_one(a, J.U, J.R, J.D, J.lamS, din, dout, fin, fout, J.F0, c);
+            double* fout = (s & 1) ? J.dFa : J.dFb;
+            double dUc[5];
+            for (int c = first; c < N; c += stride)
+                relax_one(a, J.U, J.R, J.D, J.lamS, din, dout, fin, fout, J.F0, c, dUc);
             if (!grid_barrier(bar, expected, spin_limit)) return;
             double* t = din; din = dout; dout = t;
         }
-        for (int c = first; c < N; c += stride) update_one(J.U, din, J.Wm, c);
+        if (J.k_sub > 0) {
+            for (int c = first; c < N; c += stride)
+                relax_update_one(a, J.U, J.R, J.D, J.lamS, din, (J.k_sub - 1) & 1 ? J.dFb : J.dFa, J.Wm, c);
+        } else {
+            for (int c = first; c < N; c += stride) {
+                double dUc[5];
+                for (int q = 0; q < 5; ++q) dUc[q] = din[(long long)q * N + c];
+                update_one(J.U, dUc, J.Wm, c);
+            }
+        }
         if (!grid_barrier(bar, expected, spin_limit)) return;
     }
 }
@@ -1078,7 +1239,7 @@ void macro_block(gsis_ctx* c, int steps, bool with_hot, bool time_term, bool cap
     if (path == MACRO_FUSED) {
         MacroJob J = macro_job(c, steps, time_term);
         cudaMemcpyAsync(c->d_job, &J, sizeof(MacroJob), cudaMemcpyHostToDevice, c->stream);
-        launch_macro_fused(c->d_job, 1, c->stream, fused_cluster_for(N));
+        launch_macro_fused(c->d_job, 1, c->stream, fused_cluster_for(N, c->normal_components, c->m.nbside));
         c->launches++;
         return;
     }
@@ -1089,15 +1250,14 @@ void macro_block(gsis_ctx* c, int steps, bool with_hot, bool time_term, bool cap
     const int TB = 64;
     const int nb = (N + TB - 1) / TB;
     const int ndir = c->normal_components;   // index directions that carry flux
-    const int nf = (N * ndir + c->m.nbside + TB - 1) / TB;   // faces, then the boundary sides
+    const int nf = (face_items(N, ndir) + c->m.nbside + TB - 1) / TB;   // faces, then the boundary sides
     MacroArgs a = margs(c);
     const double dt = time_term ? c->p.dt : 0.0;
     for (int it = 0; it < steps; ++it) {
         launch_gradients(c, c->Wm, false);
         k_face_flux<<<nf, TB, 0, c->stream>>>(a, c->Wm, c->gu, c->gT, c->hot, c->acell, ndir, c->Ff, c->lamf,
                                                c->wall_corr, c->Fbnd);
-        k_cell_residual<<<nb, TB, 0, c->stream>>>(a, c->Wm, c->U, c->Un, c->gu, c->gT, c->hot, c->Ff, c->lamf,
-                                                  c->Fbnd, c->p.cfl, dt, c->R, c->D, c->lamS, c->dU, c->F0,
+        k_cell_residual<<<nb, TB, 0, c->stream>>>(a, c->U, c->Un, c->Ff, c->lamf, c->Fbnd, c->p.cfl, dt, c->R, c->D, c->lamS, c->dU, c->F0,
                                                   c->p.k_sub > 0 ? c->dFa : nullptr);
         c->launches += 2;
         double* din = c->dU;
@@ -1108,7 +1268,7 @@ void macro_block(gsis_ctx* c, int steps, bool with_hot, bool time_term, bool cap
                 double* fout = (s & 1) ? c->dFa : c->dFb;
                 k_relax<<<nb, TB, 0, c->stream>>>(a, c->U, c->R, c->D, c->lamS, din, dout, fin, fout, c->F0);
             } else {
-                k_relax_update<<<nb, TB, 0, c->stream>>>(a, c->U, c->R, c->D, c->lamS, din, dout, fin, c->Wm);
+                k_relax_update<<<nb, TB, 0, c->stream>>>(a, c->U, c->R, c->D, c->lamS, din, fin, c->Wm);
             }
             c->launches++;
             double* t = din; din = dout; dout = t;
