@@ -21,258 +21,285 @@
 
 namespace gsis {
 
-struct Term { double c; int a, b, d; };
-
-__device__ static int psi_terms(int row, const double* u, Term* t, double scale) {
-    // psi_row in powers of c (c = xi - u); scale = 1 for psi, 2 for phi_4 only
-    switch (row) {
-        case 0: t[0] = {1.0, 0, 0, 0}; return 1;
-        case 1: t[0] = {1.0, 1, 0, 0}; t[1] = {u[0], 0, 0, 0}; return 2;
-        case 2: t[0] = {1.0, 0, 1, 0}; t[1] = {u[1], 0, 0, 0}; return 2;
-        case 3: t[0] = {1.0, 0, 0, 1}; t[1] = {u[2], 0, 0, 0}; return 2;
-        default: {
-            double h = 0.5 * scale;
-            t[0] = {h, 2, 0, 0}; t[1] = {h, 0, 2, 0}; t[2] = {h, 0, 0, 2};
-            t[3] = {scale * u[0], 1, 0, 0}; t[4] = {scale * u[1], 0, 1, 0}; t[5] = {scale * u[2], 0, 0, 1};
-            t[6] = {h * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]), 0, 0, 0};
-            return 7;
+// Conservation correction of one record.  C[d][k] = sum_i e_d c_d^k over the
+// axis nodes; every moment sum of the correction system is a sum of products
+// C[0][a] C[1][b] C[2][c].  Written in powers of c (the polynomials 1, c, c^2
+// span the same space as 1, xi, |xi|^2, and about u the target is (rho, 0, 0,
+// 0, 3 rho T)), the system is the Gram matrix of (1, c_x, c_y, c_z, c^2) under
+// the Maxwellian weight: symmetric positive definite, solved by an L D L^T
+// factorisation without pivoting.  On return a[5] are the coefficients of
+// (1, c, c^2) to be added to the base polynomial.
+// (The generic form -- all products of the terms of psi and phi in xi, a pivoted
+// elimination -- cost up to 250 FP64 operations per matrix entry, serially: 50 us
+// for one record.)
+__device__ __forceinline__ void correction_coefs(const RecSpec& s, const double (&C)[3][6], double wA, double* a) {
+    const double* X[3] = {C[0], C[1], C[2]};
+    double G[5][5], b[5];   // lower triangle
+    double p2[3];           // products of the other two axes: (0,0) and (2,0) + (0,2)
+    double w2[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const int e = (d + 1) % 3, f = (d + 2) % 3;
+        p2[d] = X[e][0] * X[f][0];
+        w2[d] = fma(X[e][2], X[f][0], X[e][0] * X[f][2]);
+    }
+    G[0][0] = X[0][0] * p2[0];
+    double t22 = 0.0, t4 = 0.0;   // <c_d^2 c_e^2> and <c_d^4> summed
+    G[4][0] = 0.0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        G[1 + d][0] = X[d][1] * p2[d];
+        G[1 + d][1 + d] = X[d][2] * p2[d];
+        G[4][0] += G[1 + d][1 + d];
+        G[4][1 + d] = fma(X[d][3], p2[d], X[d][1] * w2[d]);
+        t4 = fma(X[d][4], p2[d], t4);
+        t22 = fma(X[d][2], w2[d], t22);   // each pair twice
+    }
+    G[2][1] = X[0][1] * X[1][1] * X[2][0];
+    G[3][1] = X[0][1] * X[1][0] * X[2][1];
+    G[3][2] = X[0][0] * X[1][1] * X[2][1];
+    G[4][4] = t4 + t22;
+    // right-hand side: target minus the moments of the base polynomial
+    const double target = s.rho / wA;
+    b[0] = fma(-s.p0, G[0][0], target);
+    b[4] = fma(-s.p0, G[4][0], 3.0 * s.T * target);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) b[1 + d] = -s.p0 * G[1 + d][0];
+    const bool odd = s.r[0] != 0.0 || s.r[1] != 0.0 || s.r[2] != 0.0 || s.p[0] != 0.0 || s.p[1] != 0.0 || s.p[2] != 0.0;
+    const bool stress = s.P2[0] != 0.0 || s.P2[1] != 0.0 || s.P2[2] != 0.0 || s.P2[3] != 0.0 || s.P2[4] != 0.0 ||
+                        s.P2[5] != 0.0;
+    if (odd || stress) {
+        // S_de = <c_d c_e c^2>
+        double S[3][3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            S[d][d] = fma(X[d][4], p2[d], X[d][2] * w2[d]);
+            const int e = (d + 1) % 3, f = (d + 2) % 3;
+            const double v = fma(fma(X[d][3], X[e][1], X[d][1] * X[e][3]), X[f][0], X[d][1] * X[e][1] * X[f][2]);
+            S[d][e] = v;
+            S[e][d] = v;
         }
+        if (odd) {   // p.c + (r.c) c^2
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int e = (d + 1) % 3, f = (d + 2) % 3;
+                const double q4 = fma(X[e][4], X[f][0], fma(X[e][0], X[f][4], 2.0 * X[e][2] * X[f][2]));
+                const double Q = fma(X[d][5], p2[d], fma(2.0 * X[d][3], w2[d], X[d][1] * q4));   // <c_d c^4>
+                b[0] -= fma(s.p[d], G[1 + d][0], s.r[d] * G[4][1 + d]);
+                b[4] -= fma(s.p[d], G[4][1 + d], s.r[d] * Q);
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    b[1 + k] -= fma(s.p[d], k >= d ? G[1 + k][1 + d] : G[1 + d][1 + k], s.r[d] * S[k][d]);
+            }
+        }
+        if (stress) {   // c.P2.c, with P2 = (xx, yy, zz, xy, xz, yz)
+            const double P[3][3] = {{s.P2[0], s.P2[3], s.P2[4]}, {s.P2[3], s.P2[1], s.P2[5]}, {s.P2[4], s.P2[5], s.P2[2]}};
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+#pragma unroll
+                for (int e = 0; e < 3; ++e) {
+                    b[0] = fma(-P[d][e], d >= e ? G[1 + d][1 + e] : G[1 + e][1 + d], b[0]);
+                    b[4] = fma(-P[d][e], S[d][e], b[4]);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {   // <c_k c_d c_e>
+                        double m = 1.0;
+#pragma unroll
+                        for (int x = 0; x < 3; ++x) m *= X[x][(k == x) + (d == x) + (e == x)];
+                        b[1 + k] = fma(-P[d][e], m, b[1 + k]);
+                    }
+                }
+        }
+    }
+    // L D L^T
+    double L[5][5], iD[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        double V[5];
+#pragma unroll
+        for (int k = 0; k < j; ++k) V[k] = L[j][k];   // holds L[j][k] D[k] until scaled
+        double dj = G[j][j];
+#pragma unroll
+        for (int k = 0; k < j; ++k) {
+            L[j][k] = V[k] * iD[k];
+            dj = fma(-L[j][k], V[k], dj);
+        }
+        iD[j] = recip64(dj);
+#pragma unroll
+        for (int i = j + 1; i < 5; ++i) {   // column j of the rows below: G_ij - sum_k L_ik D_k L_jk
+            double v = G[i][j];
+#pragma unroll
+            for (int k = 0; k < j; ++k) v = fma(-L[i][k], L[j][k], v);
+            L[i][j] = v;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 5; ++j)
+#pragma unroll
+        for (int k = 0; k < j; ++k) b[j] = fma(-L[j][k], b[k], b[j]);
+#pragma unroll
+    for (int j = 4; j >= 0; --j) {
+        a[j] = b[j] * iD[j];
+#pragma unroll
+        for (int i = j + 1; i < 5; ++i) a[j] = fma(-L[i][j], a[i], a[j]);
     }
 }
 
-// Terms of the base polynomial with a nonzero coefficient (a Maxwellian has only
-// p0; skipping the zero terms leaves its moment sums 19 times shorter, and a
-// zero term contributes exactly zero to them).
-__device__ static int base_terms(const RecSpec& s, Term* t) {
-    const Term all[19] = {
-        {s.p0, 0, 0, 0},
-        {s.p[0], 1, 0, 0}, {s.p[1], 0, 1, 0}, {s.p[2], 0, 0, 1},
-        {s.P2[0], 2, 0, 0}, {s.P2[1], 0, 2, 0}, {s.P2[2], 0, 0, 2},
-        {2.0 * s.P2[3], 1, 1, 0}, {2.0 * s.P2[4], 1, 0, 1}, {2.0 * s.P2[5], 0, 1, 1},
-        {s.r[0], 3, 0, 0}, {s.r[0], 1, 2, 0}, {s.r[0], 1, 0, 2},
-        {s.r[1], 2, 1, 0}, {s.r[1], 0, 3, 0}, {s.r[1], 0, 1, 2},
-        {s.r[2], 2, 0, 1}, {s.r[2], 0, 2, 1}, {s.r[2], 0, 0, 3}};
-    int n = 0;
-    for (int i = 0; i < 19; ++i)
-        if (all[i].c != 0.0) t[n++] = all[i];
-    return n;
-}
-
-__device__ static double poly_moment(const Term* t1, int n1, const Term* t2, int n2, const double (*Cs)[6]) {
-    double s = 0.0;
-    for (int i = 0; i < n1; ++i)
-        for (int j = 0; j < n2; ++j)
-            s += t1[i].c * t2[j].c * (Cs[0][t1[i].a + t2[j].a] * Cs[1][t1[i].b + t2[j].b] * Cs[2][t1[i].d + t2[j].d]);
-    return s;
-}
-
-// Solve A x = b (5x5) by Gaussian elimination with partial pivoting.
-__device__ static void solve5(double A[5][5], double b[5], double x[5]) {
-    for (int col = 0; col < 5; ++col) {
-        int piv = col;
-        double best = fabs(A[col][col]);
-        for (int r = col + 1; r < 5; ++r)
-            if (fabs(A[r][col]) > best) { best = fabs(A[r][col]); piv = r; }
-        if (piv != col) {
-            for (int k = 0; k < 5; ++k) { double t = A[col][k]; A[col][k] = A[piv][k]; A[piv][k] = t; }
-            double t = b[col]; b[col] = b[piv]; b[piv] = t;
-        }
-        for (int r = col + 1; r < 5; ++r) {
-            double m = A[r][col] / A[col][col];
-            for (int k = col; k < 5; ++k) A[r][k] -= m * A[col][k];
-            b[r] -= m * b[col];
-        }
-    }
-    for (int r = 4; r >= 0; --r) {
-        double s = b[r];
-        for (int k = r + 1; k < 5; ++k) s -= A[r][k] * x[k];
-        x[r] = s / A[r][r];
-    }
-}
-
-// Four records per warp, eight lanes (a "group") per record: the FP64
-// operations of a warp instruction cost the same whatever the number of active
-// lanes, so the per-record serial parts (the 5 x 5 solve, the reductions) run
-// for four records at once.  Lanes of a group split the 1D nodes and the 30
-// entries of the correction system; every shuffle is segmented to the group.
-constexpr int REC_LANES = 8;
-constexpr int REC_PER_WARP = 32 / REC_LANES;
-
+// LPR lanes (a "group") per record: the FP64 operations of a warp instruction
+// cost the same whatever the number of active lanes, so with many records four
+// share a warp (LPR = 8) and the serial correction runs for all four at once;
+// with few, a record has the whole warp (LPR = 32: fewer nodes per lane).  The
+// records [0, n0) go to out0, [n0, nrec) to out1.
+template <int LPR>
 __device__ __forceinline__ double group_sum(double v) {
 #pragma unroll
-    for (int o = REC_LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, REC_LANES);
+    for (int o = LPR / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, LPR);
     return v;
 }
 
-__global__ void k_build_records(const RecSpec* __restrict__ specs, int nrec, Records out, VGridDev vg) {
-    const int lane = threadIdx.x & 31, sl = lane & (REC_LANES - 1);
+template <int LPR>
+__global__ void k_build_records(const RecSpec* __restrict__ specs, int nrec, int n0, Records out0, Records out1,
+                                VGridDev vg) {
+    constexpr int PER_WARP = 32 / LPR;
+    const int lane = threadIdx.x & 31, sl = lane & (LPR - 1);
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (warp * REC_PER_WARP >= nrec) return;   // the whole warp is past the last record
-    const int r0 = warp * REC_PER_WARP + (lane / REC_LANES);
+    if (warp * PER_WARP >= nrec) return;       // the whole warp is past the last record
+    const int r0 = warp * PER_WARP + (lane / LPR);
     const bool valid = r0 < nrec;              // groups past the end compute a copy and store nothing
-    const int r = valid ? r0 : nrec - 1;
-    const RecSpec s = specs[r];
+    const int rr = valid ? r0 : nrec - 1;
+    const RecSpec s = specs[rr];
+    const Records& out = rr < n0 ? out0 : out1;
+    const long long r = rr < n0 ? rr : rr - n0;
     const int NT = vg.NT, nx = vg.nx, ny = vg.ny;
-    double* tab = out.tab + (long long)r * NTAB * NT;
-    double* scal = out.scal + (long long)r * RS;
+    double* tab = out.tab + r * NTAB * NT;
+    double* scal = out.scal + r * RS;
     const double T = s.T;
-    const double A = s.rho * pow(2.0 * PI * T, -1.5);
-    double part[3][6];
+    const double ist = rsqrt(2.0 * PI * T), A = s.rho * (ist * ist * ist);   // rho (2 pi T)^(-3/2)
+    double C[3][6];
     for (int d = 0; d < 3; ++d)
-        for (int k = 0; k < 6; ++k) part[d][k] = 0.0;
+        for (int k = 0; k < 6; ++k) C[d][k] = 0.0;
     // reduced grid: the z "nodes" are the planes G (p = 0) and H (p = 1); integrating the separable form
     // over xi_z (u_z = r_z = 0 and no xz / yz stress in a flow without z dependence) leaves the same form
     // with the plane values E_z = int xi_z^{2p} e_z dxi_z = sqrt(2 pi T) (1, T), C_z = 0 and
     // C2_z = (2p + 1) T, the ratio of the Gaussian moments 3T^2 / T and T / 1
-    const double sq2piT = sqrt(2.0 * PI * T);
+    const double sq2piT = 2.0 * PI * T * ist;
     const double i2T = 0.5 / T;   // exp(-c^2 / (2T)) as exp(-c^2 * i2T): one division per record, not per node
 #pragma unroll
     for (int d = 0; d < 3; ++d) {   // the axes' node ranges in turn (static axis index for the sums)
         const int lo = d == 0 ? 0 : (d == 1 ? nx : nx + ny), hi = d == 0 ? nx : (d == 1 ? nx + ny : NT);
-        for (int idx = lo + sl; idx < hi; idx += REC_LANES) {
-            if (vg.reduced && d == 2) {
-                const int p = idx - nx - ny;
-                if (valid) {
-                    tab[idx] = p ? sq2piT * T : sq2piT;
-                    tab[2 * NT + idx] = 0.0;
-                    tab[3 * NT + idx] = p ? 3.0 * T : T;
-                }
-                continue;
-            }
-            const double c = vg.xi[idx] - s.u[d];
-            const double e = exp(-(c * c) * i2T);
-            if (valid) {
-                tab[idx] = e;
-                tab[2 * NT + idx] = c;
-                tab[3 * NT + idx] = c * c;
-            }
-            double pw = e;
-#pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                part[d][k] += pw;
-                pw *= c;
-            }
+        if (vg.reduced && d == 2) continue;
+        for (int idx = lo + sl; idx < hi; idx += LPR) {
+            const double c = vg.xi[idx] - s.u[d], c2 = c * c;
+            const double e = exp(-c2 * i2T);
+            if (valid) tab[idx] = e;
+            // e c^k for k = 0..5
+            const double e1 = e * c, e2 = e * c2, e3 = e1 * c2;
+            C[d][0] += e;
+            C[d][1] += e1;
+            C[d][2] += e2;
+            C[d][3] += e3;
+            C[d][4] = fma(e2, c2, C[d][4]);
+            C[d][5] = fma(e3, c2, C[d][5]);
         }
     }
-    double Cs[3][6];
+#pragma unroll
     for (int d = 0; d < 3; ++d)
-        for (int k = 0; k < 6; ++k) Cs[d][k] = group_sum(part[d][k]);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) C[d][k] = group_sum<LPR>(C[d][k]);
     if (vg.reduced) {   // exact xi_z integrals int c_z^k e_z dxi_z of the Gaussian (k = 0..5)
         const double zk[6] = {1.0, 0.0, T, 0.0, 3.0 * T * T, 0.0};
-        for (int k = 0; k < 6; ++k) Cs[2][k] = sq2piT * zk[k];
+        for (int k = 0; k < 6; ++k) C[2][k] = sq2piT * zk[k];
     }
-
-    // the 5 right-hand sides (entries 0-4) and 25 matrix entries (5-29) of the
-    // correction system, entry e on lane e % 8 of the group (slot e / 8), gathered
-    // on the group's first lane
-    double mine[4] = {0.0, 0.0, 0.0, 0.0};
-    if (s.correct) {
-        Term tp[7], tq[19];
-        const double wa = vg.w * A;
+    double alpha[5] = {0, 0, 0, 0, 0};
+    if (s.correct) correction_coefs(s, C, vg.w * A, alpha);
+    const double p0 = s.p0 + alpha[0];
+    double pp[3], p2d[3];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const int e = sl + REC_LANES * m;
-            if (e < 5) {
-                const int na = psi_terms(e, s.u, tp, 1.0);
-                const int nb = base_terms(s, tq);
-                mine[m] = s.U[e] - wa * poly_moment(tp, na, tq, nb, Cs);
-            } else if (e < 30) {
-                const int ra = (e - 5) / 5, rb = (e - 5) % 5;
-                const int na = psi_terms(ra, s.u, tp, 1.0);
-                const int nbb = psi_terms(rb, s.u, tq, rb == 4 ? 2.0 : 1.0);
-                mine[m] = wa * poly_moment(tp, na, tq, nbb, Cs);
-            }
-        }
+    for (int d = 0; d < 3; ++d) {
+        pp[d] = s.p[d] + alpha[1 + d];
+        p2d[d] = s.P2[d] + alpha[4];
     }
-    double Am[5][5], rhs[5];
+    if (valid && sl == 0) {
+        scal[RS_P0] = p0;
+        scal[RS_P2XY] = s.P2[3];
+        scal[RS_P2XZ] = s.P2[4];
+        scal[RS_P2YZ] = s.P2[5];
+        scal[RS_OFFD] = (s.P2[3] != 0.0 || s.P2[4] != 0.0 || s.P2[5] != 0.0) ? 1.0 : 0.0;
+        scal[RS_AMP] = A;
 #pragma unroll
-    for (int e = 0; e < 30; ++e) {
-        const double v = __shfl_sync(0xffffffffu, mine[e / REC_LANES], e % REC_LANES, REC_LANES);
-        if (e < 5) rhs[e] = v;
-        else Am[(e - 5) / 5][(e - 5) % 5] = v;
-    }
-    double coef[7];   // p0', p'(3), P2'(diag 3)
-    if (sl == 0) {
-        double pp[3] = {s.p[0], s.p[1], s.p[2]};
-        double p2d[3] = {s.P2[0], s.P2[1], s.P2[2]};
-        double p0 = s.p0;
-        double alpha[5] = {0, 0, 0, 0, 0};
-        if (s.correct) {
-            solve5(Am, rhs, alpha);
-            const double ua = alpha[1] * s.u[0] + alpha[2] * s.u[1] + alpha[3] * s.u[2];
-            const double u2 = s.u[0] * s.u[0] + s.u[1] * s.u[1] + s.u[2] * s.u[2];
-            p0 = s.p0 + alpha[0] + ua + alpha[4] * u2;
-            for (int d = 0; d < 3; ++d) {
-                pp[d] = s.p[d] + alpha[1 + d] + 2.0 * alpha[4] * s.u[d];
-                p2d[d] = s.P2[d] + alpha[4];
-            }
-        }
-        coef[0] = p0;
-        for (int d = 0; d < 3; ++d) { coef[1 + d] = pp[d]; coef[4 + d] = p2d[d]; }
-        if (valid) {
-            scal[RS_P0] = p0;
-            scal[RS_P2XY] = s.P2[3];
-            scal[RS_P2XZ] = s.P2[4];
-            scal[RS_P2YZ] = s.P2[5];
-            scal[RS_OFFD] = (s.P2[3] != 0.0 || s.P2[4] != 0.0 || s.P2[5] != 0.0) ? 1.0 : 0.0;
-            scal[RS_UX] = s.u[0];
-            scal[RS_UY] = s.u[1];
-            scal[RS_UZ] = s.u[2];
-            for (int k = 0; k < 5; ++k) scal[RS_ALPHA0 + k] = alpha[k];
-            for (int q = RS_ALPHA0 + 5; q < RS; ++q) scal[q] = 0.0;
+        for (int d = 0; d < 3; ++d) {
+            scal[RS_U + d] = s.u[d];
+            scal[RS_P + d] = pp[d];
+            scal[RS_P2D + d] = p2d[d];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) scal[RS_SUMS + 6 * d + k] = C[d][k];
         }
     }
-    for (int k = 0; k < 7; ++k) coef[k] = __shfl_sync(0xffffffffu, coef[k], 0, REC_LANES);
-    __syncwarp();   // the table values of the first loop, written by other lanes of the group, are read below
+    __syncwarp();   // the record's values written by other lanes of the group are read below
     if (valid) {
-        for (int idx = sl; idx < NT; idx += REC_LANES) {
-            const int d = idx < nx ? 0 : (idx < nx + ny ? 1 : 2);
-            const double c = tab[2 * NT + idx];
-            tab[NT + idx] = coef[1 + d] * c + coef[4 + d] * tab[3 * NT + idx];   // C2 = c^2 (plane value if reduced)
-            tab[4 * NT + idx] = s.r[d] * c;
-            if (d == 0) tab[idx] *= A;
-            if (out.tabf) {   // FP32 copies in stored units: E_x carries the VDF storage scale once
-                float* tf = out.tabf + (long long)r * NTAB * NT;
-                for (int t = 0; t < NTAB; ++t)
-                    tf[t * NT + idx] = (float)(t == 0 && d == 0 ? tab[idx] * vg.vscale : tab[t * NT + idx]);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int lo = d == 0 ? 0 : (d == 1 ? nx : nx + ny), hi = d == 0 ? nx : (d == 1 ? nx + ny : NT);
+            for (int idx = lo + sl; idx < hi; idx += LPR) {
+                double E, c, c2;
+                if (vg.reduced && d == 2) {
+                    const int p = idx - nx - ny;
+                    E = p ? sq2piT * T : sq2piT;
+                    c = 0.0;
+                    c2 = p ? 3.0 * T : T;
+                } else {
+                    E = tab[idx];
+                    c = vg.xi[idx] - s.u[d];
+                    c2 = c * c;
+                }
+                if (d == 0) E *= A;
+                const double v[NTAB] = {E, fma(pp[d], c, p2d[d] * c2), c, c2, s.r[d] * c};
+#pragma unroll
+                for (int t = 0; t < NTAB; ++t) tab[t * NT + idx] = v[t];
+                if (out.tabf) {   // FP32 copies in stored units: E_x carries the VDF storage scale once
+                    float* tf = out.tabf + r * NTAB * NT;
+#pragma unroll
+                    for (int t = 0; t < NTAB; ++t) tf[t * NT + idx] = (float)(t == 0 && d == 0 ? v[t] * vg.vscale : v[t]);
+                }
             }
         }
         if (out.scalf)
-            for (int q = sl; q < RS; q += REC_LANES) out.scalf[(long long)r * RS + q] = (float)scal[q];
+            for (int q = sl; q <= RS_OFFD; q += LPR) out.scalf[r * RS + q] = (float)scal[q];
+    }
+}
+
+// Records [0, n0) into out0 and the rest into out1.  A record per warp while the
+// warps leave sub-partitions idle (2,048 records: about three warps each), four
+// above.
+static void build_records(const RecSpec* d_specs, int nrec, int n0, const Records& out0, const Records& out1,
+                          const VGridDev& vg, cudaStream_t st) {
+    if (nrec <= 0) return;
+    const int threads = 64;
+    if (nrec <= 2048) {
+        const int blocks = (nrec * 32 + threads - 1) / threads;
+        k_build_records<32><<<blocks, threads, 0, st>>>(d_specs, nrec, n0, out0, out1, vg);
+    } else {
+        const int blocks = ((nrec + 3) / 4 * 32 + threads - 1) / threads;
+        k_build_records<8><<<blocks, threads, 0, st>>>(d_specs, nrec, n0, out0, out1, vg);
     }
 }
 
 // Context-free launcher of the record builder (caller supplies every buffer).
 void build_records_raw(const RecSpec* d_specs, int nrec, const Records& out, const VGridDev& vg, cudaStream_t st) {
-    if (nrec <= 0) return;
-    const int threads = 128;
-    const int warps = (nrec + REC_PER_WARP - 1) / REC_PER_WARP;
-    const int blocks = (warps * 32 + threads - 1) / threads;
-    k_build_records<<<blocks, threads, 0, st>>>(d_specs, nrec, out, vg);
+    build_records(d_specs, nrec, nrec, out, out, vg, st);
 }
 
 void launch_build_records(gsis_ctx* c, const Records& out, int nrec, const RecSpec* d_specs) {
     if (nrec <= 0) return;
-    const int threads = 128;
-    const int warps = (nrec + REC_PER_WARP - 1) / REC_PER_WARP;
-    const int blocks = (warps * 32 + threads - 1) / threads;
-    k_build_records<<<blocks, threads, 0, c->stream>>>(d_specs, nrec, out, c->vg);
+    build_records(d_specs, nrec, nrec, out, out, c->vg, c->stream);
     c->launches++;
 }
 
 // ---------------------------------------------------------------------------- spec builders
-__device__ static void cons_of(double rho, const double* u, double T, double* U) {
-    U[0] = rho;
-    U[1] = rho * u[0]; U[2] = rho * u[1]; U[3] = rho * u[2];
-    U[4] = rho * (1.5 * T + 0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
-}
-
 __device__ static void spec_maxwellian(RecSpec& s, double rho, const double* u, double T, int correct) {
     s.rho = rho; s.T = T;
     for (int d = 0; d < 3; ++d) { s.u[d] = u[d]; s.p[d] = 0.0; s.r[d] = 0.0; }
     for (int k = 0; k < 6; ++k) s.P2[k] = 0.0;
     s.p0 = 1.0;
-    cons_of(rho, u, T, s.U);
     s.correct = correct;
 }
 
@@ -494,12 +521,12 @@ void launch_ghost_records(gsis_ctx* c) {
     launch_build_records(c, c->recGhost, c->n_ghost, c->specs);
 }
 
-// M~(W^{n+1}) and M~(W^{n+1/2}) for Eq. updatef.
-__global__ void k_corr_specs(int Nd, const int* __restrict__ dvm_cell, const double* __restrict__ Wa,
-                             RecSpec* specs) {
+// M~(W^{n+1}) and M~(W^{n+1/2}) for Eq. updatef: specs [0, Nd) and [Nd, 2 Nd).
+__global__ void k_corr_specs(int Nd, const int* __restrict__ dvm_cell, const double* __restrict__ Wnew,
+                             const double* __restrict__ Whalf, RecSpec* specs) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= Nd) return;
-    const double* w = Wa + dvm_cell[k] * 5;
+    if (k >= 2 * Nd) return;
+    const double* w = k < Nd ? Wnew + dvm_cell[k] * 5 : Whalf + dvm_cell[k - Nd] * 5;
     const double u[3] = {w[1], w[2], w[3]};
     RecSpec s;
     spec_maxwellian(s, w[0], u, w[4], 1);
@@ -509,12 +536,9 @@ __global__ void k_corr_specs(int Nd, const int* __restrict__ dvm_cell, const dou
 void launch_correction_records(gsis_ctx* c) {
     const int Nd = (int)c->Nd;
     if (Nd == 0) return;
-    k_corr_specs<<<(Nd + 127) / 128, 128, 0, c->stream>>>(Nd, c->dvm_cell, c->W, c->specs);
-    c->launches++;
-    launch_build_records(c, c->recNew, Nd, c->specs);
-    k_corr_specs<<<(Nd + 127) / 128, 128, 0, c->stream>>>(Nd, c->dvm_cell, c->Wh, c->specs);
-    c->launches++;
-    launch_build_records(c, c->recHalf, Nd, c->specs);
+    k_corr_specs<<<(2 * Nd + 127) / 128, 128, 0, c->stream>>>(Nd, c->dvm_cell, c->W, c->Wh, c->specs);
+    build_records(c->specs, 2 * Nd, Nd, c->recNew, c->recHalf, c->vg, c->stream);
+    c->launches += 2;
 }
 
 // Seed distributions for cells entering the DVM region: Grad-13 from W and

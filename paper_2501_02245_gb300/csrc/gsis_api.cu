@@ -980,7 +980,7 @@ gsis_status gsis_set_mesh(gsis_ctx* c, const gsis_mesh_desc* md) {
     c->wall_corr = (double*)dev_alloc(c, (size_t)N * 30 * sizeof(double));
     c->has_wall = false;
     for (int s = 0; s < 6; ++s) c->has_wall = c->has_wall || md->bc_type[s] == GSIS_BC_WALL;
-    c->eps_buf = (double*)dev_alloc(c, 4 * sizeof(double));
+    c->eps_buf = (double*)dev_alloc(c, (4 + EPS_BLOCKS * 7) * sizeof(double));   // result, then partial sums
     c->flag = (uint8_t*)dev_alloc(c, N);
     c->cell2dvm = (int*)dev_alloc(c, N * sizeof(int));
     c->old_cell2dvm = (int*)dev_alloc(c, N * sizeof(int));
@@ -992,7 +992,7 @@ gsis_status gsis_set_mesh(gsis_ctx* c, const gsis_mesh_desc* md) {
     c->d_count = (int*)dev_alloc(c, 4 * sizeof(int));
     c->d_job = (gsis::MacroJob*)dev_alloc(c, sizeof(gsis::MacroJob));
     c->d_bar = (gsis::GridBarrier*)dev_alloc(c, sizeof(gsis::GridBarrier));
-    c->specs = (RecSpec*)dev_alloc(c, (size_t)std::max(N, 6) * sizeof(RecSpec));
+    c->specs = (RecSpec*)dev_alloc(c, (size_t)std::max(2 * N, 6) * sizeof(RecSpec));   // (2 N: both records of Eq. updatef)
     c->recGhost.scal = (double*)dev_alloc(c, (size_t)N * RS * sizeof(double));
     c->recBC.scal = (double*)dev_alloc(c, 6 * RS * sizeof(double));
     if (!c->d_job || !c->d_bar || !m.cen || !m.vol || !m.Sout || !m.xf || !m.lsq_w || !m.nbr || !m.side_bc || !m.hyper || !m.bside || !c->Fbnd || !c->W || !c->Wmom ||

@@ -21,16 +21,18 @@
 
 namespace gsis {
 
-constexpr int RS = 16;          // scalars per distribution record
+constexpr int RS = 40;          // scalars per distribution record
 constexpr int NTAB = 5;         // axis tables per record: E, B, C, C2, R
 constexpr int MOMN = 19;        // 13 velocity moments + 6 wall half-range fluxes
 constexpr int HOTN = 9;         // sigma xx,yy,zz,xy,xz,yz; q x,y,z
 constexpr int FIELDS_N = 15;    // derived fields per cell: constitutive sigma (6), q (3), p; wall loads
 constexpr int FIELD_WALL = 10;  // wall heat flux, pressure, shear x/y/z
 
-// record scalar slots
-enum { RS_P0 = 0, RS_P2XY = 1, RS_P2XZ = 2, RS_P2YZ = 3, RS_OFFD = 4, RS_UX = 5, RS_UY = 6, RS_UZ = 7,
-       RS_ALPHA0 = 8 };
+// record scalar slots: polynomial p0 and off-diagonal P2 (the FP32 copy holds these), then what the
+// record's velocity moments need: centre u, amplitude of E_x, p and diagonal P2 of the corrected
+// polynomial, axis sums sum_i e c^k (k < 6) of each axis
+enum { RS_P0 = 0, RS_P2XY = 1, RS_P2XZ = 2, RS_P2YZ = 3, RS_OFFD = 4, RS_U = 5, RS_AMP = 8, RS_P = 9, RS_P2D = 12,
+       RS_SUMS = 15 };
 
 // DVM side kinds
 enum { SK_NONE = 0, SK_DVM = 1, SK_GHOST = 2, SK_FAR = 3, SK_WALL = 4 };
@@ -75,11 +77,11 @@ struct Records {                 // R records
 };
 
 // Base polynomial of a record in c = xi - u:
-//   p0 + p.c + c.P2.c + (r.c) c^2, optionally conservation-corrected to U.
+//   p0 + p.c + c.P2.c + (r.c) c^2, optionally conservation-corrected to the
+// discrete mass, momentum and energy of (rho, u, T).
 struct RecSpec {
     double rho, u[3], T;         // Maxwellian factor
     double p0, p[3], P2[6], r[3];
-    double U[5];                 // target conserved moments (rho, rho u, rho E)
     int correct;
 };
 
@@ -129,6 +131,7 @@ struct MacroJob {
 };
 
 constexpr int FGEO_N = 12;      // face geometry values (MacroArgs::fgeo)
+constexpr int EPS_BLOCKS = 304;      // blocks of the residual's first launch
 constexpr int MACRO_FUSED_THREADS = 512;
 constexpr int MACRO_FUSED_MAX_CELLS = 4096;
 constexpr int MACRO_PERSISTENT_THREADS = 256;

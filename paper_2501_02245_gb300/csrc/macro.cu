@@ -1285,11 +1285,9 @@ void macro_block(gsis_ctx* c, int steps, bool with_hot, bool time_term, bool cap
 // sqrt(sum (Wn - Wp)^2 vol / sum Wp^2 vol), quantities with a zero denominator
 // left out.  out[0] = epsilon, out[1] = number of cells with non-finite or
 // non-positive rho / T in Wn.
-__global__ void k_eps(int N, const double* __restrict__ Wn, const double* __restrict__ Wp,
-                      const double* __restrict__ vol, double* __restrict__ out) {
-    __shared__ double sm[32 * 7];
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int c = threadIdx.x; c < N; c += blockDim.x) {
+__device__ __forceinline__ void eps_sums(int first, int stride, int N, const double* __restrict__ Wn,
+                                         const double* __restrict__ Wp, const double* __restrict__ vol, double* acc) {
+    for (int c = first; c < N; c += stride) {
         const double V = vol[c];
         const double* a = Wn + c * 5;
         const double* b = Wp + c * 5;
@@ -1307,19 +1305,61 @@ __global__ void k_eps(int N, const double* __restrict__ Wn, const double* __rest
         for (int i = 1; i < 4; ++i) bad = bad || !isfinite(a[i]);
         acc[6] += bad ? 1.0 : 0.0;
     }
+}
+
+__device__ __forceinline__ void eps_result(const double* acc, double* out) {
+    double e = 0.0;
+    for (int q = 0; q < 3; ++q)
+        if (acc[2 * q + 1] > 0.0) e = fmax(e, sqrt(acc[2 * q] / acc[2 * q + 1]));
+    out[0] = e;
+    out[1] = acc[6];
+}
+
+// One block (small meshes).
+__global__ void k_eps(int N, const double* __restrict__ Wn, const double* __restrict__ Wp,
+                      const double* __restrict__ vol, double* __restrict__ out) {
+    __shared__ double sm[32 * 7];
+    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
+    eps_sums(threadIdx.x, blockDim.x, N, Wn, Wp, vol, acc);
     block_sum<7>(acc, sm);
-    if (threadIdx.x == 0) {
-        double e = 0.0;
-        for (int q = 0; q < 3; ++q)
-            if (acc[2 * q + 1] > 0.0) e = fmax(e, sqrt(acc[2 * q] / acc[2 * q + 1]));
-        out[0] = e;
-        out[1] = acc[6];
-    }
+    if (threadIdx.x == 0) eps_result(acc, out);
+}
+
+// Larger meshes in two launches: the sums of each block into part[block][7],
+// then their totals, one warp per sum (fixed order).  One block alone is bound
+// by its SM's FP64 pipes: 136 us on 16,384 cells.
+__global__ void __launch_bounds__(128) k_eps_part(int N, const double* __restrict__ Wn, const double* __restrict__ Wp,
+                                                  const double* __restrict__ vol, double* __restrict__ part) {
+    __shared__ double sm[32 * 7];
+    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
+    eps_sums(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, N, Wn, Wp, vol, acc);
+    block_sum<7>(acc, sm);
+    if (threadIdx.x == 0)
+        for (int q = 0; q < 7; ++q) part[blockIdx.x * 7 + q] = acc[q];
+}
+
+__global__ void __launch_bounds__(224) k_eps_final(int nb, const double* __restrict__ part, double* __restrict__ out) {
+    __shared__ double tot[7];
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double t = 0.0;
+    for (int b = lane; b < nb; b += 32) t += part[b * 7 + q];
+    t = warp_sum(t);
+    if (lane == 0) tot[q] = t;
+    __syncthreads();
+    if (threadIdx.x == 0) eps_result(tot, out);
 }
 
 void launch_eps(gsis_ctx* c, const double* Wn, const double* Wp) {
-    k_eps<<<1, 1024, 0, c->stream>>>(c->m.N, Wn, Wp, c->m.vol, c->eps_buf);
-    c->launches++;
+    const int N = c->m.N;
+    if (N <= 1024) {
+        k_eps<<<1, 256, 0, c->stream>>>(N, Wn, Wp, c->m.vol, c->eps_buf);
+        c->launches++;
+        return;
+    }
+    const int nb = std::min(EPS_BLOCKS, (N + 127) / 128);
+    k_eps_part<<<nb, 128, 0, c->stream>>>(N, Wn, Wp, c->m.vol, c->eps_buf + 4);
+    k_eps_final<<<1, 224, 0, c->stream>>>(nb, c->eps_buf + 4, c->eps_buf);
+    c->launches += 2;
 }
 
 }  // namespace gsis

@@ -261,28 +261,20 @@ __global__ void __launch_bounds__(256, 3) k_moments(int Nd, const int* __restric
     }
 }
 
-// 1D sums of one axis table of a record about velocity u, on the lanes of
-// one warp: s[a] = sum_j c^a E_j and s[4 + a] = sum_j c^a E_j B_j, a = 0..3,
-// c = xi_j - u (valid in lane 0).
-// On the reduced grid's z axis (zplanes) c^a is the plane weight of xi_z^a.
-__device__ void axis_sums(const double* __restrict__ tab, int NT, const double* __restrict__ xi, int off, int n,
-                          double u, int lane, double* s, const VGridDev* zplanes = nullptr) {
-    double p[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int j = lane; j < n; j += 32) {
-        const double c = xi[off + j] - u, E = tab[off + j], EB = E * tab[NT + off + j];
-        double ca = 1.0;
+// 1D sums of one axis of a record about its own centre u, from the sums of the
+// record builder: s[a] = sum_j c^a E_j and s[4 + a] = sum_j c^a E_j B_j, a = 0..3,
+// c = xi_j - u, with B = p c + p2 c^2 (on the reduced grid's z axis the xi_z^a
+// weights of the planes, which the builder's Gaussian moments carry too).
+__device__ __forceinline__ void axis_sums(const double* __restrict__ scal, int d, double* s) {
+    const double amp = d == 0 ? scal[RS_AMP] : 1.0, p = scal[RS_P + d], p2 = scal[RS_P2D + d];
+    double C[6];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const double wa = zplanes ? zpow(*zplanes, j, 0.0, a) : ca;
-            p[a] += wa * E;
-            p[4 + a] += wa * EB;
-            ca *= c;
-        }
+    for (int k = 0; k < 6; ++k) C[k] = amp * scal[RS_SUMS + 6 * d + k];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        s[a] = C[a];
+        s[4 + a] = fma(p, C[a + 1], p2 * C[a + 2]);
     }
-#pragma unroll
-    for (int a = 0; a < 8; ++a) p[a] = warp_sum(p[a]);
-    if (lane == 0)
-        for (int a = 0; a < 8; ++a) s[a] = p[a];
 }
 
 // Moment c_x^a c_y^b c_z^c of a record whose value at a node is
@@ -294,7 +286,7 @@ __device__ __forceinline__ double rec_moment(const double* X, const double* Y, c
 
 // The 13 moments (layout of k_moments) of a record about the velocity its
 // axis sums were taken about.
-__device__ void rec_moments13(const double* X, const double* Y, const double* Z, double p0, double* m) {
+__device__ __forceinline__ void rec_moments13(const double* X, const double* Y, const double* Z, double p0, double* m) {
     m[0] = rec_moment(X, Y, Z, p0, 0, 0, 0);
     m[1] = rec_moment(X, Y, Z, p0, 1, 0, 0);
     m[2] = rec_moment(X, Y, Z, p0, 0, 1, 0);
@@ -314,7 +306,7 @@ __device__ void rec_moments13(const double* X, const double* Y, const double* Z,
 // re-expressed about u + d: with c' = c - d,
 //   m1' = m1 - d m0,  M' = M - d m1^T - m1 d^T + d d^T m0,
 //   Q'_i = Q_i - 2 (M d)_i + |d|^2 m1_i - d_i tr M + 2 d_i (d.m1) - |d|^2 d_i m0.
-__device__ void shift_moments13(const double* m, const double d[3], double* o) {
+__device__ __forceinline__ void shift_moments13(const double* m, const double d[3], double* o) {
     const double m0 = m[0], m1[3] = {m[1], m[2], m[3]};
     const double M[3][3] = {{m[4], m[7], m[8]}, {m[7], m[5], m[9]}, {m[8], m[9], m[6]}};
     const double dd = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
@@ -520,42 +512,42 @@ __global__ void __launch_bounds__(256) k_correct(int Nd, const int* __restrict__
     }
 }
 
+// The 13 moments (layout of k_moments, without the quadrature weight) of a
+// corrected Maxwellian record about u.
+__device__ __forceinline__ void record_moments13(const double* __restrict__ scal, const double* u, double* o) {
+    double X[8], Y[8], Z[8], m[13];
+    axis_sums(scal, 0, X);
+    axis_sums(scal, 1, Y);
+    axis_sums(scal, 2, Z);
+    rec_moments13(X, Y, Z, scal[RS_P0], m);
+    const double d[3] = {u[0] - scal[RS_U], u[1] - scal[RS_U + 1], u[2] - scal[RS_U + 2]};
+    shift_moments13(m, d, o);
+}
+
 // The 13 velocity moments of f^{n+1} about u^{n+1} that the next
-// cell-equilibrium step reads (its heat flux), one block of six warps per
-// DVM cell, with no reduction over the velocities: the moments of f^{n+1/2}
-// (taken about u^n = Wmom by the moments pass, momh) moved to u^{n+1}, plus
-// those of the two corrected Maxwellians of Eq. updatef, which factor into 1D
-// sums over each axis (warp 3 r + d: record r, axis d).
-__global__ void __launch_bounds__(192) k_corr_moments(int Nd, const int* __restrict__ dvm_cell,
-                                                      const double* __restrict__ Wnew,
-                                                      const double* __restrict__ Wmom, Records recNew,
-                                                      Records recHalf, VGridDev vg, const double* __restrict__ momh,
-                                                      double* __restrict__ mom) {
-    const int k = blockIdx.x;
+// cell-equilibrium step reads (its heat flux), one thread per DVM cell, with
+// no reduction over the velocities: the moments of f^{n+1/2} (taken about u^n
+// = Wmom by the moments pass, momh) moved to u^{n+1}, plus those of the two
+// corrected Maxwellians of Eq. updatef, products of the axis sums that the
+// record builder took.  (A block per cell that summed the axes again held the
+// FP64 pipe for 880 warp instructions per cell: 589 us on the cylinder's 10,508
+// cells.)
+__global__ void k_corr_moments(int Nd, const int* __restrict__ dvm_cell, const double* __restrict__ Wnew,
+                               const double* __restrict__ Wmom, Records recNew, Records recHalf, double w,
+                               const double* __restrict__ momh, double* __restrict__ mom) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= Nd) return;
-    __shared__ double axs[2][3][8];
     const int c = dvm_cell[k];
-    const int nx = vg.nx, ny = vg.ny, nz = vg.nz, NT = vg.NT;
-    const int w = threadIdx.x >> 5;
-    if (w < 6) {
-        const int r = w / 3, d = w % 3;
-        const double* tab = (r == 0 ? recNew.tab : recHalf.tab) + (long long)k * NTAB * NT;
-        const int off = d == 0 ? 0 : (d == 1 ? nx : nx + ny), n = d == 0 ? nx : (d == 1 ? ny : nz);
-        axis_sums(tab, NT, vg.xi, off, n, Wnew[c * 5 + 1 + d], threadIdx.x & 31, axs[r][d],
-                  (vg.reduced && d == 2) ? &vg : nullptr);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const double* mh = momh + (long long)k * MOMN;
-        double* m = mom + (long long)k * MOMN;
-        const double d[3] = {Wnew[c * 5 + 1] - Wmom[c * 5 + 1], Wnew[c * 5 + 2] - Wmom[c * 5 + 2],
-                             Wnew[c * 5 + 3] - Wmom[c * 5 + 3]};
-        double sh[13], mN[13], mH[13];
-        shift_moments13(mh, d, sh);
-        rec_moments13(axs[0][0], axs[0][1], axs[0][2], recNew.scal[(long long)k * RS + RS_P0], mN);
-        rec_moments13(axs[1][0], axs[1][1], axs[1][2], recHalf.scal[(long long)k * RS + RS_P0], mH);
-        for (int i = 0; i < 13; ++i) m[i] = sh[i] + vg.w * (mN[i] - mH[i]);
-    }
+    const double* u = Wnew + c * 5 + 1;
+    const double* um = Wmom + c * 5 + 1;
+    const double d[3] = {u[0] - um[0], u[1] - um[1], u[2] - um[2]};
+    double sh[13], mN[13], mH[13];
+    shift_moments13(momh + (long long)k * MOMN, d, sh);
+    record_moments13(rec_scal(recNew, k), u, mN);
+    record_moments13(rec_scal(recHalf, k), u, mH);
+    double* m = mom + (long long)k * MOMN;
+#pragma unroll
+    for (int i = 0; i < 13; ++i) m[i] = sh[i] + w * (mN[i] - mH[i]);
 }
 
 template <typename S, typename T>
@@ -576,8 +568,8 @@ static void correct_t(gsis_ctx* c) {
     }
     k_correct<S, T><<<Nd, 256, smem, c->stream>>>(Nd, c->dvm_cell, c->m.side_bc, c->m.Sout, (S*)c->f, c->recNew,
                                                    c->recHalf, c->vg, c->momh, c->mom);
-    k_corr_moments<<<Nd, 192, 0, c->stream>>>(Nd, c->dvm_cell, c->W, c->Wmom, c->recNew, c->recHalf, c->vg, c->momh,
-                                              c->mom);
+    k_corr_moments<<<(Nd + 63) / 64, 64, 0, c->stream>>>(Nd, c->dvm_cell, c->W, c->Wmom, c->recNew, c->recHalf, c->vg.w,
+                                                         c->momh, c->mom);
     c->launches += 2;
 }
 

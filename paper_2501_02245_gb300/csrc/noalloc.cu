@@ -55,9 +55,6 @@ __global__ void k_noalloc_specs(int n, const double* __restrict__ W, RecSpec* sp
     for (int d = 0; d < 3; ++d) { s.u[d] = w[1 + d]; s.p[d] = 0.0; s.r[d] = 0.0; }
     for (int q = 0; q < 6; ++q) s.P2[q] = 0.0;
     s.p0 = 1.0;
-    s.U[0] = w[0];
-    for (int d = 0; d < 3; ++d) s.U[1 + d] = w[0] * w[1 + d];
-    s.U[4] = w[0] * (1.5 * w[4] + 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]));
     s.correct = 1;
     specs[k] = s;
 }
