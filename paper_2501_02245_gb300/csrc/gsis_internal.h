@@ -30,9 +30,9 @@ constexpr int FIELD_WALL = 10;  // wall heat flux, pressure, shear x/y/z
 
 // record scalar slots: polynomial p0 and off-diagonal P2 (the FP32 copy holds these), then what the
 // record's velocity moments need: centre u, amplitude of E_x, p and diagonal P2 of the corrected
-// polynomial, axis sums sum_i e c^k (k < 6) of each axis
+// polynomial, axis sums sum_i e c^k (k < 6) of each axis, and r
 enum { RS_P0 = 0, RS_P2XY = 1, RS_P2XZ = 2, RS_P2YZ = 3, RS_OFFD = 4, RS_U = 5, RS_AMP = 8, RS_P = 9, RS_P2D = 12,
-       RS_SUMS = 15 };
+       RS_SUMS = 15, RS_R = 33 };
 
 // DVM side kinds
 enum { SK_NONE = 0, SK_DVM = 1, SK_GHOST = 2, SK_FAR = 3, SK_WALL = 4 };

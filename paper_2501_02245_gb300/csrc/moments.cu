@@ -24,8 +24,11 @@
 // n terms carries a relative rounding error below n * 2^-24 (< 4e-6 for
 // n = 64) of the sum of |terms|, far under the storage rounding of BF16/FP16
 // (2^-9 / 2^-12 per value) and comparable to FP32 storage rounding.
+#include <cooperative_groups.h>
 #include <type_traits>
 #include "gsis_device.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace gsis {
 
@@ -847,85 +850,181 @@ void launch_hot(gsis_ctx* c) {
 }
 
 // ---------------------------------------------------------------------------- two-VDF moments
-// Eq. getmoment for the two-VDF model, one block per state of F[n][2][Nv]
-// (f0 then f1 on a full 3D grid): rho, u from f0; then, about u, the
+// Eq. getmoment for the two-VDF model, one thread-block cluster per state of
+// F[n][2][Nv] (f0 then f1 on a full 3D grid): rho, u from f0; then, about u, the
 // pressure tensor P and heat flux q_t = 1/2 sum w c |c|^2 f0, and
 // q_r = sum w c f1, d_r/2 rho T_r = sum w f1.  out[k][18] = rho, u (3), T_t,
 // T_r, sigma (xx, yy, zz, xy, xz, yz), q_t (3), q_r (3); T_t = tr P/(3 rho),
-// sigma = P - tr P/3 I, T_r = T_t when d_r = 0.  FP64 sums in a fixed order
-// (block reduction through shared memory).
-constexpr int TWO_VDF_THREADS = 256;
+// sigma = P - tr P/3 I, T_r = T_t when d_r = 0.  FP64 sums in a fixed order.
+//
+// FP64 bound, so the sums are factored by x-rows as in k_moments (a thread owns
+// whole rows): two operations per f0 value for the mass and momentum pass, four
+// per f0 and two per f1 value for the central pass (the second read of f0 comes
+// from L2), against 29 per pair for sums formed node by node.  The rows of a
+// state are split over the CTAs of a cluster, whose partial sums meet through
+// distributed shared memory, so that a few states fill the SMs.  96 states of
+// 48 x 48 x 24 nodes: 549 us before.
+constexpr int TWO_VDF_THREADS = 128;
+constexpr int TWO_VDF_SUMS = 16;
 
-__device__ static void block_sum(double* v, int m, double* sh) {
-    // sums v[0..m) over the block into sh[0..m) (m <= 16); every thread gets the result in v
-    for (int i = 0; i < m; ++i) sh[i * TWO_VDF_THREADS + threadIdx.x] = v[i];
-    __syncthreads();
-    for (int stride = TWO_VDF_THREADS / 2; stride > 0; stride >>= 1) {
-        if (threadIdx.x < stride)
-            for (int i = 0; i < m; ++i)
-                sh[i * TWO_VDF_THREADS + threadIdx.x] += sh[i * TWO_VDF_THREADS + threadIdx.x + stride];
-        __syncthreads();
+// Sums of v[16] over the warp: lanes 2 i and 2 i + 1 return the total of v[i].
+// Each step keeps the half of the values whose index bit matches the lane's, so
+// 16 additions replace 16 five-step trees.
+__device__ __forceinline__ double warp_sum16(double (&v)[16]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int m = 8; m >= 1; m >>= 1) {
+        const bool up = (lane & (2 * m)) != 0;
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+            const double keep = up ? v[i + m] : v[i], send = up ? v[i] : v[i + m];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * m);
+        }
     }
-    for (int i = 0; i < m; ++i) v[i] = sh[i * TWO_VDF_THREADS];
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// Cluster-wide totals of v[16] (every thread's partial sums) into tot[16] of
+// every CTA.
+__device__ __forceinline__ void cluster_sum16(double (&v)[16], double (*wsum)[16], double* mine, double* tot) {
+    cg::cluster_group cl = cg::this_cluster();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double t = warp_sum16(v);
+    if (!(lane & 1)) wsum[w][lane >> 1] = t;
+    __syncthreads();
+    if (threadIdx.x < 16) {
+        double s = 0.0;
+        for (int j = 0; j < TWO_VDF_THREADS / 32; ++j) s += wsum[j][threadIdx.x];
+        mine[threadIdx.x] = s;
+    }
+    cl.sync();
+    if (threadIdx.x < 16) {
+        double s = 0.0;
+        for (unsigned r = 0; r < cl.num_blocks(); ++r) s += cl.map_shared_rank(mine, r)[threadIdx.x];
+        tot[threadIdx.x] = s;
+    }
     __syncthreads();
 }
 
+// TAB: the powers of c_x in shared memory (grids of up to TWO_VDF_TAB_NX nodes
+// along x; longer rows form them on the fly).
+constexpr int TWO_VDF_TAB_NX = 1024;
+
+template <bool TAB>
 __global__ void __launch_bounds__(TWO_VDF_THREADS) k_two_vdf_moments(int n, const double* __restrict__ F, int d_r,
                                                                      VGridDev vg, double* __restrict__ out) {
-    __shared__ double sh[16 * TWO_VDF_THREADS];
-    const int k = blockIdx.x;
-    if (k >= n) return;
+    __shared__ double wsum[TWO_VDF_THREADS / 32][16], mineA[16], mineB[16], tot[16];
+    extern __shared__ double scx[];   // [3][nx]: c_x, c_x^2, c_x^3 about the current reference
+    cg::cluster_group cl = cg::this_cluster();
+    const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank(), k = blockIdx.x / cs;
     const long long Nv = vg.Nv;
-    const int nx = vg.nx, ny = vg.ny;
+    const int nx = vg.nx, ny = vg.ny, rows = ny * vg.nz;
     const double* f0 = F + (long long)k * 2 * Nv;
     const double* f1 = f0 + Nv;
+    const int t0 = rank * TWO_VDF_THREADS + threadIdx.x, step = cs * TWO_VDF_THREADS;
+    if (TAB)
+        for (int i = threadIdx.x; i < nx; i += TWO_VDF_THREADS) scx[i] = vg.xi[i];
+    __syncthreads();
     double a[16];
-    for (int i = 0; i < 4; ++i) a[i] = 0.0;
-    for (long long v = threadIdx.x; v < Nv; v += TWO_VDF_THREADS) {
-        const int ix = (int)(v % nx);
-        const long long rr = v / nx;
-        const int iy = (int)(rr % ny), iz = (int)(rr / ny);
-        const double f = f0[v];
-        a[0] += f;
-        a[1] += vg.xi[ix] * f;
-        a[2] += vg.xi[nx + iy] * f;
-        a[3] += vg.xi[nx + ny + iz] * f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) a[i] = 0.0;
+    for (int r = t0; r < rows; r += step) {   // mass and momentum
+        const double* p = f0 + (long long)r * nx;
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
+        for (int i = 0; i < nx; ++i) {
+            const double f = p[i];
+            s0 += f;
+            s1 = fma(f, TAB ? scx[i] : vg.xi[i], s1);
+        }
+        a[0] += s0;
+        a[1] += s1;
+        a[2] = fma(s0, vg.xi[nx + r % ny], a[2]);
+        a[3] = fma(s0, vg.xi[nx + ny + r / ny], a[3]);
     }
-    block_sum(a, 4, sh);
-    const double rho = vg.w * a[0];
-    const double u[3] = {vg.w * a[1] / rho, vg.w * a[2] / rho, vg.w * a[3] / rho};
-    for (int i = 0; i < 14; ++i) a[i] = 0.0;
-    for (long long v = threadIdx.x; v < Nv; v += TWO_VDF_THREADS) {
-        const int ix = (int)(v % nx);
-        const long long rr = v / nx;
-        const int iy = (int)(rr % ny), iz = (int)(rr / ny);
-        const double c0 = vg.xi[ix] - u[0], c1 = vg.xi[nx + iy] - u[1], c2 = vg.xi[nx + ny + iz] - u[2];
-        const double f = f0[v], g = f1[v];
-        const double c2f = (c0 * c0 + c1 * c1 + c2 * c2) * f;
-        a[0] += c0 * c0 * f; a[1] += c1 * c1 * f; a[2] += c2 * c2 * f;
-        a[3] += c0 * c1 * f; a[4] += c0 * c2 * f; a[5] += c1 * c2 * f;
-        a[6] += c0 * c2f; a[7] += c1 * c2f; a[8] += c2 * c2f;
-        a[9] += g; a[10] += c0 * g; a[11] += c1 * g; a[12] += c2 * g;
+    cluster_sum16(a, wsum, mineA, tot);
+    const double rho = vg.w * tot[0];
+    const double u[3] = {vg.w * tot[1] / rho, vg.w * tot[2] / rho, vg.w * tot[3] / rho};
+    __syncthreads();   // tot and scx are rewritten
+    if (TAB)
+        for (int i = threadIdx.x; i < nx; i += TWO_VDF_THREADS) {
+            const double c = vg.xi[i] - u[0];
+            scx[i] = c;
+            scx[nx + i] = c * c;
+            scx[2 * nx + i] = c * c * c;
+        }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) a[i] = 0.0;
+    for (int r = t0; r < rows; r += step) {   // central sums
+        const double *p = f0 + (long long)r * nx, *g = f1 + (long long)r * nx;
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0, g0 = 0.0, g1 = 0.0;
+#pragma unroll 4
+        for (int i = 0; i < nx; ++i) {
+            const double f = p[i], h = g[i], c = TAB ? scx[i] : vg.xi[i] - u[0];
+            const double c2 = TAB ? scx[nx + i] : c * c, c3 = TAB ? scx[2 * nx + i] : c2 * c;
+            s0 += f;
+            s1 = fma(f, c, s1);
+            s2 = fma(f, c2, s2);
+            s3 = fma(f, c3, s3);
+            g0 += h;
+            g1 = fma(h, c, g1);
+        }
+        const double cy = vg.xi[nx + r % ny] - u[1], cz = vg.xi[nx + ny + r / ny] - u[2];
+        const double cyz = cy * cy + cz * cz, t = fma(s0, cyz, s2);   // sum of |c|^2 f over the row
+        a[0] += s2;
+        a[1] = fma(s0, cy * cy, a[1]);
+        a[2] = fma(s0, cz * cz, a[2]);
+        a[3] = fma(s1, cy, a[3]);
+        a[4] = fma(s1, cz, a[4]);
+        a[5] = fma(s0, cy * cz, a[5]);
+        a[6] += fma(s1, cyz, s3);
+        a[7] = fma(t, cy, a[7]);
+        a[8] = fma(t, cz, a[8]);
+        a[9] += g0;
+        a[10] += g1;
+        a[11] = fma(g0, cy, a[11]);
+        a[12] = fma(g0, cz, a[12]);
     }
-    block_sum(a, 13, sh);
-    if (threadIdx.x != 0) return;
+    cluster_sum16(a, wsum, mineB, tot);
+    cl.sync();   // no CTA leaves while another reads its sums
+    if (rank != 0 || threadIdx.x != 0) return;
     const double w = vg.w;
-    const double P[6] = {w * a[0], w * a[1], w * a[2], w * a[3], w * a[4], w * a[5]};
+    const double P[6] = {w * tot[0], w * tot[1], w * tot[2], w * tot[3], w * tot[4], w * tot[5]};
     const double tr = P[0] + P[1] + P[2];
     const double Tt = tr / (3.0 * rho);
     double* o = out + (long long)k * 18;
     o[0] = rho; o[1] = u[0]; o[2] = u[1]; o[3] = u[2];
     o[4] = Tt;
-    o[5] = d_r > 0 ? 2.0 * w * a[9] / (d_r * rho) : Tt;
+    o[5] = d_r > 0 ? 2.0 * w * tot[9] / (d_r * rho) : Tt;
     o[6] = P[0] - tr / 3.0; o[7] = P[1] - tr / 3.0; o[8] = P[2] - tr / 3.0;
     o[9] = P[3]; o[10] = P[4]; o[11] = P[5];
-    o[12] = 0.5 * w * a[6]; o[13] = 0.5 * w * a[7]; o[14] = 0.5 * w * a[8];
-    o[15] = w * a[10]; o[16] = w * a[11]; o[17] = w * a[12];
+    o[12] = 0.5 * w * tot[6]; o[13] = 0.5 * w * tot[7]; o[14] = 0.5 * w * tot[8];
+    o[15] = w * tot[10]; o[16] = w * tot[11]; o[17] = w * tot[12];
 }
 
 void launch_two_vdf_moments(gsis_ctx* c, const double* F, int n, int d_r, double* out) {
     if (n <= 0) return;
-    k_two_vdf_moments<<<n, TWO_VDF_THREADS, 0, c->stream>>>(n, F, d_r, c->vg, out);
+    // CTAs per state: enough for about eight blocks per SM, no more than the rows give every thread a row
+    const int rows = c->vg.ny * c->vg.nz;
+    int cs = 1;
+    while (cs < 8 && (long long)n * cs < 1216 && rows > cs * TWO_VDF_THREADS) cs *= 2;
+    const bool tab = c->vg.nx <= TWO_VDF_TAB_NX;
+    const size_t smem = tab ? (size_t)3 * c->vg.nx * sizeof(double) : 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)n * cs);
+    cfg.blockDim = dim3(TWO_VDF_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cs;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (tab) cudaLaunchKernelEx(&cfg, k_two_vdf_moments<true>, n, F, d_r, c->vg, out);
+    else cudaLaunchKernelEx(&cfg, k_two_vdf_moments<false>, n, F, d_r, c->vg, out);
     c->launches++;
 }
 
