@@ -132,7 +132,7 @@ struct MacroJob {
 
 constexpr int FGEO_N = 12;      // face geometry values (MacroArgs::fgeo)
 constexpr int EPS_BLOCKS = 304;      // blocks of the residual's first launch
-constexpr int MACRO_FUSED_THREADS = 512;
+constexpr int MACRO_FUSED_THREADS = 256;
 constexpr int MACRO_FUSED_MAX_CELLS = 4096;
 constexpr int MACRO_PERSISTENT_THREADS = 256;
 

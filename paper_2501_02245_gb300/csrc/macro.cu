@@ -24,7 +24,7 @@
 // exactly conservative and deterministic.
 #include <algorithm>
 #include <cooperative_groups.h>
-#include "gsis_device.cuh"
+#include "special.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -52,6 +52,11 @@ static MacroArgs margs(gsis_ctx* c) {
     a.mu0 = c->mu0;
     a.omega = c->p.omega;
     return a;
+}
+
+// mu0 T^omega
+__device__ __forceinline__ double viscosity_tab(double T, double mu0, double omega) {
+    return mu0 * exp_tab(omega * log_tab(T));
 }
 
 // ---------------------------------------------------------------------------- gradients
@@ -184,7 +189,7 @@ __global__ void k_nsf(int N, const double* __restrict__ Wp, const double* __rest
                       const double* __restrict__ gT, double mu0, double omega, double* __restrict__ out) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
-    const double mu = viscosity(Wp[c * 5 + 4], mu0, omega);
+    const double mu = viscosity_tab(Wp[c * 5 + 4], mu0, omega);
     double u[9], t[3];
     cell_grad(gu, gT, N, c, u, t);
     nsf_of(mu, u, t, out + (long long)c * HOTN, out + (long long)c * HOTN + 6);
@@ -315,10 +320,14 @@ __device__ __forceinline__ void half_range_add(double r, const double* u, double
 #pragma unroll
     for (int i = 1; i < ND; ++i) un += u[i] * n[i];
     // s = un / sqrt(T) and sqrt(T) = T / sqrt(T) from one reciprocal square root
-    // (instead of a square root and two FP64 divisions)
+    // (instead of a square root and two FP64 divisions).  P is the share of the
+    // Maxwellian that crosses, (1 + sign erf(s/sqrt 2))/2, from its tail
+    // q = h(|s|) exp(-s^2/2): q where the gas recedes, 1 - q where it approaches.
     const double ist = rsqrt(T), st = T * ist, s = un * ist;
-    const double P = 0.5 * (1.0 + sign * erf(s * 0.7071067811865476));        // 1/sqrt(2)
-    const double D = sign * st * exp(-0.5 * s * s) * 0.3989422804014327;       // 1/sqrt(2 pi)
+    const double e = exp_tab(-0.5 * s * s), q = mills(__longlong_as_double((long long)mag_bits(s))) * e;
+    const bool towards = (__double2hiint(s) >= 0) == (sign > 0.0);
+    const double P = towards ? 1.0 - q : q;
+    const double D = sign * st * e * 0.3989422804014327;   // 1/sqrt(2 pi)
     const double M0 = un * P + D;
     const double M1 = (un * un + T) * P + un * D;
     const double M2 = (un * un * un + 3.0 * un * T) * P + (un * un + 2.0 * T) * D;
@@ -441,7 +450,7 @@ __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* W
     // viscous + HoT
     const double uf[3] = {0.5 * (wL[1] + wR[1]), 0.5 * (wL[2] + wR[2]), 0.5 * (wL[3] + wR[3])};
     const double Tf = 0.5 * (wL[4] + wR[4]);
-    const double muf = viscosity(Tf, a.mu0, a.omega);
+    const double muf = viscosity_tab(Tf, a.mu0, a.omega);
     const double e[3] = {G[4], G[5], G[6]};
     const double dist = G[7], idist = G[8];
     // face gradients: cell average corrected along the line of centres, for every
@@ -553,7 +562,7 @@ __device__ void wall_nsf_flux(const MacroArgs& a, const double* w, const double*
         for (int i = 0; i < 3; ++i) gTw[i] = gT[i] + corr * eb[i];
     }
     double sig[6], qw[3];
-    nsf_of(viscosity(Tw, a.mu0, a.omega), guw, gTw, sig, qw);
+    nsf_of(viscosity_tab(Tw, a.mu0, a.omega), guw, gTw, sig, qw);
     const double p = w[0] * w[4];
     const double SigS[3] = {sig[0] * So[0] + sig[3] * So[1] + sig[4] * So[2],
                             sig[3] * So[0] + sig[1] * So[1] + sig[5] * So[2],
@@ -636,7 +645,7 @@ __global__ void k_constitutive(int N, const double* __restrict__ W, const double
     double sig[6], q[3];
     double u[9], t[3];
     cell_grad(gu, gT, N, c, u, t);
-    nsf_of(viscosity(W[c * 5 + 4], mu0, omega), u, t, sig, q);
+    nsf_of(viscosity_tab(W[c * 5 + 4], mu0, omega), u, t, sig, q);
     double* o = out + (long long)c * FIELDS_N;
     const double* h = hot + (long long)c * HOTN;
     for (int k = 0; k < 6; ++k) o[k] = sig[k] + h[k];
@@ -699,7 +708,7 @@ __device__ __forceinline__ void boundary_flux_one(const MacroArgs& a, const doub
         for (int q = 0; q < 5; ++q) Fb[q] += wcr[q];
     }
     const double a_c = sqrt(GAMMA * p_c / rho_c);
-    const double mu_c = viscosity(T_c, a.mu0, a.omega);
+    const double mu_c = viscosity_tab(T_c, a.mu0, a.omega);
     const double lam = fabs(u_c[0] * nn[0] + u_c[1] * nn[1] + u_c[2] * nn[2]) + a_c +
                        5.0 * mu_c / (rho_c * 2.0 * bdist);
     double* o = Fbnd + (long long)cs * 6;
@@ -822,47 +831,45 @@ __global__ void k_cell_residual(MacroArgs a, const double* __restrict__ U, const
 // (dFin); with dFout the cell's own tensor for dU_new follows for the next sweep.
 // The two sums are accumulated apart (FMA chains over the normal components
 // that can be nonzero) and combined once.
-// The loads of all sides are issued before the sums.  The new increment is
+// The loads of both sides are issued before the sums.  The new increment is
 // left in dUc (registers) and, with dUout, stored.
 template <int ND>
 __device__ __forceinline__ void relax_nd(const MacroArgs& a, const double* U, const double* R, const double* D,
                                          const double* lamS, const double* dUin, double* dUout, const double* dFin,
                                          double* dFout, const double* F0, int c, double* dUc) {
-    constexpr int NS = 2 * ND;
     const int N = a.N;
-    int n[NS];
-#pragma unroll
-    for (int d = 0; d < ND; ++d) {
-        const int2 v = *reinterpret_cast<const int2*>(a.nbr + c * 6 + 2 * d);
-        n[2 * d] = v.x;
-        n[2 * d + 1] = v.y;
-    }
-    double dF[NS][5][ND], dn[NS][5], So[NS][ND], ls[NS], Rc[5];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        const int m = n[s] >= 0 ? n[s] : c;
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-#pragma unroll
-            for (int i = 0; i < ND; ++i) dF[s][q][i] = dFin[(long long)(q * 3 + i) * N + m];
-            dn[s][q] = dUin[(long long)q * N + m];
-        }
-#pragma unroll
-        for (int i = 0; i < ND; ++i) So[s][i] = a.Sout[((long long)c * 6 + s) * 3 + i];
-        ls[s] = lamS[(long long)s * N + c];
-    }
+    double Rc[5], fs[5] = {0, 0, 0, 0, 0}, ld[5] = {0, 0, 0, 0, 0};
 #pragma unroll
     for (int q = 0; q < 5; ++q) Rc[q] = R[(long long)q * N + c];
     const double iD = D[c];   // 1 / D
-    double fs[5] = {0, 0, 0, 0, 0}, ld[5] = {0, 0, 0, 0, 0};
+    // the two sides of a direction at a time in 3D (all four at once in 2D: in 3D
+    // the six sides' values would not fit the registers)
+#pragma unroll(ND < 3 ? ND : 1)
+    for (int d = 0; d < ND; ++d) {
+        const int2 nb = *reinterpret_cast<const int2*>(a.nbr + c * 6 + 2 * d);
+        double dF[2][5][ND], dn[2][5], So[2][ND], ls[2];
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        if (n[s] < 0) continue;
+        for (int h = 0; h < 2; ++h) {
+            const int s = 2 * d + h, nn = h ? nb.y : nb.x, m = nn >= 0 ? nn : c;
 #pragma unroll
-        for (int q = 0; q < 5; ++q) {
+            for (int q = 0; q < 5; ++q) {
 #pragma unroll
-            for (int i = 0; i < ND; ++i) fs[q] = fma(dF[s][q][i], So[s][i], fs[q]);
-            ld[q] = fma(ls[s], dn[s][q], ld[q]);
+                for (int i = 0; i < ND; ++i) dF[h][q][i] = dFin[(long long)(q * 3 + i) * N + m];
+                dn[h][q] = dUin[(long long)q * N + m];
+            }
+#pragma unroll
+            for (int i = 0; i < ND; ++i) So[h][i] = a.Sout[((long long)c * 6 + s) * 3 + i];
+            ls[h] = lamS[(long long)s * N + c];
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if ((h ? nb.y : nb.x) < 0) continue;
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+#pragma unroll
+                for (int i = 0; i < ND; ++i) fs[q] = fma(dF[h][q][i], So[h][i], fs[q]);
+                ld[q] = fma(ls[h], dn[h][q], ld[q]);
+            }
         }
     }
 #pragma unroll
@@ -1257,8 +1264,8 @@ void macro_block(gsis_ctx* c, int steps, bool with_hot, bool time_term, bool cap
         launch_gradients(c, c->Wm, false);
         k_face_flux<<<nf, TB, 0, c->stream>>>(a, c->Wm, c->gu, c->gT, c->hot, c->acell, ndir, c->Ff, c->lamf,
                                                c->wall_corr, c->Fbnd);
-        k_cell_residual<<<nb, TB, 0, c->stream>>>(a, c->U, c->Un, c->Ff, c->lamf, c->Fbnd, c->p.cfl, dt, c->R, c->D, c->lamS, c->dU, c->F0,
-                                                  c->p.k_sub > 0 ? c->dFa : nullptr);
+        k_cell_residual<<<nb, TB, 0, c->stream>>>(a, c->U, c->Un, c->Ff, c->lamf, c->Fbnd, c->p.cfl, dt, c->R, c->D,
+                                                  c->lamS, c->dU, c->F0, c->p.k_sub > 0 ? c->dFa : nullptr);
         c->launches += 2;
         double* din = c->dU;
         double* dout = c->dU2;
