@@ -256,10 +256,12 @@ gsis_status gsis_debug_set_region(gsis_ctx* ctx, const uint8_t* flags);
  * tile) work items from a device counter, and the synthetic solves of all
  * meshes up to 4096 cells run in one launch (one CTA each); one iteration of
  * the whole batch is recorded once into a CUDA graph and replayed.  The tile
- * shape of the persistent sweep is picked by timing the candidates on the
- * batch itself (on a snapshot of the VDFs, restored afterwards; skipped
- * without memory for the snapshot) and cached per batch shape for the life
- * of the process.  Results are identical to iterating each solve alone.
+ * shape of the persistent sweep is that of 1D lines ("line_w4") if every
+ * member is a non-periodic line of kinetic cells, else picked by timing the
+ * candidates on the batch itself (on a snapshot of the VDFs, restored
+ * afterwards; skipped without memory for the snapshot) and cached per batch
+ * shape for the life of the process.  Results equal those of iterating each
+ * solve alone (FP64 lines: to rounding).
  *
  * ctxs: n distinct contexts on one device, each with mesh and velocity grid
  *       set, adaptive = 0 (or a region forced by gsis_debug_set_region);
@@ -286,10 +288,10 @@ gsis_status gsis_iterate_batch(gsis_ctx** ctxs, int n, int iterations, gsis_repo
  * tile shape of the persistent batched sweep instead of the autotuned one
  * (names as reported by gsis_batch_info, e.g. "vpt2_cb1_w4", or the
  * velocity-pair shapes "pair1_cb1_w4", "pair2_cb1_w4", "pair1_cb1_w8", which
- * need FP32/BF16/FP16 members with an even nx: gsis_iterate_batch then returns
- * GSIS_ERR_ARG for another batch).  NULL or "" restores autotuning.  Every
- * shape computes the same result.  GSIS_ERR_ARG for an unknown name.  The
- * paper has no counterpart. */
+ * need FP32/BF16/FP16 members with an even nx, or "line_w4", which needs 1D
+ * members: gsis_iterate_batch then returns GSIS_ERR_ARG for another batch).  NULL or "" restores autotuning.  Every
+ * shape computes the same result (the line shape: to rounding).  GSIS_ERR_ARG
+ * for an unknown name.  The paper has no counterpart. */
 gsis_status gsis_debug_set_batch_tile(const char* name);
 
 /* Test hook: run the kinetic sweep of this context with the named tile shape

@@ -1,0 +1,71 @@
+// Batched persistent sweep of 1D lines: items are (solve, warp tile) pairs drawn
+// from the ticket counter as in batch_kernel.cuh; a warp walks the line of its
+// tile with the window of sweep_line.cuh, both passes (both passes' launches
+// where walls need a refresh between them).
+#include <algorithm>
+#include "batch_kernel.cuh"
+#include "sweep_line.cuh"
+
+namespace gsis {
+
+constexpr int LINE_WPB = 4;
+
+// F64: the FP64 members' items (the others are passed over), else the
+// FP32-arithmetic ones: one kernel for both would give every item the FP64
+// code's registers.
+template <bool F64>
+__global__ void __launch_bounds__(32 * LINE_WPB, F64 ? 3 : 4) k_sweep_batch_line(const BatchSolve* __restrict__ solves,
+                                                                                 const int2* __restrict__ items,
+                                                                                 int n_items, int* __restrict__ ticket,
+                                                                                 int pass0, int pass1) {
+    // the solve's arguments, one copy per warp: registers are the limit of this
+    // kernel's occupancy (in the single launch they sit in the constant bank)
+    __shared__ SweepArgs args[LINE_WPB];
+    __shared__ LineStage stages[F64 ? 1 : LINE_WPB];
+    const int lane = threadIdx.x & 31;
+    SweepArgs& a = args[threadIdx.x >> 5];
+    LineStage* stage = &stages[F64 ? 0 : threadIdx.x >> 5];
+    for (;;) {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(ticket, 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= n_items) return;   // the counter only grows: every warp leaves after at most n_items draws
+        const int2 it = items[t];
+        const BatchSolve& B = solves[it.x];
+        const int dtype = B.dtype;
+        if ((dtype == GSIS_F64) != F64) continue;
+        __syncwarp();   // the previous item's last reads
+        for (int w = lane; w < (int)(sizeof(SweepArgs) / sizeof(int)); w += 32)
+            reinterpret_cast<int*>(&a)[w] = reinterpret_cast<const int*>(&B.a)[w];
+        __syncwarp();
+        if constexpr (F64) {
+            line_tile<double, double, LINE_ZP64>(a, (double*)B.f, B.cells, it.y, lane, pass0, pass1, stage);
+        } else {
+            if (dtype == GSIS_F32)
+                line_tile<float, float, LINE_ZP32>(a, (float*)B.f, B.cells, it.y, lane, pass0, pass1, stage);
+            else if (dtype == GSIS_BF16)
+                line_tile<__nv_bfloat16, float, LINE_ZP32>(a, (__nv_bfloat16*)B.f, B.cells, it.y, lane, pass0, pass1, stage);
+            else
+                line_tile<__half, float, LINE_ZP32>(a, (__half*)B.f, B.cells, it.y, lane, pass0, pass1, stage);
+        }
+    }
+}
+
+template <bool F64>
+static int grid_of() {
+    int dev = 0, sms = 0, per = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sweep_batch_line<F64>, 32 * LINE_WPB, 0);
+    return std::max(1, sms * std::max(1, per));
+}
+
+int batch_grid_line(bool f64) { return f64 ? grid_of<true>() : grid_of<false>(); }
+
+void batch_launch_line(const BatchSolve* s, const int2* i, int n, int* t, int grid, cudaStream_t st, int p0, int p1,
+                       bool f64) {
+    if (f64) k_sweep_batch_line<true><<<grid, 32 * LINE_WPB, 0, st>>>(s, i, n, t, p0, p1);
+    else k_sweep_batch_line<false><<<grid, 32 * LINE_WPB, 0, st>>>(s, i, n, t, p0, p1);
+}
+
+}  // namespace gsis

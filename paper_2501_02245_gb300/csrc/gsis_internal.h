@@ -274,15 +274,18 @@ size_t ring_bytes(gsis_ctx* c, int vt);
 bool launch_sweep_ring(gsis_ctx* c, const SweepArgs& a, int pass, int which);
 // sweep_col.cu (velocity columns, 2D meshes, FP64 storage)
 void launch_sweep_col(gsis_ctx* c, const SweepArgs& a, int pass, int shape);
+// sweep_line.cu (1D lines)
+void launch_sweep_line(gsis_ctx* c, const SweepArgs& a, int pass);
 // batch.cu (persistent batched sweep; BatchSolve is declared in sweep_device.cuh)
 struct BatchSolve;
 int batch_num_shapes();
 const char* batch_shape_name(int shape);
 int batch_shape_vtile(int shape);
 bool batch_shape_pair(int shape);
+bool batch_shape_line(int shape);
 int batch_grid(int shape, int nc);
 void launch_sweep_batch(int shape, int nc, const BatchSolve* d_solves, const int2* d_items, int n_items,
-                        int* d_ticket, int grid, cudaStream_t st, int pass0, int pass1);
+                        int* d_ticket, int grid, cudaStream_t st, int pass0, int pass1, int types);
 // moments.cu
 void launch_moments(gsis_ctx* c, const double* Wref, double* out);
 void launch_correct(gsis_ctx* c);

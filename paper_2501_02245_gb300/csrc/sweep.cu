@@ -252,7 +252,8 @@ SweepArgs sweep_args(gsis_ctx* c) {
 void launch_sweep(gsis_ctx* c, int pass) {
     if (c->Nd == 0) return;
     const SweepArgs a = sweep_args(c);
-    launch_sweep_shape(c, a, pass, c->sweep_shape < 0 ? 0 : c->sweep_shape);
+    if (c->normal_components == 1 && !c->sweep_forced && line_alone(c)) launch_sweep_line(c, a, pass);
+    else launch_sweep_shape(c, a, pass, c->sweep_shape < 0 ? 0 : c->sweep_shape);
     c->launches++;
     c->sweep_launches++;
 }
@@ -312,7 +313,7 @@ gsis_status tune_sweep(gsis_ctx* c) {
     c->tuned_Nd = c->Nd;
     if (c->Nd == 0 || c->normal_components == 1) {
         c->sweep_shape = 0;
-        c->sweep_info = "1D or empty: fixed shape";
+        c->sweep_info = c->Nd > 0 && line_alone(c) ? "1D line: window sweep" : "1D or empty: fixed shape";
         return GSIS_OK;
     }
     const std::string key = std::to_string(c->p.vdf_dtype) + "/" + std::to_string(c->normal_components) + "/" +

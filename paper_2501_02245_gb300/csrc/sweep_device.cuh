@@ -391,6 +391,12 @@ struct BatchSolve {
     SweepArgs a;
     void* f;      // VDF rows of this solve
     int dtype;    // GSIS_F64 / F32 / BF16 / F16
+    int cells;    // DVM cells
 };
+
+// A 1D line whose rows are its cells in order (sweep_line.cuh applies).
+bool line_ok(const gsis_ctx* c);
+bool line_alone(const gsis_ctx* c);  // ... and the faster sweep for this solve by itself
+int line_tiles(const gsis_ctx* c);   // warp tiles of its velocity grid
 
 }  // namespace gsis

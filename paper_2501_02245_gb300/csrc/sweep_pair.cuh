@@ -49,6 +49,13 @@ __device__ __forceinline__ float2 hmm2(float2 a, float2 b) {
     return make_float2(hmm_t<float>(a.x, b.x), hmm_t<float>(a.y, b.y));
 }
 
+// base + row * row_bytes in one instruction (from an element index it takes four)
+__device__ __forceinline__ char* row_at(char* base, int row, unsigned row_bytes) {
+    char* r;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(row), "r"(row_bytes), "l"(base));
+    return r;
+}
+
 // ---------------------------------------------------------------- paired storage access
 template <typename S> __device__ __forceinline__ float2 ld2(const S* p);
 template <> __device__ __forceinline__ float2 ld2<float>(const float* p) { return *reinterpret_cast<const float2*>(p); }
