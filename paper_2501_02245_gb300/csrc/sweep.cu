@@ -159,10 +159,21 @@ constexpr int kRingShapes = 3;
 // After those, for FP64 storage: the velocity columns (sweep_col.cu; 2D meshes),
 // planes per column and warps per block.
 static const char* const kColNames[] = {"col_z4_g4", "col_z4_g8", "col_z3_g4", "col_z2_g8"};
-static int col_shapes(int dtype) { return dtype == GSIS_F64 ? (int)(sizeof(kColNames) / sizeof(kColNames[0])) : 0; }
+// FP32 arithmetic: pairs on two planes (sweep_planes.cuh; 2D and 3D meshes).
+static const char* const kPlaneNames[] = {"planes"};
+static int col_shapes(int dtype) {
+    return dtype == GSIS_F64 ? (int)(sizeof(kColNames) / sizeof(kColNames[0]))
+                             : (int)(sizeof(kPlaneNames) / sizeof(kPlaneNames[0]));
+}
 // FP64 on 2D meshes (the kernels keep a row's bytes in 32 bits)
 static bool col_ok(gsis_ctx* c) {
     return c->p.vdf_dtype == GSIS_F64 && c->normal_components == 2 && (double)c->vg.Nv * sizeof(double) < 2147483648.0;
+}
+
+// FP32 arithmetic, an even nx, 2D or 3D (the same limit on a row)
+static bool planes_ok(gsis_ctx* c) {
+    return c->p.vdf_dtype != GSIS_F64 && pair_ok(c) &&
+           (double)c->vg.Nv * vdf_elem_bytes(c->p.vdf_dtype) < 2147483648.0;
 }
 
 static int base_shapes(int dtype) {
@@ -173,7 +184,7 @@ int sweep_num_shapes(int dtype) { return base_shapes(dtype) + kRingShapes + col_
 static int col_index(int dtype, int shape) { return shape - base_shapes(dtype) - kRingShapes; }
 const char* sweep_shape_name(int dtype, int shape) {
     if (shape < 0 || shape >= sweep_num_shapes(dtype)) return "?";
-    if (shape >= base_shapes(dtype) + kRingShapes) return kColNames[col_index(dtype, shape)];
+    if (shape >= base_shapes(dtype) + kRingShapes) return (dtype == GSIS_F64 ? kColNames : kPlaneNames)[col_index(dtype, shape)];
     if (shape >= base_shapes(dtype)) return kRingNames[shape - base_shapes(dtype)];
     return dtype == GSIS_F64 ? kShapesF64[shape].name : kShapesF32[shape].name;
 }
@@ -214,6 +225,13 @@ static void launch_sweep_shape(gsis_ctx* c, const SweepArgs& a, int pass, int sh
         if (col_ok(c)) {
             launch_sweep_col(c, a, pass, col_index(c->p.vdf_dtype, shape));
             return;
+        }
+        if (planes_ok(c)) {
+            switch (c->p.vdf_dtype) {
+                case GSIS_F32: launch_sweep_planes_f32(c, a, pass); return;
+                case GSIS_BF16: launch_sweep_planes_bf16(c, a, pass); return;
+                default: launch_sweep_planes_f16(c, a, pass); return;
+            }
         }
         shape = 0;
     }
@@ -271,13 +289,13 @@ static std::map<std::string, int>& sweep_cache() {
 // Shapes the autotuner times: those that win somewhere.  FP64 on 2D meshes:
 // the columns, and the wide single-velocity blocks for small velocity grids
 // (the reduced distributions' 144 tiles: g16_v1_c1 7.5 ms, best column 11.6);
-// FP32 arithmetic: the velocity pairs and the widest single-velocity tile, the
+// FP32 arithmetic: the velocity pairs, on one and on two planes, and the widest single-velocity tile, the
 // single-velocity tiles where pairs cannot run.  The shared-memory windows and
 // the remaining tiles measured slower everywhere (cylinder FP64 120 ms against
 // 51.6, FP32 37 against 6.9) and run only when forced.
 static bool tune_candidate(gsis_ctx* c, int shape) {
     const int nb = base_shapes(c->p.vdf_dtype);
-    if (shape >= nb + kRingShapes) return col_ok(c);
+    if (shape >= nb + kRingShapes) return col_ok(c) || planes_ok(c);
     if (shape >= nb) return false;
     if (c->p.vdf_dtype == GSIS_F64) return col_ok(c) ? shape >= 4 : true;
     return pair_ok(c) ? (shape == 3 || pair_shape(c->p.vdf_dtype, shape)) : shape < 4;
@@ -291,8 +309,10 @@ gsis_status force_sweep_shape(gsis_ctx* c, const char* name) {
     for (int sh = 0; sh < ns; ++sh) {
         if (std::string(sweep_shape_name(c->p.vdf_dtype, sh)) != name) continue;
         if (sh >= nb + kRingShapes) {
-            if (!col_ok(c))
-                return set_err(c, GSIS_ERR_ARG, std::string("sweep tile ") + name + " needs FP64 storage and a 2D mesh");
+            if (!col_ok(c) && !planes_ok(c))
+                return set_err(c, GSIS_ERR_ARG, std::string("sweep tile ") + name +
+                                                    (c->p.vdf_dtype == GSIS_F64 ? " needs a 2D mesh"
+                                                                                : " needs an even nx and a 2D/3D mesh"));
         } else if (sh >= nb) {
             const int which = sh - nb;
             if (ring_bytes(c, which == 2 ? 64 : 32) == 0 || (c->p.vdf_dtype == GSIS_F64 && which == 2))
