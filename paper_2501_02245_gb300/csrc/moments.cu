@@ -27,6 +27,7 @@
 #include <cooperative_groups.h>
 #include <type_traits>
 #include "gsis_device.cuh"
+#include "packed.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -98,6 +99,57 @@ __device__ __forceinline__ void psi_row(const VGridDev& vg, double x1, double x2
     a[3] = x2;
     a[4] = 0.5 * (x1 * x1 + x2 * x2);
     c[4] = 0.5;
+}
+
+// Outgoing mass flux through each wall side of a cell, row by row (mass rows
+// only): this thread's sums to acc[13 + s].
+template <typename S, typename T>
+__device__ __forceinline__ void wall_rows(const VGridDev& vg, const S* __restrict__ fk, const T* sxi, int wall_mask,
+                                          const double* __restrict__ Sc, double* acc) {
+    const int nx = vg.nx, ny = vg.ny;
+    double wsum[6] = {0, 0, 0, 0, 0, 0};
+    const int mrows = vg.reduced ? ny : ny * vg.nz;
+    for (int r = threadIdx.x; r < mrows; r += blockDim.x) {
+        const double xy = vg.xi[nx + r % ny], xz = vg.xi[nx + ny + r / ny];
+        const S* row = fk + (long long)r * nx;
+        for (int s = 0; s < 6; ++s) {
+            if (!((wall_mask >> s) & 1)) continue;
+            const double* Sw = Sc + s * 3;
+            const double rr = xy * Sw[1] + xz * Sw[2];
+            int lo, hi;
+            out_range(vg.xi, nx, Sw[0], rr, lo, hi);
+            T a0 = T(0), a1 = T(0);
+            for (int ix = lo; ix < hi; ++ix) {
+                const T fv = ldT<T, S>(row + ix);
+                a0 += fv;
+                a1 += fv * sxi[ix];
+            }
+            wsum[s] += Sw[0] * (double)a1 + rr * (double)a0;
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < 6; ++s) acc[13 + s] = wsum[s];
+}
+
+// Block reduction over the threads' rows of sums (part): lane q of each warp adds
+// moment q over the warp's threads (31 FP64 additions per warp instead of MOMN
+// five-step shuffle trees), and thread q adds the warps' totals (red).
+__device__ __forceinline__ void reduce_rows(const VGridDev& vg, const double* part, double* red, double* __restrict__ out) {
+    __syncthreads();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (lane < MOMN) {
+        const double* pw = part + w * 32 * MOMN + lane;
+        double t = 0.0;
+        for (int j = 0; j < 32; ++j) t += pw[j * MOMN];
+        red[w * MOMN + lane] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < MOMN) {
+        double t = 0.0;
+        for (int j = 0; j < nw; ++j) t += red[j * MOMN + threadIdx.x];
+        const double wv = vg.w / vg.vscale;   // stored values carry the VDF storage scale
+        out[threadIdx.x] = t * wv;
+    }
 }
 
 template <typename S, typename T>
@@ -219,49 +271,173 @@ __global__ void __launch_bounds__(256, 3) k_moments(int Nd, const int* __restric
       }
       rp = rend;
     }
-    if (wall_mask) {   // outgoing mass flux through each wall side, row by row (mass rows only)
-        double wsum[6] = {0, 0, 0, 0, 0, 0};
-        const int mrows = vg.reduced ? ny : rows;
-        for (int r = threadIdx.x; r < mrows; r += blockDim.x) {
-            const double xy = vg.xi[nx + r % ny], xz = vg.xi[nx + ny + r / ny];
-            const S* row = fk + (long long)r * nx;
-            for (int s = 0; s < 6; ++s) {
-                if (!((wall_mask >> s) & 1)) continue;
-                const double* Sw = Sout + ((long long)c * 6 + s) * 3;
-                const double rr = xy * Sw[1] + xz * Sw[2];
-                int lo, hi;
-                out_range(vg.xi, nx, Sw[0], rr, lo, hi);
-                T a0 = T(0), a1 = T(0);
-                for (int ix = lo; ix < hi; ++ix) {
-                    const T fv = ldT<T, S>(row + ix);
-                    a0 += fv;
-                    a1 += fv * sxi[ix];
+    if (wall_mask) wall_rows<S, T>(vg, fk, sxi, wall_mask, Sout + (long long)c * 18, acc);
+    reduce_rows(vg, part, red, mom + (long long)k * MOMN);
+}
+
+__device__ __forceinline__ void unpack_chunk(const float*, uint4 w, float2* v) {
+    v[0] = make_float2(__uint_as_float(w.x), __uint_as_float(w.y));
+    v[1] = make_float2(__uint_as_float(w.z), __uint_as_float(w.w));
+}
+template <typename S>
+__device__ __forceinline__ void unpack_chunk(const S*, uint4 w, float2* v) {
+    const unsigned a[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        if constexpr (std::is_same<S, __nv_bfloat16>::value)
+            v[p] = make_float2(__uint_as_float(a[p] << 16), __uint_as_float(a[p] & 0xffff0000u));
+        else
+            v[p] = __half22float2(*reinterpret_cast<const __half2*>(&a[p]));
+    }
+}
+
+// The same moments in FP32 arithmetic where the x-rows hold whole 16-byte chunks
+// (k_moments otherwise).  What limited k_moments here was the FP64 pipe (the row
+// folds, per plane and thread) and the 32 lines of each load.  Two lanes share a
+// row, so that a load takes whole 32-byte sectors; a warp takes 8 rows iy x 4
+// planes iz as two batches of 16 rows (the rows of two planes each), the lanes
+// exchange the halves of the sums, and each lane folds one row.  A lane keeps its iy
+// over the units of a strip, so it folds with the planes' z weights (shared
+// memory) only, and with the powers of c_y once per strip.  10,482 cells of 55,296
+// velocities: FP32 0.95 -> 0.72 ms, BF16 0.78 -> 0.66; 11,643 BF16 cells of 119,808: 2.24
+// -> 1.20.
+constexpr int MROW_THREADS = 128;
+template <typename S>
+__global__ void __launch_bounds__(MROW_THREADS, 6) k_moments_rows(int Nd, const int* __restrict__ dvm_cell,
+                                                               const double* __restrict__ Wref,
+                                                               const int* __restrict__ side_bc,
+                                                               const double* __restrict__ Sout,
+                                                               const S* __restrict__ f, VGridDev vg,
+                                                               double* __restrict__ mom) {
+    constexpr int V = Vec16<S>::N, H = V / 2, U = 3;
+    const int k = blockIdx.x;
+    if (k >= Nd) return;
+    extern __shared__ double sh_raw[];
+    __shared__ double red[MROW_THREADS / 32 * MOMN];
+    const int nx = vg.nx, ny = vg.ny, nz = vg.nz, nc = nx / V;
+    const int c = dvm_cell[k];
+    const double ux = Wref[c * 5 + 1], uy = Wref[c * 5 + 2], uz = Wref[c * 5 + 3];
+    float* scx = reinterpret_cast<float*>(sh_raw);   // c_x, c_x^2, c_x^3, xi_x
+    double* zt = sh_raw + 2 * nx;                     // [nz][4]: z weights of order 0..3
+    double* part = zt + 4 * nz;
+    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+        const double cx = vg.xi[i] - ux;
+        scx[i] = (float)cx;
+        scx[nx + i] = (float)(cx * cx);
+        scx[2 * nx + i] = (float)(cx * cx * cx);
+        scx[3 * nx + i] = (float)vg.xi[i];
+    }
+    for (int i = threadIdx.x; i < nz; i += blockDim.x) {
+        const double cz = vg.xi[nx + ny + i] - uz;
+        if (vg.reduced) {
+            for (int q = 0; q < 4; ++q) zt[4 * i + q] = zpow(vg, i, cz, q);
+        } else {
+            zt[4 * i] = 1.0; zt[4 * i + 1] = cz; zt[4 * i + 2] = cz * cz; zt[4 * i + 3] = cz * cz * cz;
+        }
+    }
+    double* acc = part + threadIdx.x * MOMN;
+#pragma unroll
+    for (int q = 0; q < MOMN; ++q) acc[q] = 0.0;
+    __syncthreads();
+    int wall_mask = 0;
+    for (int s = 0; s < 6; ++s)
+        if (side_bc[c * 6 + s] == GSIS_BC_WALL) wall_mask |= 1 << s;
+    const S* fk = f + (long long)k * vg.Nv;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = MROW_THREADS / 32;
+    const int j = lane & 1, ry = (lane >> 1) & 7, rz = lane >> 4;   // chunk parity, row within a batch
+    const int M = (nz + 3) / 4, units = (ny + 7) / 8 * M;
+    const int u0 = (int)((long long)units * w / nw), u1 = (int)((long long)units * (w + 1) / nw);
+    const uint4* base = reinterpret_cast<const uint4*>(fk);
+    double Z[10];
+#pragma unroll
+    for (int q = 0; q < 10; ++q) Z[q] = 0.0;
+    for (int u = u0; u < u1; ++u) {
+        const int g = u / M, m = u - g * M, iy = 8 * g + ry, iz = 4 * m + rz;
+        // batches 0, 1: row (iy, iz + 2 b); a row past the end is not read
+        const bool in0 = iy < ny && iz < nz, in1 = iy < ny && iz + 2 < nz;
+        const uint4* p0 = base + (iy + ny * iz) * nc;
+        const uint4* p1 = p0 + 2 * ny * nc;
+        float2 a[4], b[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] = b[q] = make_float2(0.0f, 0.0f);
+        for (int i0 = j; i0 < nc; i0 += 2 * U) {
+            uint4 x0[U], x1[U];
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const int ch = i0 + 2 * i;
+                x0[i] = x1[i] = make_uint4(0u, 0u, 0u, 0u);
+                if (ch < nc && in0) x0[i] = p0[ch];
+                if (ch < nc && in1) x1[i] = p1[ch];
+            }
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const int ch = i0 + 2 * i;
+                if (ch >= nc) break;
+                float2 v0[H], v1[H];
+                unpack_chunk(fk, x0[i], v0);
+                unpack_chunk(fk, x1[i], v1);
+#pragma unroll
+                for (int h = 0; h < H; h += 2) {
+                    const float4* t = reinterpret_cast<const float4*>(scx + ch * V + 2 * h);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (q == 0) {
+                            a[0] = f2add(a[0], v0[h]);
+                            a[0] = f2add(a[0], v0[h + 1]);
+                            b[0] = f2add(b[0], v1[h]);
+                            b[0] = f2add(b[0], v1[h + 1]);
+                        } else {
+                            const float4 wx = t[(q - 1) * (nx / 4)];
+                            const float2 lo = make_float2(wx.x, wx.y), hi = make_float2(wx.z, wx.w);
+                            a[q] = f2fma(v0[h], lo, a[q]);
+                            a[q] = f2fma(v0[h + 1], hi, a[q]);
+                            b[q] = f2fma(v1[h], lo, b[q]);
+                            b[q] = f2fma(v1[h + 1], hi, b[q]);
+                        }
+                    }
                 }
-                wsum[s] += Sw[0] * (double)a1 + rr * (double)a0;
             }
         }
+        double d[4];   // the row sums of batch j
 #pragma unroll
-        for (int s = 0; s < 6; ++s) acc[13 + s] = wsum[s];
+        for (int q = 0; q < 4; ++q) {
+            const float s0 = a[q].x + a[q].y, s1 = b[q].x + b[q].y;
+            const float other = __shfl_xor_sync(0xffffffffu, j ? s0 : s1, 1);
+            d[q] = (j ? s1 : s0) + other;
+        }
+        const double* z = zt + 4 * min(iz + 2 * j, nz - 1);   // (a row past the end has zero sums)
+        const double2 z01 = *reinterpret_cast<const double2*>(z), z23 = *reinterpret_cast<const double2*>(z + 2);
+        Z[0] = fma(d[0], z01.x, Z[0]);
+        Z[1] = fma(d[0], z01.y, Z[1]);
+        Z[2] = fma(d[0], z23.x, Z[2]);
+        Z[3] = fma(d[0], z23.y, Z[3]);
+        Z[4] = fma(d[1], z01.x, Z[4]);
+        Z[5] = fma(d[1], z01.y, Z[5]);
+        Z[6] = fma(d[1], z23.x, Z[6]);
+        Z[7] = fma(d[2], z01.x, Z[7]);
+        Z[8] = fma(d[2], z01.y, Z[8]);
+        Z[9] = fma(d[3], z01.x, Z[9]);
+        if (u + 1 == u1 || m + 1 == M) {   // the strip's end: fold with c_y
+            const double cy = vg.xi[nx + min(iy, ny - 1)] - uy, cy2 = cy * cy;
+            acc[0] += Z[0];
+            acc[1] += Z[4];
+            acc[2] = fma(Z[0], cy, acc[2]);
+            acc[3] += Z[1];
+            acc[4] += Z[7];
+            acc[5] = fma(Z[0], cy2, acc[5]);
+            acc[6] += Z[2];
+            acc[7] = fma(Z[4], cy, acc[7]);
+            acc[8] += Z[5];
+            acc[9] = fma(Z[1], cy, acc[9]);
+            acc[10] += fma(Z[4], cy2, Z[9] + Z[6]);                    // c_x c^2
+            acc[11] = fma(fma(Z[0], cy2, Z[7] + Z[2]), cy, acc[11]);   // c_y c^2
+            acc[12] += fma(Z[1], cy2, Z[8] + Z[3]);                    // c_z c^2
+#pragma unroll
+            for (int q = 0; q < 10; ++q) Z[q] = 0.0;
+        }
     }
-    // Block reduction over the rows of the buffer: lane q of each warp adds
-    // moment q over the warp's threads
-    // (31 FP64 additions per warp instead of MOMN five-step shuffle trees), and
-    // thread q adds the warps' totals.
-    __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (lane < MOMN) {
-        const double* pw = part + w * 32 * MOMN + lane;
-        double t = 0.0;
-        for (int j = 0; j < 32; ++j) t += pw[j * MOMN];
-        red[w * MOMN + lane] = t;
-    }
-    __syncthreads();
-    if (threadIdx.x < MOMN) {
-        double t = 0.0;
-        for (int j = 0; j < nw; ++j) t += red[j * MOMN + threadIdx.x];
-        const double wv = vg.w / vg.vscale;   // stored values carry the VDF storage scale
-        mom[(long long)k * MOMN + threadIdx.x] = t * wv;
-    }
+    if (wall_mask) wall_rows<S, float>(vg, fk, scx + 3 * nx, wall_mask, Sout + (long long)c * 18, acc);
+    reduce_rows(vg, part, red, mom + (long long)k * MOMN);
 }
 
 // 1D sums of one axis of a record about its own centre u, from the sums of the
@@ -336,13 +512,18 @@ __device__ __forceinline__ void shift_moments13(const double* m, const double d[
 // with per-x values (E, E B) and per-(y, z) values e = E_y E_z,
 // p = p0 + B_y + B_z held in shared memory each point costs
 //   a_N = E_x p_N + (E B)_x,  a_H likewise,  f += e_N a_N - e_H a_H
-// (five operations).  Where the x-rows hold whole 16-byte chunks a thread
-// loads and stores 16 bytes (2 to 8 values) at a time, two chunks in flight,
-// else four scalar points; every thread loads before it stores (the loads and
-// stores go through the same pointer, so the compiler would not move a load
-// above an earlier store).  Both forms compute the same values in the same
-// order (bitwise equal results).  A wall
-// cell adds the correction's outgoing wall sums to those of f^{n+1/2}.
+// (five operations: the bound in FP64).  Where the x-rows hold whole 16-byte
+// chunks a thread loads and stores 16 bytes (2 to 8 values) at a time, else four
+// scalar points; every thread loads before it stores (the loads and stores go
+// through the same pointer, so the compiler would not move a load above an
+// earlier store).  In FP32 arithmetic a thread keeps to one chunk position of the
+// rows, so the per-x values stay in registers, a row's values come as one 16-byte
+// word for the whole chunk and the update runs in packed pairs, with 64 to 128 bytes
+// in flight (correct_chunks; with the records it reads, 11,643 BF16 cells of 119,808
+// velocities 2.80 -> 1.77 ms, 10,482 of 55,296 1.32 -> 0.91, FP32 1.15 -> 1.06: the
+// hash of the stochastic rounding and the memory bound it now).  All forms compute the same values in the same order
+// (bitwise equal results).  A wall cell adds the correction's outgoing wall sums
+// to those of f^{n+1/2}.
 constexpr int CORR_UNROLL = 4;
 constexpr int CORR_VEC_UNROLL = 2;
 
@@ -408,8 +589,97 @@ __device__ __forceinline__ unsigned corr_key(int k, int v) {
     return (unsigned)k * 0x9e3779b9u ^ (unsigned)v * 0x85ebca6bu;
 }
 
+// A chunk of values as stored (the roundings of rounded<>).
+template <typename S>
+__device__ __forceinline__ uint4 rounded_chunk(const float2* v, int k, int v0) {
+    constexpr int V = Vec16<S>::N;
+    if constexpr (std::is_same<S, __nv_bfloat16>::value) {
+        float2 z = make_float2(0.0f, 0.0f);   // stays 0 unless a value is inf or nan
+#pragma unroll
+        for (int p = 0; p < V / 2; ++p) z = f2fma(v[p], make_float2(0.0f, 0.0f), z);
+        if (z.x + z.y == 0.0f) {
+            unsigned w[V / 2];
+#pragma unroll
+            for (int p = 0; p < V / 2; ++p) {
+                unsigned b0 = __float_as_uint(v[p].x), b1 = __float_as_uint(v[p].y);
+                b0 += mix32(corr_key(k, v0 + 2 * p) ^ b0) & 0xffffu;
+                b1 += mix32(corr_key(k, v0 + 2 * p + 1) ^ b1) & 0xffffu;
+                w[p] = __byte_perm(b0, b1, 0x7632);   // the upper halves
+            }
+            return make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+    alignas(16) S out[V];
+#pragma unroll
+    for (int p = 0; p < V / 2; ++p) {
+        out[2 * p] = rounded<float, S>(v[p].x, corr_key(k, v0 + 2 * p));
+        out[2 * p + 1] = rounded<float, S>(v[p].y, corr_key(k, v0 + 2 * p + 1));
+    }
+    return *reinterpret_cast<const uint4*>(out);
+}
+// The update of a cell by chunk positions (FP32 arithmetic; nx / V <= blockDim.x):
+// rows of velocities q0, q0 + rows per block, ...  WALL: a cell with wall sides,
+// whose outgoing sums of the increment go to acc (FP64; rows where the chunk's
+// end nodes both move inwards hold no outgoing node, xi.S being linear in xi_x).
+template <typename S, bool WALL>
+__device__ __forceinline__ void correct_chunks(S* __restrict__ fk, int k, const VGridDev& vg, const float* xa,
+                                               const float* rv, int wall_mask, const double* __restrict__ Sc,
+                                               double* acc) {
+    constexpr int V = Vec16<S>::N, H = V / 2, U = WALL ? 1 : 16 / V;
+    const int nx = vg.nx, ny = vg.ny, nyz = ny * vg.nz, nc = nx / V;
+    const int rpb = blockDim.x / nc, q0 = threadIdx.x / nc, cx = threadIdx.x - q0 * nc;
+    if (q0 >= rpb) return;
+    float2 eN[H], bN[H], eH[H], bH[H];
+#pragma unroll
+    for (int p = 0; p < H; ++p) {
+        const float2* x = reinterpret_cast<const float2*>(xa + cx * V) + p;
+        eN[p] = x[0];
+        bN[p] = x[nx / 2];
+        eH[p] = x[nx];
+        bH[p] = x[3 * nx / 2];
+    }
+    uint4* chunk = reinterpret_cast<uint4*>(fk) + cx;
+    for (int qb = q0; qb < nyz; qb += U * rpb) {
+        uint4 w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (qb + u * rpb < nyz) w[u] = chunk[(qb + u * rpb) * nc];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = qb + u * rpb;
+            if (q >= nyz) break;
+            const float4 r = reinterpret_cast<const float4*>(rv)[q];   // e_N, p_N, e_H, p_H
+            float2 v[H], d[H];
+            unpack_chunk(fk, w[u], v);
+#pragma unroll
+            for (int p = 0; p < H; ++p) {
+                const float2 aN = f2fma(eN[p], bc2(r.y), bN[p]), aH = f2fma(eH[p], bc2(r.w), bH[p]);
+                d[p] = f2fma(bc2(r.x), aN, f2mul(bc2(-r.z), aH));
+                v[p] = f2add(v[p], d[p]);
+            }
+            chunk[q * nc] = rounded_chunk<S>(v, k, q * nx + cx * V);
+            if (WALL && (!vg.reduced || q < ny)) {   // mass flux: the G plane on the reduced grid
+                const int iz = q / ny, iy = q - iz * ny;
+                const double x1 = vg.xi[nx + iy], x2 = vg.xi[nx + ny + iz];
+                const double* x0 = vg.xi + cx * V;
+#pragma unroll
+                for (int s = 0; s < 6; ++s) {
+                    if (!((wall_mask >> s) & 1)) continue;
+                    const double rr = x1 * Sc[3 * s + 1] + x2 * Sc[3 * s + 2], Sx = Sc[3 * s];
+                    if (!(fma(x0[0], Sx, rr) > 0.0) && !(fma(x0[V - 1], Sx, rr) > 0.0)) continue;
+#pragma unroll
+                    for (int j = 0; j < V; ++j) {
+                        const double xn = fma(x0[j], Sx, rr);
+                        if (xn > 0.0) acc[s] = fma(xn, (double)(j & 1 ? d[j / 2].y : d[j / 2].x), acc[s]);
+                    }
+                }
+            }
+        }
+    }
+}
+
 template <typename S, typename T>
-__global__ void __launch_bounds__(256) k_correct(int Nd, const int* __restrict__ dvm_cell,
+__global__ void __launch_bounds__(256, std::is_same<T, double>::value ? 1 : 3) k_correct(int Nd, const int* __restrict__ dvm_cell,
                                                  const int* __restrict__ side_bc, const double* __restrict__ Sout,
                                                  S* __restrict__ f, Records recNew, Records recHalf, VGridDev vg,
                                                  const double* __restrict__ momh, double* __restrict__ mom) {
@@ -418,7 +688,7 @@ __global__ void __launch_bounds__(256) k_correct(int Nd, const int* __restrict__
     extern __shared__ double sh_raw[];
     const int nx = vg.nx, ny = vg.ny, NT = vg.NT, nyz = ny * vg.nz;
     T* xa = reinterpret_cast<T*>(sh_raw);   // [4][nx]: E_N, (E B)_N, E_H, (E B)_H
-    T* rv = xa + 4 * nx;                     // [4][nyz]: e_N, p_N, e_H, p_H
+    T* rv = xa + 4 * nx;                     // [nyz][4]: e_N, p_N, e_H, p_H
     __shared__ double red[32 * 6];
     const int c = dvm_cell[k];
     const T* TN = RecT<T>::tab(recNew, k, NT);
@@ -432,10 +702,10 @@ __global__ void __launch_bounds__(256) k_correct(int Nd, const int* __restrict__
     }
     for (int q = threadIdx.x; q < nyz; q += blockDim.x) {
         const int jy = nx + q % ny, jz = nx + ny + q / ny;
-        rv[q] = TN[jy] * TN[jz];
-        rv[nyz + q] = p0N + (TN[NT + jy] + TN[NT + jz]);
-        rv[2 * nyz + q] = TH[jy] * TH[jz];
-        rv[3 * nyz + q] = p0H + (TH[NT + jy] + TH[NT + jz]);
+        rv[4 * q] = TN[jy] * TN[jz];
+        rv[4 * q + 1] = p0N + (TN[NT + jy] + TN[NT + jz]);
+        rv[4 * q + 2] = TH[jy] * TH[jz];
+        rv[4 * q + 3] = p0H + (TH[NT + jy] + TH[NT + jz]);
     }
     int wall_mask = 0;
     for (int s = 0; s < 6; ++s)
@@ -446,9 +716,9 @@ __global__ void __launch_bounds__(256) k_correct(int Nd, const int* __restrict__
     const int Nv = (int)vg.Nv, step = blockDim.x;
     // the increment at velocity (ix, q) and the outgoing wall sums of it
     auto delta = [&](int ix, int q) -> T {
-        const T aN = fma(xa[ix], rv[nyz + q], xa[nx + ix]);
-        const T aH = fma(xa[2 * nx + ix], rv[3 * nyz + q], xa[3 * nx + ix]);
-        const T dlt = fma(rv[q], aN, -(rv[2 * nyz + q] * aH));
+        const T aN = fma(xa[ix], rv[4 * q + 1], xa[nx + ix]);
+        const T aH = fma(xa[2 * nx + ix], rv[4 * q + 3], xa[3 * nx + ix]);
+        const T dlt = fma(rv[4 * q], aN, -(rv[4 * q + 2] * aH));
         if (wall_mask && (!vg.reduced || q < ny)) {   // mass flux: the G plane on the reduced grid
             const int iz = q / ny, iy = q - iz * ny;
             const double x0 = vg.xi[ix], x1 = vg.xi[nx + iy], x2 = vg.xi[nx + ny + iz];
@@ -462,9 +732,19 @@ __global__ void __launch_bounds__(256) k_correct(int Nd, const int* __restrict__
         return dlt;
     };
     constexpr int V = Vec16<S>::N;
-    if (nx % V == 0) {
-        // 16-byte chunks of V consecutive velocities (one x-row holds whole chunks;
-        // rows start on 16-byte boundaries), two chunks in flight per thread
+    // 16-byte chunks of V consecutive velocities (one x-row holds whole chunks;
+    // rows start on 16-byte boundaries)
+    bool chunks = false;
+    if constexpr (std::is_same<T, float>::value) {
+        chunks = nx % V == 0 && nx / V <= (int)blockDim.x;
+        if (chunks) {
+            const double* Sc = Sout + (long long)c * 18;
+            if (wall_mask) correct_chunks<S, true>(fk, k, vg, xa, rv, wall_mask, Sc, acc);
+            else correct_chunks<S, false>(fk, k, vg, xa, rv, 0, Sc, acc);
+        }
+    }
+    if (chunks) {
+    } else if (std::is_same<T, double>::value && nx % V == 0) {   // two chunks in flight per thread
         const int nch = Nv / V;
         for (int ch0 = threadIdx.x; ch0 < nch; ch0 += CORR_VEC_UNROLL * step) {
             T fv[CORR_VEC_UNROLL][V];
@@ -669,6 +949,15 @@ void launch_wall_rho(gsis_ctx* c) {
 template <typename S, typename T>
 static void moments_t(gsis_ctx* c, const double* Wref, double* out) {
     const int Nd = (int)c->Nd;
+    if constexpr (std::is_same<T, float>::value) {
+        const size_t sm = sizeof(double) * (2 * (size_t)c->vg.nx + 4 * (size_t)c->vg.nz + (size_t)MROW_THREADS * MOMN);
+        if (c->vg.nx % Vec16<S>::N == 0 && sm <= 48 * 1024 - MROW_THREADS / 32 * MOMN * sizeof(double)) {
+            k_moments_rows<S><<<Nd, MROW_THREADS, sm, c->stream>>>(Nd, c->dvm_cell, Wref, c->m.side_bc, c->m.Sout,
+                                                                   (const S*)c->f, c->vg, out);
+            c->launches++;
+            return;
+        }
+    }
     // threads own whole x-rows: a block size that divides the rows evenly keeps
     // every warp busy until the final reduction (256 unless 192 or 128 fits better)
     const int rows = c->vg.ny * c->vg.nz;
