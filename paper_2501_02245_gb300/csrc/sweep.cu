@@ -158,7 +158,7 @@ constexpr int kRingShapes = 3;
 
 // After those, for FP64 storage: the velocity columns (sweep_col.cu; 2D meshes),
 // planes per column and warps per block.
-static const char* const kColNames[] = {"col_z4_g4", "col_z4_g8", "col_z3_g4", "col_z2_g8"};
+static const char* const kColNames[] = {"col_z4_g4", "col_z4_g8", "col_z3_g4", "col_z2_g8", "col_z2_g12_p16"};
 // FP32 arithmetic: pairs on two planes (sweep_planes.cuh; 2D and 3D meshes).
 static const char* const kPlaneNames[] = {"planes"};
 static int col_shapes(int dtype) {
@@ -287,8 +287,9 @@ static std::map<std::string, int>& sweep_cache() {
 }
 
 // Shapes the autotuner times: those that win somewhere.  FP64 on 2D meshes:
-// the columns, and the wide single-velocity blocks for small velocity grids
-// (the reduced distributions' 144 tiles: g16_v1_c1 7.5 ms, best column 11.6);
+// the columns, and the wide single-velocity blocks for the smallest velocity
+// grids (the reduced distributions' 48 x 48 x 2: col_z2_g12_p16 6.8 ms, g16_v1_c1 7.5,
+// columns of 32 positions 11.6);
 // FP32 arithmetic: the velocity pairs, on one and on two planes, and the widest single-velocity tile, the
 // single-velocity tiles where pairs cannot run.  The shared-memory windows and
 // the remaining tiles measured slower everywhere (cylinder FP64 120 ms against

@@ -42,12 +42,14 @@ struct Column {
     int ix, iy, iz0, q[ZP];   // q = iy + ny iz
     double x0, x1;            // half of xi_x, xi_y
     int nact;            // planes to store (0: clamped position)
+    unsigned mask;       // the lanes that share this lane's cell
 };
 
-template <int ZP>
+template <int ZP, int P>
 __device__ __forceinline__ void make_column(const VGridDev& vg, double* f, int ptile, int ztile, int lane, Column<ZP>& C) {
     const int nxy = vg.nx * vg.ny;
-    const int pp = ptile * 32 + lane, p = min(pp, nxy - 1), iz0 = ztile * ZP;
+    C.mask = P == 32 ? 0xffffffffu : ((1u << (P & 31)) - 1u) << (lane & ~(P - 1));
+    const int pp = ptile * P + (lane & (P - 1)), p = min(pp, nxy - 1), iz0 = ztile * ZP;
     C.iz0 = iz0;
     C.iy = p / vg.nx;
     C.ix = p - C.iy * vg.nx;
@@ -132,7 +134,7 @@ __device__ __forceinline__ void column_load(int k, const CellMeta<double, 2>& m,
         const bool bo = oL && pos_t<double>(xH);
         double xo = oL ? mL : mH;
         out += xo;
-        if (__any_sync(0xffffffffu, bo)) {
+        if (__any_sync(C.mask, bo)) {
             if (bo) { out += xH; xo = xL - xH; }
         }
         const double iH = pos_t<double>(xH) ? 0.0 : xH;
@@ -188,11 +190,11 @@ __device__ __forceinline__ void column_apply(const SweepArgs& a, int k, const Ce
         bool dvm_h = true;
         if (!interior) {
 #pragma unroll
-            for (int hs = 0; hs < 2; ++hs) {   // (the side kinds are the same for every lane)
+            for (int hs = 0; hs < 2; ++hs) {   // (the side kinds are the same for every lane of the cell)
                 const int s = 2 * d + hs, kd = side_kind(m.kinds, s);
                 if (kd == SK_NONE || kd == SK_DVM) continue;
                 const double x = hs ? (q.oL[d] ? q.xi[d] : q.xe[d]) : (q.oL[d] ? 0.0 : q.xi[d]);   // halved, < 0 for inflow
-                if (!__any_sync(0xffffffffu, x != 0.0)) continue;
+                if (!__any_sync(C.mask, x != 0.0)) continue;
                 const double scale = kd == SK_WALL ? __ldg(a.rho_w + (long long)k * 6 + s) : 1.0;
                 double v[ZP];
                 column_record<ZP>(a, kd == SK_GHOST ? a.recGhost : a.recBC, m.rf[s], 2.0 * scale, C, v);
@@ -202,7 +204,7 @@ __device__ __forceinline__ void column_apply(const SweepArgs& a, int k, const Ce
             dvm_h = side_kind(m.kinds, 2 * d + 1) == SK_DVM;
         }
         const bool bi = dvm_h && q.xe[d] != 0.0;   // the high face is an inflow face too
-        if (__any_sync(0xffffffffu, bi)) {
+        if (__any_sync(C.mask, bi)) {
             const double ce = bi ? q.xe[d] : 0.0;
             const int r2 = dvm_h ? m.n2[2 * d + 1] : k;
             double e2[ZP];
@@ -223,16 +225,21 @@ __device__ __forceinline__ void column_apply(const SweepArgs& a, int k, const Ce
     }
 }
 
-// A block owns 32 (ix, iy) positions x ZP planes; its G warps split the cells
-// of each hyperplane.  The sweep data of a warp's next cell (also across the
+// A block owns P (ix, iy) positions x ZP planes; its G warps split the cells
+// of each hyperplane, 32 / P cells to a warp.  P = 16 serves small velocity grids,
+// whose blocks of 32 positions would leave SMs idle: the reduced grid of 48 x 48 x 2
+// on the same cylinder takes 6.8 ms with 144 blocks of 12 warps, 11.6 with 72 blocks
+// of 32 positions, 7.5 with a lane per velocity in 144 blocks of 16 warps (32 x 32 x 2:
+// 6.6, 11.6, 7.4); 8 and 16 warps take 7.6 and 7.1.  The sweep data of a warp's next cell (also across the
 // barrier: it does not change during the pass) is loaded before the current
 // cell is updated.  MINB: blocks per SM the registers are capped for.
-template <int ZP, int G, int MINB>
+template <int ZP, int G, int MINB, int P>
 __global__ void __launch_bounds__(32 * G, MINB) k_sweep_col(SweepArgs a, double* __restrict__ f, int pass, int nptile,
                                                             unsigned row_bytes) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int CG = G * (32 / P);   // cells of a hyperplane taken together
+    const int lane = threadIdx.x & 31, w = threadIdx.x / P;
     Column<ZP> C;
-    make_column<ZP>(a.vg, f, blockIdx.x % nptile, blockIdx.x / nptile, lane, C);
+    make_column<ZP, P>(a.vg, f, blockIdx.x % nptile, blockIdx.x / nptile, lane, C);
     const int h0 = pass ? a.H - 1 : 0;
     const int kb = __ldg(a.hp_off + h0);
     int n = __ldg(a.hp_off + h0 + 1) - kb;
@@ -247,9 +254,9 @@ __global__ void __launch_bounds__(32 * G, MINB) k_sweep_col(SweepArgs a, double*
             nn = __ldg(a.hp_off + h + 1) - kbn;
         }
         const int kfirst = pass ? kbn + nn - 1 - w : kbn + w;
-        for (int i = w; i < n; i += G) {
-            const bool last = i + G >= n;
-            const int kn = last ? kfirst : (pass ? k - G : k + G);
+        for (int i = w; i < n; i += CG) {
+            const bool last = i + CG >= n;
+            const int kn = last ? kfirst : (pass ? k - CG : k + CG);
             CellMeta<double, 2> mn;
             if (!last || w < nn) load_meta<double, 2>(a, kn, mn);
             Stencil<ZP> q;
@@ -267,19 +274,20 @@ __global__ void __launch_bounds__(32 * G, MINB) k_sweep_col(SweepArgs a, double*
     }
 }
 
-template <int ZP, int G, int MINB>
+template <int ZP, int G, int MINB, int P = 32>
 static void launch_col(gsis_ctx* c, const SweepArgs& a, int pass) {
-    const int nptile = (c->vg.nx * c->vg.ny + 31) / 32, nztile = (c->vg.nz + ZP - 1) / ZP;
-    k_sweep_col<ZP, G, MINB><<<nptile * nztile, 32 * G, 0, c->stream>>>(a, (double*)c->f, pass, nptile,
+    const int nptile = (c->vg.nx * c->vg.ny + P - 1) / P, nztile = (c->vg.nz + ZP - 1) / ZP;
+    k_sweep_col<ZP, G, MINB, P><<<nptile * nztile, 32 * G, 0, c->stream>>>(a, (double*)c->f, pass, nptile,
                                                                         (unsigned)(c->vg.Nv * sizeof(double)));
 }
 
-// Column shapes: planes, warps per block (names and order: kColNames in sweep.cu).
+// Column shapes: planes, warps per block, positions per block if not 32 (names and order: kColNames in sweep.cu).
 void launch_sweep_col(gsis_ctx* c, const SweepArgs& a, int pass, int shape) {
     switch (shape) {
         case 1: launch_col<4, 8, 1>(c, a, pass); break;
         case 2: launch_col<3, 4, 2>(c, a, pass); break;
         case 3: launch_col<2, 8, 1>(c, a, pass); break;
+        case 4: launch_col<2, 12, 1, 16>(c, a, pass); break;
         default: launch_col<4, 4, 3>(c, a, pass); break;
     }
 }

@@ -11,7 +11,7 @@ from helpers import run_oracle, w_rel_err, rel_err, vdf_by_cell, RTOL_W
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = ["col_z4_g4", "col_z4_g8", "col_z3_g4", "col_z2_g8"]
+SHAPES = ["col_z4_g4", "col_z4_g8", "col_z3_g4", "col_z2_g8", "col_z2_g12_p16"]
 # (nx, ny, nz): whole and partial position tiles; odd axes with a ragged plane group
 GRIDS = [(14, 12, 6), (13, 11, 7)]
 
