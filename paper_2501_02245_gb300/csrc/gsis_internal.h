@@ -275,9 +275,9 @@ bool launch_sweep_ring(gsis_ctx* c, const SweepArgs& a, int pass, int which);
 // sweep_col.cu (velocity columns, 2D meshes, FP64 storage)
 void launch_sweep_col(gsis_ctx* c, const SweepArgs& a, int pass, int shape);
 // sweep_planes_*.cu (velocity pairs on two planes, FP32 arithmetic; one unit per storage type)
-void launch_sweep_planes_f32(gsis_ctx* c, const SweepArgs& a, int pass);
-void launch_sweep_planes_bf16(gsis_ctx* c, const SweepArgs& a, int pass);
-void launch_sweep_planes_f16(gsis_ctx* c, const SweepArgs& a, int pass);
+void launch_sweep_planes_f32(gsis_ctx* c, const SweepArgs& a, int pass, int shape);
+void launch_sweep_planes_bf16(gsis_ctx* c, const SweepArgs& a, int pass, int shape);
+void launch_sweep_planes_f16(gsis_ctx* c, const SweepArgs& a, int pass, int shape);
 // sweep_line.cu (1D lines)
 void launch_sweep_line(gsis_ctx* c, const SweepArgs& a, int pass);
 // batch.cu (persistent batched sweep; BatchSolve is declared in sweep_device.cuh)

@@ -160,7 +160,7 @@ constexpr int kRingShapes = 3;
 // planes per column and warps per block.
 static const char* const kColNames[] = {"col_z4_g4", "col_z4_g8", "col_z3_g4", "col_z2_g8", "col_z2_g12_p16"};
 // FP32 arithmetic: pairs on two planes (sweep_planes.cuh; 2D and 3D meshes).
-static const char* const kPlaneNames[] = {"planes"};
+static const char* const kPlaneNames[] = {"planes", "planes_wide"};
 static int col_shapes(int dtype) {
     return dtype == GSIS_F64 ? (int)(sizeof(kColNames) / sizeof(kColNames[0]))
                              : (int)(sizeof(kPlaneNames) / sizeof(kPlaneNames[0]));
@@ -228,9 +228,9 @@ static void launch_sweep_shape(gsis_ctx* c, const SweepArgs& a, int pass, int sh
         }
         if (planes_ok(c)) {
             switch (c->p.vdf_dtype) {
-                case GSIS_F32: launch_sweep_planes_f32(c, a, pass); return;
-                case GSIS_BF16: launch_sweep_planes_bf16(c, a, pass); return;
-                default: launch_sweep_planes_f16(c, a, pass); return;
+                case GSIS_F32: launch_sweep_planes_f32(c, a, pass, col_index(c->p.vdf_dtype, shape)); return;
+                case GSIS_BF16: launch_sweep_planes_bf16(c, a, pass, col_index(c->p.vdf_dtype, shape)); return;
+                default: launch_sweep_planes_f16(c, a, pass, col_index(c->p.vdf_dtype, shape)); return;
             }
         }
         shape = 0;

@@ -22,8 +22,6 @@
 //   10,482 kinetic cells, 48 x 48 x 24 velocities (cylinder): FP32 6.75 -> 6.40 ms, BF16 6.78 ->
 //   6.11, FP16 6.58 -> 5.83;
 //   11,643 kinetic cells, 48 x 52 x 48 (sphere): BF16 30.2 -> 21.1 ms, FP32 29.4 -> 21.8;
-// small velocity grids (17 x 38 x 36: too few tiles of 128 velocities) stay with
-// eight warps per block there (2.28 ms against 2.29).
 #pragma once
 #include "sweep_pair.cuh"
 
@@ -300,9 +298,16 @@ static void launch_planes_t(gsis_ctx* c, const SweepArgs& a, int pass) {
 
 // 2D: 128 registers, 15 warps per SM (four warps of 168 registers, 12 per SM: 6.59
 // ms against 6.40 on the FP32 cylinder); 3D: 168 registers, 12 warps per SM (five
-// warps, 10 per SM: 24.7 against 21.1 on the BF16 sphere).
+// warps, 10 per SM: 24.7 against 21.1 on the BF16 sphere).  Shape 1 has wider blocks for
+// velocity grids with few tiles: 36 x 38 x 17 on 4,271 cells FP32 2.00 ms (2.33 with
+// shape 0, 2.28 with the best pair tile), 32^3 on the sphere BF16 7.1 (8.7, 10.1).
 template <typename S>
-static void launch_planes(gsis_ctx* c, const SweepArgs& a, int pass) {
+static void launch_planes(gsis_ctx* c, const SweepArgs& a, int pass, int shape) {
+    if (shape == 1) {
+        if (c->normal_components == 2) launch_planes_t<S, 2, 8, 2>(c, a, pass);
+        else launch_planes_t<S, 3, 6, 2>(c, a, pass);
+        return;
+    }
     if (c->normal_components == 2) launch_planes_t<S, 2, 5, 3>(c, a, pass);
     else launch_planes_t<S, 3, 4, 3>(c, a, pass);
 }

@@ -3,8 +3,8 @@
 
 namespace gsis {
 
-void launch_sweep_planes_bf16(gsis_ctx* c, const SweepArgs& a, int pass) {
-    launch_planes<__nv_bfloat16>(c, a, pass);
+void launch_sweep_planes_bf16(gsis_ctx* c, const SweepArgs& a, int pass, int shape) {
+    launch_planes<__nv_bfloat16>(c, a, pass, shape);
 }
 
 }  // namespace gsis
