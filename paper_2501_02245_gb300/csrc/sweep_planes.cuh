@@ -6,11 +6,13 @@
 // instructions issued and by the latency of its loads with 12 (3D) or 15 (2D) warps per SM:
 // - the update is written without selects: with m_s = max(x_s, 0) and n_s = m_s -
 //   x_s for the halved face speeds x_s = xi.S_s/(2V),
-//     num = g~/tau + sum_d (m_L - m_H) mm(c - l, h - c) + n_L (2 l + mm(l - l2, c - l))
-//                                                       + n_H (2 h + mm(h - h2, c - h)),
+//     num = g~/tau + sum_d m_L mm(c - l, h - c) + n_L (2 l + mm(l - l2, c - l))
+//                        - m_H mm(c - l, h - c) + n_H (2 h + mm(h - h2, c - h)),
 //     den = 1/tau + 2 sum (m_L + m_H),
 //   mm the minmod (a face is an outflow or an inflow face: one of its m, n is
-//   zero), instead of picking each side's upwind rows per velocity;
+//   zero), instead of picking each side's upwind rows per velocity; the sums run in
+//   the order of compute_cells, and the products with zero change nothing, so the
+//   results are those of the other tiles (to FP32 subnormals, which halving rounds);
 // - on 2D meshes m, n, den and the reciprocal do not depend on the plane and are
 //   formed once per cell;
 // - a row's address is one mad.wide from its byte pitch;
@@ -19,9 +21,9 @@
 //   the next cell's stencil or factors as well needs registers that cost more
 //   warps than it hides (2D FP32 cylinder 8.5 to 10 ms, 7.9 with the factors).
 // Per pass pair, best of sweep_pair.cuh's tiles against this one:
-//   10,482 kinetic cells, 48 x 48 x 24 velocities (cylinder): FP32 6.75 -> 6.40 ms, BF16 6.78 ->
-//   6.11, FP16 6.58 -> 5.83;
-//   11,643 kinetic cells, 48 x 52 x 48 (sphere): BF16 30.2 -> 21.1 ms, FP32 29.4 -> 21.8;
+//   10,482 kinetic cells, 48 x 48 x 24 velocities (cylinder): FP32 6.75 -> 5.9 ms, BF16 6.78 ->
+//   6.1, FP16 6.58 -> 5.6;
+//   11,643 kinetic cells, 48 x 52 x 48 (sphere): BF16 30.2 -> 21.2 ms, FP32 29.9 -> 20.3.
 #pragma once
 #include "sweep_pair.cuh"
 
@@ -153,31 +155,25 @@ __device__ __forceinline__ void load_factors(const SweepArgs& a, int k, const Pa
     g.it = __ldg(a.itauf + k);
 }
 
-// The sides of a boundary or interface cell that are not DVM sides: their
-// distributions' share of the sum.
+// Side sd of a boundary or interface cell, if it is no DVM side: its distribution's
+// share of the sum (n: its inflow, per plane on 3D meshes).
 template <typename S, int NC, int ZP>
-__device__ __forceinline__ void add_records(const SweepArgs& a, int k, int kinds, const PairColumn<S, NC, ZP>& C,
-                                         float2* num) {
-    const int NT = a.vg.NT;
-    const float* sv = static_cast<const float*>(a.sdv) + (long long)k * SD_VALS;
-    for (int s = 0; s < 2 * NC; ++s) {
-        const int kd = side_kind(kinds, s);
-        if (kd == SK_NONE || kd == SK_DVM) continue;
-        const int rec = __ldg(a.sdi + (long long)k * SD_INTS + (s < 4 ? s : 4 + s));
-        const Records& R = kd == SK_GHOST ? a.recGhost : a.recBC;
-        const float* sc = RecT<float>::scal(R, rec);
-        const float* tb = RecT<float>::tab(R, rec, NT);
-        const float w = kd == SK_WALL ? __ldg(a.rho_wf + (long long)k * 6 + s) : 1.0f;
-        const float S0 = __ldg(sv + s), S1 = NC >= 2 ? __ldg(sv + 8 + s) : 0.0f, S2 = NC >= 3 ? __ldg(sv + 16 + s) : 0.0f;
+__device__ __forceinline__ void add_record(const SweepArgs& a, int k, int kinds, int sd, const PairColumn<S, NC, ZP>& C,
+                                           const float2* n, float2* num) {
+    const int kd = side_kind(kinds, sd);
+    if (kd == SK_NONE || kd == SK_DVM) return;
+    const int NT = a.vg.NT, rec = __ldg(a.sdi + (long long)k * SD_INTS + (sd < 4 ? sd : 4 + sd));
+    const Records& R = kd == SK_GHOST ? a.recGhost : a.recBC;
+    const float* sc = RecT<float>::scal(R, rec);
+    const float* tb = RecT<float>::tab(R, rec, NT);
+    const float w = kd == SK_WALL ? __ldg(a.rho_wf + (long long)k * 6 + sd) : 1.0f;
 #pragma unroll
-        for (int u = 0; u < ZP; ++u) {
-            const int iz = min(C.iz0 + u, a.vg.nz - 1);
-            const float t = NC >= 3 ? fmaf(C.x2[u], S2, C.x1 * S1) : C.x1 * S1;
-            const float nx = fmaxf(-fmaf(C.x0.x, S0, t), 0.0f), ny = fmaxf(-fmaf(C.x0.y, S0, t), 0.0f);
-            if (!__any_sync(0xffffffffu, nx > 0.0f || ny > 0.0f)) continue;
-            num[u].x = fmaf(nx, 2.0f * w * eval_recT<float>(sc, tb, NT, a.vg.nx, a.vg.ny, C.ix, C.iy, iz), num[u].x);
-            num[u].y = fmaf(ny, 2.0f * w * eval_recT<float>(sc, tb, NT, a.vg.nx, a.vg.ny, C.ix + 1, C.iy, iz), num[u].y);
-        }
+    for (int u = 0; u < ZP; ++u) {
+        const float2 x = n[NC == 3 ? u : 0];
+        if (!__any_sync(0xffffffffu, x.x > 0.0f || x.y > 0.0f)) continue;
+        const int iz = min(C.iz0 + u, a.vg.nz - 1);
+        num[u].x = fmaf(x.x, 2.0f * w * eval_recT<float>(sc, tb, NT, a.vg.nx, a.vg.ny, C.ix, C.iy, iz), num[u].x);
+        num[u].y = fmaf(x.y, 2.0f * w * eval_recT<float>(sc, tb, NT, a.vg.nx, a.vg.ny, C.ix + 1, C.iy, iz), num[u].y);
     }
 }
 
@@ -195,53 +191,62 @@ __device__ __forceinline__ void apply_pairs(const SweepArgs& a, int k, int kinds
         num[u].y = fmaf(m.xb.w, y.w, fmaf(m.xb.z, y.z, fmaf(m.xb.y, y.y, m.xb.x * y.x)));
     }
 #pragma unroll
-    for (int z = 0; z < DZ; ++z) out[z] = make_float2(0.0f, 0.0f);
+    for (int z = 0; z < DZ; ++z) out[z] = bc2(0.5f * m.it);   // half the denominator
     const bool interior = kinds < 0;   // every side a DVM side
-    if (!interior) add_records<S, NC, ZP>(a, k, kinds, C, num);
 #pragma unroll
     for (int d = 0; d < NC; ++d) {
-        float2 co[DZ], nl[DZ], nh[DZ];
+        const float* SL = m.S[2 * d];
+        const float* SH = m.S[2 * d + 1];
+        const float2 bl = f2fma(bc2(C.x1), bc2(SL[1]), f2mul(C.x0, bc2(SL[0])));
+        const float2 bh = f2fma(bc2(C.x1), bc2(SH[1]), f2mul(C.x0, bc2(SH[0])));
+        float2 ml[DZ], mh[DZ], nl[DZ], nh[DZ];
 #pragma unroll
         for (int z = 0; z < DZ; ++z) {
-            const float* SL = m.S[2 * d];
-            const float* SH = m.S[2 * d + 1];
-            float tl = C.x1 * SL[1], th = C.x1 * SH[1];
+            float2 xl = bl, xh = bh;
             if constexpr (NC >= 3) {
-                tl = fmaf(C.x2[z], SL[NC >= 3 ? 2 : 0], tl);
-                th = fmaf(C.x2[z], SH[NC >= 3 ? 2 : 0], th);
+                xl = f2fma(bc2(C.x2[z]), bc2(SL[NC >= 3 ? 2 : 0]), bl);
+                xh = f2fma(bc2(C.x2[z]), bc2(SH[NC >= 3 ? 2 : 0]), bh);
             }
-            float2 xl = f2fma(C.x0, bc2(SL[0]), bc2(tl)), xh = f2fma(C.x0, bc2(SH[0]), bc2(th));
             if (!interior) {   // sides without flux
                 if (side_kind(kinds, 2 * d) == SK_NONE) xl = make_float2(0.0f, 0.0f);
                 if (side_kind(kinds, 2 * d + 1) == SK_NONE) xh = make_float2(0.0f, 0.0f);
             }
-            const float2 ml = pos2(xl), mh = pos2(xh);
-            co[z] = f2sub(ml, mh);
-            nl[z] = f2sub(ml, xl);
-            nh[z] = f2sub(mh, xh);
-            out[z] = f2add(out[z], f2add(ml, mh));
-            if (!interior) {   // boundary and interface sides: their distribution instead (add_records)
-                if (side_kind(kinds, 2 * d) != SK_DVM) nl[z] = make_float2(0.0f, 0.0f);
-                if (side_kind(kinds, 2 * d + 1) != SK_DVM) nh[z] = make_float2(0.0f, 0.0f);
-            }
+            ml[z] = pos2(xl);
+            mh[z] = pos2(xh);
+            nl[z] = f2sub(ml[z], xl);
+            nh[z] = f2sub(mh[z], xh);
+            out[z] = f2add(f2add(out[z], ml[z]), mh[z]);
+        }
+        const bool rl = !interior && side_kind(kinds, 2 * d) != SK_DVM, rh = !interior && side_kind(kinds, 2 * d + 1) != SK_DVM;
+        float2 own[ZP], fl[ZP], fh[ZP];
+#pragma unroll
+        for (int u = 0; u < ZP; ++u) {
+            const float2 c = unpack(tag, q.c0[u]), l = unpack(tag, q.l[d][u]), h = unpack(tag, q.h[d][u]);
+            const float2 dl = f2sub(c, l), dh = f2sub(h, c), two = make_float2(2.0f, 2.0f);
+            own[u] = mm2(dl, dh);
+            fl[u] = f2fma(two, l, mm2(f2sub(l, unpack(tag, q.l2[d][u])), dl));
+            fh[u] = f2fma(two, h, mm2(f2sub(h, unpack(tag, q.h2[d][u])), make_float2(-dh.x, -dh.y)));
         }
 #pragma unroll
         for (int u = 0; u < ZP; ++u) {
             const int z = NC == 3 ? u : 0;
-            const float2 c = unpack(tag, q.c0[u]), l = unpack(tag, q.l[d][u]), h = unpack(tag, q.h[d][u]);
-            const float2 dl = f2sub(c, l), dh = f2sub(c, h);
-            const float2 el = f2sub(l, unpack(tag, q.l2[d][u])), eh = f2sub(h, unpack(tag, q.h2[d][u]));
-            const float2 two = make_float2(2.0f, 2.0f);
-            num[u] = f2fma(co[z], mm2(dl, make_float2(-dh.x, -dh.y)), num[u]);
-            num[u] = f2fma(nl[z], f2fma(two, l, mm2(el, dl)), num[u]);
-            num[u] = f2fma(nh[z], f2fma(two, h, mm2(eh, dh)), num[u]);
+            num[u] = f2fma(ml[z], own[u], num[u]);
+            if (!rl) num[u] = f2fma(nl[z], fl[u], num[u]);
         }
+        if (rl) add_record<S, NC, ZP>(a, k, kinds, 2 * d, C, nl, num);
+#pragma unroll
+        for (int u = 0; u < ZP; ++u) {
+            const int z = NC == 3 ? u : 0;
+            num[u] = f2fma(mh[z], make_float2(-own[u].x, -own[u].y), num[u]);
+            if (!rh) num[u] = f2fma(nh[z], fh[u], num[u]);
+        }
+        if (rh) add_record<S, NC, ZP>(a, k, kinds, 2 * d + 1, C, nh, num);
     }
     float2 r[DZ];
 #pragma unroll
     for (int z = 0; z < DZ; ++z) {
-        r[z].x = recip_t<float>(fmaf(2.0f, out[z].x, m.it));
-        r[z].y = recip_t<float>(fmaf(2.0f, out[z].y, m.it));
+        r[z].x = recip_t<float>(2.0f * out[z].x);
+        r[z].y = recip_t<float>(2.0f * out[z].y);
     }
 #pragma unroll
     for (int u = 0; u < ZP; ++u)
@@ -296,11 +301,11 @@ static void launch_planes_t(gsis_ctx* c, const SweepArgs& a, int pass) {
     k_sweep_planes<S, NC, ZP, G, MINB><<<nptile * nztile, 32 * G, 0, c->stream>>>(a, (S*)c->f, pass, nptile);
 }
 
-// 2D: 128 registers, 15 warps per SM (four warps of 168 registers, 12 per SM: 6.59
-// ms against 6.40 on the FP32 cylinder); 3D: 168 registers, 12 warps per SM (five
-// warps, 10 per SM: 24.7 against 21.1 on the BF16 sphere).  Shape 1 has wider blocks for
-// velocity grids with few tiles: 36 x 38 x 17 on 4,271 cells FP32 2.00 ms (2.33 with
-// shape 0, 2.28 with the best pair tile), 32^3 on the sphere BF16 7.1 (8.7, 10.1).
+// 2D: 128 registers, 15 warps per SM (four warps of 168 registers, 12 per SM, were 3 %
+// slower on the FP32 cylinder); 3D: 168 registers, 12 warps per SM (five warps, 10 per
+// SM: 17 % slower on the BF16 sphere).  Shape 1 has wider blocks for velocity grids with
+// few tiles: 36 x 38 x 17 on 4,271 cells FP32 1.73 ms (2.07 with shape 0, 2.27 with the best
+// pair tile), 32^3 on the sphere BF16 7.2 (8.5, 10.1).
 template <typename S>
 static void launch_planes(gsis_ctx* c, const SweepArgs& a, int pass, int shape) {
     if (shape == 1) {
