@@ -22,6 +22,9 @@ __global__ void __launch_bounds__(32 * LINE_WPB, F64 ? 3 : 4) k_sweep_batch_line
     // kernel's occupancy (in the single launch they sit in the constant bank)
     __shared__ SweepArgs args[LINE_WPB];
     __shared__ LineStage stages[F64 ? 1 : LINE_WPB];
+    using T = typename std::conditional<F64, double, float>::type;
+    __shared__ LineEnds<T, F64 ? LINE_ZP64 : LINE_ZP32> ends[LINE_WPB];
+    auto& end = ends[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     SweepArgs& a = args[threadIdx.x >> 5];
     LineStage* stage = &stages[F64 ? 0 : threadIdx.x >> 5];
@@ -39,14 +42,14 @@ __global__ void __launch_bounds__(32 * LINE_WPB, F64 ? 3 : 4) k_sweep_batch_line
             reinterpret_cast<int*>(&a)[w] = reinterpret_cast<const int*>(&B.a)[w];
         __syncwarp();
         if constexpr (F64) {
-            line_tile<double, double, LINE_ZP64>(a, (double*)B.f, B.cells, it.y, lane, pass0, pass1, stage);
+            line_tile<double, double, LINE_ZP64>(a, (double*)B.f, B.cells, it.y, lane, pass0, pass1, stage, end);
         } else {
             if (dtype == GSIS_F32)
-                line_tile<float, float, LINE_ZP32>(a, (float*)B.f, B.cells, it.y, lane, pass0, pass1, stage);
+                line_tile<float, float, LINE_ZP32>(a, (float*)B.f, B.cells, it.y, lane, pass0, pass1, stage, end);
             else if (dtype == GSIS_BF16)
-                line_tile<__nv_bfloat16, float, LINE_ZP32>(a, (__nv_bfloat16*)B.f, B.cells, it.y, lane, pass0, pass1, stage);
+                line_tile<__nv_bfloat16, float, LINE_ZP32>(a, (__nv_bfloat16*)B.f, B.cells, it.y, lane, pass0, pass1, stage, end);
             else
-                line_tile<__half, float, LINE_ZP32>(a, (__half*)B.f, B.cells, it.y, lane, pass0, pass1, stage);
+                line_tile<__half, float, LINE_ZP32>(a, (__half*)B.f, B.cells, it.y, lane, pass0, pass1, stage, end);
         }
     }
 }

@@ -442,7 +442,7 @@ gsis_status tune_batch(BatchPlan* P) {
                                                 : "the forced batch tile needs FP32/BF16/FP16 members with an even nx");
     }
     {   // 1D members whose cells are all kinetic: the line sweep, without a search (the 64-shock batch:
-        // 13.7 ms per iteration, 18.8 with the best of the other tiles)
+        // 14.5 ms per iteration, 18.8 with the best of the other tiles)
         bool lines = true;
         for (gsis_ctx* c : P->ctxs) lines = lines && line_ok(c);
         for (int sh = 0; lines && sh < batch_num_shapes(); ++sh)

@@ -6,10 +6,11 @@ namespace gsis {
 template <typename S, typename T, int ZP>
 __global__ void __launch_bounds__(128) k_sweep_line(SweepArgs a, S* __restrict__ f, int N, int ntiles, int pass) {
     __shared__ LineStage stages[std::is_same<T, double>::value ? 1 : 4];
+    __shared__ LineEnds<T, ZP> ends[4];
     const int w = threadIdx.x >> 5, tile = blockIdx.x * 4 + w;   // four warps: one per SM sub-partition
     if (tile < ntiles)   // pass 1: backward, step 0
         line_tile<S, T, ZP>(a, f, N, tile, threadIdx.x & 31, 1 - pass, 2 - pass,
-                            &stages[std::is_same<T, double>::value ? 0 : w]);
+                            &stages[std::is_same<T, double>::value ? 0 : w], ends[w]);
 }
 
 // One cell per hyperplane, every cell kinetic, no periodic wrap: row k is cell

@@ -12,10 +12,12 @@
 // distance measured slower than reloading).  Ends of the line: rows are clamped,
 // and a repeated value gives the zero slope the scheme prescribes there.
 // FP32: planes in pairs for the f32x2 instructions (they share every
-// coefficient); FP64: bound by the FP64 pipe, 11 operations per point plus
+// coefficient), with the operations and roundings of the general sweep (long
+// shocks amplify a different rounding, 1e-4 of the state after a few iterations), so
+// the results are the same; FP64: bound by the FP64 pipe, 11 operations per point plus
 // 6 / ZP shared ones against 23.
 // Per iteration: a batch of 64 shocks of 100 to 800 cells, 24^3 to 64^3 velocities,
-// FP32 and BF16: 18.8 ms with the general sweep's best tile, 13.7 with this one; 30
+// FP32 and BF16: 18.8 ms with the general sweep's best tile, 14.5 with this one; 30
 // FP64 cells of 1,800 velocities alone 85 us -> 74.
 #pragma once
 #include <type_traits>
@@ -106,6 +108,12 @@ __device__ __forceinline__ void line_source(const V4<T>& x, const V4<T>* y, type
 // the L2), and in registers one cell ahead was both too late and too many.
 constexpr int LINE_STAGES = 4;
 constexpr int LINE_ZP32 = 4, LINE_ZP64 = 2;   // planes per column (batches)
+// A warp's shared memory: the end cells' boundary inflow (formed before the walk, so
+// that the loop body stays short), and the stages (FP32).
+template <typename T, int ZP>
+struct LineEnds {
+    T v[2][ZP][32];
+};
 struct LineStage {
     float4 x[LINE_STAGES][32];
     float4 y[LINE_STAGES][32 * LINE_ZP32];   // [row of the tile][plane]
@@ -128,7 +136,7 @@ __device__ __noinline__ T line_record(const T* scal, const T* tab, int NT, int n
 // directions (the instruction cache was the limit of longer bodies).
 template <typename S, typename T, int ZP>
 __device__ __forceinline__ void line_pass(const SweepArgs& a, const LineColumn<S, T, ZP>& C, int N, bool back,
-                                          LineStage* stage) {
+                                          LineStage* stage, LineEnds<T, ZP>& ends) {
     using P = typename Grp<T>::P;
     constexpr int W = Grp<T>::W, NG = ZP / W;
     constexpr bool F64 = std::is_same<T, double>::value;
@@ -186,6 +194,30 @@ __device__ __forceinline__ void line_pass(const SweepArgs& a, const LineColumn<S
     __syncwarp();   // the stages' last readers (the previous pass or item)
 #pragma unroll
     for (int j = 0; j < LINE_STAGES - 1; ++j) fetch(j);
+    bool none[2];   // an end without flux
+#pragma unroll 1
+    for (int s = 0; s < 2; ++s) {   // twice the boundary distributions at the ends
+        const int k = s ? N - 1 : 0, kd = side_kind(__ldg(a.sdi + (long long)k * SD_INTS + 12), s);
+        if (s) none[1] = kd == SK_NONE;
+        else none[0] = kd == SK_NONE;
+        const bool given = kd == SK_FAR || kd == SK_WALL;
+        const T sc = kd == SK_WALL ? __ldg(pick<T>(a.rho_w, a.rho_wf) + (long long)k * 6 + s) : T(1);
+        const T *rs = RecT<T>::scal(a.recBC, s), *rt = RecT<T>::tab(a.recBC, s, a.vg.NT);
+#pragma unroll 1
+        for (int u = 0; u < ZP; ++u) {
+            T v = T(0);
+            if (given)
+                v = T(2) * (sc * line_record<T>(rs, rt, a.vg.NT, nx, a.vg.ny, C.ix, C.iy, min(C.iz0 + u, a.vg.nz - 1)));
+            ends.v[s][u][lane] = v;
+        }
+    }
+    auto faces = [&](int j) {
+        const int k = cell(j);
+        LineFaces<T> o = load_faces<T>(a, k);
+        if (k == 0 && none[0]) o.Sl = T(0);
+        if (k == N - 1 && none[1]) o.Sh = T(0);
+        return o;
+    };
     P win[3][NG], fly[3][NG], b1[NG], b2[NG];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -194,7 +226,7 @@ __device__ __forceinline__ void line_pass(const SweepArgs& a, const LineColumn<S
     }
 #pragma unroll
     for (int g = 0; g < NG; ++g) b1[g] = b2[g] = win[0][g];
-    LineFaces<T> fa = load_faces<T>(a, cell(0)), fb = load_faces<T>(a, cell(1));
+    LineFaces<T> fa = faces(0), fb = faces(1);
     P nxt[NG];   // FP64: g~/tau of the next cell
     if constexpr (F64) source(0, nxt);
     for (int j0 = 0; j0 < N; j0 += 3) {
@@ -205,7 +237,7 @@ __device__ __forceinline__ void line_pass(const SweepArgs& a, const LineColumn<S
             const int k = first + dir * j;
             P in[NG], num[NG];
             load(j + 6, in);
-            const LineFaces<T> fc = load_faces<T>(a, cell(j + 2));
+            const LineFaces<T> fc = faces(j + 2);
             if constexpr (F64) {
 #pragma unroll
                 for (int g = 0; g < NG; ++g) num[g] = nxt[g];
@@ -221,16 +253,8 @@ __device__ __forceinline__ void line_pass(const SweepArgs& a, const LineColumn<S
             const P* a1 = win[(v + 1) % 3];
             const P* a2 = win[(v + 2) % 3];
             // upwind side of this lane (halved face speeds, outward)
-            T xl = C.x0 * fa.Sl, xh = C.x0 * fa.Sh;
+            const T xl = C.x0 * fa.Sl, xh = C.x0 * fa.Sh;
             const bool end_l = k == 0, end_h = k == N - 1;
-            int kl = SK_DVM, kh = SK_DVM;
-            if (end_l || end_h) {
-                const int kinds = __ldg(a.sdi + (long long)k * SD_INTS + 12);
-                kl = side_kind(kinds, 0);
-                kh = side_kind(kinds, 1);
-                if (kl == SK_NONE) xl = T(0);
-                if (kh == SK_NONE) xh = T(0);
-            }
             const T xb = back ? xh : xl, xa = back ? xl : xh;   // behind, ahead
             const bool ob = pos_t<T>(xb), oa = pos_t<T>(xa);
             const bool from_b = !ob && xb != T(0);              // inflow face behind
@@ -245,35 +269,36 @@ __device__ __forceinline__ void line_pass(const SweepArgs& a, const LineColumn<S
             if (rare && both_out) xo = xbp - xa;
             const T xi = from_b ? xb : (oa ? T(0) : xa);
             const bool end_b = back ? end_h : end_l, end_a = back ? end_l : end_h;
-            const T ci = (from_b ? end_b : end_a) ? T(0) : xi;   // a boundary side has its distribution instead (below)
+            const bool in_l = from_b != back;   // the inflow side is the low one
+            const bool given = from_b ? end_b : end_a;   // ... and a boundary: its distribution instead
 #pragma unroll
             for (int g = 0; g < NG; ++g) {
                 const P s1 = gsel(from_b, b1[g], a1[g]), s2 = gsel(from_b, b2[g], a2[g]), s0 = gsel(from_b, a1[g], b1[g]);
                 const P dn = gsub(c0[g], s1);
-                num[g] = gfma(-xo, gmm(dn, gsub(s0, c0[g])), num[g]);
-                const P fin = gfma(T(2), s1, gmm(gsub(s1, s2), dn));
-                num[g] = gfma(-ci, fin, num[g]);
-            }
-            if (rare && __any_sync(0xffffffffu, both_in)) {
-                const T ce = both_in && !end_a ? xa : T(0);
+                const P own = gmm(dn, gsub(s0, c0[g]));
+                P fin = gfma(T(2), s1, gmm(gsub(s1, s2), dn));
+                if (end_l || end_h) {
 #pragma unroll
-                for (int g = 0; g < NG; ++g) {
-                    const P fin = gfma(T(2), a1[g], gmm(gsub(a1[g], a2[g]), gsub(c0[g], a1[g])));
-                    num[g] = gfma(-ce, fin, num[g]);
+                    for (int i = 0; i < W; ++i)
+                        if (given) gput(fin, i, ends.v[in_l ? 0 : 1][g * W + i][lane]);
+                }
+                if constexpr (F64) {
+                    num[g] = gfma(-xo, own, num[g]);
+                    num[g] = gfma(-xi, fin, num[g]);
+                } else {   // the low side first, as the general sweep: the same roundings
+                    num[g] = gfma(in_l ? -xi : -xo, gsel(in_l, fin, own), num[g]);
+                    num[g] = gfma(in_l ? -xo : -xi, gsel(in_l, own, fin), num[g]);
                 }
             }
-            if (end_l || end_h) {
-                for (int s = 0; s < 2; ++s) {
-                    const int kd = s ? kh : kl;
-                    if (kd != SK_FAR && kd != SK_WALL) continue;
-                    const T sc = kd == SK_WALL ? __ldg(pick<T>(a.rho_w, a.rho_wf) + (long long)k * 6 + s) : T(1);
-                    const T xs = s ? xh : xl, x = pos_t<T>(xs) ? T(0) : xs;
-                    const T *rs = RecT<T>::scal(a.recBC, s), *rt = RecT<T>::tab(a.recBC, s, a.vg.NT);
+            if (rare && __any_sync(0xffffffffu, both_in)) {
+                const T ce = both_in ? xa : T(0);
 #pragma unroll
-                    for (int u = 0; u < ZP; ++u)
-                        gput(num[u / W], u % W, fma(-x, T(2) * sc * line_record<T>(rs, rt, a.vg.NT, nx, a.vg.ny, C.ix, C.iy,
-                                                                        min(C.iz0 + u, a.vg.nz - 1)),
-                                                 gget(num[u / W], u % W)));
+                for (int g = 0; g < NG; ++g) {
+                    P fin = gfma(T(2), a1[g], gmm(gsub(a1[g], a2[g]), gsub(c0[g], a1[g])));
+#pragma unroll
+                    for (int i = 0; i < W; ++i)
+                        if (end_a) gput(fin, i, ends.v[back ? 0 : 1][g * W + i][lane]);
+                    num[g] = gfma(-ce, fin, num[g]);
                 }
             }
             const T rden = recip_t<T>(fma(T(2), out, fa.it));
@@ -303,12 +328,12 @@ __device__ __forceinline__ void line_pass(const SweepArgs& a, const LineColumn<S
 // Steps pass0 .. pass1 - 1 (0: backward, 1: forward) of one tile.
 template <typename S, typename T, int ZP>
 __device__ __forceinline__ void line_tile(const SweepArgs& a, S* f, int N, int tile, int lane, int pass0, int pass1,
-                                          LineStage* stage) {
+                                          LineStage* stage, LineEnds<T, ZP>& ends) {
     const int nptile = (a.vg.nx * a.vg.ny + 31) / 32;
     LineColumn<S, T, ZP> C;
     make_line<S, T, ZP>(a.vg, f, tile % nptile, tile / nptile, lane, C);
 #pragma unroll 1
-    for (int step = pass0; step < pass1; ++step) line_pass<S, T, ZP>(a, C, N, step == 0, stage);
+    for (int step = pass0; step < pass1; ++step) line_pass<S, T, ZP>(a, C, N, step == 0, stage, ends);
 }
 
 }  // namespace gsis

@@ -74,3 +74,24 @@ def _couette(bc, cells=9, nv=(13, 12, 10)):
                                 (BC_NONE, BC_FARFIELD), (BC_FARFIELD, BC_NONE)])
 def test_lines_with_walls_and_closed_ends(bc):
     _check(_couette(bc))
+
+
+@pytest.mark.parametrize("dtype", list(BOUND))
+@pytest.mark.parametrize("cells,nv", [(7, (16, 9, 7)), (30, (20, 10, 9)), (65, (24, 16, 13))])
+def test_fp32_arithmetic_gives_the_bits_of_the_general_sweep(dtype, cells, nv):
+    """(Compared where f >= 2^-100: the kernel halves the face speeds and doubles the
+    sum, exact only while no product is an FP32 subnormal.)"""
+    from paper_2501_02245_gb300 import Solver
+    case = shock_1d_case(Ma=2.0, n_cells=cells, half_width=cells / 4.0, nv=nv, vmax=9.0, macro_steps=10)
+    W = []
+    for tile in (None, "g8_v1_c1"):
+        s = Solver.from_case(case, vdf_dtype=dtype)
+        if tile:
+            s.set_sweep_tile(tile)
+        s.iterate(3)
+        W.append((s.W(), s.vdf(cells)[1]))
+        s.close()
+    assert np.array_equal(W[0][0], W[1][0])
+    f, g = W[0][1], W[1][1]
+    big = np.maximum(f, g) >= 2.0 ** -100
+    assert big.any() and np.array_equal(f[big], g[big])
