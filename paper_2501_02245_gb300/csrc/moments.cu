@@ -296,7 +296,8 @@ __device__ __forceinline__ void unpack_chunk(const S*, uint4 w, float2* v) {
 // folds, per plane and thread) and the 32 lines of each load.  Two lanes share a
 // row, so that a load takes whole 32-byte sectors; a warp takes 8 rows iy x 4
 // planes iz as two batches of 16 rows (the rows of two planes each), the lanes
-// exchange the halves of the sums, and each lane folds one row.  A lane keeps its iy
+// exchange chunks, and each lane sums and folds one row (in the order of k_moments:
+// the same FP32 row sums).  A lane keeps its iy
 // over the units of a strip, so it folds with the planes' z weights (shared
 // memory) only, and with the powers of c_y once per strip.  10,482 cells of 55,296
 // velocities: FP32 0.95 -> 0.72 ms, BF16 0.78 -> 0.66; 11,643 BF16 cells of 119,808: 2.24
@@ -357,54 +358,47 @@ __global__ void __launch_bounds__(MROW_THREADS, 6) k_moments_rows(int Nd, const 
         const bool in0 = iy < ny && iz < nz, in1 = iy < ny && iz + 2 < nz;
         const uint4* p0 = base + (iy + ny * iz) * nc;
         const uint4* p1 = p0 + 2 * ny * nc;
-        float2 a[4], b[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) a[q] = b[q] = make_float2(0.0f, 0.0f);
-        for (int i0 = j; i0 < nc; i0 += 2 * U) {
+        float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // the sums of row j, node by node in order
+        for (int i0 = 0; i0 < nc; i0 += 2 * U) {
             uint4 x0[U], x1[U];
 #pragma unroll
             for (int i = 0; i < U; ++i) {
-                const int ch = i0 + 2 * i;
+                const int ch = i0 + 2 * i + j;
                 x0[i] = x1[i] = make_uint4(0u, 0u, 0u, 0u);
                 if (ch < nc && in0) x0[i] = p0[ch];
                 if (ch < nc && in1) x1[i] = p1[ch];
             }
 #pragma unroll
             for (int i = 0; i < U; ++i) {
-                const int ch = i0 + 2 * i;
-                if (ch >= nc) break;
-                float2 v0[H], v1[H];
-                unpack_chunk(fk, x0[i], v0);
-                unpack_chunk(fk, x1[i], v1);
+                if (i0 + 2 * i >= nc) break;
+                const uint4 give = j ? x0[i] : x1[i];
+                uint4 got;
+                got.x = __shfl_xor_sync(0xffffffffu, give.x, 1);
+                got.y = __shfl_xor_sync(0xffffffffu, give.y, 1);
+                got.z = __shfl_xor_sync(0xffffffffu, give.z, 1);
+                got.w = __shfl_xor_sync(0xffffffffu, give.w, 1);
 #pragma unroll
-                for (int h = 0; h < H; h += 2) {
-                    const float4* t = reinterpret_cast<const float4*>(scx + ch * V + 2 * h);
+                for (int e = 0; e < 2; ++e) {   // the row's chunks 2 i and 2 i + 1
+                    const int ch = i0 + 2 * i + e;
+                    if (ch >= nc) break;
+                    float2 v[H];
+                    unpack_chunk(fk, e ? (j ? x1[i] : got) : (j ? got : x0[i]), v);
+                    float w1[V], w2[V], w3[V];
+                    lds16<float, V>(scx + ch * V, w1);
+                    lds16<float, V>(scx + nx + ch * V, w2);
+                    lds16<float, V>(scx + 2 * nx + ch * V, w3);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        if (q == 0) {
-                            a[0] = f2add(a[0], v0[h]);
-                            a[0] = f2add(a[0], v0[h + 1]);
-                            b[0] = f2add(b[0], v1[h]);
-                            b[0] = f2add(b[0], v1[h + 1]);
-                        } else {
-                            const float4 wx = t[(q - 1) * (nx / 4)];
-                            const float2 lo = make_float2(wx.x, wx.y), hi = make_float2(wx.z, wx.w);
-                            a[q] = f2fma(v0[h], lo, a[q]);
-                            a[q] = f2fma(v0[h + 1], hi, a[q]);
-                            b[q] = f2fma(v1[h], lo, b[q]);
-                            b[q] = f2fma(v1[h + 1], hi, b[q]);
-                        }
+                    for (int h = 0; h < V; ++h) {
+                        const float fv = h & 1 ? v[h / 2].y : v[h / 2].x;
+                        s[0] += fv;
+                        s[1] += fv * w1[h];
+                        s[2] += fv * w2[h];
+                        s[3] += fv * w3[h];
                     }
                 }
             }
         }
-        double d[4];   // the row sums of batch j
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float s0 = a[q].x + a[q].y, s1 = b[q].x + b[q].y;
-            const float other = __shfl_xor_sync(0xffffffffu, j ? s0 : s1, 1);
-            d[q] = (j ? s1 : s0) + other;
-        }
+        const double d[4] = {s[0], s[1], s[2], s[3]};
         const double* z = zt + 4 * min(iz + 2 * j, nz - 1);   // (a row past the end has zero sums)
         const double2 z01 = *reinterpret_cast<const double2*>(z), z23 = *reinterpret_cast<const double2*>(z + 2);
         Z[0] = fma(d[0], z01.x, Z[0]);
