@@ -185,8 +185,9 @@ def traffic_per_point(config, dtype):
         return None
     with open(p) as fh:
         d = json.load(fh)
-    sha = source_sha(["paper_2501_02245_gb300/csrc/sweep.cu", "paper_2501_02245_gb300/csrc/sweep_device.cuh",
-                      "paper_2501_02245_gb300/csrc/sweep_pair.cuh", "paper_2501_02245_gb300/csrc/gsis_device.cuh"])
+    sha = source_sha(["paper_2501_02245_gb300/csrc/" + f for f in
+                      ("sweep.cu", "sweep_device.cuh", "sweep_pair.cuh", "sweep_col.cu", "sweep_planes.cuh",
+                       "sweep_line.cuh", "gsis_device.cuh")])
     if d.get("sweep_src_sha") != sha:
         return None
     return d.get("dram_bytes_per_point")
@@ -344,7 +345,7 @@ def sweep_roofline(args, rep, steps, peaks, traffic):
             peak, src = FP64_PEAK_TFLOPS, "FP64 unit counts x clock: 152 SMs x 2 DFMA/clk x 2.07 GHz (derived)"
         achieved = fpp * pts / (sweep_ms_iter * 1e-3) / 1e12
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": trf, "kernel": "k_sweep<double>", "peak_source": src,
+                "traffic": trf, "kernel": "k_sweep<double>" if args.config == "shock" else "k_sweep_col", "peak_source": src,
                 "per": "GSIS iteration: %g sweep launches (Gauss-Seidel passes) per iteration" % launches_iter,
                 "algorithmic": "%d FP64 flop per (cell, velocity) per GSIS iteration (one point update)" % fpp,
                 "per_pass": {"achieved": achieved * launches_iter, "frac": achieved * launches_iter / peak,
@@ -353,7 +354,7 @@ def sweep_roofline(args, rep, steps, peaks, traffic):
     else:
         achieved = 2 * eb * pts / (sweep_ms_iter * 1e-3) / 1e9
         roof = {"bound": "hbm", "achieved": achieved, "peak": mp["hbm_gbs"], "unit": "GB/s",
-                "frac": achieved / mp["hbm_gbs"], "traffic": trf, "kernel": "k_sweep",
+                "frac": achieved / mp["hbm_gbs"], "traffic": trf, "kernel": "k_sweep_planes",
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured copy bandwidth)",
                 "per": "GSIS iteration: %g sweep launches (Gauss-Seidel passes) per iteration" % launches_iter,
                 "algorithmic": "2 x %d bytes per (cell, velocity) per GSIS iteration (read f once, write once)" % eb,
@@ -730,7 +731,7 @@ def run_batch(args):
     achieved = bytes_alg / (sweep_ms * 1e-3) / 1e9
     roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": achieved / peaks["hbm_gbs"], "traffic": None,
-            "kernel": "k_sweep_batch (both Gauss-Seidel passes of all 64 solves, one launch)",
+            "kernel": "k_sweep_batch_line (both Gauss-Seidel passes of all 64 solves, one launch)",
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured)",
             "algorithmic": "2 passes x 2 x b bytes per (cell, velocity), b = 4 (FP32) / 2 (BF16)"}
     info = batch_info(solvers)

@@ -1292,9 +1292,9 @@ void macro_block(gsis_ctx* c, int steps, bool with_hot, bool time_term, bool cap
     const int N = c->m.N;
     if (steps <= 0) return;
     // automatic choice: the per-phase kernels above the fused kernel's limit (measured on the 16,384-cell
-    // cylinder, 100 pseudo-steps: per-phase kernels 11.1 ms, persistent kernel 13.0 ms with one CTA on
-    // each of 128 SMs and 23.8 ms with every co-resident CTA -- its 600 grid barriers cost more than
-    // the launches they replace, the phases being bound by the FP64 special functions of the fluxes)
+    // cylinder, 100 pseudo-steps, when the phases took 11.1 ms (5.95 now): persistent kernel 13.0 ms with
+    // one CTA on each of 128 SMs and 23.8 ms with every co-resident CTA -- its 600 grid barriers cost more
+    // than the launches they replace)
     int path = c->macro_path;
     if (path == MACRO_AUTO) path = N <= MACRO_FUSED_MAX_CELLS ? MACRO_FUSED : MACRO_MULTI;
     if (capturing && (path == MACRO_PERSISTENT || path == MACRO_PERSISTENT_STALL)) path = MACRO_MULTI;
