@@ -1169,7 +1169,6 @@ void launch_hot(gsis_ctx* c) {
 // distributed shared memory, so that a few states fill the SMs.  96 states of
 // 48 x 48 x 24 nodes: 549 us before.
 constexpr int TWO_VDF_THREADS = 128;
-constexpr int TWO_VDF_SUMS = 16;
 
 // Sums of v[16] over the warp: lanes 2 i and 2 i + 1 return the total of v[i].
 // Each step keeps the half of the values whose index bit matches the lane's, so
