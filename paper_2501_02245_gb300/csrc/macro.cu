@@ -218,12 +218,12 @@ __global__ void k_prim_to_cons(int N, const double* __restrict__ Wp, double* __r
 // FP64-pipe operations.)
 __device__ __forceinline__ void cons_to_prim(const double* U, double* Wp) {
     const double r = U[0], ir = recip64(r);
-    const double ux = U[1] * ir, uy = U[2] * ir, uz = U[3] * ir;
+    const double ux = __dmul_rn(U[1], ir), uy = __dmul_rn(U[2], ir), uz = __dmul_rn(U[3], ir);
     Wp[0] = r;
     Wp[1] = ux;
     Wp[2] = uy;
     Wp[3] = uz;
-    Wp[4] = (2.0 * U[4] * ir - (ux * ux + uy * uy + uz * uz)) * (1.0 / 3.0);
+    Wp[4] = fma(2.0 * U[4], ir, -fma(uz, uz, fma(ux, ux, __dmul_rn(uy, uy)))) * (1.0 / 3.0);
 }
 
 __global__ void k_cons_to_prim(int N, const double* __restrict__ U, double* __restrict__ Wp) {
@@ -307,78 +307,96 @@ void launch_cons_to_prim(gsis_ctx* c, const double* Ucons, double* Wprim) {
 }
 
 // ---------------------------------------------------------------------------- fluxes
+// a . b over the first ND components.  Every sum of products of the pseudo-steps
+// below is written out with its fused and its rounded products (fma, __dmul_rn): left
+// to the compiler, the choice depends on the code around it, and the one-lane, the two-lane,
+// the fused and the per-phase forms of a step would end in different last bits.
+template <int ND>
+__device__ __forceinline__ double dot_rn(const double* a, const double* b) {
+    if (ND == 1) return __dmul_rn(a[0], b[0]);
+    double v = fma(a[0], b[0], __dmul_rn(a[1], b[1]));
+    if (ND > 2) v = fma(a[2], b[2], v);
+    return v;
+}
+
 // Flux carried by the molecules of the Maxwellian (r, u, T) that cross a
 // face of unit normal n in the direction sign*n (half-range moments of the
-// normal Gaussian N(u.n, T); tangential thermal motion in closed form),
-// added to F.
+// normal Gaussian N(u.n, T); tangential thermal motion in closed form): c[q] X[q]
+// with c = r (mass, momentum) and r/2 (energy).
 // (ND: the normal has components 0..ND-1 only; the others are exact zeros,
 // so the terms they multiply are left out.)
 template <int ND>
-__device__ __forceinline__ void half_range_add(double r, const double* u, double T, const double* n, double sign,
-                                               double* F) {
-    double un = u[0] * n[0];
-#pragma unroll
-    for (int i = 1; i < ND; ++i) un += u[i] * n[i];
+__device__ __forceinline__ void half_range(const double* u, double T, const double* n, double sign, double* X) {
+    const double un = dot_rn<ND>(u, n);
     // s = un / sqrt(T) and sqrt(T) = T / sqrt(T) from one reciprocal square root
     // (instead of a square root and two FP64 divisions).  P is the share of the
     // Maxwellian that crosses, (1 + sign erf(s/sqrt 2))/2, from its tail
     // q = h(|s|) exp(-s^2/2): q where the gas recedes, 1 - q where it approaches.
     const double ist = rsqrt(T), st = T * ist, s = un * ist;
-    const double e = exp_tab(-0.5 * s * s), q = mills(__longlong_as_double((long long)mag_bits(s))) * e;
+    const double e = exp_tab(-0.5 * s * s), q = __dmul_rn(mills(__longlong_as_double((long long)mag_bits(s))), e);
     const bool towards = (__double2hiint(s) >= 0) == (sign > 0.0);
     const double P = towards ? 1.0 - q : q;
-    const double D = sign * st * e * 0.3989422804014327;   // 1/sqrt(2 pi)
-    const double M0 = un * P + D;
-    const double M1 = (un * un + T) * P + un * D;
-    const double M2 = (un * un * un + 3.0 * un * T) * P + (un * un + 2.0 * T) * D;
+    const double D = __dmul_rn(sign * st * e, 0.3989422804014327);   // 1/sqrt(2 pi)
+    const double M0 = fma(un, P, D);
+    const double u2 = __dmul_rn(un, un);
+    const double M1 = fma(u2 + T, P, __dmul_rn(un, D));
+    const double M2 = fma(fma(u2, un, __dmul_rn(3.0 * un, T)), P, __dmul_rn(u2 + 2.0 * T, D));
     double ut[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) ut[i] = i < ND ? u[i] - un * n[i] : u[i];
-    F[0] += r * M0;
+    for (int i = 0; i < 3; ++i) ut[i] = i < ND ? fma(-un, n[i], u[i]) : u[i];
+    X[0] = M0;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) F[1 + i] += r * (i < ND ? M1 * n[i] + ut[i] * M0 : ut[i] * M0);
-    F[4] += 0.5 * r * (M2 + (ut[0] * ut[0] + ut[1] * ut[1] + ut[2] * ut[2] + 2.0 * T) * M0);
+    for (int i = 0; i < 3; ++i) X[1 + i] = i < ND ? fma(M1, n[i], __dmul_rn(ut[i], M0)) : __dmul_rn(ut[i], M0);
+    X[4] = fma(fma(ut[2], ut[2], fma(ut[0], ut[0], __dmul_rn(ut[1], ut[1]))) + 2.0 * T, M0, M2);
 }
 
 // Kinetic flux-vector splitting per unit area through the unit normal n: the
 // left Maxwellian's molecules moving along +n plus the right one's moving
 // along -n -- the Euler flux that the discrete-velocity upwind scheme carries
-// for Maxwellian states.
+// for Maxwellian states.  The left half is rounded, the right one added with one
+// fused multiply-add: written out, so that kfvs_pair rounds the same way.
 template <int ND = 3>
 __device__ void kfvs(double rL, const double* uL, double pL, double rR, const double* uR, double pR,
                      const double* n, double* F) {
-    for (int q = 0; q < 5; ++q) F[q] = 0.0;
-    half_range_add<ND>(rL, uL, pL * recip64(rL), n, 1.0, F);
-    half_range_add<ND>(rR, uR, pR * recip64(rR), n, -1.0, F);
+    double X[5];
+    half_range<ND>(uL, __dmul_rn(pL, recip64(rL)), n, 1.0, X);
+    for (int q = 0; q < 5; ++q) F[q] = fma(q < 4 ? rL : 0.5 * rL, X[q], 0.0);
+    half_range<ND>(uR, __dmul_rn(pR, recip64(rR)), n, -1.0, X);
+    for (int q = 0; q < 5; ++q) F[q] = fma(q < 4 ? rR : 0.5 * rR, X[q], F[q]);
 }
 
 // The same sum formed by a pair of lanes (2i, 2i + 1), each with its own side's
 // state (odd lanes: the right one): the two half-range chains run side by side.
-// Both lanes get the flux, the same bits as kfvs.
+// The even lane gets the flux, the same bits as kfvs.
 template <int ND>
 __device__ __forceinline__ void kfvs_pair(double r, const double* u, double p, bool right, const double* n, double* F) {
-    double H[5] = {0, 0, 0, 0, 0};
-    half_range_add<ND>(r, u, p * recip64(r), n, right ? -1.0 : 1.0, H);
+    double X[5];
+    half_range<ND>(u, __dmul_rn(p, recip64(r)), n, right ? -1.0 : 1.0, X);
     const unsigned pair = 3u << (threadIdx.x & 30);
+    const double ro = __shfl_xor_sync(pair, r, 1);
 #pragma unroll
-    for (int q = 0; q < 5; ++q) F[q] = H[q] + __shfl_xor_sync(pair, H[q], 1);
+    for (int q = 0; q < 5; ++q)
+        F[q] = fma(q < 4 ? ro : 0.5 * ro, __shfl_xor_sync(pair, X[q], 1), fma(q < 4 ? r : 0.5 * r, X[q], 0.0));
 }
 
 // Euler flux tensor of conserved state U: F[q * 3 + i] = flux of component q
 // along axis i (so that F.S is euler_flux_dot(U, S)), one division.  Only the
 // axes i < ND are formed: on a mesh whose face normals have no component
 // along the others (ND = normal_components), F.S never reads them.
+// sub: the tensor less this one.
 template <int ND>
-__device__ __forceinline__ void euler_tensor(const double* U, double* F) {
+__device__ __forceinline__ void euler_tensor(const double* U, double* F, const double* sub = nullptr) {
     const double r = U[0], ir = recip64(r);
-    const double u[3] = {U[1] * ir, U[2] * ir, U[3] * ir};
-    const double p = (GAMMA - 1.0) * (U[4] - 0.5 * r * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
+    const double u[3] = {__dmul_rn(U[1], ir), __dmul_rn(U[2], ir), __dmul_rn(U[3], ir)};
+    const double e = fma(-(0.5 * r), dot_rn<3>(u, u), U[4]);
+    const double h = fma(GAMMA - 1.0, e, U[4]);
 #pragma unroll
     for (int i = 0; i < ND; ++i) {
-        F[i] = U[1 + i];
+        double Fi[4] = {U[1 + i], __dmul_rn(U[1], u[i]), __dmul_rn(U[2], u[i]), __dmul_rn(U[3], u[i])};
+        Fi[1 + i] = fma(GAMMA - 1.0, e, Fi[1 + i]);   // + p
 #pragma unroll
-        for (int j = 0; j < 3; ++j) F[(1 + j) * 3 + i] = U[1 + j] * u[i] + (i == j ? p : 0.0);
-        F[12 + i] = (U[4] + p) * u[i];
+        for (int q = 0; q < 4; ++q) F[q * 3 + i] = sub ? Fi[q] - sub[q * 3 + i] : Fi[q];
+        F[12 + i] = sub ? fma(h, u[i], -sub[12 + i]) : __dmul_rn(h, u[i]);
     }
 }
 
@@ -394,15 +412,29 @@ __device__ __forceinline__ void flux_change(const double* U, const double* dU, c
     double Up[5], F1[15];
 #pragma unroll
     for (int q = 0; q < 5; ++q) Up[q] = U[q] + dU[q];
-    euler_tensor<ND>(Up, F1);
+    euler_tensor<ND>(Up, F1, F0);
 #pragma unroll
     for (int q = 0; q < 5; ++q)
 #pragma unroll
-        for (int i = 0; i < ND; ++i) dF[(long long)(q * 3 + i) * N + c] = F1[q * 3 + i] - F0[q * 3 + i];
+        for (int i = 0; i < ND; ++i) dF[(long long)(q * 3 + i) * N + c] = F1[q * 3 + i];
 }
 
 __device__ __forceinline__ void prim5(const double* w, double* q) {   // (rho, u, p)
-    q[0] = w[0]; q[1] = w[1]; q[2] = w[2]; q[3] = w[3]; q[4] = w[0] * w[4];
+    q[0] = w[0]; q[1] = w[1]; q[2] = w[2]; q[3] = w[3]; q[4] = __dmul_rn(w[0], w[4]);
+}
+
+// Face state of a cell (rho, u, p: q, its primitives w) towards its neighbour on the
+// other side of the face, to which df are the differences: q +- half the minmod of
+// df and the difference to the cell beyond (wo; none: no such cell, zero slope).
+__device__ __forceinline__ void face_state(const double* q, const double* w, const double* wo, bool right, bool none,
+                                           const double* df, double* f) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const double d = k < 4 ? (right ? wo[k] - q[k] : q[k] - wo[k])
+                               : (right ? fma(wo[0], wo[4], -q[4]) : fma(-wo[0], wo[4], q[4]));
+        const double h = none ? 0.0 : hmm_t<double>(df[k], d), m = right ? -h : h;
+        f[k] = k < 4 ? q[k] + m : fma(w[0], w[4], m);
+    }
 }
 
 // Interior face between L = cell c and R = its neighbour across side 2d+1
@@ -439,7 +471,7 @@ __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* W
     const double nn[3] = {G[1], G[2], G[3]}, S[3] = {G[9], G[10], G[11]};
     // MUSCL face states: q -/+ 0.5 minmod of the one-sided differences (the
     // halved limiter on the integer pipe), first order where the second
-    // neighbour is missing (the cell itself in its place: a zero difference)
+    // neighbour is missing (the cell itself is read in its place)
     const bool right = PAIR && (threadIdx.x & 1);
     double wL[5], wR[5], qL[5], qR[5], Fv[5];
     const double *pl = Wm + (st.x >= 0 ? st.x : L) * 5, *ph = Wm + (st.z >= 0 ? st.z : Rr) * 5;
@@ -448,35 +480,25 @@ __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* W
 #pragma unroll
         for (int q = 0; q < 5; ++q) { wL[q] = pL[q]; wR[q] = pR[q]; }
     }
-    if constexpr (PAIR) {
-        double qo[5], fs[5];   // the outer neighbour and the face state of this lane's side
-        prim5(right ? ph : pl, qo);
-        prim5(wL, qL);
-        prim5(wR, qR);
+    double df[5];
+    prim5(wL, qL);
+    prim5(wR, qR);
 #pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            const double df = qR[q] - qL[q], dq = right ? qo[q] - qR[q] : qL[q] - qo[q];
-            const double m = hmm_t<double>(df, dq);
-            fs[q] = right ? qR[q] - m : qL[q] + m;
-        }
+    for (int q = 0; q < 4; ++q) df[q] = qR[q] - qL[q];
+    const double dfL = fma(wR[0], wR[4], -qL[4]), dfR = qR[4] - qL[4];   // (the two sides' roundings of the pressure's)
+    if constexpr (PAIR) {
+        double fs[5];   // the face state of this lane's side
+        df[4] = right ? dfR : dfL;
+        face_state(right ? qR : qL, right ? wR : wL, right ? ph : pl, right, (right ? st.z : st.x) < 0, df, fs);
         kfvs_pair<ND>(fs[0], fs + 1, fs[4], right, nn, Fv);
     } else {
-        double ql[5], qh[5], mL[5], mR[5];
-        prim5(pl, ql);
-        prim5(ph, qh);
-        prim5(wL, qL);
-        prim5(wR, qR);
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            const double df = qR[q] - qL[q];
-            mL[q] = hmm_t<double>(qL[q] - ql[q], df);
-            mR[q] = hmm_t<double>(df, qh[q] - qR[q]);
-        }
         double fl[5], fr[5];
-        for (int q = 0; q < 5; ++q) { fl[q] = qL[q] + mL[q]; fr[q] = qR[q] - mR[q]; }
+        df[4] = dfL;
+        face_state(qL, wL, pl, false, st.x < 0, df, fl);
+        df[4] = dfR;
+        face_state(qR, wR, ph, true, st.z < 0, df, fr);
         kfvs<ND>(fl[0], fl + 1, fl[4], fr[0], fr + 1, fr[4], nn, Fv);
     }
-    for (int q = 0; q < 5; ++q) Fv[q] *= Sabs;
     // viscous + HoT
     const double uf[3] = {0.5 * (wL[1] + wR[1]), 0.5 * (wL[2] + wR[2]), 0.5 * (wL[3] + wR[3])};
     const double Tf = 0.5 * (wL[4] + wR[4]);
@@ -489,75 +511,65 @@ __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* W
     double guf[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, gTf[3] = {0, 0, 0};
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        double gav[3], ge = 0.0;
+        double gav[3];
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
             gav[i] = 0.5 * (gu[(long long)(j * 3 + i) * N + L] + gu[(long long)(j * 3 + i) * N + Rr]);
-            ge = i == 0 ? gav[0] * e[0] : ge + gav[i] * e[i];
         }
-        const double corr = (wR[1 + j] - wL[1 + j]) * idist - ge;
+        const double corr = fma(wR[1 + j] - wL[1 + j], idist, -dot_rn<ND>(gav, e));
 #pragma unroll
-        for (int i = 0; i < ND; ++i) guf[j * 3 + i] = gav[i] + corr * e[i];
+        for (int i = 0; i < ND; ++i) guf[j * 3 + i] = fma(corr, e[i], gav[i]);
     }
     {
-        double gav[3], ge = 0.0;
+        double gav[3];
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
             gav[i] = 0.5 * (gT[(long long)i * N + L] + gT[(long long)i * N + Rr]);
-            ge = i == 0 ? gav[0] * e[0] : ge + gav[i] * e[i];
         }
-        const double corr = (wR[4] - wL[4]) * idist - ge;
+        const double corr = fma(wR[4] - wL[4], idist, -dot_rn<ND>(gav, e));
 #pragma unroll
-        for (int i = 0; i < ND; ++i) gTf[i] = gav[i] + corr * e[i];
+        for (int i = 0; i < ND; ++i) gTf[i] = fma(corr, e[i], gav[i]);
     }
     // Eq. NSF_constitutive (nsf_of) with the zero gradient entries (directions
     // i >= ND) not multiplied: the same values
-    double sig[6], qf[3];
+    const double* hL = hot + (long long)L * HOTN;
+    const double* hR = hot + (long long)Rr * HOTN;
+    double Sg[6], Q[3], hf[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) hf[q] = 0.5 * (hL[q] + hR[q]);
     {
         double div = guf[0];
         if (ND > 1) div += guf[4];
         if (ND > 2) div += guf[8];
-        const double two3 = 2.0 / 3.0, t = two3 * div;
-        sig[0] = -muf * (2.0 * guf[0] - t);
-        sig[1] = ND > 1 ? -muf * (2.0 * guf[4] - t) : -muf * (-t);
-        sig[2] = ND > 2 ? -muf * (2.0 * guf[8] - t) : -muf * (-t);
-        sig[3] = -muf * (ND > 1 ? guf[1] + guf[3] : guf[3]);   // du_x/dy + du_y/dx
-        sig[4] = -muf * (ND > 2 ? guf[2] + guf[6] : guf[6]);   // du_x/dz + du_z/dx
-        sig[5] = ND > 1 ? -muf * (ND > 2 ? guf[5] + guf[7] : guf[7]) : 0.0;   // du_y/dz + du_z/dy
+        const double two3 = 2.0 / 3.0;
+        const double t = __dmul_rn(two3, div);
+        auto stress = [&](double g, double h) { return __dmul_rn(-muf, g) + h; };
+        Sg[0] = stress(2.0 * guf[0] - t, hf[0]);
+        Sg[1] = stress(2.0 * guf[4] - t, hf[1]);
+        Sg[2] = stress(2.0 * guf[8] - t, hf[2]);
+        Sg[3] = stress(ND > 1 ? guf[1] + guf[3] : guf[3], hf[3]);   // du_x/dy + du_y/dx
+        Sg[4] = stress(ND > 2 ? guf[2] + guf[6] : guf[6], hf[4]);   // du_x/dz + du_z/dx
+        Sg[5] = ND > 1 ? stress(ND > 2 ? guf[5] + guf[7] : guf[7], hf[5]) : hf[5];   // du_y/dz + du_z/dy
         const double kap = 3.75 * muf;
 #pragma unroll
-        for (int i = 0; i < 3; ++i) qf[i] = i < ND ? -kap * gTf[i] : 0.0;
+        for (int i = 0; i < 3; ++i) Q[i] = i < ND ? fma(-kap, gTf[i], hf[6 + i]) : hf[6 + i];
     }
-    const double* hL = hot + (long long)L * HOTN;
-    const double* hR = hot + (long long)Rr * HOTN;
-    double Sg[6], Q[3];
-    for (int q = 0; q < 6; ++q) Sg[q] = sig[q] + 0.5 * (hL[q] + hR[q]);
-    for (int q = 0; q < 3; ++q) Q[q] = qf[q] + 0.5 * (hL[6 + q] + hR[6 + q]);
     // sigma . S and q . S over the normal's components 0..ND-1
     const double row[3][3] = {{Sg[0], Sg[3], Sg[4]}, {Sg[3], Sg[1], Sg[5]}, {Sg[4], Sg[5], Sg[2]}};
-    double SigS[3], QS = Q[0] * S[0];
+    double SigS[3];
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        double v = row[r][0] * S[0];
-#pragma unroll
-        for (int k = 1; k < ND; ++k) v += row[r][k] * S[k];
-        SigS[r] = v;
-    }
-#pragma unroll
-    for (int k = 1; k < ND; ++k) QS += Q[k] * S[k];
+    for (int r = 0; r < 3; ++r) SigS[r] = dot_rn<ND>(row[r], S);
     if (!right) {
         double* F = Ff + (long long)(5 * d) * N + L;
-        F[0] = Fv[0];
-        F[(long long)N] = Fv[1] + SigS[0];
-        F[(long long)2 * N] = Fv[2] + SigS[1];
-        F[(long long)3 * N] = Fv[3] + SigS[2];
-        F[(long long)4 * N] = Fv[4] + ((SigS[0] * uf[0] + SigS[1] * uf[1] + SigS[2] * uf[2]) + QS);
+        F[0] = __dmul_rn(Fv[0], Sabs);
+        F[(long long)N] = fma(Fv[1], Sabs, SigS[0]);
+        F[(long long)2 * N] = fma(Fv[2], Sabs, SigS[1]);
+        F[(long long)3 * N] = fma(Fv[3], Sabs, SigS[2]);
+        const double w = dot_rn<3>(SigS, uf);
+        F[(long long)4 * N] = fma(Fv[4], Sabs, ND == 1 ? fma(Q[0], S[0], w) : w + dot_rn<ND>(Q, S));
     }
     const double aL = acell[L], aR = acell[Rr];
-    double un = uf[0] * nn[0];
-#pragma unroll
-    for (int k = 1; k < ND; ++k) un += uf[k] * nn[k];
-    const double lam = fabs(un) + 0.5 * (aL + aR) + 5.0 * muf * recip64(0.5 * (wL[0] + wR[0]) * dist);
+    const double lam = fabs(dot_rn<ND>(uf, nn)) + 0.5 * (aL + aR) + __dmul_rn(5.0 * muf, recip64(0.5 * (wL[0] + wR[0]) * dist));
     if (!right) lamf[(long long)d * N + L] = lam * Sabs;
 }
 
@@ -732,24 +744,21 @@ __device__ __forceinline__ void boundary_flux_one(const MacroArgs& a, const doub
         } else {
             kfvs(rho_c, u_c, p_c, st[0], st + 1, st[0] * st[4], nn, Fb);
         }
-        for (int q = 0; q < 5; ++q) Fb[q] *= Sabs;
-        const double SigS[3] = {h[0] * So[0] + h[3] * So[1] + h[4] * So[2],
-                                h[3] * So[0] + h[1] * So[1] + h[5] * So[2],
-                                h[4] * So[0] + h[5] * So[1] + h[2] * So[2]};
+        const double row[3][3] = {{h[0], h[3], h[4]}, {h[3], h[1], h[5]}, {h[4], h[5], h[2]}};
+        const double SigS[3] = {dot_rn<3>(row[0], So), dot_rn<3>(row[1], So), dot_rn<3>(row[2], So)};
         const double ufb[3] = {0.5 * (u_c[0] + st[1]), 0.5 * (u_c[1] + st[2]), 0.5 * (u_c[2] + st[3])};
-        Fb[1] += SigS[0];
-        Fb[2] += SigS[1];
-        Fb[3] += SigS[2];
-        Fb[4] += (SigS[0] * ufb[0] + SigS[1] * ufb[1] + SigS[2] * ufb[2]) +
-                 (h[6] * So[0] + h[7] * So[1] + h[8] * So[2]);
+        Fb[0] = __dmul_rn(Fb[0], Sabs);
+        for (int q = 1; q < 4; ++q) Fb[q] = fma(Fb[q], Sabs, SigS[q - 1]);
+        Fb[4] = fma(Fb[4], Sabs, dot_rn<3>(SigS, ufb) + dot_rn<3>(h + 6, So));
     } else {
         wall_nsf_flux(a, wc, gu, gT, c, s, Fb);
         const double* wcr = wall_corr + (long long)cs * 5;
         for (int q = 0; q < 5; ++q) Fb[q] += wcr[q];
     }
+    if (PAIR && (threadIdx.x & 1)) return;   // (the even lane has the flux)
     const double a_c = sqrt(GAMMA * p_c / rho_c);
     const double mu_c = viscosity_tab(T_c, a.mu0, a.omega);
-    const double lam = fabs(u_c[0] * nn[0] + u_c[1] * nn[1] + u_c[2] * nn[2]) + a_c +
+    const double lam = fabs(dot_rn<3>(u_c, nn)) + a_c +
                        5.0 * mu_c / (rho_c * 2.0 * bdist);
     double* o = Fbnd + (long long)cs * 6;
     for (int q = 0; q < 5; ++q) o[q] = Fb[q];
@@ -822,11 +831,11 @@ __device__ __forceinline__ void cell_residual_nd(const MacroArgs& a, const doubl
         lamS[(long long)s * N + c] = ls[s];
         lam_sum += ls[s];
     }
-    double Dc = (1.0 / cfl + 0.5) * lam_sum;
+    double Dc = __dmul_rn(1.0 / cfl + 0.5, lam_sum);
     if (dt > 0.0) {
         const double Vdt = a.vol[c] / dt;
 #pragma unroll
-        for (int q = 0; q < 5; ++q) Rc[q] -= Vdt * (Uc[q] - Un[c * 5 + q]);
+        for (int q = 0; q < 5; ++q) Rc[q] = fma(-Vdt, Uc[q] - Un[c * 5 + q], Rc[q]);
         Dc += Vdt;
     }
     const double iD = 1.0 / Dc;
@@ -834,7 +843,7 @@ __device__ __forceinline__ void cell_residual_nd(const MacroArgs& a, const doubl
     double dUc[5];
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-        dUc[q] = Rc[q] * iD;
+        dUc[q] = __dmul_rn(Rc[q], iD);
         R[(long long)q * N + c] = Rc[q];
         dU[(long long)q * N + c] = dUc[q];
     }
@@ -917,7 +926,7 @@ __device__ __forceinline__ void relax_nd(const MacroArgs& a, const double* U, co
     }
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-        dUc[q] = (Rc[q] - 0.5 * (fs[q] - ld[q])) * iD;
+        dUc[q] = __dmul_rn(fma(-0.5, fs[q] - ld[q], Rc[q]), iD);
         if (dUout) dUout[(long long)q * N + c] = dUc[q];
     }
     if (dFout) {
