@@ -297,11 +297,11 @@ gsis_status gsis_debug_set_batch_tile(const char* name);
 /* Test hook: run the kinetic sweep of this context with the named tile shape
  * from now on instead of the autotuned one (names as reported by
  * gsis_tuning_info, e.g. "g4_v1_c1", "ring_w8_v32"); starts the context
- * (presolve, region) if needed.  Every shape computes the same result, the
- * columns, "planes" and the 1D line sweep to rounding.
+ * (presolve, region) if needed.  Every shape computes the same result, "planes"
+ * to FP32 subnormals and the 1D line sweep to rounding.
  * GSIS_ERR_ARG for an unknown name or a shape that cannot run this problem
  * (the shared-memory window shapes need a 2D mesh whose hyperplane window
- * fits in shared memory; the FP64 columns "col_*" a 2D mesh; "planes", FP32 /
+ * fits in shared memory; the columns "col_*", FP64 storage and a 2D mesh; "planes", FP32 /
  * BF16 / FP16 storage, an even nx and a 2D or 3D mesh).  The paper has no
  * counterpart. */
 gsis_status gsis_debug_set_sweep_tile(gsis_ctx* ctx, const char* name);

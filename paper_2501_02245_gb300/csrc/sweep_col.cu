@@ -13,9 +13,10 @@
 // whichever side is the inflow one: the lane loads s1, s0, s2 from rows picked
 // by its own outflow test (7 loads per point instead of 9, no selects).  The
 // halves go into x (xi is halved once per thread, exactly), so minmod needs no
-// scaling: num -= x'_o mm + x'_i (2 s1 + mm).  Both faces outflow: x'_o is
-// their difference, x'_i = 0.  Both inflow (a warp vote): the second inflow
-// face value is added.
+// scaling: num -= x'_o mm + x'_i (2 s1 + mm), the low side's term first.  Both faces
+// outflow or both inflow (a warp vote): the second one takes the place of the term
+// that is missing.  Operations, order and roundings are those of k_sweep, so the results are
+// the same to the last bit whichever tile the autotuner picks.
 //
 // What bounds it: the FP64 pipe (a warp instruction holds it for 64 cycles on
 // GB300).  A point costs 17 FP64 operations plus 12 / ZP shared ones; a lane
@@ -64,39 +65,24 @@ __device__ __forceinline__ void make_column(const VGridDev& vg, double* f, int p
     }
 }
 
-// Value of a boundary or interface record on the column's planes (eval_rec
-// with its x-y part formed once).
+// Value of a boundary or interface record on the column's planes.
 template <int ZP>
 __device__ __forceinline__ void column_record(const SweepArgs& a, const Records& R, int r, double scale,
                                               const Column<ZP>& C, double* out) {
     const double* sc = RecT<double>::scal(R, r);
     const double* tab = RecT<double>::tab(R, r, a.vg.NT);
-    const int NT = a.vg.NT, nx = a.vg.nx, jy = nx + C.iy;
-    const double e = scale * (__ldg(tab + C.ix) * __ldg(tab + jy));
-    const double b = __ldg(sc + RS_P0) + (__ldg(tab + NT + C.ix) + __ldg(tab + NT + jy));
-    const double c2 = __ldg(tab + 3 * NT + C.ix) + __ldg(tab + 3 * NT + jy);
-    const double r1 = __ldg(tab + 4 * NT + C.ix) + __ldg(tab + 4 * NT + jy);
-    double o0 = 0.0, o1 = 0.0;
-    if (__ldg(sc + RS_OFFD) != 0.0) {
-        const double cx = __ldg(tab + 2 * NT + C.ix), cy = __ldg(tab + 2 * NT + jy);
-        o0 = 2.0 * __ldg(sc + RS_P2XY) * cx * cy;
-        o1 = 2.0 * (__ldg(sc + RS_P2XZ) * cx + __ldg(sc + RS_P2YZ) * cy);
-    }
-    const double b0 = b + o0;
 #pragma unroll
-    for (int u = 0; u < ZP; ++u) {
-        const int jz = nx + a.vg.ny + min(C.iz0 + u, a.vg.nz - 1);
-        double poly = fma(r1 + __ldg(tab + 4 * NT + jz), c2 + __ldg(tab + 3 * NT + jz), b0 + __ldg(tab + NT + jz));
-        poly = fma(o1, __ldg(tab + 2 * NT + jz), poly);
-        out[u] = e * __ldg(tab + jz) * poly;
-    }
+    for (int u = 0; u < ZP; ++u)
+        out[u] = scale * eval_recT<double>(sc, tab, a.vg.NT, a.vg.nx, a.vg.ny, C.ix, C.iy, min(C.iz0 + u, a.vg.nz - 1));
 }
 
 // One cell's stencil on a column, and the column's coefficients.
 template <int ZP>
 struct Stencil {
     double c0[ZP], s1[2][ZP], s0[2][ZP], s2[2][ZP];
-    double xo[2], xi[2], xe[2], den;   // halved coefficients: outflow, inflow, second inflow face; the denominator
+    // halved coefficients: outflow, inflow face, a second face (both outflow: the high one, > 0; both inflow: the
+    // high one, < 0; else 0); the denominator
+    double xo[2], xi[2], xe[2], den;
     bool oL[2];                   // the low side is the outflow side
 };
 
@@ -114,7 +100,7 @@ __device__ __forceinline__ void column_load(int k, const CellMeta<double, 2>& m,
                                             unsigned row_bytes, Stencil<ZP>& q) {
     auto at = [&](int row, int u) { return *reinterpret_cast<const double*>(row_at(C.fz[u], row, row_bytes)); };
     const bool interior = m.kinds < 0;
-    double out = 0.0;
+    double den = m.it;
 #pragma unroll
     for (int u = 0; u < ZP; ++u) q.c0[u] = at(k, u);
 #pragma unroll
@@ -130,18 +116,16 @@ __device__ __forceinline__ void column_load(int k, const CellMeta<double, 2>& m,
             if (kh != SK_DVM) rH = nH = k;
         }
         const bool oL = pos_t<double>(xL);
-        const double mL = pos_part(xL), mH = pos_part(xH);
-        const bool bo = oL && pos_t<double>(xH);
-        double xo = oL ? mL : mH;
-        out += xo;
-        if (__any_sync(C.mask, bo)) {
-            if (bo) { out += xH; xo = xL - xH; }
+        const double mH = pos_part(xH), iH = pos_t<double>(xH) ? 0.0 : xH;
+        const double xo = oL ? xL : mH, xe = oL ? mH : iH;
+        den = fma(2.0, xo, den);
+        if (__any_sync(C.mask, oL && xe != 0.0)) {   // (the low face first, as the general update)
+            if (oL) den = fma(2.0, xe, den);
         }
-        const double iH = pos_t<double>(xH) ? 0.0 : xH;
         q.oL[d] = oL;
         q.xo[d] = xo;
         q.xi[d] = oL ? iH : xL;
-        q.xe[d] = oL ? 0.0 : iH;
+        q.xe[d] = xe;
         const int r1 = oL ? rH : rL, r0 = oL ? rL : rH, r2 = oL ? nH : nL;
 #pragma unroll
         for (int u = 0; u < ZP; ++u) {
@@ -150,7 +134,7 @@ __device__ __forceinline__ void column_load(int k, const CellMeta<double, 2>& m,
             q.s2[d][u] = at(r2, u);
         }
     }
-    q.den = fma(2.0, out, m.it);
+    q.den = den;
 }
 
 // The update of cell k from its stencil, stored.
@@ -171,41 +155,22 @@ __device__ __forceinline__ void column_apply(const SweepArgs& a, int k, const Ce
     const double rden = recip_t<double>(q.den);
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
-        double dn[ZP], dq[ZP];
+        // the own limited slope towards the outflow face (zero where a side repeats the cell) and the inflow face
+        // value (a boundary or interface side has its distribution instead)
+        double dn[ZP], dq[ZP], own[ZP], fin[ZP];
+        double co = q.xo[d], ci = q.xi[d];
+        const bool oL = q.oL[d];
 #pragma unroll
         for (int u = 0; u < ZP; ++u) {
             dn[u] = q.c0[u] - q.s1[d][u];
             dq[u] = q.s0[d][u] - q.c0[u];
-            // own limited slope towards the outflow face (zero where a side repeats the cell)
-            num[u] = fma(-q.xo[d], mm_t<double>(dn[u], dq[u]), num[u]);
+            own[u] = mm_t<double>(dn[u], dq[u]);
+            fin[u] = fma(2.0, q.s1[d][u], mm_t<double>(q.s1[d][u] - q.s2[d][u], dn[u]));
         }
-        // inflow face value; a boundary or interface side has its distribution instead
-        double ci = q.xi[d];
-        if (!interior && side_kind(m.kinds, q.oL[d] ? 2 * d + 1 : 2 * d) != SK_DVM) ci = 0.0;
-#pragma unroll
-        for (int u = 0; u < ZP; ++u) {
-            const double fin = fma(2.0, q.s1[d][u], mm_t<double>(q.s1[d][u] - q.s2[d][u], dn[u]));
-            num[u] = fma(-ci, fin, num[u]);
-        }
-        bool dvm_h = true;
-        if (!interior) {
-#pragma unroll
-            for (int hs = 0; hs < 2; ++hs) {   // (the side kinds are the same for every lane of the cell)
-                const int s = 2 * d + hs, kd = side_kind(m.kinds, s);
-                if (kd == SK_NONE || kd == SK_DVM) continue;
-                const double x = hs ? (q.oL[d] ? q.xi[d] : q.xe[d]) : (q.oL[d] ? 0.0 : q.xi[d]);   // halved, < 0 for inflow
-                if (!__any_sync(C.mask, x != 0.0)) continue;
-                const double scale = kd == SK_WALL ? __ldg(a.rho_w + (long long)k * 6 + s) : 1.0;
-                double v[ZP];
-                column_record<ZP>(a, kd == SK_GHOST ? a.recGhost : a.recBC, m.rf[s], 2.0 * scale, C, v);
-#pragma unroll
-                for (int u = 0; u < ZP; ++u) num[u] = fma(-x, v[u], num[u]);
-            }
-            dvm_h = side_kind(m.kinds, 2 * d + 1) == SK_DVM;
-        }
-        const bool bi = dvm_h && q.xe[d] != 0.0;   // the high face is an inflow face too
-        if (__any_sync(C.mask, bi)) {
-            const double ce = bi ? q.xe[d] : 0.0;
+        // a second outflow face takes the inflow term's place with the own slope the other way, a second inflow
+        // face the own term's place with its face value
+        if (__any_sync(C.mask, q.xe[d] != 0.0)) {
+            const bool both = q.xe[d] != 0.0, dvm_h = interior || side_kind(m.kinds, 2 * d + 1) == SK_DVM;
             const int r2 = dvm_h ? m.n2[2 * d + 1] : k;
             double e2[ZP];
 #pragma unroll
@@ -213,9 +178,39 @@ __device__ __forceinline__ void column_apply(const SweepArgs& a, int k, const Ce
                 e2[u] = *reinterpret_cast<const double*>(row_at(C.fz[u], r2, row_bytes));
 #pragma unroll
             for (int u = 0; u < ZP; ++u) {
-                const double fin = fma(2.0, q.s0[d][u], mm_t<double>(q.s0[d][u] - e2[u], neg_if<double>(dq[u], true)));
-                num[u] = fma(-ce, fin, num[u]);
+                const double high = fma(2.0, q.s0[d][u], mm_t<double>(q.s0[d][u] - e2[u], neg_if<double>(dq[u], true)));
+                if (both && oL) fin[u] = neg_if<double>(own[u], true);
+                if (both && !oL) own[u] = high;
             }
+            if (both && oL) ci = q.xe[d];
+            if (both && !oL) co = q.xe[d];
+        }
+        if (!interior) {
+#pragma unroll
+            for (int hs = 0; hs < 2; ++hs) {   // (the side kinds are the same for every lane of the cell)
+                const int s = 2 * d + hs, kd = side_kind(m.kinds, s);
+                if (kd == SK_NONE || kd == SK_DVM) continue;
+                // this side's inflow, and the term that carries it
+                const bool in_i = hs ? oL : !oL;
+                const double x = in_i ? q.xi[d] : (hs && !oL ? q.xe[d] : 0.0);
+                const bool in = __double_as_longlong(x) < 0 && x != 0.0;
+                if (!__any_sync(C.mask, in)) continue;
+                const double scale = kd == SK_WALL ? __ldg(a.rho_w + (long long)k * 6 + s) : 1.0;
+                double v[ZP];
+                column_record<ZP>(a, kd == SK_GHOST ? a.recGhost : a.recBC, m.rf[s], 2.0 * scale, C, v);
+#pragma unroll
+                for (int u = 0; u < ZP; ++u) {
+                    if (in && in_i) fin[u] = v[u];
+                    if (in && !in_i) own[u] = v[u];
+                }
+            }
+        }
+        // the low side first, as the general update: the same roundings
+        const double c_low = oL ? co : ci, c_high = oL ? ci : co;
+#pragma unroll
+        for (int u = 0; u < ZP; ++u) {
+            num[u] = fma(-c_low, oL ? own[u] : fin[u], num[u]);
+            num[u] = fma(-c_high, oL ? fin[u] : own[u], num[u]);
         }
     }
 #pragma unroll
