@@ -260,8 +260,8 @@ gsis_status gsis_debug_set_region(gsis_ctx* ctx, const uint8_t* flags);
  * member is a non-periodic line of kinetic cells, else picked by timing the
  * candidates on the batch itself (on a snapshot of the VDFs, restored
  * afterwards; skipped without memory for the snapshot) and cached per batch
- * shape for the life of the process.  Results equal those of iterating each
- * solve alone (FP64 lines: to rounding).
+ * shape for the life of the process.  Results are identical to iterating each
+ * solve alone.
  *
  * ctxs: n distinct contexts on one device, each with mesh and velocity grid
  *       set, adaptive = 0 (or a region forced by gsis_debug_set_region);
@@ -289,16 +289,16 @@ gsis_status gsis_iterate_batch(gsis_ctx** ctxs, int n, int iterations, gsis_repo
  * (names as reported by gsis_batch_info, e.g. "vpt2_cb1_w4", or the
  * velocity-pair shapes "pair1_cb1_w4", "pair2_cb1_w4", "pair1_cb1_w8", which
  * need FP32/BF16/FP16 members with an even nx, or "line_w4", which needs 1D
- * members: gsis_iterate_batch then returns GSIS_ERR_ARG for another batch).  NULL or "" restores autotuning.  Every
- * shape computes the same result (the line shape: to rounding).  GSIS_ERR_ARG
- * for an unknown name.  The paper has no counterpart. */
+ * members: gsis_iterate_batch then returns GSIS_ERR_ARG for another batch).
+ * NULL or "" restores autotuning.  Every shape computes the same result.
+ * GSIS_ERR_ARG for an unknown name.  The paper has no counterpart. */
 gsis_status gsis_debug_set_batch_tile(const char* name);
 
 /* Test hook: run the kinetic sweep of this context with the named tile shape
  * from now on instead of the autotuned one (names as reported by
  * gsis_tuning_info, e.g. "g4_v1_c1", "ring_w8_v32"); starts the context
- * (presolve, region) if needed.  Every shape computes the same result, "planes"
- * to FP32 subnormals and the 1D line sweep to rounding.
+ * (presolve, region) if needed.  Every shape computes the same result
+ * ("planes" and the FP32 line sweep to FP32 subnormals).
  * GSIS_ERR_ARG for an unknown name or a shape that cannot run this problem
  * (the shared-memory window shapes need a 2D mesh whose hyperplane window
  * fits in shared memory; the columns "col_*", FP64 storage and a 2D mesh; "planes", FP32 /

@@ -11,11 +11,12 @@
 // through the L1/L2) and no step waits for its load (a window without that
 // distance measured slower than reloading).  Ends of the line: rows are clamped,
 // and a repeated value gives the zero slope the scheme prescribes there.
-// FP32: planes in pairs for the f32x2 instructions (they share every
-// coefficient), with the operations and roundings of the general sweep (long
-// shocks amplify a different rounding, 1e-4 of the state after a few iterations), so
-// the results are the same; FP64: bound by the FP64 pipe, 11 operations per point plus
-// 6 / ZP shared ones against 23.
+// Operations and roundings are those of the general sweep (long shocks amplify a
+// difference in the last bit to 1e-4 of the state in a few iterations), so the results
+// are the same: FP64 to the last bit; FP32 too, except values below 2^-100, where
+// halving the face speeds meets the subnormals.  FP32: planes in pairs for the f32x2
+// instructions (they share every coefficient); FP64: bound by the FP64 pipe, 11
+// operations per point plus 6 / ZP shared ones against 23.
 // Per iteration: a batch of 64 shocks of 100 to 800 cells, 24^3 to 64^3 velocities,
 // FP32 and BF16: 18.8 ms with the general sweep's best tile, 14.5 with this one; 30
 // FP64 cells of 1,800 velocities alone 85 us -> 74.
@@ -45,6 +46,8 @@ __device__ __forceinline__ float2 gmm(float2 a, float2 b) {
 }
 __device__ __forceinline__ double gsel(bool c, double a, double b) { return c ? a : b; }
 __device__ __forceinline__ float2 gsel(bool c, float2 a, float2 b) { return make_float2(c ? a.x : b.x, c ? a.y : b.y); }
+__device__ __forceinline__ double gneg(double a) { return neg_if<double>(a, true); }
+__device__ __forceinline__ float2 gneg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ void gput(double& g, int, double v) { g = v; }
 __device__ __forceinline__ void gput(float2& g, int i, float v) {
     if (i == 0) g.x = v;
@@ -259,15 +262,17 @@ __device__ __forceinline__ void line_pass(const SweepArgs& a, const LineColumn<S
             const bool ob = pos_t<T>(xb), oa = pos_t<T>(xa);
             const bool from_b = !ob && xb != T(0);              // inflow face behind
             const T xbp = ob ? xb : T(0), xap = oa ? xa : T(0);
-            const T out = xbp + xap;
+            T den = fma(T(2), xbp + xap, fa.it);
             // s1, s2: the neighbours on the inflow side (behind if that face is an inflow face, else ahead),
-            // s0 the other one; x_o weights the own limited slope towards s0: the outflow face there, minus an
-            // outflow face on the s1 side (rare); x_i the inflow face
-            T xo = from_b ? xap : xbp;
+            // s0 the other one; x_o weights the own limited slope towards s0, at the outflow face there; x_i the
+            // inflow face value
+            T xo = from_b ? xap : xbp, xi = from_b ? xb : xa;
+            // Faces that do not oppose each other (rare): the second outflow face takes the inflow term's place with
+            // the own slope the other way, the second inflow face the own term's place with its face value
             const bool both_in = from_b && !oa && xa != T(0), both_out = !from_b && oa;
-            const bool rare = __any_sync(0xffffffffu, both_in || both_out);   // faces that do not oppose each other
-            if (rare && both_out) xo = xbp - xa;
-            const T xi = from_b ? xb : (oa ? T(0) : xa);
+            const bool rare = __any_sync(0xffffffffu, both_in || both_out);
+            if (rare && both_out) den = fma(T(2), back ? xb : xa, fma(T(2), back ? xa : xb, fa.it));   // (the low face first)
+            if (rare && both_in) xo = xa;
             const bool end_b = back ? end_h : end_l, end_a = back ? end_l : end_h;
             const bool in_l = from_b != back;   // the inflow side is the low one
             const bool given = from_b ? end_b : end_a;   // ... and a boundary: its distribution instead
@@ -275,33 +280,26 @@ __device__ __forceinline__ void line_pass(const SweepArgs& a, const LineColumn<S
             for (int g = 0; g < NG; ++g) {
                 const P s1 = gsel(from_b, b1[g], a1[g]), s2 = gsel(from_b, b2[g], a2[g]), s0 = gsel(from_b, a1[g], b1[g]);
                 const P dn = gsub(c0[g], s1);
-                const P own = gmm(dn, gsub(s0, c0[g]));
+                P own = gmm(dn, gsub(s0, c0[g]));
                 P fin = gfma(T(2), s1, gmm(gsub(s1, s2), dn));
                 if (end_l || end_h) {
 #pragma unroll
                     for (int i = 0; i < W; ++i)
                         if (given) gput(fin, i, ends.v[in_l ? 0 : 1][g * W + i][lane]);
                 }
-                if constexpr (F64) {
-                    num[g] = gfma(-xo, own, num[g]);
-                    num[g] = gfma(-xi, fin, num[g]);
-                } else {   // the low side first, as the general sweep: the same roundings
-                    num[g] = gfma(in_l ? -xi : -xo, gsel(in_l, fin, own), num[g]);
-                    num[g] = gfma(in_l ? -xo : -xi, gsel(in_l, own, fin), num[g]);
-                }
-            }
-            if (rare && __any_sync(0xffffffffu, both_in)) {
-                const T ce = both_in ? xa : T(0);
-#pragma unroll
-                for (int g = 0; g < NG; ++g) {
-                    P fin = gfma(T(2), a1[g], gmm(gsub(a1[g], a2[g]), gsub(c0[g], a1[g])));
+                if (rare) {
+                    P fa2 = gfma(T(2), a1[g], gmm(gsub(a1[g], a2[g]), gsub(c0[g], a1[g])));   // the face value ahead
 #pragma unroll
                     for (int i = 0; i < W; ++i)
-                        if (end_a) gput(fin, i, ends.v[back ? 0 : 1][g * W + i][lane]);
-                    num[g] = gfma(-ce, fin, num[g]);
+                        if (end_a) gput(fa2, i, ends.v[back ? 0 : 1][g * W + i][lane]);
+                    fin = gsel(both_out, gneg(own), fin);
+                    own = gsel(both_in, fa2, own);
                 }
+                // the low side first, as the general sweep: the same roundings
+                num[g] = gfma(in_l ? -xi : -xo, gsel(in_l, fin, own), num[g]);
+                num[g] = gfma(in_l ? -xo : -xi, gsel(in_l, own, fin), num[g]);
             }
-            const T rden = recip_t<T>(fma(T(2), out, fa.it));
+            const T rden = recip_t<T>(den);
             P fo[NG];
 #pragma unroll
             for (int u = 0; u < ZP; ++u) {
