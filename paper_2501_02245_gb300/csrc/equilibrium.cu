@@ -268,6 +268,205 @@ __global__ void k_build_records(const RecSpec* __restrict__ specs, int nrec, int
     }
 }
 
+// ---------------------------------------------------------------------------- records of lines
+// The records of a flat line of cells (face_nd = 1): the correction system in the
+// conserved quantities, entry by entry from the terms of its polynomials, and a pivoted
+// elimination.  The line's synthetic solve amplifies a difference in the last bit
+// (mu_of in macro.cu), so its records keep these operations and their order, where other
+// meshes take the shorter form above.  A warp builds one record: lanes 8 d + i add the
+// axis sums of axis d over the nodes i, i + 8, ... (eight partial sums per axis,
+// whatever the number of lanes), lane e then forms entry e of the 30 of the system.  50 to 87
+// us a launch with eight lanes and four entries on each; 25 for the short form.
+struct Term { double c; int a, b, d; };
+
+__device__ static int psi_terms(int row, const double* u, Term* t, double scale) {
+    // psi_row in powers of c (c = xi - u); scale = 1 for psi, 2 for phi_4 only
+    switch (row) {
+        case 0: t[0] = {1.0, 0, 0, 0}; return 1;
+        case 1: t[0] = {1.0, 1, 0, 0}; t[1] = {u[0], 0, 0, 0}; return 2;
+        case 2: t[0] = {1.0, 0, 1, 0}; t[1] = {u[1], 0, 0, 0}; return 2;
+        case 3: t[0] = {1.0, 0, 0, 1}; t[1] = {u[2], 0, 0, 0}; return 2;
+        default: {
+            double h = 0.5 * scale;
+            t[0] = {h, 2, 0, 0}; t[1] = {h, 0, 2, 0}; t[2] = {h, 0, 0, 2};
+            t[3] = {scale * u[0], 1, 0, 0}; t[4] = {scale * u[1], 0, 1, 0}; t[5] = {scale * u[2], 0, 0, 1};
+            t[6] = {h * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]), 0, 0, 0};
+            return 7;
+        }
+    }
+}
+
+// Terms of the base polynomial with a nonzero coefficient.
+__device__ static int base_terms(const RecSpec& s, Term* t) {
+    const Term all[19] = {
+        {s.p0, 0, 0, 0},
+        {s.p[0], 1, 0, 0}, {s.p[1], 0, 1, 0}, {s.p[2], 0, 0, 1},
+        {s.P2[0], 2, 0, 0}, {s.P2[1], 0, 2, 0}, {s.P2[2], 0, 0, 2},
+        {2.0 * s.P2[3], 1, 1, 0}, {2.0 * s.P2[4], 1, 0, 1}, {2.0 * s.P2[5], 0, 1, 1},
+        {s.r[0], 3, 0, 0}, {s.r[0], 1, 2, 0}, {s.r[0], 1, 0, 2},
+        {s.r[1], 2, 1, 0}, {s.r[1], 0, 3, 0}, {s.r[1], 0, 1, 2},
+        {s.r[2], 2, 0, 1}, {s.r[2], 0, 2, 1}, {s.r[2], 0, 0, 3}};
+    int n = 0;
+    for (int i = 0; i < 19; ++i)
+        if (all[i].c != 0.0) t[n++] = all[i];
+    return n;
+}
+
+__device__ static double poly_moment(const Term* t1, int n1, const Term* t2, int n2, const double (*Cs)[6]) {
+    double s = 0.0;
+    for (int i = 0; i < n1; ++i)
+        for (int j = 0; j < n2; ++j)
+            s += t1[i].c * t2[j].c * (Cs[0][t1[i].a + t2[j].a] * Cs[1][t1[i].b + t2[j].b] * Cs[2][t1[i].d + t2[j].d]);
+    return s;
+}
+
+// Solve A x = b (5x5) by Gaussian elimination with partial pivoting.
+__device__ static void solve5(double A[5][5], double b[5], double x[5]) {
+    for (int col = 0; col < 5; ++col) {
+        int piv = col;
+        double best = fabs(A[col][col]);
+        for (int r = col + 1; r < 5; ++r)
+            if (fabs(A[r][col]) > best) { best = fabs(A[r][col]); piv = r; }
+        if (piv != col) {
+            for (int k = 0; k < 5; ++k) { double t = A[col][k]; A[col][k] = A[piv][k]; A[piv][k] = t; }
+            double t = b[col]; b[col] = b[piv]; b[piv] = t;
+        }
+        for (int r = col + 1; r < 5; ++r) {
+            double m = A[r][col] / A[col][col];
+            for (int k = col; k < 5; ++k) A[r][k] -= m * A[col][k];
+            b[r] -= m * b[col];
+        }
+    }
+    for (int r = 4; r >= 0; --r) {
+        double s = b[r];
+        for (int k = r + 1; k < 5; ++k) s -= A[r][k] * x[k];
+        x[r] = s / A[r][r];
+    }
+}
+
+// Conserved moments (rho, rho u, rho E) of a state.
+__device__ static void cons_of(double rho, const double* u, double T, double* U) {
+    U[0] = rho;
+    U[1] = rho * u[0]; U[2] = rho * u[1]; U[3] = rho * u[2];
+    U[4] = rho * (1.5 * T + 0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
+}
+
+__global__ void k_build_records_line(const RecSpec* __restrict__ specs, int nrec, int n0, Records out0, Records out1,
+                                     VGridDev vg) {
+    const int lane = threadIdx.x & 31;
+    const int rr = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (rr >= nrec) return;   // (whole warps)
+    const RecSpec s = specs[rr];
+    const Records& out = rr < n0 ? out0 : out1;
+    const long long r = rr < n0 ? rr : rr - n0;
+    const int NT = vg.NT, nx = vg.nx, ny = vg.ny;
+    double* tab = out.tab + r * NTAB * NT;
+    double* scal = out.scal + r * RS;
+    const double T = s.T;
+    const double A = s.rho * pow(2.0 * PI * T, -1.5);
+    const double sq2piT = sqrt(2.0 * PI * T);   // (the reduced grid's planes: see k_build_records)
+    const double i2T = 0.5 / T;
+    double part[6] = {0, 0, 0, 0, 0, 0};
+    const int d = lane >> 3;
+    if (d < 3) {
+        const int lo = d == 0 ? 0 : (d == 1 ? nx : nx + ny), hi = d == 0 ? nx : (d == 1 ? nx + ny : NT);
+        for (int idx = lo + (lane & 7); idx < hi; idx += 8) {
+            if (vg.reduced && d == 2) {
+                const int p = idx - nx - ny;
+                tab[idx] = p ? sq2piT * T : sq2piT;
+                tab[2 * NT + idx] = 0.0;
+                tab[3 * NT + idx] = p ? 3.0 * T : T;
+                continue;
+            }
+            const double c = vg.xi[idx] - s.u[d];
+            const double e = exp(-(c * c) * i2T);
+            tab[idx] = e;
+            tab[2 * NT + idx] = c;
+            tab[3 * NT + idx] = c * c;
+            double pw = e;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                part[k] += pw;
+                pw *= c;
+            }
+        }
+    }
+    double Cs[3][6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        double v = part[k];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, 8);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) Cs[q][k] = __shfl_sync(0xffffffffu, v, 8 * q);
+    }
+    if (vg.reduced) {   // exact xi_z integrals int c_z^k e_z dxi_z of the Gaussian (k = 0..5)
+        const double zk[6] = {1.0, 0.0, T, 0.0, 3.0 * T * T, 0.0};
+        for (int k = 0; k < 6; ++k) Cs[2][k] = sq2piT * zk[k];
+    }
+    double alpha[5] = {0, 0, 0, 0, 0};
+    if (s.correct) {
+        Term tp[7], tq[19];
+        const double wa = vg.w * A;
+        double U[5];
+        cons_of(s.rho, s.u, T, U);
+        double mine = 0.0;   // entries 0-4: right-hand side, 5-29: the matrix by rows
+        if (lane < 5) {
+            const int na = psi_terms(lane, s.u, tp, 1.0);
+            const int nb = base_terms(s, tq);
+            mine = U[lane] - wa * poly_moment(tp, na, tq, nb, Cs);
+        } else if (lane < 30) {
+            const int ra = (lane - 5) / 5, rb = (lane - 5) % 5;
+            const int na = psi_terms(ra, s.u, tp, 1.0);
+            const int nbb = psi_terms(rb, s.u, tq, rb == 4 ? 2.0 : 1.0);
+            mine = wa * poly_moment(tp, na, tq, nbb, Cs);
+        }
+        __syncwarp();
+        double Am[5][5], rhs[5];
+#pragma unroll
+        for (int e = 0; e < 30; ++e) {
+            const double v = __shfl_sync(0xffffffffu, mine, e);
+            if (e < 5) rhs[e] = v;
+            else Am[(e - 5) / 5][(e - 5) % 5] = v;
+        }
+        solve5(Am, rhs, alpha);
+    }
+    double pp[3] = {s.p[0], s.p[1], s.p[2]};
+    double p2d[3] = {s.P2[0], s.P2[1], s.P2[2]};
+    double p0 = s.p0;
+    if (s.correct) {
+        const double ua = alpha[1] * s.u[0] + alpha[2] * s.u[1] + alpha[3] * s.u[2];
+        const double u2 = s.u[0] * s.u[0] + s.u[1] * s.u[1] + s.u[2] * s.u[2];
+        p0 = s.p0 + alpha[0] + ua + alpha[4] * u2;
+        for (int q = 0; q < 3; ++q) {
+            pp[q] = s.p[q] + alpha[1 + q] + 2.0 * alpha[4] * s.u[q];
+            p2d[q] = s.P2[q] + alpha[4];
+        }
+    }
+    if (lane == 0) {
+        scal[RS_P0] = p0;
+        scal[RS_P2XY] = s.P2[3];
+        scal[RS_P2XZ] = s.P2[4];
+        scal[RS_P2YZ] = s.P2[5];
+        scal[RS_OFFD] = (s.P2[3] != 0.0 || s.P2[4] != 0.0 || s.P2[5] != 0.0) ? 1.0 : 0.0;
+    }
+    __syncwarp();   // the record's values written by other lanes are read below
+    for (int idx = lane; idx < NT; idx += 32) {
+        const int q = idx < nx ? 0 : (idx < nx + ny ? 1 : 2);
+        const double pq = q == 0 ? pp[0] : (q == 1 ? pp[1] : pp[2]), p2q = q == 0 ? p2d[0] : (q == 1 ? p2d[1] : p2d[2]);
+        const double c = tab[2 * NT + idx];
+        tab[NT + idx] = pq * c + p2q * tab[3 * NT + idx];   // C2 = c^2 (plane value if reduced)
+        tab[4 * NT + idx] = s.r[q] * c;
+        if (q == 0) tab[idx] *= A;
+        if (out.tabf) {   // FP32 copies in stored units: E_x carries the VDF storage scale once
+            float* tf = out.tabf + r * NTAB * NT;
+            for (int t = 0; t < NTAB; ++t)
+                tf[t * NT + idx] = (float)(t == 0 && q == 0 ? tab[idx] * vg.vscale : tab[t * NT + idx]);
+        }
+    }
+    if (out.scalf && lane <= RS_OFFD) out.scalf[r * RS + lane] = (float)scal[lane];
+}
+
 // Records [0, n0) into out0 and the rest into out1.  A record per warp while the
 // warps leave sub-partitions idle (2,048 records: about three warps each), four
 // above.
@@ -289,10 +488,16 @@ void build_records_raw(const RecSpec* d_specs, int nrec, const Records& out, con
     build_records(d_specs, nrec, nrec, out, out, vg, st);
 }
 
-void launch_build_records(gsis_ctx* c, const Records& out, int nrec, const RecSpec* d_specs) {
+// Records of a context's own solve (records [0, n0) into out0, the rest into out1).
+static void solve_records(gsis_ctx* c, int nrec, int n0, const Records& out0, const Records& out1, const RecSpec* d_specs) {
     if (nrec <= 0) return;
-    build_records(d_specs, nrec, nrec, out, out, c->vg, c->stream);
+    if (c->face_nd == 1) k_build_records_line<<<(nrec + 1) / 2, 64, 0, c->stream>>>(d_specs, nrec, n0, out0, out1, c->vg);
+    else build_records(d_specs, nrec, n0, out0, out1, c->vg, c->stream);
     c->launches++;
+}
+
+void launch_build_records(gsis_ctx* c, const Records& out, int nrec, const RecSpec* d_specs) {
+    solve_records(c, nrec, nrec, out, out, d_specs);
 }
 
 // ---------------------------------------------------------------------------- spec builders
@@ -538,8 +743,8 @@ void launch_correction_records(gsis_ctx* c) {
     const int Nd = (int)c->Nd;
     if (Nd == 0) return;
     k_corr_specs<<<(2 * Nd + 127) / 128, 128, 0, c->stream>>>(Nd, c->dvm_cell, c->W, c->Wh, c->specs);
-    build_records(c->specs, 2 * Nd, Nd, c->recNew, c->recHalf, c->vg, c->stream);
-    c->launches += 2;
+    c->launches++;
+    solve_records(c, 2 * Nd, Nd, c->recNew, c->recHalf, c->specs);
 }
 
 // Seed distributions for cells entering the DVM region: Grad-13 from W and
@@ -700,7 +905,8 @@ void launch_two_vdf_reference(gsis_ctx* c, const double* S, int n, const TwoVdfG
     if (n <= 0) return;
     k_two_vdf_specs<<<(n + 127) / 128, 128, 0, c->stream>>>(n, S, g, specs);
     c->launches++;
-    launch_build_records(c, rec, 4 * n, specs);
+    build_records_raw(specs, 4 * n, rec, c->vg, c->stream);
+    c->launches++;
     const int rows = c->vg.ny * c->vg.nz;
     // row blocks: enough for eight blocks per SM, at most 256 rows (32 KB of coefficients), whole thread groups
     const int G = std::max(1, TV_THREADS / c->vg.nx);

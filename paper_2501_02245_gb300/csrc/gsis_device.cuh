@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+#include <type_traits>
 #include "gsis_internal.h"
 
 namespace gsis {
@@ -120,6 +121,23 @@ template <> __device__ __forceinline__ double mm_t<double>(double a, double b) {
     return (ia ^ ib) >= 0 ? __longlong_as_double(a_smaller ? ia : ib) : 0.0;
 }
 template <> __device__ __forceinline__ float hmm_t<float>(float a, float b) { return 0.5f * mm_t<float>(a, b); }
+// The limiter of lines (1D meshes) in FP32 arithmetic: zero also where the product of
+// the two slopes underflows (|a b| <= 2^-150, the far tails).  A line's solve amplifies a
+// difference in the last bit (mu_of in macro.cu), so its sweeps keep that form; the tiles
+// of 2D and 3D meshes do without the product.  FP64: mm_t.
+template <typename T> __device__ __forceinline__ T mm_line(T a, T b) { return mm_t<T>(a, b); }
+template <> __device__ __forceinline__ float mm_line<float>(float a, float b) {
+    const float m = fabsf(a) < fabsf(b) ? a : b;
+    return a * b > 0.0f ? m : 0.0f;
+}
+// hmm_t, or half of mm_line where LINE or line say so.
+template <typename T, bool LINE>
+__device__ __forceinline__ T hmm_of(T a, T b, bool line) {
+    if constexpr (std::is_same<T, float>::value) {
+        if (LINE || line) return 0.5f * mm_line<float>(a, b);
+    }
+    return hmm_t<T>(a, b);
+}
 template <> __device__ __forceinline__ double hmm_t<double>(double a, double b) {
     const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
     const unsigned long long ma = mag_bits(a), mb = mag_bits(b);

@@ -54,10 +54,22 @@ static MacroArgs margs(gsis_ctx* c) {
     return a;
 }
 
-// mu0 T^omega
-__device__ __forceinline__ double viscosity_tab(double T, double mu0, double omega) {
-    return mu0 * exp_tab(omega * log_tab(T));
+// A flat line of cells (fnd = 1) is solved with the library's functions and divisions,
+// meshes of two and three directions with the tables of special.cuh and recip64.  At
+// the shocks' settings (cfl = 100, four relaxation sweeps) the pseudo-time iteration of a
+// line above Mach 2 or so amplifies a difference in the last bit (1e-15 of the initial
+// state becomes 6e-7 in two GSIS iterations at Mach 5, 1e-4 in ten), so any other rounding
+// of these operations gives another trajectory; twelve sweeps, or cfl = 10, damp it.
+// The bodies' settings do not amplify.  (LINE below: fnd = 1.)
+template <bool LINE>
+__device__ __forceinline__ double mu_of(double T, double mu0, double omega) {
+    return LINE ? viscosity(T, mu0, omega) : mu0 * exp_tab(omega * log_tab(T));
 }
+__device__ __forceinline__ double mu_of(const MacroArgs& a, double T) {
+    return a.fnd == 1 ? mu_of<true>(T, a.mu0, a.omega) : mu_of<false>(T, a.mu0, a.omega);
+}
+template <bool LINE>
+__device__ __forceinline__ double quotient(double a, double b) { return LINE ? a / b : __dmul_rn(a, recip64(b)); }
 
 // ---------------------------------------------------------------------------- gradients
 // Least-squares gradient (face neighbours plus boundary face centres with the
@@ -189,7 +201,7 @@ __global__ void k_nsf(int N, const double* __restrict__ Wp, const double* __rest
                       const double* __restrict__ gT, double mu0, double omega, double* __restrict__ out) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
-    const double mu = viscosity_tab(Wp[c * 5 + 4], mu0, omega);
+    const double mu = viscosity(Wp[c * 5 + 4], mu0, omega);
     double u[9], t[3];
     cell_grad(gu, gT, N, c, u, t);
     nsf_of(mu, u, t, out + (long long)c * HOTN, out + (long long)c * HOTN + 6);
@@ -217,7 +229,7 @@ __global__ void k_prim_to_cons(int N, const double* __restrict__ Wp, double* __r
 // (One reciprocal per state, reused: on GB300 an FP64 division costs about ten
 // FP64-pipe operations.)
 __device__ __forceinline__ void cons_to_prim(const double* U, double* Wp) {
-    const double r = U[0], ir = recip64(r);
+    const double r = U[0], ir = 1.0 / r;
     const double ux = __dmul_rn(U[1], ir), uy = __dmul_rn(U[2], ir), uz = __dmul_rn(U[3], ir);
     Wp[0] = r;
     Wp[1] = ux;
@@ -325,7 +337,7 @@ __device__ __forceinline__ double dot_rn(const double* a, const double* b) {
 // with c = r (mass, momentum) and r/2 (energy).
 // (ND: the normal has components 0..ND-1 only; the others are exact zeros,
 // so the terms they multiply are left out.)
-template <int ND>
+template <int ND, bool LINE>
 __device__ __forceinline__ void half_range(const double* u, double T, const double* n, double sign, double* X) {
     const double un = dot_rn<ND>(u, n);
     // s = un / sqrt(T) and sqrt(T) = T / sqrt(T) from one reciprocal square root
@@ -333,9 +345,16 @@ __device__ __forceinline__ void half_range(const double* u, double T, const doub
     // Maxwellian that crosses, (1 + sign erf(s/sqrt 2))/2, from its tail
     // q = h(|s|) exp(-s^2/2): q where the gas recedes, 1 - q where it approaches.
     const double ist = rsqrt(T), st = T * ist, s = un * ist;
-    const double e = exp_tab(-0.5 * s * s), q = __dmul_rn(mills(__longlong_as_double((long long)mag_bits(s))), e);
-    const bool towards = (__double2hiint(s) >= 0) == (sign > 0.0);
-    const double P = towards ? 1.0 - q : q;
+    double e, P;
+    if constexpr (LINE) {
+        e = exp(-0.5 * s * s);
+        P = 0.5 * (1.0 + sign * erf(s * 0.7071067811865476));   // 1/sqrt(2)
+    } else {
+        e = exp_tab(-0.5 * s * s);
+        const double q = __dmul_rn(mills(__longlong_as_double((long long)mag_bits(s))), e);
+        const bool towards = (__double2hiint(s) >= 0) == (sign > 0.0);
+        P = towards ? 1.0 - q : q;
+    }
     const double D = __dmul_rn(sign * st * e, 0.3989422804014327);   // 1/sqrt(2 pi)
     const double M0 = fma(un, P, D);
     const double u2 = __dmul_rn(un, un);
@@ -355,23 +374,23 @@ __device__ __forceinline__ void half_range(const double* u, double T, const doub
 // along -n -- the Euler flux that the discrete-velocity upwind scheme carries
 // for Maxwellian states.  The left half is rounded, the right one added with one
 // fused multiply-add: written out, so that kfvs_pair rounds the same way.
-template <int ND = 3>
-__device__ void kfvs(double rL, const double* uL, double pL, double rR, const double* uR, double pR,
+template <int ND, bool LINE>
+__device__ __forceinline__ void kfvs(double rL, const double* uL, double pL, double rR, const double* uR, double pR,
                      const double* n, double* F) {
     double X[5];
-    half_range<ND>(uL, __dmul_rn(pL, recip64(rL)), n, 1.0, X);
+    half_range<ND, LINE>(uL, quotient<LINE>(pL, rL), n, 1.0, X);
     for (int q = 0; q < 5; ++q) F[q] = fma(q < 4 ? rL : 0.5 * rL, X[q], 0.0);
-    half_range<ND>(uR, __dmul_rn(pR, recip64(rR)), n, -1.0, X);
+    half_range<ND, LINE>(uR, quotient<LINE>(pR, rR), n, -1.0, X);
     for (int q = 0; q < 5; ++q) F[q] = fma(q < 4 ? rR : 0.5 * rR, X[q], F[q]);
 }
 
 // The same sum formed by a pair of lanes (2i, 2i + 1), each with its own side's
 // state (odd lanes: the right one): the two half-range chains run side by side.
 // The even lane gets the flux, the same bits as kfvs.
-template <int ND>
+template <int ND, bool LINE>
 __device__ __forceinline__ void kfvs_pair(double r, const double* u, double p, bool right, const double* n, double* F) {
     double X[5];
-    half_range<ND>(u, __dmul_rn(p, recip64(r)), n, right ? -1.0 : 1.0, X);
+    half_range<ND, LINE>(u, quotient<LINE>(p, r), n, right ? -1.0 : 1.0, X);
     const unsigned pair = 3u << (threadIdx.x & 30);
     const double ro = __shfl_xor_sync(pair, r, 1);
 #pragma unroll
@@ -386,7 +405,7 @@ __device__ __forceinline__ void kfvs_pair(double r, const double* u, double p, b
 // sub: the tensor less this one.
 template <int ND>
 __device__ __forceinline__ void euler_tensor(const double* U, double* F, const double* sub = nullptr) {
-    const double r = U[0], ir = recip64(r);
+    const double r = U[0], ir = quotient<ND == 1>(1.0, r);
     const double u[3] = {__dmul_rn(U[1], ir), __dmul_rn(U[2], ir), __dmul_rn(U[3], ir)};
     const double e = fma(-(0.5 * r), dot_rn<3>(u, u), U[4]);
     const double h = fma(GAMMA - 1.0, e, U[4]);
@@ -459,6 +478,7 @@ template <int ND, bool PAIR>
 __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* Wm, const double* gu,
                                              const double* gT, const double* hot, const double* acell,
                                              double* Ff, double* lamf, int t) {
+    constexpr bool LINE = ND == 1;
     const int N = a.N, d = t / N, L = t - d * N;
     const int4 st = a.fst[(long long)L * 3 + d];
     const int Rr = st.y;
@@ -490,19 +510,19 @@ __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* W
         double fs[5];   // the face state of this lane's side
         df[4] = right ? dfR : dfL;
         face_state(right ? qR : qL, right ? wR : wL, right ? ph : pl, right, (right ? st.z : st.x) < 0, df, fs);
-        kfvs_pair<ND>(fs[0], fs + 1, fs[4], right, nn, Fv);
+        kfvs_pair<ND, LINE>(fs[0], fs + 1, fs[4], right, nn, Fv);
     } else {
         double fl[5], fr[5];
         df[4] = dfL;
         face_state(qL, wL, pl, false, st.x < 0, df, fl);
         df[4] = dfR;
         face_state(qR, wR, ph, true, st.z < 0, df, fr);
-        kfvs<ND>(fl[0], fl + 1, fl[4], fr[0], fr + 1, fr[4], nn, Fv);
+        kfvs<ND, LINE>(fl[0], fl + 1, fl[4], fr[0], fr + 1, fr[4], nn, Fv);
     }
     // viscous + HoT
     const double uf[3] = {0.5 * (wL[1] + wR[1]), 0.5 * (wL[2] + wR[2]), 0.5 * (wL[3] + wR[3])};
     const double Tf = 0.5 * (wL[4] + wR[4]);
-    const double muf = viscosity_tab(Tf, a.mu0, a.omega);
+    const double muf = mu_of<LINE>(Tf, a.mu0, a.omega);
     const double e[3] = {G[4], G[5], G[6]};
     const double dist = G[7], idist = G[8];
     // face gradients: cell average corrected along the line of centres, for every
@@ -569,7 +589,7 @@ __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* W
         F[(long long)4 * N] = fma(Fv[4], Sabs, ND == 1 ? fma(Q[0], S[0], w) : w + dot_rn<ND>(Q, S));
     }
     const double aL = acell[L], aR = acell[Rr];
-    const double lam = fabs(dot_rn<ND>(uf, nn)) + 0.5 * (aL + aR) + __dmul_rn(5.0 * muf, recip64(0.5 * (wL[0] + wR[0]) * dist));
+    const double lam = fabs(dot_rn<ND>(uf, nn)) + 0.5 * (aL + aR) + quotient<LINE>(5.0 * muf, 0.5 * (wL[0] + wR[0]) * dist);
     if (!right) lamf[(long long)d * N + L] = lam * Sabs;
 }
 
@@ -607,7 +627,7 @@ __device__ void wall_nsf_flux(const MacroArgs& a, const double* w, const double*
         for (int i = 0; i < 3; ++i) gTw[i] = gT[i] + corr * eb[i];
     }
     double sig[6], qw[3];
-    nsf_of(viscosity_tab(Tw, a.mu0, a.omega), guw, gTw, sig, qw);
+    nsf_of(mu_of(a, Tw), guw, gTw, sig, qw);
     const double p = w[0] * w[4];
     const double SigS[3] = {sig[0] * So[0] + sig[3] * So[1] + sig[4] * So[2],
                             sig[3] * So[0] + sig[1] * So[1] + sig[5] * So[2],
@@ -690,7 +710,7 @@ __global__ void k_constitutive(int N, const double* __restrict__ W, const double
     double sig[6], q[3];
     double u[9], t[3];
     cell_grad(gu, gT, N, c, u, t);
-    nsf_of(viscosity_tab(W[c * 5 + 4], mu0, omega), u, t, sig, q);
+    nsf_of(viscosity(W[c * 5 + 4], mu0, omega), u, t, sig, q);
     double* o = out + (long long)c * FIELDS_N;
     const double* h = hot + (long long)c * HOTN;
     for (int k = 0; k < 6; ++k) o[k] = sig[k] + h[k];
@@ -740,9 +760,11 @@ __device__ __forceinline__ void boundary_flux_one(const MacroArgs& a, const doub
         if constexpr (PAIR) {
             const bool right = threadIdx.x & 1;
             const double u[3] = {right ? st[1] : u_c[0], right ? st[2] : u_c[1], right ? st[3] : u_c[2]};
-            kfvs_pair<3>(right ? st[0] : rho_c, u, right ? st[0] * st[4] : p_c, right, nn, Fb);
+            if (a.fnd == 1) kfvs_pair<3, true>(right ? st[0] : rho_c, u, right ? st[0] * st[4] : p_c, right, nn, Fb);
+            else kfvs_pair<3, false>(right ? st[0] : rho_c, u, right ? st[0] * st[4] : p_c, right, nn, Fb);
         } else {
-            kfvs(rho_c, u_c, p_c, st[0], st + 1, st[0] * st[4], nn, Fb);
+            if (a.fnd == 1) kfvs<3, true>(rho_c, u_c, p_c, st[0], st + 1, st[0] * st[4], nn, Fb);
+            else kfvs<3, false>(rho_c, u_c, p_c, st[0], st + 1, st[0] * st[4], nn, Fb);
         }
         const double row[3][3] = {{h[0], h[3], h[4]}, {h[3], h[1], h[5]}, {h[4], h[5], h[2]}};
         const double SigS[3] = {dot_rn<3>(row[0], So), dot_rn<3>(row[1], So), dot_rn<3>(row[2], So)};
@@ -757,7 +779,7 @@ __device__ __forceinline__ void boundary_flux_one(const MacroArgs& a, const doub
     }
     if (PAIR && (threadIdx.x & 1)) return;   // (the even lane has the flux)
     const double a_c = sqrt(GAMMA * p_c / rho_c);
-    const double mu_c = viscosity_tab(T_c, a.mu0, a.omega);
+    const double mu_c = mu_of(a, T_c);
     const double lam = fabs(dot_rn<3>(u_c, nn)) + a_c +
                        5.0 * mu_c / (rho_c * 2.0 * bdist);
     double* o = Fbnd + (long long)cs * 6;

@@ -683,7 +683,7 @@ template <typename S, typename T>
 __global__ void __launch_bounds__(256, std::is_same<T, double>::value ? 1 : 3) k_correct(int Nd, const int* __restrict__ dvm_cell,
                                                  const int* __restrict__ side_bc, const double* __restrict__ Sout,
                                                  S* __restrict__ f, Records recNew, Records recHalf, VGridDev vg,
-                                                 const double* __restrict__ momh, double* __restrict__ mom) {
+                                                 const double* __restrict__ momh, double* __restrict__ mom, bool line) {
     const int k = blockIdx.x;
     if (k >= Nd) return;
     extern __shared__ double sh_raw[];
@@ -696,7 +696,7 @@ __global__ void __launch_bounds__(256, std::is_same<T, double>::value ? 1 : 3) k
     int wall_mask = 0;
     for (int s = 0; s < 6; ++s)
         if (side_bc[c * 6 + s] == GSIS_BC_WALL) wall_mask |= 1 << s;
-    const bool products = F64 && wall_mask == 0;
+    const bool products = F64 && wall_mask == 0 && !line;
     const T* TN = RecT<T>::tab(recNew, k, NT);
     const T* TH = RecT<T>::tab(recHalf, k, NT);
     const T p0N = RecT<T>::scal(recNew, k)[RS_P0], p0H = RecT<T>::scal(recHalf, k)[RS_P0];
@@ -751,7 +751,7 @@ __global__ void __launch_bounds__(256, std::is_same<T, double>::value ? 1 : 3) k
     // rows start on 16-byte boundaries)
     bool chunks = false;
     if constexpr (std::is_same<T, float>::value) {
-        chunks = nx % V == 0 && nx / V <= (int)blockDim.x;
+        chunks = nx % V == 0 && nx / V <= (int)blockDim.x && !(line && wall_mask);
         if (chunks) {
             const double* Sc = Sout + (long long)c * 18;
             if (wall_mask) correct_chunks<S, true>(fk, k, vg, xa, rv, wall_mask, Sc, acc);
@@ -759,7 +759,7 @@ __global__ void __launch_bounds__(256, std::is_same<T, double>::value ? 1 : 3) k
         }
     }
     if (chunks) {
-    } else if (std::is_same<T, double>::value && nx % V == 0) {   // two chunks in flight per thread
+    } else if ((std::is_same<T, double>::value || line) && nx % V == 0) {   // two chunks in flight per thread
         const int nch = Nv / V;
         for (int ch0 = threadIdx.x; ch0 < nch; ch0 += CORR_VEC_UNROLL * step) {
             T fv[CORR_VEC_UNROLL][V];
@@ -848,6 +848,59 @@ __global__ void k_corr_moments(int Nd, const int* __restrict__ dvm_cell, const d
     for (int i = 0; i < 13; ++i) m[i] = sh[i] + w * (mN[i] - mH[i]);
 }
 
+// The same on a flat line (face_nd = 1), whose solve keeps the order of its sums (see
+// mu_of in macro.cu): one block of six warps per cell, warp 3 r + d adds the sums of axis
+// d of record r about u^{n+1}, from the record's tables.
+// s[a] = sum_j c^a E_j and s[4 + a] = sum_j c^a E_j B_j, a = 0..3, valid in lane 0 (on the
+// reduced grid's z axis, zplanes, c^a is the plane weight of xi_z^a).
+__device__ static void table_sums(const double* __restrict__ tab, int NT, const double* __restrict__ xi, int off, int n,
+                                  double u, int lane, double* s, const VGridDev* zplanes) {
+    double p[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (int j = lane; j < n; j += 32) {
+        const double c = xi[off + j] - u, E = tab[off + j], EB = E * tab[NT + off + j];
+        double ca = 1.0;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const double wa = zplanes ? zpow(*zplanes, j, 0.0, a) : ca;
+            p[a] += wa * E;
+            p[4 + a] += wa * EB;
+            ca *= c;
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 8; ++a) p[a] = warp_sum(p[a]);
+    if (lane == 0)
+        for (int a = 0; a < 8; ++a) s[a] = p[a];
+}
+
+__global__ void __launch_bounds__(192) k_corr_moments_line(int Nd, const int* __restrict__ dvm_cell,
+                                                           const double* __restrict__ Wnew,
+                                                           const double* __restrict__ Wmom, Records recNew,
+                                                           Records recHalf, VGridDev vg,
+                                                           const double* __restrict__ momh, double* __restrict__ mom) {
+    const int k = blockIdx.x;
+    if (k >= Nd) return;
+    __shared__ double axs[2][3][8];
+    const int nx = vg.nx, ny = vg.ny, nz = vg.nz, NT = vg.NT;
+    const int c = dvm_cell[k];
+    const int w = threadIdx.x >> 5, r = w / 3, d = w % 3;
+    const double* tab = (r == 0 ? recNew.tab : recHalf.tab) + (long long)k * NTAB * NT;
+    const int off = d == 0 ? 0 : (d == 1 ? nx : nx + ny), n = d == 0 ? nx : (d == 1 ? ny : nz);
+    table_sums(tab, NT, vg.xi, off, n, Wnew[c * 5 + 1 + d], threadIdx.x & 31, axs[r][d],
+               (vg.reduced && d == 2) ? &vg : nullptr);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    const double* mh = momh + (long long)k * MOMN;
+    double* m = mom + (long long)k * MOMN;
+    const double dl[3] = {Wnew[c * 5 + 1] - Wmom[c * 5 + 1], Wnew[c * 5 + 2] - Wmom[c * 5 + 2],
+                          Wnew[c * 5 + 3] - Wmom[c * 5 + 3]};
+    double sh[13], mN[13], mH[13];
+    shift_moments13(mh, dl, sh);
+    rec_moments13(axs[0][0], axs[0][1], axs[0][2], recNew.scal[(long long)k * RS + RS_P0], mN);
+    rec_moments13(axs[1][0], axs[1][1], axs[1][2], recHalf.scal[(long long)k * RS + RS_P0], mH);
+    for (int i = 0; i < 13; ++i) m[i] = sh[i] + vg.w * (mN[i] - mH[i]);
+}
+
 template <typename S, typename T>
 static void correct_t(gsis_ctx* c) {
     const int Nd = (int)c->Nd;
@@ -864,10 +917,15 @@ static void correct_t(gsis_ctx* c) {
         }
         configured = smem;
     }
+    const bool line = c->face_nd == 1;
     k_correct<S, T><<<Nd, 256, smem, c->stream>>>(Nd, c->dvm_cell, c->m.side_bc, c->m.Sout, (S*)c->f, c->recNew,
-                                                   c->recHalf, c->vg, c->momh, c->mom);
-    k_corr_moments<<<(Nd + 63) / 64, 64, 0, c->stream>>>(Nd, c->dvm_cell, c->W, c->Wmom, c->recNew, c->recHalf, c->vg.w,
-                                                         c->momh, c->mom);
+                                                   c->recHalf, c->vg, c->momh, c->mom, line);
+    if (line)
+        k_corr_moments_line<<<Nd, 192, 0, c->stream>>>(Nd, c->dvm_cell, c->W, c->Wmom, c->recNew, c->recHalf, c->vg,
+                                                       c->momh, c->mom);
+    else
+        k_corr_moments<<<(Nd + 63) / 64, 64, 0, c->stream>>>(Nd, c->dvm_cell, c->W, c->Wmom, c->recNew, c->recHalf,
+                                                             c->vg.w, c->momh, c->mom);
     c->launches += 2;
 }
 
@@ -966,7 +1024,7 @@ static void moments_t(gsis_ctx* c, const double* Wref, double* out) {
     const int Nd = (int)c->Nd;
     if constexpr (std::is_same<T, float>::value) {
         const size_t sm = sizeof(double) * (2 * (size_t)c->vg.nx + 4 * (size_t)c->vg.nz + (size_t)MROW_THREADS * MOMN);
-        if (c->vg.nx % Vec16<S>::N == 0 && sm <= 48 * 1024 - MROW_THREADS / 32 * MOMN * sizeof(double)) {
+        if (c->face_nd != 1 && c->vg.nx % Vec16<S>::N == 0 && sm <= 48 * 1024 - MROW_THREADS / 32 * MOMN * sizeof(double)) {
             k_moments_rows<S><<<Nd, MROW_THREADS, sm, c->stream>>>(Nd, c->dvm_cell, Wref, c->m.side_bc, c->m.Sout,
                                                                    (const S*)c->f, c->vg, out);
             c->launches++;

@@ -187,6 +187,8 @@ __device__ __forceinline__ void compute_cells(const SweepArgs& a, const int* kk,
                                               const T (*lo)[NC][VPT], const T (*hi)[NC][VPT],
                                               const T (*lo2)[NC][VPT], const T (*hi2)[NC][VPT], T (*fo)[VPT]) {
     const int NT = a.vg.NT, nx = a.vg.nx, ny = a.vg.ny;
+    // (a batch runs lines in its 3-direction kernels too, always by the general update)
+    const bool line = !INTERIOR && a.nc == 1;
 #pragma unroll
     for (int b = 0; b < CB; ++b) {
         if (!kon[b]) continue;
@@ -226,7 +228,7 @@ __device__ __forceinline__ void compute_cells(const SweepArgs& a, const int* kk,
                 const T dl = c0 - vl, dh = vh - c0;
                 // half the cell's own limited slope (outgoing face values c0 -+ hown);
                 // zero next to a side that is not a DVM side (its value repeats c0)
-                const T hown = hmm_t<T>(dl, dh);
+                const T hown = hmm_of<T, NC == 1>(dl, dh, line);
                 if constexpr (INTERIOR && std::is_same<T, double>::value) {
                     // (FP64 arithmetic, where the FP64 pipe bounds the sweep; in FP32
                     // the votes and selects cost more issue slots than they save.)
@@ -272,7 +274,7 @@ __device__ __forceinline__ void compute_cells(const SweepArgs& a, const int* kk,
                     if constexpr (NC >= 3) xn = fma(V.x2[u], m[b].S[2 * d][NC >= 3 ? 2 : 0], xn);
                     T fin;
                     if (kl == SK_DVM) {   // neighbour's face value: its value plus half its limited slope
-                        fin = vl + hmm_t<T>(vl - lo2[b][d][u], dl);
+                        fin = vl + hmm_of<T, NC == 1>(vl - lo2[b][d][u], dl, line);
                     } else {
                         const int iz = V.q[u] / ny;
                         fin = scl * eval_recT<T>(bsl, btl, NT, nx, ny, V.ix[u], V.q[u] - ny * iz, iz);
@@ -287,7 +289,7 @@ __device__ __forceinline__ void compute_cells(const SweepArgs& a, const int* kk,
                     if constexpr (NC >= 3) xn = fma(V.x2[u], m[b].S[2 * d + 1][NC >= 3 ? 2 : 0], xn);
                     T fin;
                     if (kh == SK_DVM) {
-                        fin = vh - hmm_t<T>(dh, hi2[b][d][u] - vh);
+                        fin = vh - hmm_of<T, NC == 1>(dh, hi2[b][d][u] - vh, line);
                     } else {
                         const int iz = V.q[u] / ny;
                         fin = sch * eval_recT<T>(bsh, bth, NT, nx, ny, V.ix[u], V.q[u] - ny * iz, iz);

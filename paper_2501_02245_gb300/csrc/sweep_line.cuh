@@ -42,7 +42,7 @@ __device__ __forceinline__ double gfma(double a, double b, double c) { return fm
 __device__ __forceinline__ float2 gfma(float a, float2 b, float2 c) { return f2fma(bc2(a), b, c); }
 __device__ __forceinline__ double gmm(double a, double b) { return mm_t<double>(a, b); }
 __device__ __forceinline__ float2 gmm(float2 a, float2 b) {
-    return make_float2(mm_t<float>(a.x, b.x), mm_t<float>(a.y, b.y));
+    return make_float2(mm_line<float>(a.x, b.x), mm_line<float>(a.y, b.y));
 }
 __device__ __forceinline__ double gsel(bool c, double a, double b) { return c ? a : b; }
 __device__ __forceinline__ float2 gsel(bool c, float2 a, float2 b) { return make_float2(c ? a.x : b.x, c ? a.y : b.y); }

@@ -14,8 +14,9 @@
 
 namespace gsis {
 
-__device__ __forceinline__ float2 hmm2(float2 a, float2 b) {
-    return make_float2(hmm_t<float>(a.x, b.x), hmm_t<float>(a.y, b.y));
+template <bool LINE>
+__device__ __forceinline__ float2 hmm2(float2 a, float2 b, bool line) {
+    return make_float2(hmm_of<float, LINE>(a.x, b.x, line), hmm_of<float, LINE>(a.y, b.y, line));
 }
 
 // base + row * row_bytes in one instruction (from an element index it takes four)
@@ -105,6 +106,7 @@ __device__ __forceinline__ void compute_cells2(const SweepArgs& a, const int* kk
                                                const float2 (*hi)[NC][VPT], const float2 (*lo2)[NC][VPT],
                                                const float2 (*hi2)[NC][VPT], float2 (*fo)[VPT]) {
     const int NT = a.vg.NT, nx = a.vg.nx, ny = a.vg.ny;
+    const bool line = !INTERIOR && a.nc == 1;
 #pragma unroll
     for (int b = 0; b < CB; ++b) {
         if (!kon[b]) continue;
@@ -140,12 +142,12 @@ __device__ __forceinline__ void compute_cells2(const SweepArgs& a, const int* kk
             for (int u = 0; u < VPT; ++u) {
                 const float2 c0 = fc[b][u], vl = lo[b][d][u], vh = hi[b][d][u];
                 const float2 dl = f2sub(c0, vl), dh = f2sub(vh, c0);
-                const float2 hown = hmm2(dl, dh);
+                const float2 hown = hmm2<NC == 1>(dl, dh, line);
                 if (kl != SK_NONE) {
                     const float2 xn = normal2<NC>(V, u, m[b].S[2 * d]);
                     float2 fin;
                     if (kl == SK_DVM) {
-                        fin = f2add(vl, hmm2(f2sub(vl, lo2[b][d][u]), dl));
+                        fin = f2add(vl, hmm2<NC == 1>(f2sub(vl, lo2[b][d][u]), dl, line));
                     } else {
                         const int iz = V.q[u] / ny, iy = V.q[u] - ny * iz;
                         fin = make_float2(scl * eval_recT<float>(bsl, btl, NT, nx, ny, V.ix[u], iy, iz),
@@ -161,7 +163,7 @@ __device__ __forceinline__ void compute_cells2(const SweepArgs& a, const int* kk
                     const float2 xn = normal2<NC>(V, u, m[b].S[2 * d + 1]);
                     float2 fin;
                     if (kh == SK_DVM) {
-                        fin = f2sub(vh, hmm2(dh, f2sub(hi2[b][d][u], vh)));
+                        fin = f2sub(vh, hmm2<NC == 1>(dh, f2sub(hi2[b][d][u], vh), line));
                     } else {
                         const int iz = V.q[u] / ny, iy = V.q[u] - ny * iz;
                         fin = make_float2(sch * eval_recT<float>(bsh, bth, NT, nx, ny, V.ix[u], iy, iz),
