@@ -414,12 +414,23 @@ std::vector<int2> batch_items(const std::vector<gsis_ctx*>& cs, int shape) {
 std::string batch_signature(const std::vector<gsis_ctx*>& cs, int nc) {
     std::vector<std::string> parts;
     for (gsis_ctx* c : cs)
-        parts.push_back(std::to_string(c->Nd) + "x" + std::to_string(c->vg.Nv) + "x" + std::to_string(c->p.vdf_dtype) +
-                        "x" + std::to_string(c->m.H));
+        parts.push_back(std::to_string(c->Nd) + "x" + std::to_string(c->vg.nx) + "." + std::to_string(c->vg.ny) + "." +
+                        std::to_string(c->vg.nz) + "x" + std::to_string(c->p.vdf_dtype) + "x" +
+                        std::to_string(c->normal_components) + "x" + std::to_string(c->m.H));
     std::sort(parts.begin(), parts.end());
     std::string s = "nc" + std::to_string(nc);
     for (auto& p : parts) s += "|" + p;
     return s;
+}
+
+// Whether every member of the batch can run the tile shape: the pair shapes need FP32 /
+// BF16 / FP16 storage and an even nx, the line shape 1D lines whose cells are all kinetic.
+bool batch_shape_fits(const BatchPlan* P, int shape) {
+    for (gsis_ctx* c : P->ctxs) {
+        if (batch_shape_pair(shape) && (c->p.vdf_dtype == GSIS_F64 || c->vg.nx % 2 != 0)) return false;
+        if (batch_shape_line(shape) && !line_ok(c)) return false;
+    }
+    return true;
 }
 
 // Autotuner: time every tile shape on the batch itself (one warm-up and two
@@ -428,33 +439,26 @@ std::string batch_signature(const std::vector<gsis_ctx*>& cs, int nc) {
 gsis_status tune_batch(BatchPlan* P) {
     gsis_ctx* o = P->owner;
     if (forced_batch_shape() >= 0) {   // test hook: the named shape, if this batch can run it
-        bool pairs_ok = true, lines_ok = true;
-        for (gsis_ctx* c : P->ctxs) {
-            pairs_ok = pairs_ok && c->p.vdf_dtype != GSIS_F64 && c->vg.nx % 2 == 0;
-            lines_ok = lines_ok && line_ok(c);
-        }
-        if (!(batch_shape_pair(forced_batch_shape()) && !pairs_ok) && !(batch_shape_line(forced_batch_shape()) && !lines_ok)) {
+        if (batch_shape_fits(P, forced_batch_shape())) {
             P->shape = forced_batch_shape();
             P->tuned = false;
             return GSIS_OK;
         }
-        return set_err(o, GSIS_ERR_ARG, pairs_ok ? "the forced batch tile needs 1D members whose cells are all kinetic"
-                                                : "the forced batch tile needs FP32/BF16/FP16 members with an even nx");
+        return set_err(o, GSIS_ERR_ARG, batch_shape_line(forced_batch_shape())
+                                            ? "the forced batch tile needs 1D members whose cells are all kinetic"
+                                            : "the forced batch tile needs FP32/BF16/FP16 members with an even nx");
     }
-    {   // 1D members whose cells are all kinetic: the line sweep, without a search (the 64-shock batch:
-        // 14.5 ms per iteration, 18.8 with the best of the other tiles)
-        bool lines = true;
-        for (gsis_ctx* c : P->ctxs) lines = lines && line_ok(c);
-        for (int sh = 0; lines && sh < batch_num_shapes(); ++sh)
-            if (batch_shape_line(sh)) {
-                P->shape = sh;
-                P->tuned = false;
-                return GSIS_OK;
-            }
-    }
+    // 1D members whose cells are all kinetic: the line sweep, without a search (the 64-shock batch:
+    // 14.5 ms per iteration, 18.8 with the best of the other tiles)
+    for (int sh = 0; sh < batch_num_shapes(); ++sh)
+        if (batch_shape_line(sh) && batch_shape_fits(P, sh)) {
+            P->shape = sh;
+            P->tuned = false;
+            return GSIS_OK;
+        }
     const std::string sig = batch_signature(P->ctxs, P->nc);
     auto hit = tuned_shapes().find(sig);
-    if (hit != tuned_shapes().end()) {
+    if (hit != tuned_shapes().end() && batch_shape_fits(P, hit->second)) {
         P->shape = hit->second;
         P->tuned = true;
         return GSIS_OK;
@@ -484,10 +488,8 @@ gsis_status tune_batch(BatchPlan* P) {
     int best = 1;
     double best_ms = 1e300;
     int2* d_it = nullptr;
-    bool pairs_ok = true;   // the pair shapes need FP32 / BF16 / FP16 storage and an even nx in every member
-    for (gsis_ctx* c : P->ctxs) pairs_ok = pairs_ok && c->p.vdf_dtype != GSIS_F64 && c->vg.nx % 2 == 0;
     for (int sh = 0; sh < ns; ++sh) {
-        if ((batch_shape_pair(sh) && !pairs_ok) || batch_shape_line(sh)) continue;   // (not all members are lines here)
+        if (!batch_shape_fits(P, sh)) continue;
         std::vector<int2> it = batch_items(P->ctxs, sh);
         d_it = (int2*)dev_alloc(o, std::max<size_t>(1, it.size()) * sizeof(int2));
         if (!d_it) break;

@@ -338,7 +338,8 @@ gsis_status tune_sweep(gsis_ctx* c) {
         return GSIS_OK;
     }
     const std::string key = std::to_string(c->p.vdf_dtype) + "/" + std::to_string(c->normal_components) + "/" +
-                            std::to_string(c->Nd) + "/" + std::to_string(c->vg.Nv) + "/" + std::to_string(c->m.H);
+                            std::to_string(c->Nd) + "/" + std::to_string(c->vg.nx) + "x" + std::to_string(c->vg.ny) + "x" +
+                            std::to_string(c->vg.nz) + "/" + std::to_string(c->m.H);
     auto hit = sweep_cache().find(key);
     if (hit != sweep_cache().end()) {
         c->sweep_shape = hit->second;
