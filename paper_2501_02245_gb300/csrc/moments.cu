@@ -25,6 +25,8 @@
 // n = 64) of the sum of |terms|, far under the storage rounding of BF16/FP16
 // (2^-9 / 2^-12 per value) and comparable to FP32 storage rounding.
 #include <cooperative_groups.h>
+#include <map>
+#include <mutex>
 #include <type_traits>
 #include "gsis_device.cuh"
 #include "packed.cuh"
@@ -901,21 +903,33 @@ __global__ void __launch_bounds__(192) k_corr_moments_line(int Nd, const int* __
     for (int i = 0; i < 13; ++i) m[i] = sh[i] + vg.w * (mN[i] - mH[i]);
 }
 
+// Raises a kernel's limit of dynamic shared memory to `bytes`; the limit belongs to the
+// device, and host threads may launch on several.
+static bool allow_smem(const void* kernel, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<const void*, int>, size_t> limit;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    size_t& have = limit[{kernel, dev}];
+    if (bytes <= have) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    have = bytes;
+    return true;
+}
+
 template <typename S, typename T>
 static void correct_t(gsis_ctx* c) {
     const int Nd = (int)c->Nd;
     const long long nyz = (long long)c->vg.ny * c->vg.nz;
     const size_t smem = (size_t)4 * (c->vg.nx + nyz) * sizeof(T);
-    static size_t configured = 0;   // per instantiation: the largest dynamic size set so far
-    if (smem > configured) {
-        if (cudaFuncSetAttribute(k_correct<S, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            set_err(c, GSIS_ERR_UNSUPPORTED, "velocity grid too large for the correction pass's tables");
-            c->broken = true;
-            return;
-        }
-        configured = smem;
+    if (!allow_smem((const void*)k_correct<S, T>, smem)) {
+        set_err(c, GSIS_ERR_UNSUPPORTED, "velocity grid too large for the correction pass's tables");
+        c->broken = true;
+        return;
     }
     const bool line = c->face_nd == 1;
     k_correct<S, T><<<Nd, 256, smem, c->stream>>>(Nd, c->dvm_cell, c->m.side_bc, c->m.Sout, (S*)c->f, c->recNew,
@@ -1037,8 +1051,19 @@ static void moments_t(gsis_ctx* c, const double* Wref, double* out) {
     int tb = 256;
     for (int b : {256, 192, 128})
         if ((rows + b - 1) / b * b - rows < (rows + tb - 1) / tb * tb - rows) tb = b;
-    // c_x tables, then one row of MOMN sums per thread for the block reduction
-    const size_t smem = ((size_t)4 * c->vg.nx * sizeof(T) + 7) / 8 * 8 + (size_t)tb * MOMN * sizeof(double);
+    // c_x tables, then one row of MOMN sums per thread for the block reduction: long x axes take smaller
+    // blocks (above 168 FP64 or 336 FP32 nodes 256 threads pass 48 KB), then a larger limit
+    auto bytes = [&](int t) {
+        return ((size_t)4 * c->vg.nx * sizeof(T) + 7) / 8 * 8 + (size_t)t * MOMN * sizeof(double);
+    };
+    const size_t room = 48 * 1024 - 32 * MOMN * sizeof(double);
+    while (tb > 128 && bytes(tb) > room) tb -= 64;
+    const size_t smem = bytes(tb);
+    if (smem > room && !allow_smem((const void*)k_moments<S, T>, smem)) {
+        set_err(c, GSIS_ERR_UNSUPPORTED, "velocity grid too large for the moment pass's tables");
+        c->broken = true;
+        return;
+    }
     k_moments<S, T><<<Nd, tb, smem, c->stream>>>(Nd, c->dvm_cell, Wref, c->m.side_bc, c->m.Sout, (const S*)c->f,
                                                   c->vg, out);
     c->launches++;
