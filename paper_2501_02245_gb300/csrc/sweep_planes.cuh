@@ -11,8 +11,10 @@
 //     den = 1/tau + 2 sum (m_L + m_H),
 //   mm the minmod (a face is an outflow or an inflow face: one of its m, n is
 //   zero), instead of picking each side's upwind rows per velocity; the sums run in
-//   the order of compute_cells, and the products with zero change nothing, so the
-//   results are those of the other tiles (to FP32 subnormals, which halving rounds);
+//   the order of compute_cells, and the products of finite values with zero change
+//   nothing, so the results are those of the other tiles (to FP32 subnormals, which
+//   halving rounds); a pair whose sum is not a number, as where a value downstream has
+//   overflowed its storage to an infinity, is formed again by compute_cells;
 // - on 2D meshes m, n, den and the reciprocal do not depend on the plane and are
 //   formed once per cell;
 // - a row's address is one mad.wide from its byte pitch;
@@ -177,8 +179,23 @@ __device__ __forceinline__ void add_record(const SweepArgs& a, int k, int kinds,
     }
 }
 
+// The general update of one cell at the velocities v and v + 1 (a pair whose product
+// form met an infinity; out of line).
+template <typename S, int NC>
+__device__ __noinline__ void redo_pair(const SweepArgs& a, S* f, int k, int v) {
+    const bool on = true;
+    CellMeta<float, NC> m;
+    load_meta<float, NC>(a, k, m);
+#pragma unroll 1
+    for (int j = 0; j < 2; ++j) {
+        Vel<float, 1> V;
+        make_vel<float, 1, false>(a.vg, v + j, 0, V);
+        update_cells_k<S, float, NC, 1, 1, false>(a, f, &k, &on, V, &m);
+    }
+}
+
 template <typename S, int NC, int ZP>
-__device__ __forceinline__ void apply_pairs(const SweepArgs& a, int k, int kinds, const PairFactors<NC, ZP>& m,
+__device__ __forceinline__ void apply_pairs(const SweepArgs& a, S* f, int k, int kinds, const PairFactors<NC, ZP>& m,
                                             const PairColumn<S, NC, ZP>& C, unsigned row_bytes,
                                             const PairStencil<S, NC, ZP>& q) {
     constexpr int DZ = NC == 3 ? ZP : 1;   // coefficients per plane on 3D meshes
@@ -248,13 +265,26 @@ __device__ __forceinline__ void apply_pairs(const SweepArgs& a, int k, int kinds
         r[z].x = recip_t<float>(2.0f * out[z].x);
         r[z].y = recip_t<float>(2.0f * out[z].y);
     }
+    float2 v[ZP];
+    float t = 0.0f;   // NaN if any value is
+#pragma unroll
+    for (int u = 0; u < ZP; ++u) {
+        v[u] = f2mul(num[u], r[NC == 3 ? u : 0]);
+        t += v[u].x + v[u].y;
+    }
+    if (t != t) {
+#pragma unroll 1
+        for (int u = 0; u < C.nact; ++u) redo_pair<S, NC>(a, f, k, C.ix + a.vg.nx * (u == 0 ? C.q[0] : C.q[ZP - 1]));
+        return;
+    }
 #pragma unroll
     for (int u = 0; u < ZP; ++u)
-        if (u < C.nact) st2<S>(reinterpret_cast<S*>(row_at(C.fz[u], k, row_bytes)), f2mul(num[u], r[NC == 3 ? u : 0]));
+        if (u < C.nact) st2<S>(reinterpret_cast<S*>(row_at(C.fz[u], k, row_bytes)), v[u]);
 }
 
 template <typename S, int NC, int ZP, int G, int MINB>
-__global__ void __launch_bounds__(32 * G, MINB) k_sweep_planes(SweepArgs a, S* __restrict__ f, int pass, int nptile) {
+__global__ void __launch_bounds__(32 * G, MINB) k_sweep_planes(const __grid_constant__ SweepArgs a, S* __restrict__ f,
+                                                               int pass, int nptile) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned row_bytes = (unsigned)(a.vg.Nv * sizeof(S));
     PairColumn<S, NC, ZP> C;
@@ -282,7 +312,7 @@ __global__ void __launch_bounds__(32 * G, MINB) k_sweep_planes(SweepArgs a, S* _
             load_stencil(k, r, C, row_bytes, q);
             load_factors(a, k, C, g);
             if (more || w < nn) load_rows<NC>(a, kn, r);
-            apply_pairs<S, NC, ZP>(a, k, kinds, g, C, row_bytes, q);
+            apply_pairs<S, NC, ZP>(a, f, k, kinds, g, C, row_bytes, q);
             k = kn;
         }
         if (w >= n && w < nn) {
