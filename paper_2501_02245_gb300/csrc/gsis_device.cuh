@@ -156,9 +156,9 @@ __device__ __forceinline__ double viscosity(double T, double mu0, double omega) 
     return mu0 * exp(omega * log(T));
 }
 
-// 1 / x to within two units in the last place (x a normal number, not 0): the
-// hardware's double-precision seed (20 bits) and two Newton-Raphson steps, four
-// FP64 operations where the division takes about ten.
+// 1 / x to within one unit in the last place for |x| from 2^-1022 to 2^1021 (NaN for 0
+// and the infinities): the hardware's double-precision seed (20 bits) and two
+// Newton-Raphson steps, four FP64 operations where the division takes about ten.
 __device__ __forceinline__ double recip64(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));

@@ -10,10 +10,11 @@
 //  * mills: h(t) = (1/2) erfc(t/sqrt 2) exp(t^2/2) for 0 <= t <= 10 as its Taylor
 //    series of degree 6 about the nearest multiple of 1/64; h satisfies
 //    h' = t h - 1/sqrt(2 pi), so (n+1) c_{n+1} = t c_n + c_{n-1}.
-// Largest errors against 40-digit values over the arguments of the flux, in units
-// in the last place: exp 0.75, T^0.81 3.4 (the library's exp and log composed the
-// same way: 3.4), h 3.2 (half of 1 - erf loses the tail's relative accuracy
-// altogether).
+// Errors in units in the last place, bound (largest seen over every table interval, by
+// tests/test_gpu_special.py): exp 0.85 (0.80); log 0.55 plus 2^-58, absolute near log x = 0, where the
+// table value cancels e ln 2 (0.50); h 4 (3.2; half of 1 - erf loses the tail's relative accuracy
+// altogether); T^0.81 for 0.05 <= T <= 20 5 (3.5).  Outside their ranges exp and log
+// are the library's, and h keeps its value at 10.
 #pragma once
 #include "gsis_device.cuh"
 
@@ -231,7 +232,7 @@ __device__ __forceinline__ double exp_tab(double y) {
     return __hiloint2double(__double2hiint(v) + (k >> 6) * (1 << 20), __double2loint(v));
 }
 
-// log(x)
+// log(x); near x = 1 the error is absolute (2^-58), not relative: enough for x^omega
 __device__ __forceinline__ double log_tab(double x) {
     const unsigned hi = (unsigned)__double2hiint(x);
     if (hi - 0x00100000u >= 0x7fe00000u) return log(x);   // not a positive normal number
