@@ -176,19 +176,39 @@ def source_sha(files):
     return h.hexdigest()[:16]
 
 
-def traffic_per_point(config, dtype):
+# the sources that the sweep kernels are made of
+SWEEP_SOURCES = ("sweep.cu", "sweep_col.cu", "sweep_ring.cu", "sweep_line.cu", "sweep_line.cuh", "sweep_planes.cuh",
+                 "sweep_planes_f32.cu", "sweep_planes_bf16.cu", "sweep_planes_f16.cu", "sweep_pair.cuh",
+                 "sweep_device.cuh", "packed.cuh", "gsis_device.cuh")
+
+
+def sweep_tile(tuning):
+    """Name of the tile in Solver.tuning_info()'s text ("tile NAME (autotuned; ...)"); "" where it names none."""
+    return tuning.split()[1] if tuning.startswith("tile ") else ""
+
+
+def sweep_kernel(tuning):
+    """The sweep kernel that ran, from Solver.tuning_info()'s text."""
+    if tuning.startswith("1D line"):
+        return "k_sweep_line"
+    for prefix, kernel in (("col_", "k_sweep_col"), ("planes", "k_sweep_planes"), ("ring_", "k_sweep_ring"),
+                           ("p", "k_sweep2")):
+        if sweep_tile(tuning).startswith(prefix):
+            return kernel
+    return "k_sweep"
+
+
+def traffic_per_point(config, dtype, tuning):
     """DRAM bytes per (cell, velocity) point of one sweep launch, from the
-    committed ncu summary, if it was taken on the current sweep source (else
-    None)."""
+    committed ncu summary, if it was taken on the current sweep sources and
+    the tile that ran (else None)."""
     p = os.path.join(ROOT, "profiles", "sweep_%s_%s.json" % (config, dtype))
     if not os.path.exists(p):
         return None
     with open(p) as fh:
         d = json.load(fh)
-    sha = source_sha(["paper_2501_02245_gb300/csrc/" + f for f in
-                      ("sweep.cu", "sweep_device.cuh", "sweep_pair.cuh", "sweep_col.cu", "sweep_planes.cuh",
-                       "sweep_line.cuh", "gsis_device.cuh")])
-    if d.get("sweep_src_sha") != sha:
+    sha = source_sha(["paper_2501_02245_gb300/csrc/" + f for f in SWEEP_SOURCES])
+    if d.get("sweep_src_sha") != sha or d.get("tile") != sweep_tile(tuning):
         return None
     return d.get("dram_bytes_per_point")
 
@@ -324,7 +344,7 @@ def measured_alu_peaks(stream, local):
     return out
 
 
-def sweep_roofline(args, rep, steps, peaks, traffic):
+def sweep_roofline(args, rep, steps, peaks, traffic, kernel):
     """Roofline of the dominant kernel (the kinetic sweep) in the unit of one
     GSIS iteration -- every (cell, velocity) point updated once: read f once,
     write f once (2b bytes), one point update's flops -- over the measured
@@ -345,7 +365,7 @@ def sweep_roofline(args, rep, steps, peaks, traffic):
             peak, src = FP64_PEAK_TFLOPS, "FP64 unit counts x clock: 152 SMs x 2 DFMA/clk x 2.07 GHz (derived)"
         achieved = fpp * pts / (sweep_ms_iter * 1e-3) / 1e12
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": trf, "kernel": "k_sweep<double>" if args.config == "shock" else "k_sweep_col", "peak_source": src,
+                "traffic": trf, "kernel": kernel, "peak_source": src,
                 "per": "GSIS iteration: %g sweep launches (Gauss-Seidel passes) per iteration" % launches_iter,
                 "algorithmic": "%d FP64 flop per (cell, velocity) per GSIS iteration (one point update)" % fpp,
                 "per_pass": {"achieved": achieved * launches_iter, "frac": achieved * launches_iter / peak,
@@ -354,7 +374,7 @@ def sweep_roofline(args, rep, steps, peaks, traffic):
     else:
         achieved = 2 * eb * pts / (sweep_ms_iter * 1e-3) / 1e9
         roof = {"bound": "hbm", "achieved": achieved, "peak": mp["hbm_gbs"], "unit": "GB/s",
-                "frac": achieved / mp["hbm_gbs"], "traffic": trf, "kernel": "k_sweep_planes",
+                "frac": achieved / mp["hbm_gbs"], "traffic": trf, "kernel": kernel,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured copy bandwidth)",
                 "per": "GSIS iteration: %g sweep launches (Gauss-Seidel passes) per iteration" % launches_iter,
                 "algorithmic": "2 x %d bytes per (cell, velocity) per GSIS iteration (read f once, write once)" % eb,
@@ -414,7 +434,8 @@ def run_gsis(args):
             peaks = measured_alu_peaks(stream, local)
         except Exception as exc:   # the roofline then falls back to the derived FP64 peak, and says so
             peaks = {"error": str(exc)}
-    roof = sweep_roofline(args, rep, args.steps, peaks, traffic_per_point(args.config, args.dtype))
+    roof = sweep_roofline(args, rep, args.steps, peaks, traffic_per_point(args.config, args.dtype, tuning),
+                          sweep_kernel(tuning))
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": t_max / args.steps, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": args.dtype, "data": "synthetic",
@@ -729,12 +750,13 @@ def run_batch(args):
     with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
         peaks = json.load(fh)
     achieved = bytes_alg / (sweep_ms * 1e-3) / 1e9
+    info = batch_info(solvers)
     roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": achieved / peaks["hbm_gbs"], "traffic": None,
-            "kernel": "k_sweep_batch_line (both Gauss-Seidel passes of all 64 solves, one launch)",
+            "kernel": "%s (both Gauss-Seidel passes of all 64 solves, one launch)"
+                      % ("k_sweep_batch_line" if "tile=line" in info else "k_sweep_batch"),
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured)",
             "algorithmic": "2 passes x 2 x b bytes per (cell, velocity), b = 4 (FP32) / 2 (BF16)"}
-    info = batch_info(solvers)
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": t_max / args.steps, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f32/bf16", "data": "synthetic",
