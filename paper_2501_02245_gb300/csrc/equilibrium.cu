@@ -273,10 +273,11 @@ __global__ void k_build_records(const RecSpec* __restrict__ specs, int nrec, int
 // conserved quantities, entry by entry from the terms of its polynomials, and a pivoted
 // elimination.  The line's synthetic solve amplifies a difference in the last bit
 // (mu_of in macro.cu), so its records keep these operations and their order, where other
-// meshes take the shorter form above.  A warp builds one record: lanes 8 d + i add the
-// axis sums of axis d over the nodes i, i + 8, ... (eight partial sums per axis,
-// whatever the number of lanes), lane e then forms entry e of the 30 of the system.  50 to 87
-// us a launch with eight lanes and four entries on each; 25 for the short form.
+// meshes take the shorter form above.  LPR lanes build one record.  The axis sums are
+// eight partial sums per axis, over the nodes i, i + 8, ..., whatever LPR: with 32 lanes
+// those 8 d + i have axis d and each lane one of the 30 entries of the system, with 8 every
+// lane its share of each axis and four entries.  50 to 87 us a launch with 8; 25 for
+// the short form.
 struct Term { double c; int a, b, d; };
 
 __device__ static int psi_terms(int row, const double* u, Term* t, double scale) {
@@ -351,11 +352,16 @@ __device__ static void cons_of(double rho, const double* u, double T, double* U)
     U[4] = rho * (1.5 * T + 0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
 }
 
+template <int LPR>
 __global__ void k_build_records_line(const RecSpec* __restrict__ specs, int nrec, int n0, Records out0, Records out1,
                                      VGridDev vg) {
-    const int lane = threadIdx.x & 31;
-    const int rr = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (rr >= nrec) return;   // (whole warps)
+    constexpr int AXES = LPR == 32 ? 1 : 3, SLOTS = LPR == 32 ? 1 : 4;   // axes and entries of the system per lane
+    const int lane = threadIdx.x & (LPR - 1);
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (warp * (32 / LPR) >= nrec) return;   // (whole warps)
+    const int r0 = warp * (32 / LPR) + (threadIdx.x & 31) / LPR;
+    const bool valid = r0 < nrec;   // groups past the end compute a copy and store nothing
+    const int rr = valid ? r0 : nrec - 1;
     const RecSpec s = specs[rr];
     const Records& out = rr < n0 ? out0 : out1;
     const long long r = rr < n0 ? rr : rr - n0;
@@ -366,40 +372,54 @@ __global__ void k_build_records_line(const RecSpec* __restrict__ specs, int nrec
     const double A = s.rho * pow(2.0 * PI * T, -1.5);
     const double sq2piT = sqrt(2.0 * PI * T);   // (the reduced grid's planes: see k_build_records)
     const double i2T = 0.5 / T;
-    double part[6] = {0, 0, 0, 0, 0, 0};
-    const int d = lane >> 3;
-    if (d < 3) {
+    double part[AXES][6];
+#pragma unroll
+    for (int q = 0; q < AXES; ++q) {
+        const int d = LPR == 32 ? lane >> 3 : q;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) part[q][k] = 0.0;
+        if (d > 2) continue;
         const int lo = d == 0 ? 0 : (d == 1 ? nx : nx + ny), hi = d == 0 ? nx : (d == 1 ? nx + ny : NT);
         for (int idx = lo + (lane & 7); idx < hi; idx += 8) {
             if (vg.reduced && d == 2) {
                 const int p = idx - nx - ny;
-                tab[idx] = p ? sq2piT * T : sq2piT;
-                tab[2 * NT + idx] = 0.0;
-                tab[3 * NT + idx] = p ? 3.0 * T : T;
+                if (valid) {
+                    tab[idx] = p ? sq2piT * T : sq2piT;
+                    tab[2 * NT + idx] = 0.0;
+                    tab[3 * NT + idx] = p ? 3.0 * T : T;
+                }
                 continue;
             }
             const double c = vg.xi[idx] - s.u[d];
             const double e = exp(-(c * c) * i2T);
-            tab[idx] = e;
-            tab[2 * NT + idx] = c;
-            tab[3 * NT + idx] = c * c;
+            if (valid) {
+                tab[idx] = e;
+                tab[2 * NT + idx] = c;
+                tab[3 * NT + idx] = c * c;
+            }
             double pw = e;
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
-                part[k] += pw;
+                part[q][k] += pw;
                 pw *= c;
             }
         }
     }
     double Cs[3][6];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        double v = part[k];
+    for (int q = 0; q < AXES; ++q)
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, 8);
+        for (int k = 0; k < 6; ++k) {
+            double v = part[q][k];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) Cs[q][k] = __shfl_sync(0xffffffffu, v, 8 * q);
-    }
+            for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, 8);
+            if (LPR == 32) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) Cs[d][k] = __shfl_sync(0xffffffffu, v, 8 * d);
+            } else {
+                Cs[q][k] = v;
+            }
+        }
     if (vg.reduced) {   // exact xi_z integrals int c_z^k e_z dxi_z of the Gaussian (k = 0..5)
         const double zk[6] = {1.0, 0.0, T, 0.0, 3.0 * T * T, 0.0};
         for (int k = 0; k < 6; ++k) Cs[2][k] = sq2piT * zk[k];
@@ -410,22 +430,27 @@ __global__ void k_build_records_line(const RecSpec* __restrict__ specs, int nrec
         const double wa = vg.w * A;
         double U[5];
         cons_of(s.rho, s.u, T, U);
-        double mine = 0.0;   // entries 0-4: right-hand side, 5-29: the matrix by rows
-        if (lane < 5) {
-            const int na = psi_terms(lane, s.u, tp, 1.0);
-            const int nb = base_terms(s, tq);
-            mine = U[lane] - wa * poly_moment(tp, na, tq, nb, Cs);
-        } else if (lane < 30) {
-            const int ra = (lane - 5) / 5, rb = (lane - 5) % 5;
-            const int na = psi_terms(ra, s.u, tp, 1.0);
-            const int nbb = psi_terms(rb, s.u, tq, rb == 4 ? 2.0 : 1.0);
-            mine = wa * poly_moment(tp, na, tq, nbb, Cs);
+        double mine[SLOTS];   // entries 0-4: right-hand side, 5-29: the matrix by rows
+#pragma unroll
+        for (int m = 0; m < SLOTS; ++m) {
+            const int e = lane + LPR * m;
+            mine[m] = 0.0;
+            if (e < 5) {
+                const int na = psi_terms(e, s.u, tp, 1.0);
+                const int nb = base_terms(s, tq);
+                mine[m] = U[e] - wa * poly_moment(tp, na, tq, nb, Cs);
+            } else if (e < 30) {
+                const int ra = (e - 5) / 5, rb = (e - 5) % 5;
+                const int na = psi_terms(ra, s.u, tp, 1.0);
+                const int nbb = psi_terms(rb, s.u, tq, rb == 4 ? 2.0 : 1.0);
+                mine[m] = wa * poly_moment(tp, na, tq, nbb, Cs);
+            }
         }
         __syncwarp();
         double Am[5][5], rhs[5];
 #pragma unroll
         for (int e = 0; e < 30; ++e) {
-            const double v = __shfl_sync(0xffffffffu, mine, e);
+            const double v = __shfl_sync(0xffffffffu, mine[e / LPR], e % LPR, LPR);
             if (e < 5) rhs[e] = v;
             else Am[(e - 5) / 5][(e - 5) % 5] = v;
         }
@@ -443,7 +468,7 @@ __global__ void k_build_records_line(const RecSpec* __restrict__ specs, int nrec
             p2d[q] = s.P2[q] + alpha[4];
         }
     }
-    if (lane == 0) {
+    if (valid && lane == 0) {
         scal[RS_P0] = p0;
         scal[RS_P2XY] = s.P2[3];
         scal[RS_P2XZ] = s.P2[4];
@@ -451,7 +476,8 @@ __global__ void k_build_records_line(const RecSpec* __restrict__ specs, int nrec
         scal[RS_OFFD] = (s.P2[3] != 0.0 || s.P2[4] != 0.0 || s.P2[5] != 0.0) ? 1.0 : 0.0;
     }
     __syncwarp();   // the record's values written by other lanes are read below
-    for (int idx = lane; idx < NT; idx += 32) {
+    if (!valid) return;
+    for (int idx = lane; idx < NT; idx += LPR) {
         const int q = idx < nx ? 0 : (idx < nx + ny ? 1 : 2);
         const double pq = q == 0 ? pp[0] : (q == 1 ? pp[1] : pp[2]), p2q = q == 0 ? p2d[0] : (q == 1 ? p2d[1] : p2d[2]);
         const double c = tab[2 * NT + idx];
@@ -488,10 +514,17 @@ void build_records_raw(const RecSpec* d_specs, int nrec, const Records& out, con
     build_records(d_specs, nrec, nrec, out, out, vg, st);
 }
 
+// Records up to which a line's have a warp each: a few leave SMs idle (30 cells 2.27 ms a
+// case, 2.33 with four to a warp); more fill the FP64 pipes, which four to a warp
+// share (64 shocks of 100 to 800 cells 126 ms, 134 with a warp each).
+constexpr int LINE_WARP_RECORDS = 304;
 // Records of a context's own solve (records [0, n0) into out0, the rest into out1).
 static void solve_records(gsis_ctx* c, int nrec, int n0, const Records& out0, const Records& out1, const RecSpec* d_specs) {
     if (nrec <= 0) return;
-    if (c->face_nd == 1) k_build_records_line<<<(nrec + 1) / 2, 64, 0, c->stream>>>(d_specs, nrec, n0, out0, out1, c->vg);
+    if (c->face_nd == 1 && nrec <= LINE_WARP_RECORDS)
+        k_build_records_line<32><<<(nrec + 1) / 2, 64, 0, c->stream>>>(d_specs, nrec, n0, out0, out1, c->vg);
+    else if (c->face_nd == 1)
+        k_build_records_line<8><<<(nrec + 7) / 8, 64, 0, c->stream>>>(d_specs, nrec, n0, out0, out1, c->vg);
     else build_records(d_specs, nrec, n0, out0, out1, c->vg, c->stream);
     c->launches++;
 }
