@@ -189,7 +189,7 @@ def sweep_tile(tuning):
 
 def sweep_kernel(tuning):
     """The sweep kernel that ran, from Solver.tuning_info()'s text."""
-    if tuning.startswith("1D line"):
+    if tuning.startswith("1D line: window"):
         return "k_sweep_line"
     for prefix, kernel in (("col_", "k_sweep_col"), ("planes", "k_sweep_planes"), ("ring_", "k_sweep_ring"),
                            ("p", "k_sweep2")):

@@ -256,8 +256,9 @@ gsis_status gsis_debug_set_region(gsis_ctx* ctx, const uint8_t* flags);
  * tile) work items from a device counter, and the synthetic solves of all
  * meshes up to 4096 cells run in one launch (one CTA each); one iteration of
  * the whole batch is recorded once into a CUDA graph and replayed.  The tile
- * shape of the persistent sweep is that of 1D lines ("line_w4") if every
- * member is a non-periodic line of kinetic cells, else picked by timing the
+ * shape of the persistent sweep is that of 1D lines ("line_w4", or "line1_w4"
+ * for few FP64 tiles) if every member is a non-periodic line of kinetic cells
+ * and all have FP64 or all FP32 arithmetic, else picked by timing the
  * candidates on the batch itself (on a snapshot of the VDFs, restored
  * afterwards; skipped without memory for the snapshot) and cached per batch
  * shape for the life of the process.  Results are identical to iterating each
@@ -288,7 +289,8 @@ gsis_status gsis_iterate_batch(gsis_ctx** ctxs, int n, int iterations, gsis_repo
  * tile shape of the persistent batched sweep instead of the autotuned one
  * (names as reported by gsis_batch_info, e.g. "vpt2_cb1_w4", or the
  * velocity-pair shapes "pair1_cb1_w4", "pair2_cb1_w4", "pair1_cb1_w8", which
- * need FP32/BF16/FP16 members with an even nx, or "line_w4", which needs 1D
+ * need FP32/BF16/FP16 members with an even nx, or "line_w4" and "line1_w4"
+ * (two planes or one per column of FP64 members), which need 1D
  * members: gsis_iterate_batch then returns GSIS_ERR_ARG for another batch).
  * NULL or "" restores autotuning.  Every shape computes the same result.
  * GSIS_ERR_ARG for an unknown name.  The paper has no counterpart. */

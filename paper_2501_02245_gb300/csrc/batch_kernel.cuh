@@ -214,8 +214,9 @@ void batch_launch_nc3(int shape, const BatchSolve* s, const int2* i, int n, int*
 int batch_grid_nc1(int shape);
 int batch_grid_nc3(int shape);
 // batch_line.cu
+// (planes64: planes per column of the FP64 members' launch, 1 or 2; 0: the FP32-arithmetic members' launch)
 void batch_launch_line(const BatchSolve* s, const int2* i, int n, int* t, int grid, cudaStream_t st, int p0, int p1,
-                       bool f64);
-int batch_grid_line(bool f64);
+                       int planes64);
+int batch_grid_line(int planes64);
 
 }  // namespace gsis

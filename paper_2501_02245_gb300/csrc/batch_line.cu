@@ -10,20 +10,21 @@ namespace gsis {
 
 constexpr int LINE_WPB = 4;
 
-// F64: the FP64 members' items (the others are passed over), else the
-// FP32-arithmetic ones: one kernel for both would give every item the FP64
-// code's registers.
-template <bool F64>
-__global__ void __launch_bounds__(32 * LINE_WPB, F64 ? 3 : 4) k_sweep_batch_line(const BatchSolve* __restrict__ solves,
+// Z64: the FP64 members' items with Z64 planes per column (the others are passed
+// over), 0: the FP32-arithmetic ones; one kernel for both would give every item the
+// FP64 code's registers.
+template <int Z64>
+__global__ void __launch_bounds__(32 * LINE_WPB, Z64 ? 3 : 4) k_sweep_batch_line(const BatchSolve* __restrict__ solves,
                                                                                  const int2* __restrict__ items,
                                                                                  int n_items, int* __restrict__ ticket,
                                                                                  int pass0, int pass1) {
+    constexpr bool F64 = Z64 > 0;
     // the solve's arguments, one copy per warp: registers are the limit of this
     // kernel's occupancy (in the single launch they sit in the constant bank)
     __shared__ SweepArgs args[LINE_WPB];
     __shared__ LineStage stages[F64 ? 1 : LINE_WPB];
     using T = typename std::conditional<F64, double, float>::type;
-    __shared__ LineEnds<T, F64 ? LINE_ZP64 : LINE_ZP32> ends[LINE_WPB];
+    __shared__ LineEnds<T, F64 ? Z64 : LINE_ZP32> ends[LINE_WPB];
     auto& end = ends[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     SweepArgs& a = args[threadIdx.x >> 5];
@@ -42,7 +43,7 @@ __global__ void __launch_bounds__(32 * LINE_WPB, F64 ? 3 : 4) k_sweep_batch_line
             reinterpret_cast<int*>(&a)[w] = reinterpret_cast<const int*>(&B.a)[w];
         __syncwarp();
         if constexpr (F64) {
-            line_tile<double, double, LINE_ZP64>(a, (double*)B.f, B.cells, it.y, lane, pass0, pass1, stage, end);
+            line_tile<double, double, Z64>(a, (double*)B.f, B.cells, it.y, lane, pass0, pass1, stage, end);
         } else {
             if (dtype == GSIS_F32)
                 line_tile<float, float, LINE_ZP32>(a, (float*)B.f, B.cells, it.y, lane, pass0, pass1, stage, end);
@@ -54,21 +55,22 @@ __global__ void __launch_bounds__(32 * LINE_WPB, F64 ? 3 : 4) k_sweep_batch_line
     }
 }
 
-template <bool F64>
+template <int Z64>
 static int grid_of() {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sweep_batch_line<F64>, 32 * LINE_WPB, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sweep_batch_line<Z64>, 32 * LINE_WPB, 0);
     return std::max(1, sms * std::max(1, per));
 }
 
-int batch_grid_line(bool f64) { return f64 ? grid_of<true>() : grid_of<false>(); }
+int batch_grid_line(int planes64) { return planes64 == 2 ? grid_of<2>() : (planes64 == 1 ? grid_of<1>() : grid_of<0>()); }
 
 void batch_launch_line(const BatchSolve* s, const int2* i, int n, int* t, int grid, cudaStream_t st, int p0, int p1,
-                       bool f64) {
-    if (f64) k_sweep_batch_line<true><<<grid, 32 * LINE_WPB, 0, st>>>(s, i, n, t, p0, p1);
-    else k_sweep_batch_line<false><<<grid, 32 * LINE_WPB, 0, st>>>(s, i, n, t, p0, p1);
+                       int planes64) {
+    if (planes64 == 2) k_sweep_batch_line<2><<<grid, 32 * LINE_WPB, 0, st>>>(s, i, n, t, p0, p1);
+    else if (planes64 == 1) k_sweep_batch_line<1><<<grid, 32 * LINE_WPB, 0, st>>>(s, i, n, t, p0, p1);
+    else k_sweep_batch_line<0><<<grid, 32 * LINE_WPB, 0, st>>>(s, i, n, t, p0, p1);
 }
 
 }  // namespace gsis

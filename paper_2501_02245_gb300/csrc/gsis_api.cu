@@ -405,7 +405,7 @@ std::vector<int2> batch_items(const std::vector<gsis_ctx*>& cs, int shape) {
     std::vector<int2> items;
     for (int s : order) {
         if (cs[s]->Nd == 0) continue;
-        const long long nt = batch_shape_line(shape) ? line_tiles(cs[s]) : (cs[s]->vg.Nv + vt - 1) / vt;
+        const long long nt = batch_shape_line(shape) ? line_tiles(cs[s], batch_shape_planes64(shape)) : (cs[s]->vg.Nv + vt - 1) / vt;
         for (long long t = 0; t < nt; ++t) items.push_back(make_int2(s, (int)t));
     }
     return items;
@@ -448,10 +448,15 @@ gsis_status tune_batch(BatchPlan* P) {
                                             ? "the forced batch tile needs 1D members whose cells are all kinetic"
                                             : "the forced batch tile needs FP32/BF16/FP16 members with an even nx");
     }
-    // 1D members whose cells are all kinetic: the line sweep, without a search (the 64-shock batch:
-    // 14.5 ms per iteration, 18.8 with the best of the other tiles)
+    // 1D members whose cells are all kinetic, of one arithmetic: the line sweep, without a search (64 FP32 and
+    // BF16 shocks: 14.5 ms per iteration, 18.8 with the best of the other tiles), FP64 members with one plane per
+    // column while that gives no sub-partition two warps.  FP32 and FP64 lines together take two launches
+    // there, one after the other, so they are searched (2 + 2 of 200 cells, 24^3: 1.60 ms, the general sweep 1.05).
+    long long one_plane = 0;
+    for (gsis_ctx* c : P->ctxs) one_plane += c->p.vdf_dtype == GSIS_F64 ? line_tiles(c, 1) : 0;
+    const int planes64 = P->types == 2 && one_plane <= fp64_pipes() ? 1 : 2;
     for (int sh = 0; sh < batch_num_shapes(); ++sh)
-        if (batch_shape_line(sh) && batch_shape_fits(P, sh)) {
+        if (batch_shape_line(sh) && batch_shape_planes64(sh) == planes64 && P->types != 3 && batch_shape_fits(P, sh)) {
             P->shape = sh;
             P->tuned = false;
             return GSIS_OK;

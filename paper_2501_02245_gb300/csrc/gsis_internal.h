@@ -287,6 +287,7 @@ const char* batch_shape_name(int shape);
 int batch_shape_vtile(int shape);
 bool batch_shape_pair(int shape);
 bool batch_shape_line(int shape);
+int batch_shape_planes64(int shape);
 int batch_grid(int shape, int nc);
 void launch_sweep_batch(int shape, int nc, const BatchSolve* d_solves, const int2* d_items, int n_items,
                         int* d_ticket, int grid, cudaStream_t st, int pass0, int pass1, int types);

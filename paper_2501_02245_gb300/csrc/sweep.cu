@@ -334,7 +334,9 @@ gsis_status tune_sweep(gsis_ctx* c) {
     c->tuned_Nd = c->Nd;
     if (c->Nd == 0 || c->normal_components == 1) {
         c->sweep_shape = 0;
-        c->sweep_info = c->Nd > 0 && line_alone(c) ? "1D line: window sweep" : "1D or empty: fixed shape";
+        c->sweep_info = line_alone(c) ? "1D line: window sweep"
+                        : line_ok(c) && line_tiles(c, 2) >= 2 * fp64_pipes() ? "1D line: general sweep (tiles uneven over the SMs)"
+                                                                           : "1D or empty: fixed shape";
         return GSIS_OK;
     }
     const std::string key = std::to_string(c->p.vdf_dtype) + "/" + std::to_string(c->normal_components) + "/" +

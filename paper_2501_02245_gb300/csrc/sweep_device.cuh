@@ -399,6 +399,7 @@ struct BatchSolve {
 // A 1D line whose rows are its cells in order (sweep_line.cuh applies).
 bool line_ok(const gsis_ctx* c);
 bool line_alone(const gsis_ctx* c);  // ... and the faster sweep for this solve by itself
-int line_tiles(const gsis_ctx* c);   // warp tiles of its velocity grid
+int line_tiles(const gsis_ctx* c, int planes64);   // warp tiles of its velocity grid (planes64: per FP64 column)
+int fp64_pipes();   // SM sub-partitions of the current device
 
 }  // namespace gsis

@@ -22,16 +22,31 @@ bool line_ok(const gsis_ctx* c) {
 }
 
 static int tiles(const gsis_ctx* c, int zp) { return (c->vg.nx * c->vg.ny + 31) / 32 * ((c->vg.nz + zp - 1) / zp); }
-int line_tiles(const gsis_ctx* c) { return tiles(c, c->p.vdf_dtype == GSIS_F64 ? LINE_ZP64 : LINE_ZP32); }
+int line_tiles(const gsis_ctx* c, int planes64) { return tiles(c, c->p.vdf_dtype == GSIS_F64 ? planes64 : LINE_ZP32); }
 
-// Planes per column of an FP64 line alone, 0 for the general sweep.  Two planes
-// take 15 FP64 operations per point, one plane and the general sweep 18.  A single
-// warp fills only 60 % of its sub-partition's FP64 pipe, so two planes need two
-// warps for each of the 608 sub-partitions; one plane wins while no sub-partition
-// has two warps (30 cells, 1,800 velocities: 74 us against 83); between them
-// the general sweep's five-value loads cost nothing (200 cells, 27,648
-// velocities: 518 us against 622).
-static int line_planes64(const gsis_ctx* c) { return tiles(c, 2) >= 1216 ? 2 : (tiles(c, 1) <= 608 ? 1 : 0); }
+int fp64_pipes() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return 4 * sms;
+}
+
+// Planes per column of an FP64 line alone, 0 for the general sweep.  One plane and the
+// general sweep take 18 FP64 operations per point, two planes 15.  One plane wins while no
+// sub-partition has two warps (30 cells, 1,800 velocities, 63 tiles on 608 sub-partitions:
+// 74 us against 85; 200 cells, 15,360 velocities, 480 tiles: 405 against 476).  With two
+// planes the busiest sub-partition's warps set the time, 0.46 ms for each on 200 cells; the
+// general sweep has twice the tiles and evens out at 0.56 ms for each warp of two planes that a
+// sub-partition would have in the mean.  So two planes are taken where the most is at most 1.2
+// times the mean: 1,296 tiles (3 and 2.1) 1.39 ms against 1.20, 1,728 (3 and 2.8) 1.39
+// against 1.58, 2,304 (4 and 3.8) 1.85 against 2.25, 4,096 (7 and 6.7) 3.22 against 3.71.  Below
+// two warps each the general sweep's five-value loads cost nothing (27,648 velocities: 0.52
+// ms against 0.62).
+static int line_planes64(const gsis_ctx* c) {
+    const int n = tiles(c, 2), pipes = fp64_pipes(), most = (n + pipes - 1) / pipes;
+    if (n >= 2 * pipes) return 5LL * most * pipes <= 6LL * n ? 2 : 0;
+    return tiles(c, 1) <= pipes ? 1 : 0;
+}
 
 bool line_alone(const gsis_ctx* c) {
     return line_ok(c) && (c->p.vdf_dtype != GSIS_F64 || line_planes64(c) > 0);

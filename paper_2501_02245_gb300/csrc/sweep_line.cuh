@@ -110,7 +110,7 @@ __device__ __forceinline__ void line_source(const V4<T>& x, const V4<T>* y, type
 // the y-z entries of its few rows: they come from far (the table is larger than
 // the L2), and in registers one cell ahead was both too late and too many.
 constexpr int LINE_STAGES = 4;
-constexpr int LINE_ZP32 = 4, LINE_ZP64 = 2;   // planes per column (batches)
+constexpr int LINE_ZP32 = 4;   // planes per FP32 column (FP64: one or two)
 // A warp's shared memory: the end cells' boundary inflow (formed before the walk, so
 // that the loop body stays short), and the stages (FP32).
 template <typename T, int ZP>

@@ -14,6 +14,7 @@ CSRC = os.path.join(bench.ROOT, "paper_2501_02245_gb300", "csrc")
 
 @pytest.mark.parametrize("tuning,kernel", [
     ("1D line: window sweep", "k_sweep_line"), ("1D or empty: fixed shape", "k_sweep"),
+    ("1D line: general sweep (tiles uneven over the SMs)", "k_sweep"),
     ("tile col_z2_g12_p16 (autotuned; tile timings (ms per pass pair): g16_v1_c1=7.5)", "k_sweep_col"),
     ("tile planes_wide (cached)", "k_sweep_planes"), ("tile p5_v2_c1 (autotuned; x)", "k_sweep2"),
     ("tile g4_v1_c1 (not tuned: no memory for a snapshot)", "k_sweep"), ("tile ring_w8_v32 (forced)", "k_sweep_ring")])

@@ -48,6 +48,38 @@ def test_fp64_lines_give_the_bits_of_the_general_sweep(name):
     assert all(np.array_equal(a, b) for a, b in zip(*out))
 
 
+@pytest.mark.parametrize("tile", ["line_w4", "line1_w4", "vpt1_cb1_w4"])
+def test_batch_tiles_of_lines_give_the_same_bits(tile):
+    from paper_2501_02245_gb300 import Solver, iterate_batch, batch_info
+    from paper_2501_02245_gb300.gsis import set_batch_tile
+    members = [(CASES[n](), d) for n in ("shock", "walls", "closed") for d in ("f64", "f32")]
+    set_batch_tile(tile)
+    try:
+        batch = [Solver.from_case(c, vdf_dtype=d) for c, d in members]
+        iterate_batch(batch, 3)
+        assert "tile=" + tile + " " in batch_info(batch)
+    finally:
+        set_batch_tile(None)
+    for b, (c, d) in zip(batch, members):
+        s = Solver.from_case(c, vdf_dtype=d)
+        s.iterate(3)
+        assert np.array_equal(b.W(), s.W()), (c.name, d)
+        s.close()
+        b.close()
+
+
+def test_few_fp64_tiles_take_one_plane_and_mixed_lines_are_searched():
+    from paper_2501_02245_gb300 import Solver, iterate_batch, batch_info
+    few, many = _shock(), _shock(12, (48, 40, 20))   # 42 and 1,200 one-plane tiles
+    for members, tile in (([(few, "f64")] * 2, "line1_w4 (default)"), ([(many, "f64")], "line_w4 (default)"),
+                          ([(few, "f32")] * 2, "line_w4 (default)"), ([(few, "f64"), (few, "f32")], "(autotuned)")):
+        batch = [Solver.from_case(c, vdf_dtype=d) for c, d in members]
+        iterate_batch(batch, 1)
+        assert tile in batch_info(batch)
+        for b in batch:
+            b.close()
+
+
 @pytest.mark.parametrize("mixed", [False, True])
 def test_batches_give_the_bits_of_their_members_alone(mixed):
     """mixed: with a 2D member every line runs in the 3-direction kernels."""
