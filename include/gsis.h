@@ -254,8 +254,9 @@ gsis_status gsis_debug_set_region(gsis_ctx* ctx, const uint8_t* flags);
  * Per iteration the per-solve stages run for every solve, the kinetic sweeps
  * of ALL solves run in one persistent launch that draws (solve, velocity
  * tile) work items from a device counter, and the synthetic solves of all
- * meshes up to 4096 cells run in one launch (one CTA each); one iteration of
- * the whole batch is recorded once into a CUDA graph and replayed.  The tile
+ * meshes up to 4096 cells run in one launch per cluster size (one to eight
+ * CTAs for each solve); one iteration of the whole batch is recorded once into
+ * a CUDA graph and replayed.  The tile
  * shape of the persistent sweep is that of 1D lines ("line_w4", or "line1_w4"
  * for few FP64 tiles) if every member is a non-periodic line of kinetic cells
  * and all have FP64 or all FP32 arithmetic, else picked by timing the

@@ -449,7 +449,7 @@ gsis_status tune_batch(BatchPlan* P) {
                                             : "the forced batch tile needs FP32/BF16/FP16 members with an even nx");
     }
     // 1D members whose cells are all kinetic, of one arithmetic: the line sweep, without a search (64 FP32 and
-    // BF16 shocks: 14.5 ms per iteration, 18.8 with the best of the other tiles), FP64 members with one plane per
+    // BF16 shocks: 15.2 ms per iteration, 20.0 with the best of the other tiles), FP64 members with one plane per
     // column while that gives no sub-partition two warps.  FP32 and FP64 lines together take two launches
     // there, one after the other, so they are searched (2 + 2 of 200 cells, 24^3: 1.60 ms, the general sweep 1.05).
     long long one_plane = 0;

@@ -60,7 +60,8 @@ static MacroArgs margs(gsis_ctx* c) {
 // line above Mach 2 or so amplifies a difference in the last bit (1e-15 of the initial
 // state becomes 6e-7 in two GSIS iterations at Mach 5, 1e-4 in ten), so any other rounding
 // of these operations gives another trajectory; twelve sweeps, or cfl = 10, damp it.
-// The bodies' settings do not amplify.  (LINE below: fnd = 1.)
+// The bodies' settings do not amplify.  (LINE below: fnd = 1.  50 pseudo-steps of 200
+// cells take 1.60 ms, 1.48 with the tables.)
 template <bool LINE>
 __device__ __forceinline__ double mu_of(double T, double mu0, double omega) {
     return LINE ? viscosity(T, mu0, omega) : mu0 * exp_tab(omega * log_tab(T));
@@ -472,8 +473,8 @@ __device__ __forceinline__ void face_state(const double* q, const double* w, con
 // stored, the others come from recip64, and the limiter runs on the integer pipe.
 // PAIR: a pair of lanes takes the face (kfvs_pair), each with one side's face state;
 // the rest is formed by both and stored by the even one.  The same values.  For
-// solves that leave sub-partitions idle: 200 cells 1.64 -> 1.48 ms per block of
-// pseudo-steps, 30 cells 0.71 -> 0.66.
+// solves that leave sub-partitions idle: 200 cells 1.72 -> 1.60 ms per block of
+// pseudo-steps, 30 cells 0.85 -> 0.75.
 template <int ND, bool PAIR>
 __device__ __forceinline__ void face_flux_nd(const MacroArgs& a, const double* Wm, const double* gu,
                                              const double* gT, const double* hot, const double* acell,

@@ -293,8 +293,9 @@ __device__ __forceinline__ void unpack_chunk(const S*, uint4 w, float2* v) {
     }
 }
 
-// The same moments in FP32 arithmetic where the x-rows hold whole 16-byte chunks
-// (k_moments otherwise).  What limited k_moments here was the FP64 pipe (the row
+// The same moments in FP32 arithmetic on 2D and 3D meshes where the x-rows hold whole
+// 16-byte chunks (k_moments otherwise; lines keep its order of the FP64 folds, see mu_of
+// in macro.cu).  What limited k_moments here was the FP64 pipe (the row
 // folds, per plane and thread) and the 32 lines of each load.  Two lanes share a
 // row, so that a load takes whole 32-byte sectors; a warp takes 8 rows iy x 4
 // planes iz as two batches of 16 rows (the rows of two planes each), the lanes
@@ -524,9 +525,11 @@ __device__ __forceinline__ void shift_moments13(const double* m, const double d[
 // word for the whole chunk and the update runs in packed pairs, with 64 to 128 bytes
 // in flight (correct_chunks; with the records it reads, 11,643 BF16 cells of 119,808
 // velocities 2.80 -> 1.77 ms, 10,482 of 55,296 1.32 -> 0.91, FP32 1.15 -> 1.06: the
-// hash of the stochastic rounding and the memory bound it now).  All forms compute the same values in the same order
-// (bitwise equal results).  A wall cell adds the correction's outgoing wall sums
-// to those of f^{n+1/2}.
+// hash of the stochastic rounding and the memory bound it now).  In FP32 all forms
+// compute the same values in the same order (bitwise equal results); lines take the
+// five operations in FP64 too and sum their walls in the order of the 16-byte form (mu_of
+// in macro.cu).  A wall cell adds the correction's outgoing wall sums to those of
+// f^{n+1/2}.
 constexpr int CORR_UNROLL = 4;
 constexpr int CORR_VEC_UNROLL = 2;
 

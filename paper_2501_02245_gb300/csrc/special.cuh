@@ -1,5 +1,5 @@
-// Special functions of the synthetic solve's face flux, by table and short
-// polynomial: on GB300 every FP64 instruction of a warp holds its sub-partition's
+// Special functions of the synthetic solve's face flux on 2D and 3D meshes, by table
+// and short polynomial: on GB300 every FP64 instruction of a warp holds its sub-partition's
 // FP64 pipe for 64 cycles, and the library's erf, exp and log spend 45, 17 and
 // 25 of them.
 //  * exp_tab, log_tab: Tang's table-driven method (P. T. P. Tang, ACM TOMS 15

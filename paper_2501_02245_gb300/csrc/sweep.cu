@@ -288,12 +288,12 @@ static std::map<std::string, int>& sweep_cache() {
 
 // Shapes the autotuner times: those that win somewhere.  FP64 on 2D meshes:
 // the columns, and the wide single-velocity blocks for the smallest velocity
-// grids (the reduced distributions' 48 x 48 x 2: col_z2_g12_p16 6.8 ms, g16_v1_c1 7.5,
-// columns of 32 positions 11.6);
+// grids (the reduced distributions' 48 x 48 x 2: col_z2_g12_p16 7.25 ms, g16_v1_c1 7.46,
+// columns of 32 positions 11.7);
 // FP32 arithmetic: the velocity pairs, on one and on two planes, and the widest single-velocity tile, the
 // single-velocity tiles where pairs cannot run.  The shared-memory windows and
 // the remaining tiles measured slower everywhere (cylinder FP64 120 ms against
-// 51.6, FP32 37 against 6.9) and run only when forced.
+// 52.6, FP32 37 against 5.7) and run only when forced.
 static bool tune_candidate(gsis_ctx* c, int shape) {
     const int nb = base_shapes(c->p.vdf_dtype);
     if (shape >= nb + kRingShapes) return col_ok(c) || planes_ok(c);

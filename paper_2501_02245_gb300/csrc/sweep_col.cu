@@ -23,8 +23,9 @@
 // per velocity (k_sweep) costs 30.  Measured on the 128 x 128 cylinder, 48 x
 // 48 x 24 velocities, 10,482 DVM cells, ms per pass pair: lane per velocity
 // 81.8 (97.9 before the limiter's absolute values left the FP64 pipe, see
-// mag_bits), columns of two planes 64.6, of three 55.8, of four 51.6 at three
-// blocks per SM (68.7 at two, where 432 blocks take two waves).
+// mag_bits), columns of two planes 70.2, of three 57.6, of four 52.6 at three
+// blocks per SM (at two, 432 blocks take two waves); 51.6 with the outflow
+// term first whichever side is low, which rounds differently.
 // FP32 arithmetic gains nothing here (7.1 ms against 6.9 for the velocity
 // pairs: it waits for loads, not for arithmetic) and keeps its own tiles.
 #include "sweep_device.cuh"
@@ -223,9 +224,9 @@ __device__ __forceinline__ void column_apply(const SweepArgs& a, int k, const Ce
 // A block owns P (ix, iy) positions x ZP planes; its G warps split the cells
 // of each hyperplane, 32 / P cells to a warp.  P = 16 serves small velocity grids,
 // whose blocks of 32 positions would leave SMs idle: the reduced grid of 48 x 48 x 2
-// on the same cylinder takes 6.8 ms with 144 blocks of 12 warps, 11.6 with 72 blocks
-// of 32 positions, 7.5 with a lane per velocity in 144 blocks of 16 warps (32 x 32 x 2:
-// 6.6, 11.6, 7.4); 8 and 16 warps take 7.6 and 7.1.  The sweep data of a warp's next cell (also across the
+// on the same cylinder takes 7.25 ms with 144 blocks of 12 warps, 11.7 with 72 blocks
+// of 32 positions, 7.46 with a lane per velocity in 144 blocks of 16 warps (32 x 32 x 2:
+// 6.9, 11.7, 7.4).  The sweep data of a warp's next cell (also across the
 // barrier: it does not change during the pass) is loaded before the current
 // cell is updated.  MINB: blocks per SM the registers are capped for.
 template <int ZP, int G, int MINB, int P>

@@ -1,4 +1,5 @@
 // Single-solve launch of the 1D line sweep (sweep_line.cuh): one warp per tile.
+#include <algorithm>
 #include "sweep_line.cuh"
 
 namespace gsis {
@@ -28,7 +29,7 @@ int fp64_pipes() {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return 4 * sms;
+    return 4 * std::max(1, sms);
 }
 
 // Planes per column of an FP64 line alone, 0 for the general sweep.  One plane and the

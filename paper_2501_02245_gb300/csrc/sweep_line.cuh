@@ -18,8 +18,8 @@
 // instructions (they share every coefficient); FP64: bound by the FP64 pipe, 11
 // operations per point plus 6 / ZP shared ones against 23.
 // Per iteration: a batch of 64 shocks of 100 to 800 cells, 24^3 to 64^3 velocities,
-// FP32 and BF16: 18.8 ms with the general sweep's best tile, 14.5 with this one; 30
-// FP64 cells of 1,800 velocities alone 85 us -> 74.
+// FP32 and BF16: 20.0 ms with the general sweep's best tile, 15.2 with this one; 30
+// FP64 cells of 1,800 velocities alone 85 us -> 75.
 #pragma once
 #include <type_traits>
 #include "sweep_pair.cuh"

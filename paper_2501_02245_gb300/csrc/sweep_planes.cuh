@@ -23,9 +23,9 @@
 //   the next cell's stencil or factors as well needs registers that cost more
 //   warps than it hides (2D FP32 cylinder 8.5 to 10 ms, 7.9 with the factors).
 // Per pass pair, best of sweep_pair.cuh's tiles against this one:
-//   10,482 kinetic cells, 48 x 48 x 24 velocities (cylinder): FP32 6.75 -> 5.9 ms, BF16 6.78 ->
-//   6.1, FP16 6.58 -> 5.6;
-//   11,643 kinetic cells, 48 x 52 x 48 (sphere): BF16 30.2 -> 21.2 ms, FP32 29.9 -> 20.3.
+//   10,499 kinetic cells, 48 x 48 x 24 velocities (cylinder): FP32 7.25 -> 5.7 ms, BF16 6.84 ->
+//   6.05, FP16 6.72 -> 5.8;
+//   11,643 kinetic cells, 48 x 48 x 48 (sphere): BF16 31.4 -> 21.4 ms, FP32 31.2 -> 21.0.
 #pragma once
 #include "sweep_pair.cuh"
 
@@ -334,8 +334,8 @@ static void launch_planes_t(gsis_ctx* c, const SweepArgs& a, int pass) {
 // 2D: 128 registers, 15 warps per SM (four warps of 168 registers, 12 per SM, were 3 %
 // slower on the FP32 cylinder); 3D: 168 registers, 12 warps per SM (five warps, 10 per
 // SM: 17 % slower on the BF16 sphere).  Shape 1 has wider blocks for velocity grids with
-// few tiles: 36 x 38 x 17 on 4,271 cells FP32 1.73 ms (2.07 with shape 0, 2.27 with the best
-// pair tile), 32^3 on the sphere BF16 7.2 (8.5, 10.1).
+// few tiles: 36 x 38 x 17 on 4,335 cells FP32 1.74 ms (2.09 with shape 0, 2.26 with the best
+// pair tile), 32^3 on the sphere BF16 7.1 (8.9, 10.3).
 template <typename S>
 static void launch_planes(gsis_ctx* c, const SweepArgs& a, int pass, int shape) {
     if (shape == 1) {
